@@ -588,8 +588,8 @@ static lbm_status fields_to_device(lbm_ctx* c, double* rho, double* vx, double* 
     const size_t B = c->N * sizeof(double);
     if (!is_fp64(c)) {
         CK(launch_macro_mixed((const float*)c->f[c->cur], c->m_rh, c->m_rl, c->m_Fx, c->m_Fy,
-                              rho, vx, vy, c->nx, c->ny, c->plane, c->stream));
-        if (mu) CK(launch_f_to_double<float>(c->m_dxx, mu, c->N, c->stream));  // holds mu-hat
+                              c->m_dxx /* holds mu-hat */, rho, vx, vy, mu, c->nx, c->ny,
+                              c->plane, c->stream));
         return LBM_OK;
     }
     if (vx || vy) {

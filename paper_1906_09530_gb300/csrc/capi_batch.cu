@@ -591,11 +591,10 @@ lbm_status lbm_batch_fields(lbm_batch* b, int32_t i, double* h_rho, double* h_vx
     CK(cudaSetDevice(b->dev));
     double* sg = (double*)h.f[1 - b->cur];  // idle buffer: >= 4 N doubles
     const size_t N = h.N;
-    if (h_rho || h_vx || h_vy)
-        CK(launch_macro_mixed(h.f[b->cur], h.rh, h.rl, h.Fx, h.Fy, h_rho ? sg : nullptr,
-                              h_vx ? sg + N : nullptr, h_vy ? sg + 2 * N : nullptr, h.nx, h.ny,
-                              h.plane, b->stream));
-    if (h_mu) CK(launch_f_to_double<float>(h.dxx, sg + 3 * N, N, b->stream));  // mu-hat
+    CK(launch_macro_mixed(h.f[b->cur], h.rh, h.rl, h.Fx, h.Fy, h.dxx /* holds mu-hat */,
+                          h_rho ? sg : nullptr, h_vx ? sg + N : nullptr,
+                          h_vy ? sg + 2 * N : nullptr, h_mu ? sg + 3 * N : nullptr, h.nx, h.ny,
+                          h.plane, b->stream));
     lbm_status st = wait_stream(b);
     if (st) return st;
     const size_t B = N * sizeof(double);

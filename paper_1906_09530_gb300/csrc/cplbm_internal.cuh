@@ -136,8 +136,9 @@ cudaError_t launch_init_mixed(const double* rho, const double* ux, const double*
 cudaError_t launch_rho_from_f_mixed(const float* f, float* rh, float* rl, int nx, int ny,
                                     size_t plane, cudaStream_t s);
 cudaError_t launch_macro_mixed(const float* f, const float* rh, const float* rl,
-                               const float* Fx, const float* Fy, double* rho, double* vx,
-                               double* vy, int nx, int ny, size_t plane, cudaStream_t s);
+                               const float* Fx, const float* Fy, const float* mu, double* rho,
+                               double* vx, double* vy, double* mu_out, int nx, int ny,
+                               size_t plane, cudaStream_t s);
 cudaError_t launch_diag_mixed(const float* f, const float* rh, const float* rl, const float* Fx,
                               const float* Fy, int nx, int ny, size_t plane, double* partials,
                               int nparts, DevState* st, cudaStream_t s);

@@ -67,5 +67,45 @@ __device__ __forceinline__ df sum9_exact(const float g[9]) {
     return quick_two_sum(s, e);
 }
 
+// A float as a double, by integer operations: the conversion instruction runs on the
+// FP64 pipe (2 lanes a clock and SM).  Zeros and subnormals, infinities and NaN take it.
+__device__ __forceinline__ double widen(float x) {
+    const unsigned u = __float_as_uint(x), e = u & 0x7fffffffu;
+    if (e - 0x00800000u >= 0x7f000000u) return e == 0 ? __hiloint2double((int)u, 0) : (double)x;
+    return __hiloint2double((int)((u & 0x80000000u) | ((e >> 3) + 0x38000000u)), (int)(u << 29));
+}
+
+// Unevaluated sum of three floats: about 72 significant bits, more than a double's 53.
+struct tf {
+    float a, b, c;
+};
+__device__ __forceinline__ void tf_add(tf& s, float x) {
+    const df h = two_sum(s.a, x), l = two_sum(s.b, h.lo);
+    s.a = h.hi;
+    s.b = l.hi;
+    s.c = __fadd_rn(s.c, l.lo);
+}
+// n / r to about 68 bits, rounded once to double: three quotient digits of one float
+// each, the remainder after the first kept as hi + lo.  inv: 1 / r.hi to a float's
+// accuracy.  Finite n and finite r with r.hi > 0.
+__device__ __forceinline__ double tf_div(tf n, df r, float inv) {
+    df s = quick_two_sum(n.a, n.b);  // normalised: the head holds a float's accuracy
+    const float q0 = __fmul_rn(s.hi, inv);
+    const float p = __fmul_rn(q0, r.hi), t = __fmul_rn(q0, r.lo);
+    float lo = __fsub_rn(n.c, fmaf(q0, r.lo, -t));
+    df m = two_sum(__fsub_rn(s.hi, p), -fmaf(q0, r.hi, -p));
+    lo = __fadd_rn(lo, m.lo);
+    m = two_sum(m.hi, s.lo);
+    lo = __fadd_rn(lo, m.lo);
+    m = two_sum(m.hi, -t);
+    lo = __fadd_rn(lo, m.lo);
+    const float q1 = __fmul_rn(__fadd_rn(m.hi, lo), inv);
+    const float p1 = __fmul_rn(q1, r.hi);
+    float rem = __fsub_rn(m.hi, p1);
+    rem = __fsub_rn(rem, fmaf(q1, r.hi, -p1));
+    rem = __fadd_rn(rem, fmaf(-q1, r.lo, lo));
+    const float q2 = __fmul_rn(rem, inv);
+    return __dadd_rn(widen(q0), __dadd_rn(widen(q1), widen(q2)));
+}
 
 }  // namespace cplbm

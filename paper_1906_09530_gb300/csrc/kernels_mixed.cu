@@ -352,22 +352,54 @@ __global__ void k_rho_from_f_mixed(const float* __restrict__ f, float* __restric
     }
 }
 
-// FP64 outputs of the mixed state: rho = hi + lo, v = u + F/(2 rho), mu-hat.
+// The velocity v = u + F/(2 rho) of a mixed node in FP64: the momentum's seven float
+// terms and the quotient are carried as triple-floats on the FP32 pipe and each component
+// is rounded once.  GB300 has 2 FP64 lanes a clock and SM; in FP64 arithmetic (13
+// conversions, 14 sums, 2 divisions) the fields of a 1024^2 grid took 108 us, of which its
+// 84 bytes a node are 13.  Here 5 sums a node are left on that
+// pipe: 4096^2 took 1335 us and takes 258 (5.5 TB/s of its 84 bytes a node).
+__device__ __forceinline__ void velocity_mixed(const float (&g)[9], df r, float fx, float fy,
+                                               double& vx, double& vy) {
+    tf jx{g[1], 0.0f, 0.0f}, jy{g[2], 0.0f, 0.0f};
+    tf_add(jx, -g[3]);
+    tf_add(jy, -g[4]);
+    tf_add(jx, g[5]);
+    tf_add(jy, g[5]);
+    tf_add(jx, -g[6]);
+    tf_add(jy, g[6]);
+    tf_add(jx, -g[7]);
+    tf_add(jy, -g[7]);
+    tf_add(jx, g[8]);
+    tf_add(jy, -g[8]);
+    tf_add(jx, __fmul_rn(0.5f, fx));
+    tf_add(jy, __fmul_rn(0.5f, fy));
+    const float inv = __frcp_rn(r.hi);
+    vx = tf_div(jx, r, inv);
+    vy = tf_div(jy, r, inv);
+}
+
+// FP64 outputs of the mixed state: rho = hi + lo, v = u + F/(2 rho), mu-hat; each output
+// may be null (vx and vy together).
 __global__ void k_macro_mixed(const float* __restrict__ f, const float* __restrict__ rh,
                               const float* __restrict__ rl, const float* __restrict__ Fx,
-                              const float* __restrict__ Fy, double* rho_o, double* vx, double* vy,
-                              size_t N, size_t plane) {
+                              const float* __restrict__ Fy, const float* __restrict__ mu,
+                              double* rho_o, double* vx, double* vy, double* mu_o, size_t N,
+                              size_t plane) {
     for (size_t n = blockIdx.x * (size_t)blockDim.x + threadIdx.x; n < N;
          n += (size_t)gridDim.x * blockDim.x) {
-        double g[9];
+        const df r{rh[n], rl[n]};
+        const float m = mu_o ? mu[n] : 0.0f;
+        if (vx || vy) {
+            float g[9];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) g[i] = (double)f[i * plane + n];
-        const double r = (double)rh[n] + (double)rl[n];
-        const double jx = (g[1] + g[5] + g[8]) - (g[3] + g[6] + g[7]);
-        const double jy = (g[2] + g[5] + g[6]) - (g[4] + g[7] + g[8]);
-        if (rho_o) rho_o[n] = r;
-        if (vx) vx[n] = (jx + 0.5 * (double)Fx[n]) / r;
-        if (vy) vy[n] = (jy + 0.5 * (double)Fy[n]) / r;
+            for (int i = 1; i < 9; ++i) g[i] = f[i * plane + n];
+            double u, v;
+            velocity_mixed(g, r, Fx[n], Fy[n], u, v);
+            if (vx) vx[n] = u;
+            if (vy) vy[n] = v;
+        }
+        if (rho_o) rho_o[n] = __dadd_rn(widen(r.hi), widen(r.lo));
+        if (mu_o) mu_o[n] = widen(m);
     }
 }
 
@@ -429,21 +461,21 @@ __global__ void __launch_bounds__(kDiagT)
     double s = 0.0, vmax = 0.0, rmin = DBL_MAX, rmax = -DBL_MAX;
     for (size_t n = blockIdx.x * (size_t)blockDim.x + threadIdx.x; n < N;
          n += (size_t)gridDim.x * blockDim.x) {
-        double g[9];
+        float g[9];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) g[i] = (double)f[i * plane + n];
-        const double r = (double)rh[n] + (double)rl[n];
-        const double jx = (g[1] + g[5] + g[8]) - (g[3] + g[6] + g[7]);
-        const double jy = (g[2] + g[5] + g[6]) - (g[4] + g[7] + g[8]);
-        const double u = (jx + 0.5 * (double)Fx[n]) / r, v = (jy + 0.5 * (double)Fy[n]) / r;
+        for (int i = 1; i < 9; ++i) g[i] = f[i * plane + n];
+        const df rd{rh[n], rl[n]};
+        double u, v;
+        velocity_mixed(g, rd, Fx[n], Fy[n], u, v);
+        const double r = __dadd_rn(widen(rd.hi), widen(rd.lo));
         s += r;
-        vmax = fmax(vmax, sqrt(u * u + v * v));
+        vmax = fmax(vmax, u * u + v * v);  // the square: one root a thread
         rmin = fmin(rmin, r);
         rmax = fmax(rmax, r);
     }
     __shared__ double sh[4][kDiagT];
     sh[0][threadIdx.x] = s;
-    sh[1][threadIdx.x] = vmax;
+    sh[1][threadIdx.x] = sqrt(vmax);
     sh[2][threadIdx.x] = rmin;
     sh[3][threadIdx.x] = rmax;
     __syncthreads();
@@ -578,10 +610,12 @@ cudaError_t launch_rho_from_f_mixed(const float* f, float* rh, float* rl, int nx
 }
 
 cudaError_t launch_macro_mixed(const float* f, const float* rh, const float* rl,
-                               const float* Fx, const float* Fy, double* rho, double* vx,
-                               double* vy, int nx, int ny, size_t plane, cudaStream_t s) {
+                               const float* Fx, const float* Fy, const float* mu, double* rho,
+                               double* vx, double* vy, double* mu_out, int nx, int ny,
+                               size_t plane, cudaStream_t s) {
     const size_t N = (size_t)nx * ny;
-    k_macro_mixed<<<grid_for(N, 256), 256, 0, s>>>(f, rh, rl, Fx, Fy, rho, vx, vy, N, plane);
+    k_macro_mixed<<<grid_for(N, 256), 256, 0, s>>>(f, rh, rl, Fx, Fy, mu, rho, vx, vy, mu_out, N,
+                                                   plane);
     return cudaGetLastError();
 }
 
