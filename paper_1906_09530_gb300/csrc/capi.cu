@@ -3,11 +3,12 @@
 // error flag and bounded waits.
 //
 // FP64 path: one time step is five device passes (all on the caller's stream):
-//   1 collide-stream      f^t, F^t           -> f^{t+1}, rho^{t+1}      Eqs. 1-5
-//   2 x-lines of rho      rho                -> d_x rho, d_xx rho       Eqs. 37-39
+//   1 collide-stream      f^t, rho^t, F^t    -> f^{t+1}                 Eqs. 1, 2, 5
+//   2 x-lines of rho      f^{t+1}            -> rho, d_x rho, d_xx rho  Eqs. 3, 37-39
 //   3 y-lines of rho      rho, d_xx rho      -> d_y rho, mu-hat         Eqs. 21, 33, Sec. 5.6
 //   4 x-lines of mu-hat   mu, rho, d_x rho   -> F_x                     Eq. 12
 //   5 y-lines of mu-hat   mu, rho, d_y rho   -> F_y                     Eq. 12
+// with passes 4 and 5 in one launch (two when each is timed).
 // Mixed path: four passes -- collide-stream; the x- and y-lines of rho in one
 // launch (d_x, d_xx, d_y, d_yy rho); mu-hat pointwise (stored over d_xx rho);
 // the x- and y-lines of mu-hat in one launch with the force epilogue.
@@ -127,8 +128,9 @@ lbm_status use_dev(lbm_ctx* c) {
     return LBM_OK;
 }
 
-// Passes 2-5 on the current density.  `timed` records an event after each.
-lbm_status enqueue_force(lbm_ctx* c, cudaStream_t s, int bump, cudaEvent_t* ev = nullptr) {
+// Passes 2-5 on the density of f[fcur].  `ev` records an event after each.
+lbm_status enqueue_force(lbm_ctx* c, cudaStream_t s, int bump, int fcur,
+                         cudaEvent_t* ev = nullptr) {
     const int nx = c->nx, ny = c->ny, o = c->fd_order;
     launch_pdl_on() = c->pdl_now;
     auto mark = [&](int i) { return ev ? cudaEventRecord(ev[i], s) : cudaSuccess; };
@@ -149,15 +151,21 @@ lbm_status enqueue_force(lbm_ctx* c, cudaStream_t s, int bump, cudaEvent_t* ev =
         CK(mark(3));
         return LBM_OK;
     }
-    CK(lines_fp64_rho_x(c->rho, c->dxr, c->dxx, nx, ny, o, c->dst, bump, s));
+    CK(lines_fp64_rho_x((const double*)c->f[fcur], c->plane, c->rho, c->dxr, c->dxx, nx, ny, o,
+                        c->dst, bump, s));
     CK(mark(0));
     CK(lines_fp64_rho_y_mu(c->rho, c->dxx, c->dyr, c->mu, nx, ny, o, c->phys, c->dst, s,
                            c->walls_y));
     CK(mark(1));
-    CK(lines_fp64_force(c->mu, c->rho, c->dxr, c->Fx, nx, ny, 0, o, s));
-    CK(mark(2));
-    CK(lines_fp64_force(c->mu, c->rho, c->dyr, c->Fy, nx, ny, 1, o, s, c->walls_y));
-    CK(mark(3));
+    if (ev) {
+        CK(lines_fp64_force(c->mu, c->rho, c->dxr, nullptr, c->Fx, nullptr, nx, ny, o, s));
+        CK(mark(2));
+        CK(lines_fp64_force(c->mu, c->rho, nullptr, c->dyr, nullptr, c->Fy, nx, ny, o, s,
+                            c->walls_y));
+        CK(mark(3));
+        return LBM_OK;
+    }
+    CK(lines_fp64_force(c->mu, c->rho, c->dxr, c->dyr, c->Fx, c->Fy, nx, ny, o, s, c->walls_y));
     return LBM_OK;
 }
 
@@ -166,10 +174,9 @@ lbm_status enqueue_collide(lbm_ctx* c, cudaStream_t s, int from) {
     const int to = 1 - from;
     launch_pdl_on() = c->pdl_now;
     if (is_fp64(c))
-        CK(launch_collide_stream<double>((const double*)c->f[from], (double*)c->f[to], c->Fx,
-                                         c->Fy, c->rho, c->nx, c->ny, c->plane,
-                                         c->phys.omega, c->mrt ? &c->rates : nullptr, c->dst,
-                                         s, c->walls));
+        CK(launch_collide_stream((const double*)c->f[from], (double*)c->f[to], c->Fx, c->Fy,
+                                 c->rho, c->nx, c->ny, c->plane, c->phys.omega,
+                                 c->mrt ? &c->rates : nullptr, c->dst, s, c->walls));
     else
         CK(launch_cs_mixed((const float*)c->f[from], (float*)c->f[to], c->m_Fx, c->m_Fy,
                            c->m_rh, c->m_rl, c->nx, c->ny, c->plane, c->phys.omega,
@@ -181,7 +188,7 @@ lbm_status enqueue_collide(lbm_ctx* c, cudaStream_t s, int from) {
 lbm_status enqueue_step(lbm_ctx* c, cudaStream_t s, int from) {
     lbm_status st = enqueue_collide(c, s, from);
     if (st) return st;
-    return enqueue_force(c, s, 1);
+    return enqueue_force(c, s, 1, 1 - from);
 }
 
 // Steps in the long graph: even, so a replay ends on the buffer it started from.
@@ -479,12 +486,11 @@ static lbm_status init_from_device_fields(lbm_ctx* c, const double* rho, const d
     lbm_status st = reset_state(c, 0);
     if (st) return st;
     if (is_fp64(c))
-        CK(launch_init_feq<double>(rho, ux, uy, (double*)c->f[0], c->rho, c->nx, c->ny,
-                                   c->plane, c->stream));
+        CK(launch_init_feq(rho, ux, uy, (double*)c->f[0], c->nx, c->ny, c->plane, c->stream));
     else
         CK(launch_init_mixed(rho, ux, uy, (float*)c->f[0], c->m_rh, c->m_rl, c->nx, c->ny,
                              c->plane, c->stream));
-    st = enqueue_force(c, c->stream, 0);
+    st = enqueue_force(c, c->stream, 0, c->cur);
     if (st) return st;
     c->ready = true;
     return LBM_OK;
@@ -573,7 +579,7 @@ lbm_status lbm_step_timed(lbm_ctx* c, float* pass_ms) {
     st = enqueue_collide(c, s, from);
     if (st) return st;
     CK(cudaEventRecord(c->tev[1], s));
-    st = enqueue_force(c, s, 1, c->tev + 2);
+    st = enqueue_force(c, s, 1, to, c->tev + 2);
     if (st) return st;
     c->cur = to;
     c->t += 1;
@@ -593,8 +599,8 @@ static lbm_status fields_to_device(lbm_ctx* c, double* rho, double* vx, double* 
         return LBM_OK;
     }
     if (vx || vy) {
-        CK(launch_macro<double>((const double*)c->f[c->cur], c->Fx, c->Fy, vx, vy, c->nx,
-                                c->ny, c->plane, c->stream));
+        CK(launch_macro((const double*)c->f[c->cur], c->rho, c->Fx, c->Fy, vx, vy, c->nx, c->ny,
+                        c->plane, c->stream));
     }
     if (rho) CK(cudaMemcpyAsync(rho, c->rho, B, cudaMemcpyDeviceToDevice, c->stream));
     if (mu) CK(cudaMemcpyAsync(mu, c->mu, B, cudaMemcpyDeviceToDevice, c->stream));
@@ -643,7 +649,7 @@ lbm_status lbm_get_populations(lbm_ctx* c, double* h_f, int64_t* t) {
             CK(cudaMemcpyAsync(sg, (const double*)c->f[c->cur] + i * c->plane, B,
                                cudaMemcpyDeviceToDevice, c->stream));
         else
-            CK(launch_f_to_double<float>((const float*)c->f[c->cur] + i * c->plane, sg, c->N,
+            CK(launch_f_to_double((const float*)c->f[c->cur] + i * c->plane, sg, c->N,
                                          c->stream));
         st = wait_stream(c);
         if (st) return st;
@@ -670,19 +676,16 @@ lbm_status lbm_set_populations(lbm_ctx* c, const double* h_f, int64_t t) {
             CK(cudaMemcpyAsync((double*)c->f[0] + i * c->plane, sg, B, cudaMemcpyDeviceToDevice,
                                c->stream));
         else
-            CK(launch_f_from_double<float>(sg, (float*)c->f[0] + i * c->plane, c->N, c->stream));
+            CK(launch_f_from_double(sg, (float*)c->f[0] + i * c->plane, c->N, c->stream));
         st = wait_stream(c);
         if (st) return st;
     }
     st = reset_state(c, t);
     if (st) return st;
-    if (is_fp64(c))
-        CK(launch_rho_from_f<double>((const double*)c->f[0], c->rho, c->nx, c->ny, c->plane,
-                                     c->stream));
-    else
+    if (!is_fp64(c))  // (the FP64 path's x-lines take the density from the populations)
         CK(launch_rho_from_f_mixed((const float*)c->f[0], c->m_rh, c->m_rl, c->nx, c->ny,
                                    c->plane, c->stream));
-    st = enqueue_force(c, c->stream, 0);
+    st = enqueue_force(c, c->stream, 0, c->cur);
     if (st) return st;
     c->ready = true;
     return read_state(c);
@@ -698,7 +701,7 @@ lbm_status cplbm_diag_with_partials(lbm_ctx* c, double* partials, int nparts, do
     lbm_status st = use_dev(c);
     if (st) return st;
     if (is_fp64(c))
-        CK(launch_diag<double>((const double*)c->f[c->cur], c->rho, c->Fx, c->Fy, c->nx, c->ny,
+        CK(launch_diag((const double*)c->f[c->cur], c->rho, c->Fx, c->Fy, c->nx, c->ny,
                                c->plane, partials, nparts, c->dst, c->stream));
     else
         CK(launch_diag_mixed((const float*)c->f[c->cur], c->m_rh, c->m_rl, c->m_Fx, c->m_Fy,

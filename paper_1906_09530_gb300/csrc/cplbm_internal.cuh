@@ -87,35 +87,22 @@ struct Walls {
     double u[2] = {0.0, 0.0};
 };
 
-// Launchers (all asynchronous on `s`).  Fields are FP64 [ny][nx]; populations
-// are [9][plane] of TF with plane >= nx*ny.
-template <typename TF>
-cudaError_t launch_collide_stream(const TF* fin, TF* fout, const double* Fx, const double* Fy,
-                                  double* rho_out, int nx, int ny, size_t plane, double omega,
-                                  const MrtRates* mrt, DevState* st, cudaStream_t s,
-                                  const Walls& walls = Walls());
-
-template <typename TF>
-cudaError_t launch_init_feq(const double* rho, const double* ux, const double* uy, TF* f,
-                            double* rho_out, int nx, int ny, size_t plane, cudaStream_t s);
-
-template <typename TF>
-cudaError_t launch_rho_from_f(const TF* f, double* rho, int nx, int ny, size_t plane,
-                              cudaStream_t s);
-
-template <typename TF>
-cudaError_t launch_macro(const TF* f, const double* Fx, const double* Fy, double* vx,
-                         double* vy, int nx, int ny, size_t plane, cudaStream_t s);
-
-template <typename TF>
-cudaError_t launch_diag(const TF* f, const double* rho, const double* Fx, const double* Fy,
+// Launchers (all asynchronous on `s`).  FP64 path: fields are [ny][nx], populations
+// [9][plane] with plane >= nx*ny.
+cudaError_t launch_collide_stream(const double* fin, double* fout, const double* Fx,
+                                  const double* Fy, const double* rho, int nx, int ny,
+                                  size_t plane, double omega, const MrtRates* mrt, DevState* st,
+                                  cudaStream_t s, const Walls& walls = Walls());
+cudaError_t launch_init_feq(const double* rho, const double* ux, const double* uy, double* f,
+                            int nx, int ny, size_t plane, cudaStream_t s);
+cudaError_t launch_macro(const double* f, const double* rho, const double* Fx, const double* Fy,
+                         double* vx, double* vy, int nx, int ny, size_t plane, cudaStream_t s);
+cudaError_t launch_diag(const double* f, const double* rho, const double* Fx, const double* Fy,
                         int nx, int ny, size_t plane, double* partials, int nparts,
                         DevState* st, cudaStream_t s);
-
-template <typename TF>
-cudaError_t launch_f_to_double(const TF* f, double* out, size_t n, cudaStream_t s);
-template <typename TF>
-cudaError_t launch_f_from_double(const double* in, TF* f, size_t n, cudaStream_t s);
+// FP32 populations <-> FP64 host layout
+cudaError_t launch_f_to_double(const float* f, double* out, size_t n, cudaStream_t s);
+cudaError_t launch_f_from_double(const double* in, float* f, size_t n, cudaStream_t s);
 
 cudaError_t launch_diag_final(const double* partials, int nparts, DevState* st, cudaStream_t s);
 
@@ -256,19 +243,20 @@ cudaError_t lines_batch_launch(LineBatchKind kind, const void* d_desc, const int
 // above it, in double-float wherever a window spans more than a factor 32.
 constexpr double kDfRatio = 1e4;
 
-// Warp-cooperative compact-FD line solves (kernels_lines.cu).  With walls_y the
-// y-lines are extended evenly about both walls (a periodic line of period
-// 2 ny, the first ghost equal to its fluid neighbour, Sec. 5.5).  axis 0: lines
-// along x, 1: along y.  Passes 2-5 of the FP64 path and of the mixed path, and
-// the stand-alone derivatives.
-cudaError_t lines_fp64_rho_x(const double* rho, double* dxr, double* dxx, int nx, int ny,
-                             int order, DevState* st, int bump, cudaStream_t s);
-cudaError_t lines_fp64_rho_y_mu(const double* rho, const double* dxx, double* dyr, double* mu,
+// Compact-FD line solves.  With walls_y the y-lines are extended evenly about both
+// walls (a periodic line of period 2 ny, the first ghost equal to its fluid neighbour,
+// Sec. 5.5).  axis 0: lines along x, 1: along y.
+// FP64 path (lines64.cu).  z: a derivative without its factor c1 (c1^2 for a second one).
+// The x-lines take the density as the sum of the populations and store it.
+cudaError_t lines_fp64_rho_x(const double* f, size_t plane, double* rho, double* zx, double* zxx,
+                             int nx, int ny, int order, DevState* st, int bump, cudaStream_t s);
+cudaError_t lines_fp64_rho_y_mu(const double* rho, const double* zxx, double* zy, double* mu,
                                 int nx, int ny, int order, const PhysParams& p, DevState* st,
                                 cudaStream_t s, bool walls_y = false);
-cudaError_t lines_fp64_force(const double* mu, const double* rho, const double* dr, double* F,
-                             int nx, int ny, int axis, int order, cudaStream_t s,
-                             bool walls_y = false);
+// the x- and y-lines of mu-hat in one launch; zx or zy null: the other direction alone
+cudaError_t lines_fp64_force(const double* mu, const double* rho, const double* zx,
+                             const double* zy, double* Fx, double* Fy, int nx, int ny, int order,
+                             cudaStream_t s, bool walls_y = false);
 cudaError_t lines_fp64_plain(const double* u, double* d1, double* d2, int nx, int ny, int axis,
                              int order, cudaStream_t s);
 // Mixed path, merged launches: the x- and y-lines of rho together (first and

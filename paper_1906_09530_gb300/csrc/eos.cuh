@@ -12,23 +12,29 @@
 
 namespace cplbm {
 
-__device__ __forceinline__ float rn_log(float x) { return logf(x); }
-__device__ __forceinline__ double rn_log(double x) { return log(x); }
+// Logarithm and division of the FP32 evaluation.
+struct MathF {
+    __device__ __forceinline__ float log(float x) const { return logf(x); }
+    __device__ __forceinline__ float div(float a, float b) const { return rn_div(a, b); }
+    __device__ __forceinline__ bool pos(float x) const { return x > 0.0f; }
+};
 
-template <class T>
-__device__ __forceinline__ T eos_mu0(const EosC<T>& e, T r, bool& bad) {
+template <class T, class Math>
+__device__ __forceinline__ T eos_mu0(const EosC<T>& e, T r, bool& bad, const Math& M) {
+    auto rn_log = [&](T x) { return M.log(x); };
+    auto rn_div = [&](T a, T b) { return M.div(a, b); };
     if (e.kind == LBM_EOS_CS) {
         const T eta = rn_mul(e.b, r);  // e.b holds b/4
         const T om = rn_sub(T(1), eta);
         const T z = rn_add(rn_add(rn_div(rn_sub(T(3), eta), rn_mul(rn_mul(om, om), om)),
                                   rn_log(r)),
                            T(1));
-        bad |= !(r > T(0) && eta < T(1));
+        bad |= !(M.pos(r) && M.pos(om));
         return rn_fma(e.rt, z, -rn_mul(e.a2, r));
     }
     const T br = rn_mul(e.b, r);
     const T om = rn_sub(T(1), br);
-    bad |= !(r > T(0) && om > T(0));
+    bad |= !(M.pos(r) && M.pos(om));
     const T lr = rn_log(rn_div(r, om));  // ln(rho / (1 - b rho))
     const T inv = rn_div(T(1), om);      // 1 / (1 - b rho)
     if (e.kind == LBM_EOS_VDW) return rn_fma(e.rt, rn_add(lr, inv), -rn_mul(e.a2, r));
@@ -62,7 +68,7 @@ __device__ __forceinline__ bool eos_at_pole(const EosC<T>& e, T r) {
 __device__ __forceinline__ float mu_node(float r, float xx, float yy, const MuConstF& p,
                                          bool capped, bool& bad) {
     bool b0 = false;
-    const float mu0 = eos_mu0(p.e, r, b0);
+    const float mu0 = eos_mu0(p.e, r, b0, MathF());
     float m = rn_fma(p.k2, mu0, -rn_mul(p.kappa, rn_add(xx, yy)));
     if (capped) {
         if (eos_at_pole(p.e, r)) {  // mu0 = +infinity: the limit takes the node

@@ -1,44 +1,24 @@
-// kernels_lbm.cu -- lattice kernels: fused collide-stream (Eqs. 1-5),
-// equilibrium initialisation, moments, output velocity and diagnostics.
+// kernels_lbm.cu -- lattice kernels of the FP64 path: collide-stream (Eqs. 1, 2, 5),
+// equilibrium initialisation, output velocity and diagnostics.
 //
 // Populations are structure-of-arrays, f[i*plane + y*nx + x], i in the velocity
-// order of Sec. 2.  TF is the storage and arithmetic type of the populations:
-// double (FP64 path) or float (mixed path).  The density and force fields are
-// always FP64.
+// order of Sec. 2.
 #include <cfloat>
 #include <climits>
 
 #include "cplbm_internal.cuh"
+#include "fp64_math.cuh"
 #include "lattice.cuh"
 
 namespace cplbm {
 namespace {
 
-// D2Q9 velocity set and weights (Sec. 2).  Called with compile-time i inside
-// fully unrolled loops, so they fold to constants.
-__host__ __device__ __forceinline__ constexpr int ex(int i) {
-    return (i == 1 || i == 5 || i == 8) ? 1 : ((i == 3 || i == 6 || i == 7) ? -1 : 0);
-}
-__host__ __device__ __forceinline__ constexpr int ey(int i) {
-    return (i == 2 || i == 5 || i == 6) ? 1 : ((i == 4 || i == 7 || i == 8) ? -1 : 0);
-}
-template <typename T>
-__host__ __device__ __forceinline__ constexpr T wq(int i) {
-    return i == 0 ? T(4.0 / 9.0) : (i < 5 ? T(1.0 / 9.0) : T(1.0 / 36.0));
-}
-
-
-template <typename T>
-__device__ __forceinline__ T sum9(const T f[9]) {
-    return ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
-}
-
 // Second-order equilibrium of Eq. 2 with c_s^2 = 1/3:
 //   f_i^eq = w_i rho (1 + 3 e.u + 9/2 (e.u)^2 - 3/2 u.u).
-template <typename T>
-__device__ __forceinline__ T feq(int i, T rho, T ux, T uy, T uu) {
-    const T eu = T(ex(i)) * ux + T(ey(i)) * uy;
-    return wq<T>(i) * rho * (T(1) + T(3) * eu + T(4.5) * eu * eu - T(1.5) * uu);
+__device__ __forceinline__ double feq(int i, double rho, double ux, double uy, double uu) {
+    const double w = i == 0 ? 4.0 / 9.0 : (i < 5 ? 1.0 / 9.0 : 1.0 / 36.0);
+    const double eu = q_ex(i) * ux + q_ey(i) * uy;
+    return w * rho * (1.0 + 3.0 * eu + 4.5 * eu * eu - 1.5 * uu);
 }
 
 __device__ __forceinline__ void raise_flag(DevState* st, unsigned bits, int64_t t) {
@@ -46,123 +26,124 @@ __device__ __forceinline__ void raise_flag(DevState* st, unsigned bits, int64_t 
     atomicMin(&st->failed_t, (unsigned long long)t);
 }
 
+// In-place BGK collision with exact-difference forcing (Eqs. 1, 2, 5), with j = rho u,
+// m = j + F, keep = 1 - 1/tau, g = m - keep j and P = (m m - keep j j)/rho:
+//   f_i* = keep f_i + w_i [omega rho + 3 e.g + 9/2 (e e : P) - 3/2 tr P],
+// in moments, so that the velocity is never formed and opposite directions share all but
+// the sign of one term: 60 FP64 instructions.  (Pair by pair in u and v it is 84.)
+__device__ __forceinline__ void collide_bgk(double (&f)[9], double rho, double Fx, double Fy,
+                                            double omega) {
+    const double keep = rn_sub(1.0, omega);
+    const double d57 = rn_sub(f[5], f[7]), d68 = rn_sub(f[6], f[8]);
+    const double jx = rn_add(rn_sub(f[1], f[3]), rn_sub(d57, d68));
+    const double jy = rn_add(rn_sub(f[2], f[4]), rn_add(d57, d68));
+    const double inv = rcp64(rho);
+    const double mx = rn_add(jx, Fx), my = rn_add(jy, Fy);
+    const double kx = rn_mul(keep, jx), ky = rn_mul(keep, jy);
+    const double pxx = rn_mul(rn_fma(mx, mx, -rn_mul(kx, jx)), inv);
+    const double pyy = rn_mul(rn_fma(my, my, -rn_mul(ky, jy)), inv);
+    const double pxy = rn_mul(rn_fma(mx, my, -rn_mul(kx, jy)), inv);
+    const double s = rn_add(pxx, pyy);
+    const double e1 = rn_mul(rn_fma(-1.5, s, rn_mul(omega, rho)), 1.0 / 9.0);
+    f[0] = rn_fma(keep, f[0], rn_mul(4.0, e1));
+    const double bx = rn_mul(rn_sub(mx, kx), 1.0 / 3.0), by = rn_mul(rn_sub(my, ky), 1.0 / 3.0);
+    auto pair = [&](int i, int j, double even, double c, double odd) {
+        f[i] = rn_fma(c, odd, rn_fma(keep, f[i], even));
+        f[j] = rn_fma(-c, odd, rn_fma(keep, f[j], even));
+    };
+    pair(1, 3, rn_fma(0.5, pxx, e1), 1.0, bx);
+    pair(2, 4, rn_fma(0.5, pyy, e1), 1.0, by);
+    const double e2 = rn_fma(0.125, s, rn_mul(0.25, e1));
+    pair(5, 7, rn_fma(0.25, pxy, e2), 0.25, rn_add(bx, by));
+    pair(6, 8, rn_fma(-0.25, pxy, e2), 0.25, rn_sub(by, bx));
+}
+
 // ---------------------------------------------------------------------------
-// Pass 1, FP64: fused collide + stream (pull from a shared-memory tile).
-// A block owns a BX x BY tile of destination nodes.  It first collides the
-// tile plus a one-node periodic halo (post-collision values to shared memory),
-// then every destination node gathers f_i*(x - e_i) from shared memory, writes
-// its nine populations once (coalesced, aligned) and its new density.
+// Pass 1, FP64: collide a node and push its populations to its neighbours.  A thread
+// per node; each plane is written by a warp as one row piece shifted by e_i.  What bounds
+// it is the FP64 pipe, so no node is collided twice: a tile pulling from a collided halo
+// (32 x 16 nodes, 1.2 collisions a node) took 251 us at 1024^2, this takes 123.  The new
+// density is summed by the pass that needs it first (the x-lines).
 // ---------------------------------------------------------------------------
-template <typename TF, int BX, int BY, bool MRT, bool WALLS>
-__global__ void __launch_bounds__(BX* BY)
-    k_collide_stream(const TF* __restrict__ fin, TF* __restrict__ fout,
+constexpr int kCsT = 128;
+
+template <bool MRT, bool WALLS>
+__global__ void __launch_bounds__(kCsT)
+    k_collide_stream(const double* __restrict__ fin, double* __restrict__ fout,
                      const double* __restrict__ Fx, const double* __restrict__ Fy,
-                     double* __restrict__ rho_out, int nx, int ny, size_t plane, TF omega,
-                     TF se, TF seps, TF sq, TF uwb6, TF uwt6,
+                     const double* __restrict__ rho, int nx, int ny, size_t plane, double omega,
+                     double se, double seps, double sq, double uwb6, double uwt6,
                      DevState* __restrict__ st) {
-    constexpr int HX = BX + 2, HY = BY + 2, HN = HX * HY;
-    __shared__ TF sf[9][HN];
-    const int tid = threadIdx.x + BX * threadIdx.y;
-    const int gx0 = blockIdx.x * BX - 1, gy0 = blockIdx.y * BY - 1;
-    bool ok = true;
-    for (int k = tid; k < HN; k += BX * BY) {
-        const int ly = k / HX, lx = k - ly * HX;
-        const int gx = wrap_near(gx0 + lx, nx), gy = wrap_near(gy0 + ly, ny);
-        const size_t n = (size_t)gy * nx + gx;
-        TF f[9];
+    const long long n = blockIdx.x * (long long)kCsT + threadIdx.x;
+    if (n >= (long long)nx * ny) return;
+    const int y = (int)(n / nx), x = (int)(n - (long long)y * nx);
+    double f[9];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) f[i] = fin[i * plane + n];
-        if constexpr (MRT)
-            ok &= collide_mrt<TF>(f, (TF)Fx[n], (TF)Fy[n], omega, (TF)FLT_MAX, se, seps, sq);
-        else
-            ok &= collide_pairs<TF>(f, (TF)Fx[n], (TF)Fy[n], omega, (TF)FLT_MAX);
+    for (int i = 0; i < 9; ++i) f[i] = fin[i * plane + n];
+    const double r = rho[n];
+    bool ok = positive64(r);
+    if constexpr (MRT)
+        ok &= collide_mrt<double>(f, Fx[n], Fy[n], omega, (double)FLT_MAX, se, seps, sq);
+    else
+        collide_bgk(f, r, Fx[n], Fy[n], omega);
+    const int xs[3] = {x > 0 ? x - 1 : nx - 1, x, x + 1 < nx ? x + 1 : 0};
+    const int ys[3] = {y > 0 ? y - 1 : ny - 1, y, y + 1 < ny ? y + 1 : 0};
+    // the node's density, for the momentum a moving wall gives
+    const bool bottom = WALLS && y == 0, top = WALLS && y == ny - 1;
+    double rw = 0.0;
+    if (WALLS && (bottom || top)) {
 #pragma unroll
-        for (int i = 0; i < 9; ++i) sf[i][k] = f[i];
+        for (int i = 0; i < 9; ++i) rw += f[i];
     }
-    __syncthreads();
-    const int x = blockIdx.x * BX + threadIdx.x, y = blockIdx.y * BY + threadIdx.y;
-    if (x < nx && y < ny) {
-        const int lx = threadIdx.x + 1, ly = threadIdx.y + 1;
-        const size_t n = (size_t)y * nx + x;
-        TF g[9];
-        // the node's density, for the momentum a moving wall gives
-        TF rw = TF(0);
-        if (WALLS && (y == 0 || y == ny - 1)) {
 #pragma unroll
-            for (int i = 0; i < 9; ++i) rw += sf[i][ly * HX + lx];
-        }
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const int ys = y - q_ey(i);
-            // halfway bounce-back at walls: the node's own opposite population,
-            // plus e_x rho U / 6 on the diagonals from a wall moving at U (Ladd)
-            if (WALLS && (ys < 0 || ys >= ny))
-                g[i] = sf[q_opp(i)][ly * HX + lx] + TF(q_ex(i)) * rw * (ys < 0 ? uwb6 : uwt6);
-            else
-                g[i] = sf[i][(ly - q_ey(i)) * HX + (lx - q_ex(i))];
-            fout[i * plane + n] = g[i];
-        }
-        rho_out[n] = (double)sum9(g);
+    for (int i = 0; i < 9; ++i) {
+        // halfway bounce-back at walls: the node keeps the population, reversed, plus
+        // e_x rho U / 6 on the diagonals from a wall moving at U (Ladd)
+        if (WALLS && ((q_ey(i) < 0 && bottom) || (q_ey(i) > 0 && top)))
+            fout[q_opp(i) * plane + n] =
+                f[i] - (double)q_ex(i) * rw * (q_ey(i) < 0 ? uwb6 : uwt6);
+        else
+            fout[i * plane + (size_t)ys[q_ey(i) + 1] * nx + xs[q_ex(i) + 1]] = f[i];
     }
     if (!ok) raise_flag(st, FLAG_RHO, st->t);
 }
 
-// f_i = f_i^eq(rho, u) (Eq. 2) in FP64, stored as TF; rho_out = sum of the
-// stored populations (the density every later pass sees).
-template <typename TF>
+// f_i = f_i^eq(rho, u) (Eq. 2).
 __global__ void k_init_feq(const double* __restrict__ rho, const double* __restrict__ ux,
-                           const double* __restrict__ uy, TF* __restrict__ f,
-                           double* __restrict__ rho_out, size_t N, size_t plane) {
+                           const double* __restrict__ uy, double* __restrict__ f, size_t N,
+                           size_t plane) {
     for (size_t n = blockIdx.x * (size_t)blockDim.x + threadIdx.x; n < N;
          n += (size_t)gridDim.x * blockDim.x) {
         const double r = rho[n];
         const double u = ux ? ux[n] : 0.0, v = uy ? uy[n] : 0.0;
         const double uu = u * u + v * v;
-        TF g[9];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            g[i] = (TF)feq<double>(i, r, u, v, uu);
-            f[i * plane + n] = g[i];
-        }
-        rho_out[n] = (double)sum9(g);
+        for (int i = 0; i < 9; ++i) f[i * plane + n] = feq(i, r, u, v, uu);
     }
 }
 
-template <typename TF>
-__global__ void k_rho_from_f(const TF* __restrict__ f, double* __restrict__ rho, size_t N,
-                             size_t plane) {
-    for (size_t n = blockIdx.x * (size_t)blockDim.x + threadIdx.x; n < N;
-         n += (size_t)gridDim.x * blockDim.x) {
-        TF g[9];
-#pragma unroll
-        for (int i = 0; i < 9; ++i) g[i] = f[i * plane + n];
-        rho[n] = (double)sum9(g);
-    }
-}
-
-// Output velocity v = u + F/(2 rho) (Sec. 2, after Eq. 5), in FP64.
-template <typename TF>
-__device__ __forceinline__ void node_velocity(const TF* __restrict__ f, size_t plane, size_t n,
-                                              double Fx, double Fy, double& rho, double& vx,
+// Output velocity v = u + F/(2 rho) (Sec. 2, after Eq. 5).
+__device__ __forceinline__ void node_velocity(const double* __restrict__ f, size_t plane, size_t n,
+                                              double rho, double Fx, double Fy, double& vx,
                                               double& vy) {
     double g[9];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) g[i] = (double)f[i * plane + n];
-    rho = sum9(g);
+    for (int i = 1; i < 9; ++i) g[i] = f[i * plane + n];
     const double jx = (g[1] + g[5] + g[8]) - (g[3] + g[6] + g[7]);
     const double jy = (g[2] + g[5] + g[6]) - (g[4] + g[7] + g[8]);
-    vx = (jx + 0.5 * Fx) / rho;
-    vy = (jy + 0.5 * Fy) / rho;
+    const double inv = rcp64(rho);
+    vx = div64(jx + 0.5 * Fx, rho, inv);
+    vy = div64(jy + 0.5 * Fy, rho, inv);
 }
 
-template <typename TF>
-__global__ void k_macro(const TF* __restrict__ f, const double* __restrict__ Fx,
-                        const double* __restrict__ Fy, double* __restrict__ vx,
-                        double* __restrict__ vy, size_t N, size_t plane) {
+__global__ void k_macro(const double* __restrict__ f, const double* __restrict__ rho,
+                        const double* __restrict__ Fx, const double* __restrict__ Fy,
+                        double* __restrict__ vx, double* __restrict__ vy, size_t N,
+                        size_t plane) {
     for (size_t n = blockIdx.x * (size_t)blockDim.x + threadIdx.x; n < N;
          n += (size_t)gridDim.x * blockDim.x) {
-        double r, u, v;
-        node_velocity(f, plane, n, Fx[n], Fy[n], r, u, v);
+        double u, v;
+        node_velocity(f, plane, n, rho[n], Fx[n], Fy[n], u, v);
         if (vx) vx[n] = u;
         if (vy) vy[n] = v;
     }
@@ -171,25 +152,24 @@ __global__ void k_macro(const TF* __restrict__ f, const double* __restrict__ Fx,
 // Diagnostics, two deterministic stages: per-block partials, then one block.
 constexpr int kDiagThreads = 256;
 
-template <typename TF>
 __global__ void __launch_bounds__(kDiagThreads)
-    k_diag_partial(const TF* __restrict__ f, const double* __restrict__ rho,
+    k_diag_partial(const double* __restrict__ f, const double* __restrict__ rho,
                    const double* __restrict__ Fx, const double* __restrict__ Fy, size_t N,
                    size_t plane, double* __restrict__ partials) {
     double s = 0.0, vmax = 0.0, rmin = DBL_MAX, rmax = -DBL_MAX;
     for (size_t n = blockIdx.x * (size_t)blockDim.x + threadIdx.x; n < N;
          n += (size_t)gridDim.x * blockDim.x) {
-        double r, u, v;
-        node_velocity(f, plane, n, Fx[n], Fy[n], r, u, v);
+        double u, v;
         const double rf = rho[n];
+        node_velocity(f, plane, n, rf, Fx[n], Fy[n], u, v);
         s += rf;
-        vmax = fmax(vmax, sqrt(u * u + v * v));
+        vmax = fmax(vmax, u * u + v * v);  // the square: one root a thread
         rmin = fmin(rmin, rf);
         rmax = fmax(rmax, rf);
     }
     __shared__ double sh[4][kDiagThreads];
     sh[0][threadIdx.x] = s;
-    sh[1][threadIdx.x] = vmax;
+    sh[1][threadIdx.x] = sqrt(vmax);
     sh[2][threadIdx.x] = rmin;
     sh[3][threadIdx.x] = rmax;
     __syncthreads();
@@ -236,18 +216,16 @@ __global__ void __launch_bounds__(kDiagThreads)
     }
 }
 
-template <typename TF>
-__global__ void k_f_to_double(const TF* __restrict__ f, double* __restrict__ out, size_t n) {
+__global__ void k_f_to_double(const float* __restrict__ f, double* __restrict__ out, size_t n) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
          i += (size_t)gridDim.x * blockDim.x)
-        out[i] = (double)f[i];
+        out[i] = widen(f[i]);
 }
 
-template <typename TF>
-__global__ void k_f_from_double(const double* __restrict__ in, TF* __restrict__ f, size_t n) {
+__global__ void k_f_from_double(const double* __restrict__ in, float* __restrict__ f, size_t n) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
          i += (size_t)gridDim.x * blockDim.x)
-        f[i] = (TF)in[i];
+        f[i] = (float)in[i];
 }
 
 inline unsigned grid_for(size_t n, int threads) {
@@ -257,68 +235,43 @@ inline unsigned grid_for(size_t n, int threads) {
 
 }  // namespace
 
-// Tile of the collide-stream pass: 32 x 8 destination nodes per block.
-constexpr int kCsBX = 32, kCsBY = 16;
+cudaError_t launch_collide_stream(const double* fin, double* fout, const double* Fx,
+                                  const double* Fy, const double* rho, int nx, int ny,
+                                  size_t plane, double omega, const MrtRates* mrt, DevState* st,
+                                  cudaStream_t s, const Walls& walls) {
+    const unsigned grid = (unsigned)(((long long)nx * ny + kCsT - 1) / kCsT);
+    const double se = mrt ? mrt->se : 0.0, seps = mrt ? mrt->seps : 0.0, sq = mrt ? mrt->sq : 0.0;
+    auto go = [&](auto kern) {
+        kern<<<grid, kCsT, 0, s>>>(fin, fout, Fx, Fy, rho, nx, ny, plane, omega, se, seps, sq,
+                                   walls.u[0] / 6.0, walls.u[1] / 6.0, st);
+        return cudaGetLastError();
+    };
+    if (mrt)
+        return walls.on ? go(k_collide_stream<true, true>) : go(k_collide_stream<true, false>);
+    return walls.on ? go(k_collide_stream<false, true>) : go(k_collide_stream<false, false>);
+}
 
-template <typename TF>
-cudaError_t launch_collide_stream(const TF* fin, TF* fout, const double* Fx, const double* Fy,
-                                  double* rho_out, int nx, int ny, size_t plane, double omega,
-                                  const MrtRates* mrt, DevState* st, cudaStream_t s,
-                                  const Walls& walls) {
-    const TF ub = (TF)(walls.u[0] / 6.0), ut = (TF)(walls.u[1] / 6.0);
-    dim3 block(kCsBX, kCsBY);
-    dim3 grid((nx + kCsBX - 1) / kCsBX, (ny + kCsBY - 1) / kCsBY);
-    const TF se = mrt ? (TF)mrt->se : TF(0), seps = mrt ? (TF)mrt->seps : TF(0),
-             sq = mrt ? (TF)mrt->sq : TF(0);
-#define CPLBM_CS(M, W)                                                                    \
-    k_collide_stream<TF, kCsBX, kCsBY, M, W><<<grid, block, 0, s>>>(                      \
-        fin, fout, Fx, Fy, rho_out, nx, ny, plane, (TF)omega, se, seps, sq, ub, ut, st)
-    if (mrt && walls.on)
-        CPLBM_CS(true, true);
-    else if (mrt)
-        CPLBM_CS(true, false);
-    else if (walls.on)
-        CPLBM_CS(false, true);
-    else
-        CPLBM_CS(false, false);
-#undef CPLBM_CS
+cudaError_t launch_init_feq(const double* rho, const double* ux, const double* uy, double* f,
+                            int nx, int ny, size_t plane, cudaStream_t s) {
+    const size_t N = (size_t)nx * ny;
+    k_init_feq<<<grid_for(N, 256), 256, 0, s>>>(rho, ux, uy, f, N, plane);
     return cudaGetLastError();
 }
 
-template <typename TF>
-cudaError_t launch_init_feq(const double* rho, const double* ux, const double* uy, TF* f,
-                            double* rho_out, int nx, int ny, size_t plane, cudaStream_t s) {
-    size_t N = (size_t)nx * ny;
-    k_init_feq<TF><<<grid_for(N, 256), 256, 0, s>>>(rho, ux, uy, f, rho_out, N, plane);
+cudaError_t launch_macro(const double* f, const double* rho, const double* Fx, const double* Fy,
+                         double* vx, double* vy, int nx, int ny, size_t plane, cudaStream_t s) {
+    const size_t N = (size_t)nx * ny;
+    k_macro<<<grid_for(N, 256), 256, 0, s>>>(f, rho, Fx, Fy, vx, vy, N, plane);
     return cudaGetLastError();
 }
 
-template <typename TF>
-cudaError_t launch_rho_from_f(const TF* f, double* rho, int nx, int ny, size_t plane,
-                              cudaStream_t s) {
-    size_t N = (size_t)nx * ny;
-    k_rho_from_f<TF><<<grid_for(N, 256), 256, 0, s>>>(f, rho, N, plane);
-    return cudaGetLastError();
-}
-
-template <typename TF>
-cudaError_t launch_macro(const TF* f, const double* Fx, const double* Fy, double* vx,
-                         double* vy, int nx, int ny, size_t plane, cudaStream_t s) {
-    size_t N = (size_t)nx * ny;
-    k_macro<TF><<<grid_for(N, 256), 256, 0, s>>>(f, Fx, Fy, vx, vy, N, plane);
-    return cudaGetLastError();
-}
-
-template <typename TF>
-cudaError_t launch_diag(const TF* f, const double* rho, const double* Fx, const double* Fy,
+cudaError_t launch_diag(const double* f, const double* rho, const double* Fx, const double* Fy,
                         int nx, int ny, size_t plane, double* partials, int nparts,
                         DevState* st, cudaStream_t s) {
-    size_t N = (size_t)nx * ny;
-    k_diag_partial<TF><<<nparts, kDiagThreads, 0, s>>>(f, rho, Fx, Fy, N, plane, partials);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_diag_final<<<1, kDiagThreads, 0, s>>>(partials, nparts, st);
-    return cudaGetLastError();
+    const size_t N = (size_t)nx * ny;
+    k_diag_partial<<<nparts, kDiagThreads, 0, s>>>(f, rho, Fx, Fy, N, plane, partials);
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : launch_diag_final(partials, nparts, st, s);
 }
 
 cudaError_t launch_diag_final(const double* partials, int nparts, DevState* st, cudaStream_t s) {
@@ -326,37 +279,14 @@ cudaError_t launch_diag_final(const double* partials, int nparts, DevState* st, 
     return cudaGetLastError();
 }
 
-template <typename TF>
-cudaError_t launch_f_to_double(const TF* f, double* out, size_t n, cudaStream_t s) {
-    k_f_to_double<TF><<<grid_for(n, 256), 256, 0, s>>>(f, out, n);
+cudaError_t launch_f_to_double(const float* f, double* out, size_t n, cudaStream_t s) {
+    k_f_to_double<<<grid_for(n, 256), 256, 0, s>>>(f, out, n);
     return cudaGetLastError();
 }
 
-template <typename TF>
-cudaError_t launch_f_from_double(const double* in, TF* f, size_t n, cudaStream_t s) {
-    k_f_from_double<TF><<<grid_for(n, 256), 256, 0, s>>>(in, f, n);
+cudaError_t launch_f_from_double(const double* in, float* f, size_t n, cudaStream_t s) {
+    k_f_from_double<<<grid_for(n, 256), 256, 0, s>>>(in, f, n);
     return cudaGetLastError();
 }
-
-#define CPLBM_INST(TF)                                                                       \
-    template cudaError_t launch_collide_stream<TF>(const TF*, TF*, const double*,            \
-                                                   const double*, double*, int, int, size_t, \
-                                                   double, const MrtRates*, DevState*,       \
-                                                   cudaStream_t, const Walls&);              \
-    template cudaError_t launch_init_feq<TF>(const double*, const double*, const double*,    \
-                                             TF*, double*, int, int, size_t, cudaStream_t);  \
-    template cudaError_t launch_rho_from_f<TF>(const TF*, double*, int, int, size_t,         \
-                                               cudaStream_t);                                \
-    template cudaError_t launch_macro<TF>(const TF*, const double*, const double*, double*,  \
-                                          double*, int, int, size_t, cudaStream_t);          \
-    template cudaError_t launch_diag<TF>(const TF*, const double*, const double*,            \
-                                         const double*, int, int, size_t, double*, int,      \
-                                         DevState*, cudaStream_t);                           \
-    template cudaError_t launch_f_to_double<TF>(const TF*, double*, size_t, cudaStream_t);   \
-    template cudaError_t launch_f_from_double<TF>(const double*, TF*, size_t, cudaStream_t);
-
-CPLBM_INST(double)
-CPLBM_INST(float)
-#undef CPLBM_INST
 
 }  // namespace cplbm

@@ -1,6 +1,5 @@
-// kernels_lines.cu -- warp-cooperative compact-FD line solves (Eqs. 37-39) with
-// the fused chemical-potential (Eqs. 21, 33, Sec. 5.6) and force (Eq. 12)
-// epilogues, for both the FP64 and the mixed path.
+// kernels_lines.cu -- warp-cooperative compact-FD line solves (Eqs. 37-39) of the mixed
+// path, with the fused force (Eq. 12) epilogue.  (The FP64 path's are in lines64.cu.)
 //
 // The periodic compact scheme is the circulant system A d = B u with
 //   (A d)_i = alpha d_{i-1} + d_i + alpha d_{i+1},
@@ -26,7 +25,7 @@
 // a double recursion in each direction whose chunk-joining map is
 // (v, w) -> (m v, m (C v + w)).
 //
-// Arithmetic policies: PolD (FP64), PolF (FP32), PolDF (double-float pairs).
+// Arithmetic policies: PolF (FP32), PolDF (double-float pairs).
 // The mixed path uses PolDF for the first derivative of the density and PolF for
 // everything else (see kernels_mixed.cu for why).
 #include <cuda.h>  // CUtensorMap and its encoder's types (the encoder is fetched at run time)
@@ -46,25 +45,6 @@ namespace cplbm {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-
-struct PolD {
-    using V = double;
-    using K = double;
-    using O = double;  // stored result
-    static __device__ __forceinline__ V zero() { return 0.0; }
-    static __device__ __forceinline__ V sub(V a, V b) { return a - b; }
-    static __device__ __forceinline__ V mulc(V a, K c) { return a * c; }
-    static __device__ __forceinline__ V fmac(V a, K c, V b) { return fma(a, c, b); }
-    static __device__ __forceinline__ V up(V a, int o) { return __shfl_up_sync(kFull, a, o); }
-    static __device__ __forceinline__ V down(V a, int o) { return __shfl_down_sync(kFull, a, o); }
-    static __device__ __forceinline__ O out(V a) { return a; }
-    static K konst(double v) { return v; }
-    // shared-memory staging: one plane of S
-    using S = double;
-    static constexpr int kPlanes = 1;
-    static __device__ __forceinline__ V sget(const S* t, int i, int) { return t[i]; }
-    static __device__ __forceinline__ void sput(S* t, int i, int, V v) { t[i] = v; }
-};
 
 struct PolF {
     using V = float;
@@ -119,8 +99,6 @@ struct PolDF {
 
 // value of the second-derivative arithmetic from the first's right-hand side
 template <class P2>
-__device__ __forceinline__ typename P2::V to2(double v) { return (typename P2::V)v; }
-template <class P2>
 __device__ __forceinline__ typename P2::V to2(float v) { return (typename P2::V)v; }
 template <class P2>
 __device__ __forceinline__ typename P2::V to2(df v) { return (typename P2::V)v.hi; }
@@ -165,10 +143,6 @@ struct LineGeo {
 __device__ __forceinline__ void cp_async4(void* sdst, const void* gsrc) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(sdst);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async8(void* sdst, const void* gsrc) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(sdst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gsrc) : "memory");
 }
 __device__ __forceinline__ void cp_async16(void* sdst, const void* gsrc) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(sdst);
@@ -229,18 +203,6 @@ __device__ __forceinline__ void tma_load_2d(void* sdst, const CUtensorMap* map, 
 
 // Input fields: stage(t, i, ps, o) copies the element at global offset o into
 // staging slot i (planes `ps` apart).
-struct InD {
-    const double* p;
-    __device__ __forceinline__ void init(const DevState*) {}
-    __device__ __forceinline__ void stage(double* t, int i, int, size_t o) {
-        cp_async8(t + i, p + o);
-    }
-    __device__ __forceinline__ void stage4(double* t, int i, int, size_t o) {
-        cp_async16(t + i, p + o);
-        cp_async16(t + i + 2, p + o + 2);
-    }
-    __device__ __forceinline__ bool flagged() const { return false; }
-};
 struct InF {
     const float* p;
     __device__ __forceinline__ void init(const DevState*) {}
@@ -1073,48 +1035,6 @@ struct EpiStore {
     }
 };
 
-// mu-hat = k^2 mu0(rho) - kappa (d_xx + d_yy) rho, Eq. 33 with the mu0 of
-// Eqs. 15, 17, 19 or 21, limited from above while t < cap_steps (Sec. 5.6).  R
-// is the arithmetic of the EOS.
-template <class R, class O, class RhoT>
-struct EpiMu {
-    static constexpr int kBatch = 4;
-    O* dyr;
-    O* mu;
-    const RhoT* __restrict__ rho;
-    const O* __restrict__ dxx;
-    EosC<R> e;
-    R k2, kappa, cap;
-    int64_t cap_steps;
-    bool capped;
-    struct Ops {
-        RhoT r;
-        O xx;
-    };
-    struct Ops4 {};  // the FP64 path has no vector epilogue
-    __device__ __forceinline__ Ops4 fetch4(size_t) const { return Ops4{}; }
-    __device__ __forceinline__ bool put4(size_t, float4, float4, const Ops4&) { return false; }
-    // the time level is read on the device: graph replays reuse the arguments
-    __device__ __forceinline__ void init(const DevState* st) { capped = st->t < cap_steps; }
-    __device__ __forceinline__ Ops fetch(size_t o) const { return Ops{__ldg(rho + o), __ldg(dxx + o)}; }
-    __device__ __forceinline__ bool operator()(size_t o, O d1, O d2, const Ops& op) {
-        dyr[o] = d1;
-        bool bad = false;
-        const R mu0 = eos_mu0(e, (R)op.r, bad);
-        R m = rn_fma(k2, mu0, -rn_mul(kappa, rn_add((R)op.xx, (R)d2)));
-        if (capped) {
-            if (eos_at_pole(e, (R)op.r)) {  // mu0 = +infinity: the limit takes the node
-                m = cap;
-                bad = false;
-            } else {
-                m = m < cap ? m : cap;
-            }
-        }
-        mu[o] = (O)m;
-        return bad || !(m > -R(1e30) && m < R(1e30));
-    }
-};
-
 // F = -rho d(mu-hat) + c_s^2 d(rho), Eq. 12.  In FP32, c_s^2 = 1/3 as a constant is 3e-8
 // too large, a bias that the populations' pressure does not share and that moves the dilute
 // gas at high density ratios.  So c_s^2 = hi + lo, and the sum is rounded once.
@@ -1122,9 +1042,6 @@ __device__ __forceinline__ float force_term(float r, float dmu, float d) {
     constexpr float hi = 1.0f / 3.0f;
     constexpr float lo = (float)(1.0 / 3.0 - (double)hi);
     return rn_fma(d, hi, rn_fma(-r, dmu, rn_mul(d, lo)));
-}
-__device__ __forceinline__ double force_term(double r, double dmu, double d) {
-    return rn_fma(-r, dmu, rn_mul(d, 1.0 / 3.0));
 }
 
 template <class O, class RhoT>
@@ -1381,7 +1298,7 @@ cudaError_t launch_lines(In in, int nx, int ny, int axis, int order, double eps1
 }
 
 // rounding levels the recursions are cut at
-constexpr double kEpsD = 1e-17, kEpsDF = 1e-15, kEpsF = 1e-8;
+constexpr double kEpsDF = 1e-15, kEpsF = 1e-8;
 
 // ---- batched mixed line passes ----
 using RhoInst = LinesXYInst<InDF, EpiStore<float, float>, InDF, EpiStore<float, float>>;
@@ -1415,35 +1332,6 @@ cudaError_t launch_batch_t(const Inst* d, const int* map, int nblocks, int order
 }
 
 }  // namespace
-
-// ---- FP64 path ----
-cudaError_t lines_fp64_rho_x(const double* rho, double* dxr, double* dxx, int nx, int ny,
-                             int order, DevState* st, int bump, cudaStream_t s) {
-    return launch_lines<PolD, PolD, true>(InD{rho}, nx, ny, 0, order, kEpsD, kEpsD,
-                                          EpiStore<double, double>{dxr, dxx}, st, bump, s);
-}
-cudaError_t lines_fp64_rho_y_mu(const double* rho, const double* dxx, double* dyr, double* mu,
-                                int nx, int ny, int order, const PhysParams& p, DevState* st,
-                                cudaStream_t s, bool walls_y) {
-    EpiMu<double, double, double> epi{dyr, mu, rho, dxx, eos_const<double>(p), p.k2, p.kappa,
-                                      p.mu_cap, p.cap_steps, false};
-    return launch_lines<PolD, PolD, true>(InD{rho}, nx, ny, 1, order, kEpsD, kEpsD, epi, st, 0, s,
-                                          walls_y);
-}
-cudaError_t lines_fp64_force(const double* mu, const double* rho, const double* dr, double* F,
-                             int nx, int ny, int axis, int order, cudaStream_t s, bool walls_y) {
-    return launch_lines<PolD, PolD, false>(InD{mu}, nx, ny, axis, order, kEpsD, kEpsD,
-                                           EpiForce<double, double>{F, rho, dr}, nullptr, 0, s,
-                                           walls_y);
-}
-cudaError_t lines_fp64_plain(const double* u, double* d1, double* d2, int nx, int ny, int axis,
-                             int order, cudaStream_t s) {
-    if (d2)
-        return launch_lines<PolD, PolD, true>(InD{u}, nx, ny, axis, order, kEpsD, kEpsD,
-                                              EpiStore<double, double>{d1, d2}, nullptr, 0, s);
-    return launch_lines<PolD, PolD, false>(InD{u}, nx, ny, axis, order, kEpsD, kEpsD,
-                                           EpiStore<double, double>{d1, nullptr}, nullptr, 0, s);
-}
 
 // ---- mixed path ----
 cudaError_t lines_mixed_rho_xy(const float* rh, const float* rl, float* dxr, float* dxx,
