@@ -179,42 +179,60 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs g) {
 //
 // k_umma_rows: D[M x 256] = A[M x K] Bt[256 x K]^T, K = 64 or 256: the forward
 // products (A = the layer input, Bt = the transposed weights) and the input
-// gradients (A = the backward signal, Bt = the weights as stored).  Persistent:
-// one CTA per SM walks 128-row tiles of A.  Warp 8 (one thread) streams the
-// 64-wide K chunks of A and Bt (Bt is re-read from L2 for every tile) through a
-// three-stage ring; warp 9 (one thread) issues the MMAs (128 x 256 x 16 each)
-// into one of two 256-column accumulators; warps 0-7 drain the other
-// accumulator (the previous tile) meanwhile, two warps per quarter of the
-// tensor-memory lanes, one per half of the columns.  The epilogue stages each
-// 32-row x 16-column block in shared memory so that its global loads and stores
-// are row pieces of 64 (FP32) or 32 (BF16) bytes.
+// gradients (A = the backward signal, Bt = the weights as stored).  A CTA computes tiles
+// of 128 rows x kNT columns (grid.y: column blocks) and walks the rows.
+// Warp 8 (one thread) loads the CTA's columns of Bt once, which stay in shared memory, and
+// streams the 64-wide K chunks of A through a ring; warp 9 (one thread) issues the MMAs (128 x kNT x 16
+// each) into one of two accumulators; warps 0-7 drain the other accumulator (the previous
+// tile) meanwhile, two warps per quarter of the tensor-memory lanes, one per half of the
+// columns.  The epilogue bounds it: it stages each 32-row x 32-column block in shared
+// memory so that its global loads and stores are row pieces of 128 (FP32) or 64 (BF16)
+// bytes.
 //
-// k_umma_wgrad: the weight gradient dW[fi x 256] = A^T D over the batch, as
-// At[fi x K] Dt[256 x K]^T with K the batch: the epilogues above also write the
-// transposed BF16 copies At and Dt.  K is split into slices (grid.y) so that the
-// product fills the GPU; each CTA streams its slice through a four-stage ring
-// of 64-wide K chunks (warp 4 loads, warp 5 issues the MMAs) and writes an FP32
-// partial; k_wgrad_reduce adds the partials in a fixed order (deterministic).
+// k_umma_wgrad: the weight gradients dW[fi x 256] = A^T D over the batch, of all four
+// layers in one launch.  Both operands are read as the row kernel left them, [batch][256],
+// so K (the batch) is their slow dimension: the MN-major 128-byte-swizzle layout, 64
+// columns a row of 128 bytes, 8 batch rows a group of 1024 bytes, the next 64 columns one
+// box further.  (Transposed copies for a K-major product cost the row kernel's epilogue
+// sixteen 2-byte stores a chunk.)  K is split into slices (grid.y); each CTA streams its
+// slice through a four-stage ring of 64-row chunks (warp 4 loads, warp 5 issues the MMAs)
+// and writes an FP32 partial; k_gradient adds the partials in a fixed order
+// (deterministic) and, in training, applies Adam to each entry as it gets it.
+//
+// The kernels of a call are launched with programmatic serialization: each sets up its
+// barriers and tensor memory while the one before it finishes.  An Adam step at batch 256
+// takes 48 us (174 with products of 2 CTAs and eighteen launches), at 32768 158 us (297).
 // ---------------------------------------------------------------------------
 constexpr int UM = 128, UN = 256;
 constexpr unsigned kUmmaSpins = 1u << 22;
-constexpr int kS32 = 20, kS16 = 24;  // padded rows of the epilogue's staging blocks
+constexpr int kS32 = 36, kS16 = 40;  // padded rows of the epilogue's staging blocks
 constexpr int kKC = 64;              // K chunk of the streamed operands
 // k_umma_rows: 8 epilogue warps (two per tensor-memory lane quarter, one per
-// half of the 256 columns), a loader warp and an MMA warp; 3-stage ring
-constexpr int kRowEpi = 8, kRowStages = 3;
+// half of the columns), a loader warp and an MMA warp; a ring of A chunks (two CTAs an SM with
+// two stages each were no faster)
+constexpr int kRowEpi = 8, kRowStages = 5, kRowsPerSm = 1;
 constexpr int kRowsThreads = 32 * (kRowEpi + 2);
 // k_umma_wgrad: 4 epilogue warps, a loader warp and an MMA warp; 4-stage ring
 constexpr int kWgEpi = 4, kStages = 4;
 constexpr int kWgThreads = 32 * (kWgEpi + 2);
 constexpr int kRowGridCap = 256;  // most CTAs of a k_umma_rows launch
-constexpr size_t kChunkBytes = (size_t)(UM + UN) * kKC * 2;
-// (+1024: the stages are aligned to 1024 bytes inside the dynamic allocation)
-constexpr size_t kRowsSmem = 1024 + kRowStages * kChunkBytes +
-                             (size_t)kRowEpi * 32 * (kS32 * 4 + kS16 * 2) + UN * 4 +
-                             (size_t)kRowEpi * (UN / 2) * 4;
+constexpr int kBox = 64;                              // rows of a tensor-copy box
+constexpr unsigned kBoxBytes = kBox * kKC * 2;        // 64 x 64 BF16
+// columns of a row kernel's tile: narrow, so that the two row tiles of a batch of 256 use
+// eight SMs, and because 256 row tiles then divide evenly (7 quarter tiles for the busiest
+// of 152 SMs against 2 whole ones): Adam step 49 / 205 us at batch 256 / 32768 with 64
+// columns, 63 / 222 with 128, 91 / 249 with 256 (before the steps that followed).
+constexpr int kNT = 64;
+// the stages are aligned to 1024 bytes inside the dynamic allocation (hence + 1024)
+constexpr size_t kRowChunk = (size_t)UM * kKC * 2;                  // of A
+constexpr size_t kRowB = (size_t)kNT * kW * 2;                       // Bt, all of K
+constexpr size_t kRowsSmem = 1024 + kRowStages * kRowChunk + kRowB +
+                             (size_t)kRowEpi * 32 * kS32 * 4 + kNT * 4 +
+                             (size_t)kRowEpi * (kNT / 2) * 4;
+constexpr size_t kChunkBytes = (size_t)(UM + UN) * kKC * 2;  // of the weight gradient
 constexpr size_t kWgSmem = 1024 + kStages * kChunkBytes + (size_t)kWgEpi * 32 * kS32 * 4;
-static_assert(kRowsSmem <= 227 * 1024 - 1024, "row kernel shared memory");
+static_assert(kRowsPerSm * (kRowsSmem + 1024) <= 227 * 1024, "row kernel shared memory");
+static_assert(kNT == 2 * 32, "an epilogue warp takes one 32-column chunk of a tile");
 static_assert(kWgSmem <= 227 * 1024 - 1024, "weight-gradient kernel shared memory");
 
 struct RowArgs {
@@ -229,16 +247,19 @@ struct RowArgs {
     int ld32;
     __nv_bfloat16* out16;   // [M][ld16] or null
     int ld16;
-    __nv_bfloat16* out16t;  // [256][ldt] (column c of D at row c) or null
-    int ldt, rows_t;        // transposed copy: entries m < rows_t written, zero for m >= M
     int* err;
 };
 
+// 128-row tiles of dW: one of layer 0 (its 4 rows padded), two of each further layer
+constexpr int kWgTiles = 7;
+__host__ __device__ constexpr int wg_row0(int l) { return l == 0 ? 0 : UM + (l - 1) * kW; }
+struct WgMaps {
+    CUtensorMap a[kLayers], d[kLayers];  // layer inputs and signals, [batch][K or 256]
+};
 struct WgArgs {
-    int mtiles;       // 128-row tiles of At (fi rows)
-    int chunks;       // K chunks (64 wide) in all
+    int chunks;       // K chunks (64 batch rows) in all
     int per_slice;    // K chunks per slice
-    float* part;      // [slices][mtiles * 128][256]
+    float* part;      // [slices][kWgTiles * 128][256]
     int* err;
 };
 
@@ -289,19 +310,28 @@ __device__ __forceinline__ void tma2(void* dst, const CUtensorMap* map, int k, i
 // shared-memory matrix descriptor of a K-major operand in the 128-byte swizzle
 // layout: start address, leading byte offset 16 (unused by this layout), stride
 // byte offset 1024 (one 8-row group), descriptor version 1, layout type 2
-__device__ __forceinline__ uint64_t umma_desc(unsigned addr) {
+__device__ __forceinline__ uint64_t umma_desc(unsigned addr) {  // K-major
     return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
            ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
-// instruction descriptor: D f32 (bits 4-5), A and B bf16 (7-9, 10-12), both
-// K-major, N >> 3 at bit 17, M >> 4 at bit 24
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(UN >> 3) << 17) |
-                            ((uint32_t)(UM >> 4) << 24);
+// the same of an MN-major operand: 64 columns a 128-byte row, leading byte offset from one
+// 64-column box to the next, stride byte offset from one group of 8 K rows to the next
+__device__ __forceinline__ uint64_t umma_desc_mn(unsigned addr) {
+    return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)(kBoxBytes >> 4) << 16) |
+           ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+// instruction descriptor: D f32 (bits 4-5), A and B bf16 (7-9, 10-12), A and B
+// MN-major (15, 16), N >> 3 at bit 17, M >> 4 at bit 24
+constexpr uint32_t idesc(int n, bool mn) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | (mn ? 3u << 15 : 0u) |
+           ((uint32_t)(n >> 3) << 17) | ((uint32_t)(UM >> 4) << 24);
+}
+template <uint32_t IDESC>
 __device__ __forceinline__ void umma(uint32_t tmem, uint64_t da, uint64_t db, bool acc) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
         " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-        "l"(da), "l"(db), "r"(kIdesc), "r"(acc ? 1u : 0u)
+        "l"(da), "l"(db), "r"(IDESC), "r"(acc ? 1u : 0u)
         : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
@@ -316,16 +346,21 @@ __device__ __forceinline__ void tc_fence_before() {
 __device__ __forceinline__ void tc_fence_after() {
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 }
-// kNC consecutive accumulator columns of this warp's 32 lanes (one row a thread)
-constexpr int kNC = 16;
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* x) {
-    uint32_t v[16];
+// kNC consecutive accumulator columns of this warp's 32 lanes (one row a thread).  32, so
+// that the FP32 row pieces of the epilogue are 128 bytes: in 64-byte pieces the hidden
+// layers of a batch of 32768 wrote 2.8 TB/s (Adam step there 205 -> 179 us).
+constexpr int kNC = 32;
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, float* x) {
+    uint32_t v[32];
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
-        "%13,%14,%15}, [%16];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
+        "%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
         : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
           "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
-          "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+          "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]),
+          "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
+          "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]),
+          "=r"(v[31])
         : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
@@ -335,7 +370,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* x) {
 // this warp's 32 rows [r0, r0 + 32) x kNC columns [c, c + kNC) of a row-major
 // FP32 matrix (row stride ld): thread `lane` holds row r0 + lane in x.  Stores
 // and loads go through the warp's staging block s (32 rows of kS32 floats), so
-// that the global accesses are 64-byte row pieces, eight rows an instruction.
+// that the global accesses are 128-byte row pieces, four rows an instruction.
 __device__ __forceinline__ void rows_store32(float* s, const float* x, float* out, long long ld,
                                              int r0, int c, int M, int lane) {
 #pragma unroll
@@ -344,8 +379,8 @@ __device__ __forceinline__ void rows_store32(float* s, const float* x, float* ou
             make_float4(x[4 * j], x[4 * j + 1], x[4 * j + 2], x[4 * j + 3]);
     __syncwarp();
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int rr = 8 * j + (lane >> 2), q = lane & 3;
+    for (int j = 0; j < 8; ++j) {
+        const int rr = 4 * j + (lane >> 3), q = lane & 7;
         if (r0 + rr < M)
             *reinterpret_cast<float4*>(out + (long long)(r0 + rr) * ld + c + 4 * q) =
                 *reinterpret_cast<const float4*>(s + rr * kS32 + 4 * q);
@@ -355,61 +390,69 @@ __device__ __forceinline__ void rows_store32(float* s, const float* x, float* ou
 
 // coalesced loads of this warp's 32 rows x kNC columns of a row-major FP32
 // matrix [M][256], issued ahead of use (rows >= M read as zero): piece j holds
-// row 8 j + lane / 4, columns 4 (lane % 4) .. + 3
+// row 4 j + lane / 8, columns 4 (lane % 8) .. + 3
 __device__ __forceinline__ void aux_fetch(float4* pf, const float* in, int r0, int c, int M,
                                           int lane) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int rr = 8 * j + (lane >> 2), q = lane & 3;
+    for (int j = 0; j < 8; ++j) {
+        const int rr = 4 * j + (lane >> 3), q = lane & 7;
         pf[j] = r0 + rr < M
                     ? __ldg(reinterpret_cast<const float4*>(in + (long long)(r0 + rr) * UN + c +
                                                             4 * q))
                     : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
-// the fetched pieces -> row r0 + lane in aux, through the staging block s
-__device__ __forceinline__ void aux_rows(const float4* pf, float* s, float* aux, int lane) {
+// the fetched pieces into the staging block s, row r0 + i of the matrix in its row i
+__device__ __forceinline__ void aux_stage(const float4* pf, float* s, int lane) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-        *reinterpret_cast<float4*>(s + (8 * j + (lane >> 2)) * kS32 + 4 * (lane & 3)) = pf[j];
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < kNC / 4; ++j) {
-        const float4 a = *reinterpret_cast<const float4*>(s + lane * kS32 + 4 * j);
-        aux[4 * j] = a.x;
-        aux[4 * j + 1] = a.y;
-        aux[4 * j + 2] = a.z;
-        aux[4 * j + 3] = a.w;
-    }
+    for (int j = 0; j < 8; ++j)
+        *reinterpret_cast<float4*>(s + (4 * j + (lane >> 3)) * kS32 + 4 * (lane & 7)) = pf[j];
     __syncwarp();
 }
 
 // The epilogue of one kNC-column chunk [c, c + kNC) of a warp's 32 rows (x: row
-// r0 + lane; aux: the same entries of aprev, for EPI_TANH_BACK and EPI_LOSS).
-// Column sums of the result over the warp's rows are added to bsum[0..kNC).
-__device__ __forceinline__ void rows_epilogue(const RowArgs& g, float* x, const float* aux,
-                                              const float* bias_s, float* s32,
-                                              __nv_bfloat16* s16, int r0, int c, int lane,
-                                              float* bsum, double& sse) {
+// r0 + lane; bias_c: the biases of its columns; for EPI_TANH_BACK and EPI_LOSS the
+// staging block s holds the same entries of aprev).  Column sums of the result over the
+// warp's rows are added to bsum[0..kNC).
+__device__ __forceinline__ void rows_epilogue(const RowArgs& g, float* x, const float* bias_c,
+                                              float* s32, int r0, int c, int lane, float* bsum,
+                                              double& sse) {
     const bool live = r0 + lane < g.M;
+    __nv_bfloat16* s16 = reinterpret_cast<__nv_bfloat16*>(s32);
+    // this lane's row of the staged operand, four entries at a time
+    auto aux = [&](int j) { return *reinterpret_cast<const float4*>(s32 + lane * kS32 + j); };
     if (g.epi == EPI_TANH_BACK) {
 #pragma unroll
-        for (int j = 0; j < kNC; ++j) x[j] *= 1.0f - aux[j] * aux[j];
+        for (int j = 0; j < kNC; j += 4) {
+            const float4 a = aux(j);
+            x[j] *= 1.0f - a.x * a.x;
+            x[j + 1] *= 1.0f - a.y * a.y;
+            x[j + 2] *= 1.0f - a.z * a.z;
+            x[j + 3] *= 1.0f - a.w * a.w;
+        }
     } else if (g.epi == EPI_BIAS_TANH) {
 #pragma unroll
-        for (int j = 0; j < kNC; ++j) x[j] = tanh_act(x[j] + bias_s[c + j]);
+        for (int j = 0; j < kNC; ++j) x[j] = tanh_act(x[j] + bias_c[j]);
     } else if (g.epi == EPI_BIAS) {
 #pragma unroll
-        for (int j = 0; j < kNC; ++j) x[j] += bias_s[c + j];
+        for (int j = 0; j < kNC; ++j) x[j] += bias_c[j];
     } else if (g.epi == EPI_LOSS) {
-        float e2 = 0.0f;
 #pragma unroll
-        for (int j = 0; j < kNC; ++j) {
-            const float e = live ? x[j] + bias_s[c + j] - aux[j] : 0.0f;
-            e2 = fmaf(e, e, e2);
-            x[j] = 2.0f * e * g.scale;
+        for (int h = 0; h < kNC; h += 16) {
+            float e2 = 0.0f;
+#pragma unroll
+            for (int j = h; j < h + 16; j += 4) {
+                const float4 a = aux(j);
+                const float t[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float e = live ? x[j + k] + bias_c[j + k] - t[k] : 0.0f;
+                    e2 = fmaf(e, e, e2);
+                    x[j + k] = 2.0f * e * g.scale;
+                }
+            }
+            sse += (double)e2;
         }
-        sse += (double)e2;
     }
     if (!live) {
 #pragma unroll
@@ -423,8 +466,8 @@ __device__ __forceinline__ void rows_epilogue(const RowArgs& g, float* x, const 
         __syncwarp();
         if (g.out32) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int rr = 8 * j + (lane >> 2), q = lane & 3;
+            for (int j = 0; j < 8; ++j) {
+                const int rr = 4 * j + (lane >> 3), q = lane & 7;
                 if (r0 + rr < g.M)
                     *reinterpret_cast<float4*>(g.out32 + (long long)(r0 + rr) * g.ld32 + c +
                                                4 * q) =
@@ -432,63 +475,50 @@ __device__ __forceinline__ void rows_epilogue(const RowArgs& g, float* x, const 
             }
         }
         if (g.bpart) {
-            // lane l adds column l % 16 over rows 16 (l / 16) .. + 15, then the halves
-            const int col = lane & (kNC - 1), h = lane >> 4;
-            float cs = 0.0f;
+            // lane l adds column l over rows 0 .. 15 and 16 .. 31, then the halves
+            float cs[2] = {0.0f, 0.0f};
 #pragma unroll
-            for (int r = 0; r < 16; ++r) cs += s32[(16 * h + r) * kS32 + col];
-            cs += __shfl_down_sync(0xffffffffu, cs, 16);
-            if (lane < kNC) bsum[lane] += cs;
+            for (int r = 0; r < 32; ++r) cs[r >> 4] += s32[r * kS32 + lane];
+            bsum[lane] += cs[0] + cs[1];
         }
         __syncwarp();
     }
-    if (!g.out16 && !g.out16t) return;
-    __nv_bfloat16 hv[kNC];
+    if (!g.out16) return;
+    __align__(16) __nv_bfloat16 hv[kNC];
 #pragma unroll
     for (int j = 0; j < kNC; ++j) hv[j] = __float2bfloat16_rn(x[j]);
-    if (g.out16) {
 #pragma unroll
-        for (int j = 0; j < kNC / 8; ++j)
-            *reinterpret_cast<uint4*>(s16 + lane * kS16 + 8 * j) =
-                *reinterpret_cast<const uint4*>(hv + 8 * j);
-        __syncwarp();
+    for (int j = 0; j < kNC / 8; ++j)
+        *reinterpret_cast<uint4*>(s16 + lane * kS16 + 8 * j) =
+            *reinterpret_cast<const uint4*>(hv + 8 * j);
+    __syncwarp();
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int rr = 16 * j + (lane >> 1), q = lane & 1;
-            if (r0 + rr < g.M)
-                *reinterpret_cast<uint4*>(g.out16 + (long long)(r0 + rr) * g.ld16 + c + 8 * q) =
-                    *reinterpret_cast<const uint4*>(s16 + rr * kS16 + 8 * q);
-        }
-        __syncwarp();
+    for (int j = 0; j < 4; ++j) {
+        const int rr = 8 * j + (lane >> 2), q = lane & 3;
+        if (r0 + rr < g.M)
+            *reinterpret_cast<uint4*>(g.out16 + (long long)(r0 + rr) * g.ld16 + c + 8 * q) =
+                *reinterpret_cast<const uint4*>(s16 + rr * kS16 + 8 * q);
     }
-    if (g.out16t) {
-        // column c + j of D is row c + j of the copy: the warp writes 64 bytes a
-        // column (zeros, set above, for rows in [M, rows_t))
-        const int m = r0 + lane;
-        if (m < g.rows_t) {
-#pragma unroll
-            for (int j = 0; j < kNC; ++j) g.out16t[(long long)(c + j) * g.ldt + m] = hv[j];
-        }
-    }
+    __syncwarp();
 }
 
-__global__ void __launch_bounds__(kRowsThreads, 1)
+__global__ void __launch_bounds__(kRowsThreads, kRowsPerSm)
     k_umma_rows(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
                 RowArgs g) {
     extern __shared__ __align__(1024) unsigned char usm_raw[];
     // the swizzle pattern repeats every 1024 bytes: stages start on such a boundary
     unsigned char* usm = usm_raw + ((1024u - (su32(usm_raw) & 1023u)) & 1023u);
     const int nkc = g.K / kKC;  // 64-wide chunks: K = 64 or 256
-    constexpr unsigned abytes = UM * kKC * 2;
-    // stage s: A chunk (UM x kc) then Bt chunk (UN x kc), kChunkBytes apart
-    float* st32 = reinterpret_cast<float*>(usm + kRowStages * kChunkBytes);
-    __nv_bfloat16* st16 = reinterpret_cast<__nv_bfloat16*>(st32 + kRowEpi * 32 * kS32);
-    float* bias_s = reinterpret_cast<float*>(st16 + kRowEpi * 32 * kS16);
-    float* bsum_s = bias_s + UN;  // [kRowEpi][128]: column sums of each warp's half
-    // [0..2] stage full, [3..5] stage free, [6..7] accumulator 0/1 full,
-    // [8..9] accumulator 0/1 drained
-    constexpr int F0 = 0, E0 = kRowStages, AF = 2 * kRowStages, AE = AF + 2;
-    __shared__ __align__(8) uint64_t bar[2 * kRowStages + 4];
+    constexpr unsigned bbytes = kNT * kKC * 2;  // a K chunk of Bt
+    const int col0 = blockIdx.y * kNT;
+    // the A ring, Bt chunk after chunk, the epilogue's staging blocks
+    unsigned char* bsm = usm + kRowStages * kRowChunk;
+    float* st32 = reinterpret_cast<float*>(bsm + kRowB);
+    float* bias_s = st32 + kRowEpi * 32 * kS32;
+    float* bsum_s = bias_s + kNT;  // [kRowEpi][kNT / 2]: column sums of each warp's half
+    // stages full, stages free, accumulator 0/1 full, Bt there, accumulator 0/1 drained
+    constexpr int F0 = 0, E0 = kRowStages, AF = 2 * kRowStages, BF = AF + 2, AE = BF + 1;
+    __shared__ __align__(8) uint64_t bar[AE + 2];
     __shared__ uint32_t tbase;
     __shared__ int abort_s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -496,7 +526,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
                          su32(&tbase)),
-                     "r"(2 * UN)
+                     "r"(2 * kNT)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
@@ -507,8 +537,9 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         abort_s = 0;
     }
-    for (int i = tid; i < UN; i += blockDim.x) bias_s[i] = g.bias ? g.bias[i] : 0.0f;
-    for (int i = tid; i < kRowEpi * (UN / 2); i += blockDim.x) bsum_s[i] = 0.0f;
+    for (int i = tid; i < kRowEpi * (kNT / 2); i += blockDim.x) bsum_s[i] = 0.0f;
+    pdl_prologue();  // what follows reads what the kernels before this one wrote
+    for (int i = tid; i < kNT; i += blockDim.x) bias_s[i] = g.bias ? g.bias[col0 + i] : 0.0f;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -516,25 +547,30 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     volatile int* abort_v = &abort_s;
     if (warp == kRowEpi) {
         if (lane == 0) {
-            // loader: every chunk of every tile through the ring
+            // loader: Bt, then every chunk of every tile through the ring
             int q = 0;  // chunks issued
             bool ok = true;
+            mb_expect(&bar[BF], nkc * bbytes);
+            for (int j = 0; j < nkc; ++j)
+                for (int r = 0; r < kNT; r += kBox)
+                    tma2(bsm + j * bbytes + r * kKC * 2, &tb, j * kKC, col0 + r, &bar[BF]);
             for (int t = blockIdx.x; ok && t < ntiles; t += gridDim.x)
                 for (int j = 0; j < nkc; ++j, ++q) {
                     const int st = q % kRowStages;
                     if (q >= kRowStages)
                         ok = mb_wait(&bar[E0 + st], ((q / kRowStages) - 1) & 1, abort_v);
                     if (!ok) break;
-                    unsigned char* A = usm + st * kChunkBytes;
-                    mb_expect(&bar[F0 + st], (unsigned)kChunkBytes);
-                    tma2(A, &ta, j * kKC, t * UM, &bar[F0 + st]);
-                    tma2(A + abytes, &tb, j * kKC, 0, &bar[F0 + st]);
+                    unsigned char* A = usm + st * kRowChunk;
+                    mb_expect(&bar[F0 + st], (unsigned)kRowChunk);
+                    for (int r = 0; r < UM; r += kBox)
+                        tma2(A + r * kKC * 2, &ta, j * kKC, t * UM + r, &bar[F0 + st]);
                 }
             if (!ok) {
                 atomicExch(g.err, 1);
                 *abort_v = 1;
             }
             // the copies issued last complete before the CTA leaves (bounded)
+            mb_wait(&bar[BF], 0, nullptr);
             for (int r = (q > kRowStages ? q - kRowStages : 0); r < q; ++r)
                 mb_wait(&bar[F0 + r % kRowStages], (r / kRowStages) & 1, nullptr);
         }
@@ -542,20 +578,21 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
         if (lane == 0) {
             // MMA issuer: one accumulator per tile, alternating
             int q = 0, i = 0, committed = -1;
-            bool ok = true;
+            const unsigned B = su32(bsm);
+            bool ok = mb_wait(&bar[BF], 0, abort_v);
             for (int t = blockIdx.x; ok && t < ntiles; t += gridDim.x, ++i) {
                 if (i >= 2) ok = mb_wait(&bar[AE + (i & 1)], ((i - 2) >> 1) & 1, abort_v);
                 if (!ok) break;
-                const uint32_t acc = tmem + (uint32_t)((i & 1) * UN);
+                const uint32_t acc = tmem + (uint32_t)((i & 1) * kNT);
                 for (int j = 0; j < nkc; ++j, ++q) {
                     const int st = q % kRowStages;
                     ok = mb_wait(&bar[F0 + st], (q / kRowStages) & 1, abort_v);
                     if (!ok) break;
                     tc_fence_after();
-                    const unsigned A = su32(usm + st * kChunkBytes);
+                    const unsigned A = su32(usm + st * kRowChunk);
                     for (int kk = 0; kk < kKC / 16; ++kk)
-                        umma(acc, umma_desc(A + kk * 32), umma_desc(A + abytes + kk * 32),
-                             j > 0 || kk > 0);
+                        umma<idesc(kNT, false)>(acc, umma_desc(A + kk * 32),
+                                                umma_desc(B + j * bbytes + kk * 32), j > 0 || kk > 0);
                     umma_commit(&bar[E0 + st]);
                     committed = q;
                 }
@@ -572,13 +609,16 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
         }
     } else {
         float* s32 = st32 + warp * 32 * kS32;
-        __nv_bfloat16* s16 = st16 + warp * 32 * kS16;
-        float* bsum = bsum_s + warp * (UN / 2);
-        const int quarter = warp & 3, c0 = (warp >> 2) * (UN / 2);
+        float* bsum = bsum_s + warp * (kNT / 2);
+        const int quarter = warp & 3, c0 = (warp >> 2) * (kNT / 2);
         const bool need_aux = g.epi == EPI_TANH_BACK || g.epi == EPI_LOSS;
         double sse = 0.0;
         int i = 0;
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
+            // the operand does not depend on the product: on its way during the wait
+            const int r0 = t * UM + quarter * 32;
+            float4 pf[8];
+            if (need_aux) aux_fetch(pf, g.aprev, r0, col0 + c0, g.M, lane);
             bool ok = mb_wait(&bar[AF + (i & 1)], (i >> 1) & 1, abort_v);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) {
@@ -590,28 +630,19 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
             }
             tc_fence_after();
             const uint32_t acc =
-                tmem + (uint32_t)((i & 1) * UN) + ((uint32_t)(quarter * 32) << 16);
-            const int r0 = t * UM + quarter * 32;
-            float4 pf[4];
-            if (need_aux) aux_fetch(pf, g.aprev, r0, c0, g.M, lane);
-            for (int c = c0; c < c0 + UN / 2; c += kNC) {
-                float x[kNC], aux[kNC];
-                tmem_ld16(acc + (uint32_t)c, x);
-                if (need_aux) {
-                    aux_rows(pf, s32, aux, lane);
-                    // the next chunk's operand is on its way while this one is worked
-                    if (c + kNC < c0 + UN / 2) aux_fetch(pf, g.aprev, r0, c + kNC, g.M, lane);
-                }
-                rows_epilogue(g, x, aux, bias_s, s32, s16, r0, c, lane, bsum + (c - c0), sse);
-            }
+                tmem + (uint32_t)((i & 1) * kNT) + ((uint32_t)(quarter * 32) << 16);
+            if (need_aux) aux_stage(pf, s32, lane);
+            float x[kNC];
+            tmem_ld(acc + (uint32_t)c0, x);
+            rows_epilogue(g, x, bias_s + c0, s32, r0, col0 + c0, lane, bsum, sse);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mb_arrive(&bar[AE + (i & 1)]);
         }
         __syncwarp();
         if (g.bpart)
-            for (int j = lane; j < UN / 2; j += 32)
-                g.bpart[((long long)blockIdx.x * 4 + quarter) * UN + c0 + j] = bsum[j];
+            for (int j = lane; j < kNT / 2; j += 32)
+                g.bpart[((long long)blockIdx.x * 4 + quarter) * UN + col0 + c0 + j] = bsum[j];
         if (g.sse) {
             for (int o = 16; o > 0; o >>= 1) sse += __shfl_down_sync(0xffffffffu, sse, o);
             if (lane == 0) atomicAdd(g.sse, sse);
@@ -621,13 +652,12 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
-                     "r"(2 * UN)
+                     "r"(2 * kNT)
                      : "memory");
 }
 
 __global__ void __launch_bounds__(kWgThreads, 1)
-    k_umma_wgrad(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
-                 WgArgs g) {
+    k_umma_wgrad(const __grid_constant__ WgMaps maps, WgArgs g) {
     extern __shared__ __align__(1024) unsigned char usm_raw[];
     unsigned char* usm = usm_raw + ((1024u - (su32(usm_raw) & 1023u)) & 1023u);
     // stage s: A chunk (UM x kKC) then B chunk (UN x kKC)
@@ -640,6 +670,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     __shared__ int abort_s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int mt = blockIdx.x, slice = blockIdx.y;
+    const int layer = (mt + 1) / 2, m0 = mt == 0 ? 0 : ((mt - 1) & 1) * UM;
     const int j0 = slice * g.per_slice;
     const int nk = min(g.per_slice, g.chunks - j0);  // >= 1 by the host's choice of slices
     if (warp == 0) {
@@ -654,6 +685,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         abort_s = 0;
     }
+    pdl_prologue();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -670,8 +702,10 @@ __global__ void __launch_bounds__(kWgThreads, 1)
                 if (!ok) break;
                 unsigned char* A = usm + (size_t)s * (kAbytes + kBbytes);
                 mb_expect(&bar[s], kAbytes + kBbytes);
-                tma2(A, &ta, (j0 + j) * kKC, mt * UM, &bar[s]);
-                tma2(A + kAbytes, &tb, (j0 + j) * kKC, 0, &bar[s]);
+                for (int c = 0; c < UM; c += kKC)
+                    tma2(A + c * kBox * 2, &maps.a[layer], m0 + c, (j0 + j) * kBox, &bar[s]);
+                for (int c = 0; c < UN; c += kKC)
+                    tma2(A + kAbytes + c * kBox * 2, &maps.d[layer], c, (j0 + j) * kBox, &bar[s]);
                 loaded = j + 1;
             }
             if (!ok) {
@@ -694,8 +728,8 @@ __global__ void __launch_bounds__(kWgThreads, 1)
                 tc_fence_after();
                 const unsigned A = su32(usm + (size_t)s * (kAbytes + kBbytes));
                 for (int kk = 0; kk < kKC / 16; ++kk)
-                    umma(tmem, umma_desc(A + kk * 32), umma_desc(A + kAbytes + kk * 32),
-                         j > 0 || kk > 0);
+                    umma<idesc(UN, true)>(tmem, umma_desc_mn(A + kk * 2048),
+                                          umma_desc_mn(A + kAbytes + kk * 2048), j > 0 || kk > 0);
                 umma_commit(&bar[kStages + s]);
                 issued = j + 1;
             }
@@ -717,11 +751,11 @@ __global__ void __launch_bounds__(kWgThreads, 1)
             float* s32 = st32 + warp * 32 * kS32;
             const uint32_t acc = tmem + ((uint32_t)(warp * 32) << 16);
             const int r0 = mt * UM + warp * 32;
-            float* out = g.part + (long long)slice * g.mtiles * UM * UN;
+            float* out = g.part + (long long)slice * kWgTiles * UM * UN;
             for (int c = 0; c < UN; c += kNC) {
                 float x[kNC];
-                tmem_ld16(acc + (uint32_t)c, x);
-                rows_store32(s32, x, out, UN, r0, c, g.mtiles * UM, lane);
+                tmem_ld(acc + (uint32_t)c, x);
+                rows_store32(s32, x, out, UN, r0, c, kWgTiles * UM, lane);
             }
         } else if (lane == 0) {
             atomicExch(g.err, 1);
@@ -736,72 +770,136 @@ __global__ void __launch_bounds__(kWgThreads, 1)
                      : "memory");
 }
 
-// dW[k][n] = sum over slices of part[s][k][n] (k < fi), and db[n] = sum of
-// the nb column-sum rows bpart[p][n] the row kernel left.  A block takes 32
-// outputs with 8 threads each: thread phase y adds rows y, y + 8, ..., and the
-// eight phase sums are added in phase order, so the result does not depend on
-// timing.
-__global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ part, int slices,
-                                                      int rows, int fi, float* __restrict__ gw,
-                                                      const float* __restrict__ bpart, int nb,
-                                                      float* __restrict__ gb) {
-    __shared__ float acc[8][33];
-    const int o = blockIdx.x * 32 + threadIdx.x, y = threadIdx.y;
-    float s = 0.0f;
-    if (o < fi * UN) {
-        for (int q = y; q < slices; q += 8) s += part[(long long)q * rows * UN + o];
-    } else if (o < fi * UN + UN) {
-        const int n = o - fi * UN;
-        for (int q = y; q < nb; q += 8) s += bpart[(long long)q * UN + n];
-    }
-    acc[y][threadIdx.x] = s;
-    __syncthreads();
-    if (y == 0 && o < fi * UN + UN) {
-        float t = acc[0][threadIdx.x];
-        for (int p = 1; p < 8; ++p) t += acc[p][threadIdx.x];
-        if (o < fi * UN) gw[o] = t;
-        else gb[o - fi * UN] = t;
+// One Adam step of one parameter.
+__device__ __forceinline__ float adam(float p, float gi, float* m, float* v, float lr, float c1,
+                                      float c2) {
+    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+    const float mi = b1 * *m + (1.0f - b1) * gi;
+    const float vi = b2 * *v + (1.0f - b2) * gi * gi;
+    *m = mi;
+    *v = vi;
+    return p - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+}
+
+// where the BF16 copies of parameter k of layer l's weights (k = row * 256 + column) go
+__device__ __forceinline__ void store_w16(int l, int k, float p, __nv_bfloat16* w16,
+                                          __nv_bfloat16* w16t) {
+    const __nv_bfloat16 h = __float2bfloat16_rn(p);
+    const int row = k / kW, n = k - row * kW;
+    if (l == 0) {
+        w16[k] = h;
+        w16t[n * kK0 + row] = h;
+    } else {
+        w16[kInPad * kW + (l - 1) * kW * kW + k] = h;
+        w16t[kK0 * kW + (l - 1) * kW * kW + n * kW + row] = h;
     }
 }
 
-// x [B][4] FP32 -> BF16 [B][kK0], zero-padded, and (x16t not null) its transpose
-// [16][ldt] with zeros for b in [B, rows_t)
-__global__ void k_input(const float* __restrict__ x, __nv_bfloat16* __restrict__ x16, int B,
-                        __nv_bfloat16* __restrict__ x16t, int ldt, int rows_t) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < B * kK0) {
-        const int b = i / kK0, k = i - b * kK0;
-        x16[i] = __float2bfloat16_rn(k < kIn ? x[b * kIn + k] : 0.0f);
-    }
-    if (x16t && i < kInPad * rows_t) {
-        const int k = i / rows_t, b = i - k * rows_t;
-        x16t[(long long)k * ldt + b] =
-            __float2bfloat16_rn(k < kIn && b < B ? x[b * kIn + k] : 0.0f);
+struct GradArgs {
+    const float* part;    // [slices][kWgTiles * 128][256]
+    int slices;
+    const float* bpart;   // [layers][kRowGridCap * 4][256]: column sums of each signal
+    int nb;               // rows of it in use
+    float* grad;          // !ADAM: the gradient
+    float *p, *m, *v;     // ADAM: parameters and moments
+    float lr, c1, c2;
+    __nv_bfloat16 *w16, *w16t;
+};
+
+// The parameter's new value from its gradient, or the gradient itself.
+template <bool ADAM>
+__device__ __forceinline__ void take_gradient(const GradArgs& g, int l, int k, bool weight,
+                                              float t) {
+    const int i = (int)param_offset(l) + k;
+    if constexpr (ADAM) {
+        const float p = adam(g.p[i], t, g.m + i, g.v + i, g.lr, g.c1, g.c2);
+        g.p[i] = p;
+        if (weight) store_w16(l, k, p, g.w16, g.w16t);
+    } else {
+        g.grad[i] = t;
     }
 }
 
-// FP32 master weights -> BF16 copies ([fan_in padded][fan_out] for layer 0),
-// and the same transposed ([fan_out][fan_in padded]) for the tensor-core
-// products, whose second operand is K-major
-__global__ void k_weights16(const float* __restrict__ p, __nv_bfloat16* __restrict__ w16,
-                            __nv_bfloat16* __restrict__ w16t) {
-    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const long long n16 = (long long)kInPad * kW + 3LL * kW * kW;
-    if (i >= n16) return;
-    if (i < (long long)kInPad * kW) {
-        const int k = (int)(i / kW), n = (int)(i - (long long)k * kW);
-        const __nv_bfloat16 v = __float2bfloat16_rn(k < kIn ? p[k * kW + n] : 0.0f);
-        w16[i] = v;
-        w16t[(long long)n * kK0 + k] = v;  // columns 16..63 stay zero
+// The gradient: dW[k][n] = sum of part[s][row][n] over the slices, db[n] = sum of the
+// column-sum rows.  Eight running sums (rows q, q + 8, ...) added in order at the end, so
+// the result does not depend on timing: a weight's in one thread (the first kGradW blocks),
+// a bias's in eight (a large batch has 152 rows to add; in one thread they set the kernel's
+// time).  ADAM: the parameter and its BF16 copies are updated with it, which a launch of
+// its own would read back.  65 us at batch 32768 with a bias in one thread, 6.4 so.
+constexpr int kGradW = (kIn * kW + (kLayers - 1) * kW * kW) / 256;  // blocks of weights
+constexpr int kGradB = kLayers * kW / 32;                           // blocks of biases
+template <bool ADAM>
+__global__ void __launch_bounds__(256) k_gradient(GradArgs g) {
+    pdl_prologue();
+    if ((int)blockIdx.x < kGradW) {
+        int k = blockIdx.x * 256 + threadIdx.x, l = 0;
+        if (k >= kIn * kW) {
+            k -= kIn * kW;
+            l = 1 + k / (kW * kW);
+            k -= (l - 1) * kW * kW;
+        }
+        const float* src = g.part + (long long)wg_row0(l) * UN + k;
+        constexpr long long stride = (long long)kWgTiles * UM * UN;
+        float acc[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 2
+        for (int q = 0; q < g.slices; q += 8) {
+            float r[8];
+#pragma unroll
+            for (int y = 0; y < 8; ++y) r[y] = q + y < g.slices ? src[(q + y) * stride] : 0.0f;
+#pragma unroll
+            for (int y = 0; y < 8; ++y) acc[y] += r[y];
+        }
+        float t = acc[0];
+#pragma unroll
+        for (int y = 1; y < 8; ++y) t += acc[y];
+        take_gradient<ADAM>(g, l, k, true, t);
         return;
     }
-    const long long j = i - (long long)kInPad * kW;  // layers 1..3
-    const int l = 1 + (int)(j / (kW * kW));
-    const long long r = j - (long long)(l - 1) * kW * kW;
-    const int k = (int)(r / kW), n = (int)(r - (long long)k * kW);
-    const __nv_bfloat16 v = __float2bfloat16_rn(p[param_offset(l) + r]);
-    w16[i] = v;
-    w16t[(long long)kK0 * kW + (long long)(l - 1) * kW * kW + (long long)n * kW + k] = v;
+    __shared__ float acc[8][33];
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    const int o = ((int)blockIdx.x - kGradW) * 32 + x, l = o / kW, n = o - l * kW;
+    const float* src = g.bpart + (long long)l * kRowGridCap * 4 * UN + n;
+    float s = 0.0f;
+#pragma unroll 8
+    for (int q = y; q < g.nb; q += 8) s += src[q * UN];
+    acc[y][x] = s;
+    __syncthreads();
+    if (y == 0) {
+        float t = acc[0][x];
+#pragma unroll
+        for (int p = 1; p < 8; ++p) t += acc[p][x];
+        take_gradient<ADAM>(g, l, (l == 0 ? kIn : kW) * kW + n, false, t);
+    }
+}
+
+// x [B][4] FP32 -> BF16 [B][kK0], zero-padded; the squared-error sum (not null) cleared
+__global__ void k_input(const float* __restrict__ x, __nv_bfloat16* __restrict__ x16, int B,
+                        double* sse) {
+    pdl_prologue();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0 && sse) *sse = 0.0;
+    // eight of a row's kK0 entries a thread
+    if (i < B * (kK0 / 8)) {
+        const int b = i / (kK0 / 8), k = 8 * (i - b * (kK0 / 8));
+        __align__(16) __nv_bfloat16 h[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            h[j] = __float2bfloat16_rn(k + j < kIn ? x[b * kIn + k + j] : 0.0f);
+        *reinterpret_cast<uint4*>(x16 + (long long)b * kK0 + k) = *reinterpret_cast<uint4*>(h);
+    }
+}
+
+// FP32 master weights -> BF16 copies ([fan_in padded][fan_out] for layer 0; the
+// padding stays zero), and the same transposed ([fan_out][fan_in padded]) for the
+// tensor-core products, whose second operand is K-major
+__global__ void k_weights16(const float* __restrict__ p, __nv_bfloat16* __restrict__ w16,
+                            __nv_bfloat16* __restrict__ w16t) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= kParams) return;
+    int l = 0;
+    while (l + 1 < kLayers && i >= param_offset(l + 1)) ++l;
+    const int k = i - (int)param_offset(l);
+    if (k < (l == 0 ? kIn : kW) * kW) store_w16(l, k, p[i], w16, w16t);
 }
 
 // dL/dy = 2 (y - t) / (B N) (FP32 and BF16), and the squared-error sum
@@ -837,16 +935,9 @@ __global__ void k_bias_grad(const float* __restrict__ d, int B, int N, float* __
 
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                        float* __restrict__ v, long long n, float lr, float c1, float c2) {
-    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.0f - b1) * gi;
-        const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    }
+         i += (long long)gridDim.x * blockDim.x)
+        p[i] = adam(p[i], g[i], m + i, v + i, lr, c1, c2);
 }
 
 }  // namespace
@@ -859,15 +950,13 @@ struct lbm_mlp;
 namespace {
 
 // tensor maps of the tcgen05 products for one batch size (they depend on the
-// batch through the row and K extents)
+// batch through the row extents), all with boxes of 64 x 64
 struct TcMaps {
     int B = -1;
-    CUtensorMap fwdA[kLayers];    // x16, a16[0..2]: [B][K], boxes 128 rows x 64
-    CUtensorMap fwdB[kLayers];    // w16t of each layer: [256][K], boxes 256 x 64
-    CUtensorMap sigA[2];          // d16, e16 (the backward signal as the A operand)
-    CUtensorMap sigB[kLayers];    // w16 of layers 1..3 ([fi][fo] = [256][K = fo])
-    CUtensorMap wgA[kLayers];     // x16t, a16t[0..2]: [fi rows][K = batch], 64-wide K boxes
-    CUtensorMap wgB[2];           // d16t, e16t
+    WgMaps wg;               // a: x16, a16[0..2], also the forward A operands;
+                             // d: the backward signals, also the input gradients' A
+    CUtensorMap wt[kLayers]; // w16t of each layer: [256][K]
+    CUtensorMap w[kLayers];  // w16 of layers 1..3 ([fi][fo] = [256][K = fo])
 };
 
 }  // namespace
@@ -881,20 +970,14 @@ struct lbm_mlp {
     int* err;                    // device word: a tensor-core product's wait ran out
     int* h_err;                  // pinned mirror
     __nv_bfloat16* x16;          // [R][kK0]
-    __nv_bfloat16* x16t;         // [16][R]
     float* a32[kLayers];         // layer outputs, FP32 [R][256]
     __nv_bfloat16* a16[kLayers - 1];   // hidden outputs, BF16 (inputs of the next product)
-    __nv_bfloat16* a16t[kLayers - 1];  // the same transposed, [256][R]
-    float* d32;                  // backward signal, FP32 [R][256]
-    __nv_bfloat16* d16;          // its BF16 copy
-    __nv_bfloat16* d16t;         // transposed, [256][R]
-    float* e32;                  // the previous layer's signal
-    __nv_bfloat16* e16;
-    __nv_bfloat16* e16t;
-    float* part;                 // weight-gradient partials [slices][256][256]
-    float* bpart;                // bias-gradient partials [slices][256]
+    __nv_bfloat16* sig[kLayers]; // backward signal at each layer's output, BF16 [R][256]
+    float *d32, *e32;            // the same in FP32 (mma.sync kernel only), alternating
+    float* part;                 // weight-gradient partials [slices][kWgTiles * 128][256]
+    float* bpart;                // bias-gradient partials [layers][kRowGridCap * 4][256]
     double* sse;                 // device scalar
-    double* h_sse;               // pinned mirror
+    double* h_sse;               // pinned mirror of both
     long long step;
     bool tensor_cores;           // forward and input-gradient products by tcgen05
     TcMaps maps;
@@ -905,25 +988,22 @@ namespace {
 size_t al(size_t v) { return (v + 255) / 256 * 256; }
 
 struct MlpLayout {
-    size_t p, g, m, v, w16, w16t, x16, x16t, a32, a16, a16t, d32, d16, d16t, e32, e16, e16t,
-        part, bpart, sse, err, total;
+    size_t p, g, m, v, w16, w16t, x16, a32, a16, sig, d32, e32, part, bpart, sse, total;
 };
 
-// Rows of the batch-sized buffers: a multiple of 8, so that the tensor copies of
-// 8-row core matrices stay inside the buffers and the transposed copies' rows
-// are whole 16-byte pieces.
-int rows_of(int B) { return (B + 7) / 8 * 8; }
+int rows_of(int B) { return (B + 7) / 8 * 8; }  // rows of the batch-sized buffers
 
-// K slices of the weight gradient for a batch of B: 64-wide chunks, at most
-// kWgSlices slices of equal whole-chunk length
-constexpr int kWgSlices = 74;
+// K slices of the weight gradients for a batch of B: 64-row chunks, one a slice up to
+// kWgSlices; larger batches take as many as make one wave of the launch's CTAs, kWgTiles
+// a slice, which also keeps the partials small (at 32768: 21 slices, 19 MB for all layers).
+constexpr int kWgSlices = 74, kWgWave = 21;
 struct Slicing {
     int chunks, per_slice, slices;
 };
 Slicing slicing(int B) {
     Slicing s;
-    s.chunks = (rows_of(B) + kKC - 1) / kKC;
-    s.per_slice = (s.chunks + kWgSlices - 1) / kWgSlices;
+    s.chunks = (B + kBox - 1) / kBox;
+    s.per_slice = s.chunks <= kWgSlices ? 1 : (s.chunks + kWgWave - 1) / kWgWave;
     s.slices = (s.chunks + s.per_slice - 1) / s.per_slice;
     return s;
 }
@@ -947,20 +1027,14 @@ MlpLayout mlp_layout(int B0) {
     L.w16 = take(((size_t)kInPad * kW + 3ull * kW * kW) * 2);
     L.w16t = take(((size_t)kK0 * kW + 3ull * kW * kW) * 2);
     L.x16 = take(B * kK0 * 2);
-    L.x16t = take(B * kInPad * 2);
     L.a32 = take((size_t)kLayers * B * kW * 4);
     L.a16 = take((size_t)(kLayers - 1) * B * kW * 2);
-    L.a16t = take((size_t)(kLayers - 1) * B * kW * 2);
+    L.sig = take((size_t)kLayers * B * kW * 2);
     L.d32 = take(B * kW * 4);
-    L.d16 = take(B * kW * 2);
-    L.d16t = take(B * kW * 2);
     L.e32 = take(B * kW * 4);
-    L.e16 = take(B * kW * 2);
-    L.e16t = take(B * kW * 2);
-    L.part = take(S * kW * UN * 4);
-    L.bpart = take((size_t)kRowGridCap * 4 * UN * 4);
-    L.sse = take(8);
-    L.err = take(4);
+    L.part = take(S * kWgTiles * UM * UN * 4);
+    L.bpart = take((size_t)kLayers * kRowGridCap * 4 * UN * 4);
+    L.sse = take(16);  // the squared-error sum and the error word, read back together
     L.total = o;
     return L;
 }
@@ -987,7 +1061,7 @@ const __nv_bfloat16* w16t_of(const lbm_mlp* n, int l) {
 // Drain the stream; a tensor-core product whose bounded wait ran out since the
 // last check makes this LBM_ETIMEOUT (and the word is cleared).
 lbm_status sync(lbm_mlp* n) {
-    if (cudaMemcpyAsync(n->h_err, n->err, sizeof(int), cudaMemcpyDeviceToHost, n->stream) !=
+    if (cudaMemcpyAsync(n->h_sse, n->sse, 16, cudaMemcpyDeviceToHost, n->stream) !=
             cudaSuccess ||
         cudaStreamSynchronize(n->stream) != cudaSuccess)
         return LBM_ECUDA;
@@ -1020,15 +1094,15 @@ EncodeTiledFn encoder() {
     return fn;
 }
 
-// Tensor map of a BF16 matrix [rows][kext] (row stride ld elements, a multiple
-// of 8) whose boxes of 64 (K) x box_rows land in shared memory in the
-// 128-byte-swizzle layout; parts of a box outside the matrix arrive as zeros.
-bool sw128_map(const __nv_bfloat16* A, int rows, int kext, int ld, int box_rows, CUtensorMap* m) {
+// Tensor map of a BF16 matrix [rows][cols] (cols a multiple of 8) whose boxes of 64
+// columns x 64 rows land in shared memory in the 128-byte-swizzle layout; parts of a
+// box outside the matrix arrive as zeros.
+bool sw128_map(const __nv_bfloat16* A, int rows, int cols, CUtensorMap* m) {
     const EncodeTiledFn enc = encoder();
     if (!enc) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)kext, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kKC, (cuuint32_t)box_rows};
+    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
+    const cuuint32_t box[2] = {(cuuint32_t)kKC, (cuuint32_t)kBox};
     const cuuint32_t estr[2] = {1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<__nv_bfloat16*>(A), dims,
                strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -1042,20 +1116,14 @@ bool prepare_maps(lbm_mlp* n, int B) {
     TcMaps& t = n->maps;
     if (t.B == B) return true;
     t.B = -1;
-    const int kB = rows_of(B);
     bool ok = true;
     for (int l = 0; l < kLayers; ++l) {
         const int K = l == 0 ? kK0 : kW;
-        ok = ok && sw128_map(l == 0 ? n->x16 : n->a16[l - 1], B, K, K, UM, &t.fwdA[l]);
-        ok = ok && sw128_map(w16t_of(n, l), UN, K, K, UN, &t.fwdB[l]);
-        if (l > 0) ok = ok && sw128_map(w16_of(n, l), UN, kW, kW, UN, &t.sigB[l]);
-        ok = ok && sw128_map(l == 0 ? n->x16t : n->a16t[l - 1], l == 0 ? kInPad : kW, kB, n->R,
-                             UM, &t.wgA[l]);
+        ok = ok && sw128_map(l == 0 ? n->x16 : n->a16[l - 1], B, K, &t.wg.a[l]);
+        ok = ok && sw128_map(n->sig[l], B, kW, &t.wg.d[l]);
+        ok = ok && sw128_map(w16t_of(n, l), UN, K, &t.wt[l]);
+        if (l > 0) ok = ok && sw128_map(w16_of(n, l), UN, kW, &t.w[l]);
     }
-    ok = ok && sw128_map(n->d16, B, kW, kW, UM, &t.sigA[0]);
-    ok = ok && sw128_map(n->e16, B, kW, kW, UM, &t.sigA[1]);
-    ok = ok && sw128_map(n->d16t, UN, kB, n->R, UN, &t.wgB[0]);
-    ok = ok && sw128_map(n->e16t, UN, kB, n->R, UN, &t.wgB[1]);
     if (ok) t.B = B;
     return ok;
 }
@@ -1073,54 +1141,50 @@ cudaError_t set_smem_attrs(int dev) {
     return e;
 }
 
-// CTAs of the persistent row kernel for M rows: one per SM at most, and at
-// most kRowGridCap (the rows of column sums it leaves are sized by that)
-int rows_grid(const lbm_mlp* n, int M) {
+// a launch with programmatic serialization (every kernel here starts with pdl_prologue)
+template <typename... KArgs, typename... Args>
+cudaError_t launch(void (*kern)(KArgs...), dim3 grid, int block, size_t smem, cudaStream_t s,
+                   Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+
+// CTAs that walk the row tiles of one column block for M rows: together kRowsPerSm per SM
+// at most, and at most kRowGridCap (the rows of column sums they leave are sized by that)
+int row_walkers(const lbm_mlp* n, int M) {
     const int tiles = (M + UM - 1) / UM;
-    const int cap = n->nsm < kRowGridCap ? n->nsm : kRowGridCap;
+    int cap = kRowsPerSm * n->nsm / (UN / kNT);
+    cap = cap < 1 ? 1 : (cap < kRowGridCap ? cap : kRowGridCap);
     return tiles < cap ? tiles : cap;
 }
 
 // D[M x 256] = A Bt^T with the epilogue of g
 cudaError_t rows_tc(lbm_mlp* n, const CUtensorMap& ta, const CUtensorMap& tb, const RowArgs& g) {
-    k_umma_rows<<<rows_grid(n, g.M), kRowsThreads, kRowsSmem, n->stream>>>(ta, tb, g);
-    return cudaGetLastError();
+    return launch(k_umma_rows, dim3(row_walkers(n, g.M), UN / kNT), kRowsThreads, kRowsSmem,
+                  n->stream, ta, tb, g);
 }
 
-// gw [fi][256] = A^T D over a batch of B, and gb [256] from the nb column-sum
-// rows that the kernel producing D left in n->bpart
-cudaError_t wgrad_tc(lbm_mlp* n, const CUtensorMap& ta, const CUtensorMap& tb, int fi, int B,
-                     float* gw, int nb, float* gb) {
-    const Slicing sl = slicing(B);
-    const int mtiles = (fi + UM - 1) / UM;
-    WgArgs w;
-    w.mtiles = mtiles;
-    w.chunks = sl.chunks;
-    w.per_slice = sl.per_slice;
-    w.part = n->part;
-    w.err = n->err;
-    k_umma_wgrad<<<dim3(mtiles, sl.slices), kWgThreads, kWgSmem, n->stream>>>(ta, tb, w);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_wgrad_reduce<<<(fi * UN + UN + 31) / 32, dim3(32, 8), 0, n->stream>>>(
-        n->part, sl.slices, mtiles * UM, fi, gw, n->bpart, nb, gb);
-    return cudaGetLastError();
-}
+float* bpart_of(const lbm_mlp* n, int l) { return n->bpart + (size_t)l * kRowGridCap * 4 * UN; }
 
 // forward pass on tcgen05.  t null: inference, only the output (written to y).
 // t not null: training; the hidden layers keep what the backward pass needs
-// (FP32 activations, transposed BF16 copies), and the last layer's epilogue
-// turns its output straight into the loss signal dL/dy (BF16, transposed BF16,
-// column sums) and the squared-error sum, without storing y.
+// (FP32 activations), and the last layer's epilogue turns its output straight into
+// the loss signal dL/dy (BF16, column sums) and the squared-error sum, without
+// storing y.
 lbm_status forward_tc(lbm_mlp* n, const float* x, int B, const float* t, float* y) {
     cudaStream_t s = n->stream;
     const bool train = t != nullptr;
-    const int kB = rows_of(B);
-    const int threads = kK0 * B > kInPad * kB ? kK0 * B : kInPad * kB;
-    k_input<<<(threads + 255) / 256, 256, 0, s>>>(x, n->x16, B, train ? n->x16t : nullptr, n->R,
-                                                  kB);
-    CK(cudaGetLastError());
-    if (train) CK(cudaMemsetAsync(n->sse, 0, sizeof(double), s));
+    CK(launch(k_input, dim3((B * (kK0 / 8) + 255) / 256), 256, 0, s, x, n->x16, B,
+              train ? n->sse : nullptr));
     for (int l = 0; l < kLayers; ++l) {
         const bool hidden = l < kLayers - 1;
         RowArgs g{};
@@ -1129,66 +1193,66 @@ lbm_status forward_tc(lbm_mlp* n, const float* x, int B, const float* t, float* 
         g.bias = n->p + param_offset(l) + (long long)kFanIn[l] * kFanOut[l];
         g.ld32 = kW;
         g.ld16 = kW;
-        g.ldt = n->R;
-        g.rows_t = kB;
         g.err = n->err;
         if (hidden) {
             g.epi = EPI_BIAS_TANH;
             g.out32 = train ? n->a32[l] : nullptr;
             g.out16 = n->a16[l];
-            g.out16t = train ? n->a16t[l] : nullptr;
         } else if (train) {
             g.epi = EPI_LOSS;
             g.aprev = t;
             g.scale = 1.0f / ((float)B * kOut);
             g.sse = n->sse;
-            g.out16 = n->d16;
-            g.out16t = n->d16t;
-            g.bpart = n->bpart;
+            g.out16 = n->sig[l];
+            g.bpart = bpart_of(n, l);
         } else {
             g.epi = EPI_BIAS;
             g.out32 = y;
         }
-        CK(rows_tc(n, n->maps.fwdA[l], n->maps.fwdB[l], g));
+        CK(rows_tc(n, n->maps.wg.a[l], n->maps.wt[l], g));
     }
     return LBM_OK;
 }
 
-// the gradient on tcgen05, after forward_tc with targets
+// the backward pass on tcgen05, after forward_tc with targets: the signals of the hidden
+// layers and the partial weight gradients
 lbm_status backward_tc(lbm_mlp* n, int B) {
-    int sig = 0;  // which of (d, e) holds the current signal
-    for (int l = kLayers - 1; l >= 0; --l) {
-        const int fi = kFanIn[l], fo = kFanOut[l];
-        float* gw = n->g + param_offset(l);
-        float* gb = gw + (long long)fi * fo;
-        // dW = A_{l-1}^T D from the transposed copies; db from the column sums
-        CK(wgrad_tc(n, n->maps.wgA[l], n->maps.wgB[sig], fi, B, gw, 4 * rows_grid(n, B), gb));
-        if (l == 0) break;
-        // D_{l-1} = (D W_l^T) (1 - A_{l-1}^2): K-major operands are D [B][fo] and
+    for (int l = kLayers - 1; l > 0; --l) {
+        // D_{l-1} = (D_l W_l^T) (1 - A_{l-1}^2): K-major operands are D [B][fo] and
         // W_l itself ([fi][fo])
         RowArgs g{};
         g.M = B;
-        g.K = fo;
+        g.K = kW;
         g.epi = EPI_TANH_BACK;
         g.aprev = n->a32[l - 1];
-        g.out16 = sig == 0 ? n->e16 : n->d16;
-        g.ld16 = fi;
-        g.out16t = sig == 0 ? n->e16t : n->d16t;
-        g.ldt = n->R;
-        g.rows_t = rows_of(B);
-        g.bpart = n->bpart;
+        g.out16 = n->sig[l - 1];
+        g.ld16 = kW;
+        g.bpart = bpart_of(n, l - 1);
         g.err = n->err;
-        CK(rows_tc(n, n->maps.sigA[sig], n->maps.sigB[l], g));
-        sig ^= 1;
+        CK(rows_tc(n, n->maps.wg.d[l], n->maps.w[l], g));
     }
+    const Slicing sl = slicing(B);
+    const WgArgs w{sl.chunks, sl.per_slice, n->part, n->err};
+    CK(launch(k_umma_wgrad, dim3(kWgTiles, sl.slices), kWgThreads, kWgSmem, n->stream,
+              n->maps.wg, w));
+    return LBM_OK;
+}
+
+// the gradient from the partial sums of backward_tc: into grad, or (grad null) into one
+// Adam step of the parameters
+lbm_status gradient_tc(lbm_mlp* n, int B, float* grad, float lr, float c1, float c2) {
+    const GradArgs g{n->part, slicing(B).slices, n->bpart, 4 * row_walkers(n, B), grad,
+                     n->p, n->m, n->v, lr, c1, c2, n->w16, n->w16t};
+    CK(launch(grad ? k_gradient<false> : k_gradient<true>, dim3(kGradW + kGradB), 256, 0,
+              n->stream, g));
     return LBM_OK;
 }
 
 // the mma.sync forward pass (every layer's FP32 output kept)
 lbm_status forward_ms(lbm_mlp* n, const float* x, int B) {
     cudaStream_t s = n->stream;
-    k_input<<<(B * kK0 + 255) / 256, 256, 0, s>>>(x, n->x16, B, nullptr, 0, 0);
-    CK(cudaGetLastError());
+    CK(launch(k_input, dim3((B * (kK0 / 8) + 255) / 256), 256, 0, s, x, n->x16, B,
+              (double*)nullptr));
     for (int l = 0; l < kLayers; ++l) {
         GemmArgs g{};
         g.A = l == 0 ? n->x16 : n->a16[l - 1];
@@ -1229,12 +1293,12 @@ lbm_status backward_ms(lbm_mlp* n, const float* t, int B) {
     CK(cudaMemsetAsync(n->sse, 0, sizeof(double), s));
     const int total = B * kOut;
     k_loss_grad<<<(total + 255) / 256 < 1024 ? (total + 255) / 256 : 1024, 256, 0, s>>>(
-        n->a32[kLayers - 1], t, total, 1.0f / (float)total, n->d32, n->d16, n->sse);
+        n->a32[kLayers - 1], t, total, 1.0f / (float)total, n->d32, n->sig[1], n->sse);
     CK(cudaGetLastError());
     float* d32 = n->d32;
-    __nv_bfloat16* d16 = n->d16;
+    __nv_bfloat16* d16 = n->sig[1];
     float* e32 = n->e32;
-    __nv_bfloat16* e16 = n->e16;
+    __nv_bfloat16* e16 = n->sig[0];
     for (int l = kLayers - 1; l >= 0; --l) {
         const int fi = kFanIn[l], fo = kFanOut[l];
         float* gw = n->g + param_offset(l);
@@ -1280,10 +1344,54 @@ lbm_status backward_ms(lbm_mlp* n, const float* t, int B) {
 }
 
 lbm_status refresh_w16(lbm_mlp* n) {
-    const long long n16 = (long long)kInPad * kW + 3LL * kW * kW;
-    k_weights16<<<(unsigned)((n16 + 255) / 256), 256, 0, n->stream>>>(n->p, n->w16, n->w16t);
+    k_weights16<<<(unsigned)((kParams + 255) / 256), 256, 0, n->stream>>>(n->p, n->w16, n->w16t);
     CK(cudaGetLastError());
     return LBM_OK;
+}
+
+// Forward and backward pass of a batch, then one of: the gradient into d_grad, the
+// gradient kept inside (d_grad null), an Adam step (lr > 0); and the loss (h_loss not
+// null, which waits).
+lbm_status train(lbm_mlp* n, const float* x, const float* t, int B, float lr, float* d_grad,
+                 double* h_loss) {
+    if (!n || !x || !t || B < 1 || B > n->max_batch) return LBM_EINVAL;
+    CK(cudaSetDevice(n->dev));
+    lbm_status st = LBM_OK;
+    const bool tc = use_tc(n, B, &st);
+    if (st) return st;
+    auto loss = [&]() -> lbm_status {
+        if (!h_loss) return LBM_OK;
+        const lbm_status w = sync(n);
+        if (w) return w;
+        *h_loss = *n->h_sse / ((double)B * kOut);
+        return LBM_OK;
+    };
+    float c1 = 0.0f, c2 = 0.0f;
+    auto corrections = [&] {
+        n->step += 1;
+        c1 = (float)(1.0 - std::pow(0.9, (double)n->step));
+        c2 = (float)(1.0 - std::pow(0.999, (double)n->step));
+    };
+    if (tc) {
+        st = forward_tc(n, x, B, t, nullptr);
+        if (!st) st = backward_tc(n, B);
+        if (!st && !(lr > 0)) st = gradient_tc(n, B, d_grad ? d_grad : n->g, 0.0f, 0.0f, 0.0f);
+        if (!st) st = loss();  // (a wait that ran out is reported before the step is taken)
+        if (st || !(lr > 0)) return st;
+        corrections();
+        return gradient_tc(n, B, nullptr, lr, c1, c2);
+    }
+    st = forward_ms(n, x, B);
+    if (!st) st = backward_ms(n, t, B);
+    if (st) return st;
+    if (d_grad)
+        CK(cudaMemcpyAsync(d_grad, n->g, kParams * 4, cudaMemcpyDeviceToDevice, n->stream));
+    st = loss();
+    if (st || !(lr > 0)) return st;
+    corrections();
+    k_adam<<<592, 256, 0, n->stream>>>(n->p, n->g, n->m, n->v, kParams, lr, c1, c2);
+    CK(cudaGetLastError());
+    return refresh_w16(n);
 }
 
 }  // namespace
@@ -1321,24 +1429,18 @@ lbm_status lbm_mlp_init(lbm_mlp** out, int32_t max_batch, void* d_ws, size_t byt
     n->w16 = (__nv_bfloat16*)(w + L.w16);
     n->w16t = (__nv_bfloat16*)(w + L.w16t);
     n->x16 = (__nv_bfloat16*)(w + L.x16);
-    n->x16t = (__nv_bfloat16*)(w + L.x16t);
     n->R = rows_of(max_batch);
     const size_t R = (size_t)n->R;
     for (int l = 0; l < kLayers; ++l) n->a32[l] = (float*)(w + L.a32) + (size_t)l * R * kW;
-    for (int l = 0; l < kLayers - 1; ++l) {
+    for (int l = 0; l < kLayers - 1; ++l)
         n->a16[l] = (__nv_bfloat16*)(w + L.a16) + (size_t)l * R * kW;
-        n->a16t[l] = (__nv_bfloat16*)(w + L.a16t) + (size_t)l * R * kW;
-    }
-    n->err = (int*)(w + L.err);
+    for (int l = 0; l < kLayers; ++l) n->sig[l] = (__nv_bfloat16*)(w + L.sig) + (size_t)l * R * kW;
     n->d32 = (float*)(w + L.d32);
-    n->d16 = (__nv_bfloat16*)(w + L.d16);
-    n->d16t = (__nv_bfloat16*)(w + L.d16t);
     n->e32 = (float*)(w + L.e32);
-    n->e16 = (__nv_bfloat16*)(w + L.e16);
-    n->e16t = (__nv_bfloat16*)(w + L.e16t);
     n->part = (float*)(w + L.part);
     n->bpart = (float*)(w + L.bpart);
     n->sse = (double*)(w + L.sse);
+    n->err = (int*)(n->sse + 1);
     n->step = 0;
     n->tensor_cores = true;
     if (cudaDeviceGetAttribute(&n->nsm, cudaDevAttrMultiProcessorCount, n->dev) != cudaSuccess ||
@@ -1346,15 +1448,11 @@ lbm_status lbm_mlp_init(lbm_mlp** out, int32_t max_batch, void* d_ws, size_t byt
         delete n;
         return LBM_ECUDA;
     }
-    if (cudaMallocHost((void**)&n->h_sse, sizeof(double)) != cudaSuccess) {
+    if (cudaMallocHost((void**)&n->h_sse, 16) != cudaSuccess) {
         delete n;
         return LBM_ECUDA;
     }
-    if (cudaMallocHost((void**)&n->h_err, sizeof(int)) != cudaSuccess) {
-        cudaFreeHost(n->h_sse);
-        delete n;
-        return LBM_ECUDA;
-    }
+    n->h_err = (int*)(n->h_sse + 1);
     if (cudaMemsetAsync(w, 0, L.total, n->stream) != cudaSuccess) {
         lbm_mlp_free(n);
         return LBM_ECUDA;
@@ -1375,7 +1473,6 @@ void lbm_mlp_free(lbm_mlp* n) {
     if (!n) return;
     cudaSetDevice(n->dev);
     if (n->h_sse) cudaFreeHost(n->h_sse);
-    if (n->h_err) cudaFreeHost(n->h_err);
     delete n;
 }
 
@@ -1413,41 +1510,13 @@ lbm_status lbm_mlp_forward(lbm_mlp* n, const float* d_x, int32_t batch, float* d
 
 lbm_status lbm_mlp_loss_grad(lbm_mlp* n, const float* d_x, const float* d_t, int32_t batch,
                              double* h_loss, float* d_grad) {
-    if (!n || !d_x || !d_t || batch < 1 || batch > n->max_batch) return LBM_EINVAL;
-    CK(cudaSetDevice(n->dev));
-    lbm_status st = LBM_OK;
-    const bool tc = use_tc(n, batch, &st);
-    if (st) return st;
-    if (tc) {
-        st = forward_tc(n, d_x, batch, d_t, nullptr);
-        if (!st) st = backward_tc(n, batch);
-    } else {
-        st = forward_ms(n, d_x, batch);
-        if (!st) st = backward_ms(n, d_t, batch);
-    }
-    if (st) return st;
-    if (d_grad)
-        CK(cudaMemcpyAsync(d_grad, n->g, kParams * 4, cudaMemcpyDeviceToDevice, n->stream));
-    if (h_loss) {
-        CK(cudaMemcpyAsync(n->h_sse, n->sse, 8, cudaMemcpyDeviceToHost, n->stream));
-        st = sync(n);
-        if (st) return st;
-        *h_loss = *n->h_sse / ((double)batch * kOut);
-    }
-    return LBM_OK;
+    return train(n, d_x, d_t, batch, 0.0f, d_grad, h_loss);
 }
 
 lbm_status lbm_mlp_train_step(lbm_mlp* n, const float* d_x, const float* d_t, int32_t batch,
                               float lr, double* h_loss) {
     if (!n || !(lr > 0)) return LBM_EINVAL;
-    lbm_status st = lbm_mlp_loss_grad(n, d_x, d_t, batch, h_loss, nullptr);
-    if (st) return st;
-    n->step += 1;
-    const float c1 = (float)(1.0 - std::pow(0.9, (double)n->step));
-    const float c2 = (float)(1.0 - std::pow(0.999, (double)n->step));
-    k_adam<<<592, 256, 0, n->stream>>>(n->p, n->g, n->m, n->v, kParams, lr, c1, c2);
-    CK(cudaGetLastError());
-    return refresh_w16(n);
+    return train(n, d_x, d_t, batch, lr, nullptr, h_loss);
 }
 
 }  // extern "C"
