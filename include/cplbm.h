@@ -146,7 +146,7 @@ lbm_status lbm_set_fields_device(lbm_ctx *ctx, const double *d_rho, const double
                                  const double *d_uy);
 
 /* Advance n >= 0 time steps.  Steps are enqueued (in CUDA graphs of two
- * steps); the call then waits for the stream and checks the device error
+ * steps; small periodic MIXED grids run many steps in one launch); the call then waits for the stream and checks the device error
  * flag.  LBM_EUNSTABLE: some step produced a bad value, lbm_failed_step()
  * names the first time level flagged, and the state is undefined until the
  * next lbm_set_fields. */
@@ -193,7 +193,9 @@ lbm_status lbm_set_collide_form(lbm_ctx *ctx, int32_t ring_rows);
  *   single_graph  1: a lone step (lbm_step_async of one step, or the odd last
  *                 step of a longer call) replays a captured one-step CUDA graph;
  *                 0: its passes are launched directly.  Longer calls always
- *                 replay graphs of 2 and 16 steps.
+ *                 replay graphs of 2 and 16 steps.  Periodic MIXED grids of a few
+ *                 thousand nodes (at most 8192) with FP32 density lines run
+ *                 whole steps in one cluster launch instead, in every mode.
  *   pdl_direct, pdl_graphs  programmatic dependent launch between the kernels
  *                 of a mixed step, for direct launches and for graph-captured
  *                 ones: each kernel lets the next be scheduled once all of its
@@ -363,7 +365,8 @@ lbm_status lbm_batch_autotune(lbm_batch *b, int32_t reps);
 /* The strip height in use for instance i (rows of the collide-stream warps). */
 int32_t lbm_batch_tile_rows(const lbm_batch *b, int32_t i);
 
-/* Lines per block (8 or 16) of the batch's FP32 line launches: the density
+/* Lines per block (8 or 16 full-length windows; short lines share a block in larger
+ * numbers) of the batch's FP32 line launches: the density
  * lines of the instances below the double-float ratio, and every instance's
  * force lines (lbm_batch_autotune times both and keeps the faster; the
  * double-float density lines always take 8).  Results do not depend on it.

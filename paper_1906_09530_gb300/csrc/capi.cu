@@ -12,6 +12,7 @@
 // Mixed path: four passes -- collide-stream; the x- and y-lines of rho in one
 // launch (d_x, d_xx, d_y, d_yy rho); mu-hat pointwise (stored over d_xx rho);
 // the x- and y-lines of mu-hat in one launch with the force epilogue.
+// Small periodic grids run whole steps of these passes in one launch (lines32.cu).
 // Passes after the first compute the force of the new time level;
 // lbm_set_fields runs them once on the initial density.  Each needs its input
 // complete over whole lines or all nodes, so they are separate launches.
@@ -66,6 +67,7 @@ struct lbm_ctx {
     int64_t t;
     int64_t failed;
     bool ready;      // fields set
+    bool small;      // steps run whole in one launch (launch_small_steps)
     cudaGraphExec_t graph[2];    // two steps, starting from f[0] / f[1]
     cudaGraphExec_t graph16[2];  // kLongGraph steps, likewise (fewer graph launches)
     cudaGraphExec_t graph1[2];   // one step, for single steps when single_graph is set
@@ -135,18 +137,26 @@ lbm_status enqueue_force(lbm_ctx* c, cudaStream_t s, int bump, int fcur,
     launch_pdl_on() = c->pdl_now;
     auto mark = [&](int i) { return ev ? cudaEventRecord(ev[i], s) : cudaSuccess; };
     if (!is_fp64(c)) {
+        const bool lines32 = (long long)nx * ny <= kLines32Nodes;
         // x|y lines of rho together, mu-hat pointwise, x|y lines of mu-hat + force
         if (c->rho_df)
             CK(lines_mixed_rho_xy(c->m_rh, c->m_rl, c->m_dxr, c->m_dxx, c->m_dyr, c->m_dyy, nx,
                                   ny, o, c->dst, bump, s, c->walls_y));
+        else if (lines32)
+            CK(lines32_rho(c->m_rh, c->m_dxr, c->m_dxx, c->m_dyr, c->m_dyy, nx, ny, o, c->dst,
+                           bump, s, c->walls_y));
         else
             CK(lines_mixed_rho_xy_f32(c->m_rh, c->m_dxr, c->m_dxx, c->m_dyr, c->m_dyy, nx, ny, o,
                                       c->dst, bump, s, c->walls_y));
         CK(mark(0));
         CK(launch_mu_mixed(c->m_rh, c->m_dxx, c->m_dyy, nx, ny, c->phys, c->dst, s));
         CK(mark(1));
-        CK(lines_mixed_force_xy(c->m_dxx, c->m_rh, c->m_dxr, c->m_dyr, c->m_Fx, c->m_Fy, nx, ny,
-                                o, s, c->walls_y, c->dst));
+        if (lines32)
+            CK(lines32_force(c->m_dxx, c->m_rh, c->m_dxr, c->m_dyr, c->m_Fx, c->m_Fy, nx, ny, o,
+                             c->dst, s, c->walls_y));
+        else
+            CK(lines_mixed_force_xy(c->m_dxx, c->m_rh, c->m_dxr, c->m_dyr, c->m_Fx, c->m_Fy, nx,
+                                    ny, o, s, c->walls_y, c->dst));
         CK(mark(2));
         CK(mark(3));
         return LBM_OK;
@@ -182,6 +192,14 @@ lbm_status enqueue_collide(lbm_ctx* c, cudaStream_t s, int from) {
                            c->m_rh, c->m_rl, c->nx, c->ny, c->plane, c->phys.omega,
                            c->mrt ? &c->rates : nullptr, c->dst, s, c->walls, c->ring_rows));
     return LBM_OK;
+}
+
+// the context as launch_small_steps takes it
+SmallStep small_step(const lbm_ctx* c) {
+    return SmallStep{{(float*)c->f[0], (float*)c->f[1]},
+                     MixedLinesView{c->m_rh, c->m_rl, c->m_dxr, c->m_dyr, c->m_dxx, c->m_dyy,
+                                    c->m_Fx, c->m_Fy, c->nx, c->ny, c->dst},
+                     c->plane, c->phys, c->mrt ? &c->rates : nullptr, c->fd_order};
 }
 
 // One full time step starting from f[from]; leaves the state in f[1-from].
@@ -404,6 +422,7 @@ lbm_status lbm_init(lbm_ctx** out, const lbm_grid* grid, const lbm_eos* eos, dou
     c->failed = -1;
     c->timeout_s = 600.0;
     c->cur = 0;
+    c->small = !is_fp64(c) && !c->rho_df && !c->walls_y && small_steps_fit(small_step(c));
     if (cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev, cudaEventDisableTiming) != cudaSuccess ||
         cudaMallocHost((void**)&c->hst, sizeof(DevState)) != cudaSuccess) {
@@ -529,6 +548,12 @@ lbm_status lbm_step_async(lbm_ctx* c, int64_t n) {
     lbm_status st = use_dev(c);
     if (st) return st;
     int64_t left = n;
+    if (c->small) {
+        CK(launch_small_steps(small_step(c), c->cur, n, c->stream));
+        c->cur = (int)((c->cur + n) & 1);
+        c->t += n;
+        return LBM_OK;
+    }
     if (left >= kLongGraph) {
         st = build_graph(c, c->cur, kLongGraph, &c->graph16[c->cur]);
         if (st) return st;

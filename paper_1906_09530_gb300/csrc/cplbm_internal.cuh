@@ -213,7 +213,7 @@ struct MixedLinesView {
 CsArgs cs_mixed_args(const float* fin, float* fout, const float* Fx, const float* Fy,
                      float* rh, float* rl, int nx, int ny, size_t plane, double omega,
                      const MrtRates* mrt, DevState* st,
-                     int rows,  // rows <= 0: the default choice
+                     int rows,  // 0: the default of a batch member, < 0: of a lone grid
                      const Walls& walls = Walls());
 int cs_mixed_blocks(const CsArgs& a);
 cudaError_t launch_cs_mixed_args(const CsArgs& a, cudaStream_t s);
@@ -222,6 +222,62 @@ cudaError_t launch_cs_mixed_batch(const CsBatchInst* d, const int* map, int nblo
 MuConstF mu_mixed_const(const PhysParams& p);
 cudaError_t launch_mu_mixed_batch(const MuBatchInst* d, const int* map, int nblocks,
                                   cudaStream_t s);
+// ---- FP32 line solves (lines32.cuh, lines32.cu) ----
+constexpr int kC32 = 19;  // positions of a chunk (odd: chunk starts hit distinct banks)
+// One direction's windows; see lines32.cuh.
+struct Geo32 {
+    int n, nlines;            // line length, lines
+    long long ps, ls;         // stride along a line, between lines
+    int H, own, nwin;         // halo, owned positions of a window, windows a line
+    int nch;                  // chunks solved of a window's 32
+    int nl, ngroups;          // lines a block, line groups
+    int vec;                  // nx a multiple of 4: 16-byte pieces
+    int period, mirror;       // n, or 2 n with positions n .. 2n-1 reading 2n-1-p (walls)
+    int lift;                 // multiple of the period that makes window starts positive
+    unsigned magic;           // ceil(2^32 / period) for periods shorter than a window, else 0
+};
+struct Dir32 {
+    Geo32 g;
+    const float* u;           // the field solved (density, or mu-hat)
+    const float *rho, *dr;    // force: density and its derivative along the line
+    float *o1, *o2;           // first and second derivative, or the force
+};
+struct Lines32Inst {          // one instance of a batch
+    Dir32 x, y;
+    int nbx, blk0;            // x-line blocks, first block in the launch
+    DevState* st;
+};
+cudaError_t lines32_rho(const float* rh, float* dxr, float* dxx, float* dyr, float* dyy, int nx,
+                        int ny, int order, DevState* st, int bump, cudaStream_t s,
+                        bool walls_y = false);
+cudaError_t lines32_force(const float* mu, const float* rh, const float* dxr, const float* dyr,
+                          float* Fx, float* Fy, int nx, int ny, int order, DevState* st,
+                          cudaStream_t s, bool walls_y = false);
+// Grids whose FP32 lines they solve.  Larger ones keep the full windows of
+// kernels_lines.cu: 1024^2 37.1 us a step against 35.4, 4096^2 499 against 471; 512^2 17.4
+// against 20.1.
+constexpr long long kLines32Nodes = 1LL << 19;
+// nl (8 or 16): blocks of 32 nl threads
+int lines32_batch_blocks(int nx, int ny, int order, bool second, int nl);
+Lines32Inst lines32_batch_inst(const MixedLinesView& v, int order, bool second, int blk0, int nl);
+cudaError_t lines32_batch_launch(const Lines32Inst* d, const int* map, int nblocks, int order,
+                                 bool second, int bump, int nl, cudaStream_t s);
+
+// Whole steps of a small periodic grid in one launch (FP32 density lines).
+struct SmallStep {
+    float* f[2];
+    MixedLinesView v;
+    size_t plane;
+    PhysParams phys;
+    const MrtRates* mrt;
+    int order;
+};
+constexpr long long kSmallNodes = 1 << 13;  // largest grid it is used for
+constexpr int64_t kSmallSteps = 512;        // steps a launch (a few milliseconds)
+// whether the grid and the device allow it (also makes the kernel ready to launch)
+bool small_steps_fit(const SmallStep& p);
+cudaError_t launch_small_steps(const SmallStep& p, int from, int64_t steps, cudaStream_t s);
+
 // Line passes: descriptor size per instance, blocks per instance, descriptor
 // written to host memory (copied to the device by the caller), the launches.
 enum class LineBatchKind {

@@ -507,11 +507,19 @@ bool& launch_pdl_on() {
 CsArgs cs_mixed_args(const float* fin, float* fout, const float* Fx, const float* Fy,
                      float* rh, float* rl, int nx, int ny, size_t plane, double omega,
                      const MrtRates* mrt, DevState* st, int rows, const Walls& walls) {
-    // rows per warp: 32 on large grids, fewer on small ones to keep >= ~4k warps
     const int nstrips = (nx + 29) / 30;
     if (rows <= 0) {
+        // rows per warp: 32 on large grids, fewer on smaller ones to keep >= ~4k warps, down
+        // to 8 (each warp also collides a row on either side); a lone grid (rows < 0) that
+        // still leaves the SMs short of warps goes on to 4, 2 and 1, as long as there are
+        // fewer than 1300.  Steps with 8 / 4 / 2 / 1 rows: 8 x 400 14.1 / 12.7 / 11.9 / 11.7
+        // us, 128^2 15.1 / 13.1 / 12.2 / 11.7, 333 x 277 20.4 / 18.7 / 17.9 / 18.3, 512^2
+        // 17.4 / 16.3 / 16.4 / 17.9.
+        auto warps = [&](int r) { return (long long)nstrips * ((ny + r - 1) / r); };
+        const bool lone = rows < 0;
         rows = 32;
-        while (rows > 8 && (long long)nstrips * ((ny + rows - 1) / rows) < 4096) rows /= 2;
+        while (rows > 8 && warps(rows) < 4096) rows /= 2;
+        while (lone && rows > 1 && warps(rows) < 1300) rows /= 2;
     }
     CsArgs a{fin, fout, Fx, Fy, rh, rl, nx, ny, plane, (float)omega, nstrips,
              (ny + rows - 1) / rows, rows, st, mrt ? 1 : 0,
@@ -561,7 +569,7 @@ cudaError_t launch_cs_mixed(const float* fin, float* fout, const float* Fx, cons
                             const MrtRates* mrt, DevState* st, cudaStream_t s,
                             const Walls& walls, int ring_rows) {
     const CsArgs a =
-        cs_mixed_args(fin, fout, Fx, Fy, rh, rl, nx, ny, plane, omega, mrt, st, 0, walls);
+        cs_mixed_args(fin, fout, Fx, Fy, rh, rl, nx, ny, plane, omega, mrt, st, -1, walls);
     if (!cs_ring_used(nx, ny, plane, fin, Fx, Fy, walls.on, ring_rows))
         return launch_cs_mixed_args(a, s);
     const CsArgs r = cs_ring_args(a, ring_rows);
@@ -627,7 +635,8 @@ MuConstF mu_mixed_const(const PhysParams& p) {
 cudaError_t launch_mu_mixed(const float* rh, float* dxx_mu, const float* dyy, int nx, int ny,
                             const PhysParams& p, DevState* st, cudaStream_t s) {
     const size_t N = (size_t)nx * ny;
-    return launch_pdl(k_mu_mixed, grid_for((N + 3) / 4, 256), 256, 0, s, rh, dxx_mu, dyy, N,
+    // (blocks of 128: with 256 a grid of 3e5 nodes took 8.1 us with the PR EOS instead of 6.2)
+    return launch_pdl(k_mu_mixed, grid_for((N + 3) / 4, 128), 128, 0, s, rh, dxx_mu, dyy, N,
                       mu_mixed_const(p), st);
 }
 
