@@ -124,6 +124,8 @@ Layout layout(int nx, int ny, int prec) {
     } while (0)
 
 bool is_fp64(const lbm_ctx* c) { return c->prec == LBM_PREC_FP64; }
+// the density's low part, where the line solves read it (null: not kept by the steps)
+float* rl_of(const lbm_ctx* c) { return c->rho_df ? c->m_rl : nullptr; }
 
 lbm_status use_dev(lbm_ctx* c) {
     CK(cudaSetDevice(c->dev));
@@ -140,8 +142,8 @@ lbm_status enqueue_force(lbm_ctx* c, cudaStream_t s, int bump, int fcur,
         const bool lines32 = (long long)nx * ny <= kLines32Nodes;
         // x|y lines of rho together, mu-hat pointwise, x|y lines of mu-hat + force
         if (c->rho_df)
-            CK(lines_mixed_rho_xy(c->m_rh, c->m_rl, c->m_dxr, c->m_dxx, c->m_dyr, c->m_dyy, nx,
-                                  ny, o, c->dst, bump, s, c->walls_y));
+            CK(lines_df_rho(c->m_rh, c->m_rl, c->m_dxr, c->m_dxx, c->m_dyr, c->m_dyy, nx, ny, o,
+                            c->dst, bump, s, c->walls_y));
         else if (lines32)
             CK(lines32_rho(c->m_rh, c->m_dxr, c->m_dxx, c->m_dyr, c->m_dyy, nx, ny, o, c->dst,
                            bump, s, c->walls_y));
@@ -189,7 +191,7 @@ lbm_status enqueue_collide(lbm_ctx* c, cudaStream_t s, int from) {
                                  c->mrt ? &c->rates : nullptr, c->dst, s, c->walls));
     else
         CK(launch_cs_mixed((const float*)c->f[from], (float*)c->f[to], c->m_Fx, c->m_Fy,
-                           c->m_rh, c->m_rl, c->nx, c->ny, c->plane, c->phys.omega,
+                           c->m_rh, rl_of(c), c->nx, c->ny, c->plane, c->phys.omega,
                            c->mrt ? &c->rates : nullptr, c->dst, s, c->walls, c->ring_rows));
     return LBM_OK;
 }
@@ -253,7 +255,9 @@ lbm_status wait_stream(lbm_ctx* c) {
         const double el =
             std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
         if (el > c->timeout_s) return LBM_ETIMEOUT;
-        std::this_thread::sleep_for(std::chrono::microseconds(el < 0.01 ? 5 : 200));
+        // a sleep of 5 us takes about 60: short waits are polled through
+        if (el > 3e-4)
+            std::this_thread::sleep_for(std::chrono::microseconds(el < 0.01 ? 5 : 200));
     }
 }
 
@@ -618,7 +622,7 @@ static lbm_status fields_to_device(lbm_ctx* c, double* rho, double* vx, double* 
                                    double* mu) {
     const size_t B = c->N * sizeof(double);
     if (!is_fp64(c)) {
-        CK(launch_macro_mixed((const float*)c->f[c->cur], c->m_rh, c->m_rl, c->m_Fx, c->m_Fy,
+        CK(launch_macro_mixed((const float*)c->f[c->cur], c->m_rh, rl_of(c), c->m_Fx, c->m_Fy,
                               c->m_dxx /* holds mu-hat */, rho, vx, vy, mu, c->nx, c->ny,
                               c->plane, c->stream));
         return LBM_OK;
@@ -729,7 +733,7 @@ lbm_status cplbm_diag_with_partials(lbm_ctx* c, double* partials, int nparts, do
         CK(launch_diag((const double*)c->f[c->cur], c->rho, c->Fx, c->Fy, c->nx, c->ny,
                                c->plane, partials, nparts, c->dst, c->stream));
     else
-        CK(launch_diag_mixed((const float*)c->f[c->cur], c->m_rh, c->m_rl, c->m_Fx, c->m_Fy,
+        CK(launch_diag_mixed((const float*)c->f[c->cur], c->m_rh, rl_of(c), c->m_Fx, c->m_Fy,
                              c->nx, c->ny, c->plane, partials, nparts, c->dst, c->stream));
     st = read_state(c);
     if (st) return st;
@@ -769,8 +773,8 @@ lbm_status lbm_cfd_df(const float* d_hi, const float* d_lo, float* d_d1, float* 
     for (const void* o : outs)
         if (o && (o == (const void*)d_hi || o == (const void*)d_lo)) return LBM_EINVAL;
     if (d_d2 == d_d1) return LBM_EINVAL;
-    CK(lines_mixed_plain(d_hi, d_lo, d_d1, d_d2, nx, ny, axis, fd_order,
-                         (cudaStream_t)cuda_stream));
+    CK(lines_df_plain(d_hi, d_lo, d_d1, d_d2, nx, ny, axis, fd_order,
+                      (cudaStream_t)cuda_stream));
     return LBM_OK;
 }
 

@@ -48,6 +48,9 @@ struct InstHost {
     int rows;     // collide-stream strip height (0: the single-instance default)
 };
 
+// the density's low part, where the line solves read it (null: not kept by the steps)
+float* rl_of(const InstHost& h) { return h.rho_df ? h.rl : nullptr; }
+
 struct Region {
     size_t plane, f_bytes, field_bytes, parts_off, total;
 };
@@ -101,7 +104,7 @@ Tables table_layout(const lbm_instance* inst, int n, int order, size_t base) {
         const int nx = inst[i].grid.nx, ny = inst[i].grid.ny;
         cs_max += cs_blocks_for(nx, ny, kRowChoices[0]);
         mu += mu_blocks_for((size_t)nx * ny);
-        rho += std::max(lines_batch_blocks(nx, ny, order, LineBatchKind::kRhoDF),
+        rho += std::max(lines_df_batch_blocks(nx, ny, order),
                         f32_blocks(l32, nx, ny, order, LineBatchKind::kRhoF32, 8));
         force += f32_blocks(l32, nx, ny, order, LineBatchKind::kForce, 8);
     }
@@ -114,7 +117,7 @@ Tables table_layout(const lbm_instance* inst, int n, int order, size_t base) {
     };
     t.cs = take(n * sizeof(CsBatchInst));
     t.mu = take(n * sizeof(MuBatchInst));
-    t.rho_df = take(n * lines_batch_desc_bytes(LineBatchKind::kRhoDF));
+    t.rho_df = take(n * sizeof(Lines32Inst));
     t.rho_f32 = take(n * f32_desc_bytes(l32, LineBatchKind::kRhoF32));
     t.force = take(n * f32_desc_bytes(l32, LineBatchKind::kForce));
     t.state = take(n * sizeof(DevState));
@@ -147,8 +150,8 @@ struct lbm_batch {
     bool mrt;  // MRT collision (Eq. 4) for every instance
     bool l32;  // FP32 line passes by Lines32Inst (every grid small enough)
     MrtRates rates;
-    cudaStream_t stream, cap_stream;
-    cudaEvent_t ev, tev[5];
+    cudaStream_t stream, cap_stream, side_stream;  // the last two for graph capture only
+    cudaEvent_t ev, tev[5], fork_ev, join_ev;
     char* ws;
     std::vector<InstHost> inst;
     std::vector<int> order_by_size;  // instance indices, largest grid first
@@ -175,7 +178,9 @@ lbm_status wait_stream(lbm_batch* b) {
         const double el =
             std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
         if (el > b->timeout_s) return LBM_ETIMEOUT;
-        std::this_thread::sleep_for(std::chrono::microseconds(el < 0.01 ? 5 : 200));
+        // a sleep of 5 us takes about 60: short waits are polled through
+        if (el > 3e-4)
+            std::this_thread::sleep_for(std::chrono::microseconds(el < 0.01 ? 5 : 200));
     }
 }
 
@@ -197,7 +202,7 @@ MixedLinesView view_of(const lbm_batch* b, int i) {
 lbm_status upload_tables(lbm_batch* b) {
     Tables& t = b->tb;
     const int n = b->n;
-    const size_t bdf = lines_batch_desc_bytes(LineBatchKind::kRhoDF);
+    const size_t bdf = sizeof(Lines32Inst);
     const size_t bf = f32_desc_bytes(b->l32, LineBatchKind::kRhoF32);
     const size_t bfo = f32_desc_bytes(b->l32, LineBatchKind::kForce);
     // one instance's descriptor of an FP32 line pass, and its blocks in the map
@@ -221,7 +226,7 @@ lbm_status upload_tables(lbm_batch* b) {
         const InstHost& h = b->inst[i];
         DevState* st = b->dst + i;
         CsBatchInst c;
-        c.a = cs_mixed_args(h.f[0], h.f[1], h.Fx, h.Fy, h.rh, h.rl, h.nx, h.ny, h.plane,
+        c.a = cs_mixed_args(h.f[0], h.f[1], h.Fx, h.Fy, h.rh, rl_of(h), h.nx, h.ny, h.plane,
                             h.phys.omega, b->mrt ? &b->rates : nullptr, st, h.rows);
         c.f[0] = h.f[0];
         c.f[1] = h.f[1];
@@ -234,10 +239,10 @@ lbm_status upload_tables(lbm_batch* b) {
         mu[i] = m;
 
         if (h.rho_df) {
-            lines_batch_fill(LineBatchKind::kRhoDF, view_of(b, i), b->order, (int)mrdf.size(),
-                             rdf.data() + i * bdf);
-            mrdf.insert(mrdf.end(),
-                        lines_batch_blocks(h.nx, h.ny, b->order, LineBatchKind::kRhoDF), i);
+            const Lines32Inst d =
+                lines_df_batch_inst(view_of(b, i), b->order, (int)mrdf.size());
+            std::memcpy(rdf.data() + i * bdf, &d, sizeof(d));
+            mrdf.insert(mrdf.end(), lines_df_batch_blocks(h.nx, h.ny, b->order), i);
         } else {
             fill(LineBatchKind::kRhoF32, i, mrf, rf.data() + i * bf);
         }
@@ -289,16 +294,30 @@ cudaError_t f32_lines(const lbm_batch* b, LineBatchKind kind, int bump, cudaStre
     return lines_batch_launch(kind, d, map, nb, b->order, bump, s, b->line_nl);
 }
 
-lbm_status enqueue_step(lbm_batch* b, cudaStream_t s, int from, cudaEvent_t* ev = nullptr) {
+// `side` (while capturing): another stream, on which the double-float density lines run
+// beside the FP32 ones (they are other instances'; one after the other they took 17 and 15
+// us of the 24-instance batch's 92)
+lbm_status enqueue_step(lbm_batch* b, cudaStream_t s, int from, cudaEvent_t* ev = nullptr,
+                        cudaStream_t side = nullptr) {
     const Tables& t = b->tb;
     auto mark = [&](int i) { return ev ? cudaEventRecord(ev[i], s) : cudaSuccess; };
     CK(launch_cs_mixed_batch(at<CsBatchInst>(b, t.cs), at<int>(b, t.map_cs), t.nb_cs, from,
                              b->mrt, s));
     CK(mark(1));
     // every instance is in exactly one of the two density launches
+    const bool fork = side && t.nb_rho_df > 0 && t.nb_rho_f32 > 0;
+    cudaStream_t sd = fork ? side : s;
+    if (fork) {
+        CK(cudaEventRecord(b->fork_ev, s));
+        CK(cudaStreamWaitEvent(side, b->fork_ev, 0));
+    }
+    CK(lines_df_batch_launch(at<Lines32Inst>(b, t.rho_df), at<int>(b, t.map_rho_df), t.nb_rho_df,
+                             b->order, 1, sd));
     CK(f32_lines(b, LineBatchKind::kRhoF32, 1, s));
-    CK(lines_batch_launch(LineBatchKind::kRhoDF, b->ws + t.rho_df, at<int>(b, t.map_rho_df),
-                          t.nb_rho_df, b->order, 1, s));
+    if (fork) {
+        CK(cudaEventRecord(b->join_ev, side));
+        CK(cudaStreamWaitEvent(s, b->join_ev, 0));
+    }
     CK(mark(2));
     CK(launch_mu_mixed_batch(at<MuBatchInst>(b, t.mu), at<int>(b, t.map_mu), t.nb_mu, s));
     CK(mark(3));
@@ -311,8 +330,8 @@ lbm_status build_graph(lbm_batch* b, int from) {
     if (b->graph[from]) return LBM_OK;
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
-    lbm_status st = enqueue_step(b, b->cap_stream, from);
-    if (st == LBM_OK) st = enqueue_step(b, b->cap_stream, 1 - from);
+    lbm_status st = enqueue_step(b, b->cap_stream, from, nullptr, b->side_stream);
+    if (st == LBM_OK) st = enqueue_step(b, b->cap_stream, 1 - from, nullptr, b->side_stream);
     cudaError_t e = cudaStreamEndCapture(b->cap_stream, &g);
     if (st != LBM_OK) {
         if (g) cudaGraphDestroy(g);
@@ -376,8 +395,7 @@ lbm_status instance_force(lbm_batch* b, int i) {
     DevState* st = b->dst + i;
     cudaStream_t s = b->stream;
     if (h.rho_df)
-        CK(lines_mixed_rho_xy(h.rh, h.rl, h.dxr, h.dxx, h.dyr, h.dyy, h.nx, h.ny, b->order, st,
-                              0, s));
+        CK(lines_df_rho(h.rh, h.rl, h.dxr, h.dxx, h.dyr, h.dyy, h.nx, h.ny, b->order, st, 0, s));
     else if (b->l32)
         CK(lines32_rho(h.rh, h.dxr, h.dxx, h.dyr, h.dyy, h.nx, h.ny, b->order, st, 0, s));
     else
@@ -450,8 +468,8 @@ lbm_status lbm_batch_init(lbm_batch** out, const lbm_instance* inst, int32_t n,
     b->failed_step = -1;
     b->cur = 0;
     b->graph[0] = b->graph[1] = nullptr;
-    b->cap_stream = nullptr;
-    b->ev = nullptr;
+    b->cap_stream = b->side_stream = nullptr;
+    b->ev = b->fork_ev = b->join_ev = nullptr;
     for (auto& e : b->tev) e = nullptr;
     b->hst = nullptr;
     if (cudaGetDevice(&b->dev) != cudaSuccess) {
@@ -509,6 +527,9 @@ lbm_status lbm_batch_init(lbm_batch** out, const lbm_instance* inst, int32_t n,
                      [&](int x, int y) { return b->inst[x].N > b->inst[y].N; });
 
     if (cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&b->side_stream, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&b->fork_ev, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&b->join_ev, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) != cudaSuccess ||
         cudaMallocHost((void**)&b->hst, n * sizeof(DevState)) != cudaSuccess) {
         lbm_batch_free(b);
@@ -534,10 +555,12 @@ void lbm_batch_free(lbm_batch* b) {
     if (!b) return;
     cudaSetDevice(b->dev);
     drop_graphs(b);
-    if (b->ev) cudaEventDestroy(b->ev);
+    for (cudaEvent_t e : {b->ev, b->fork_ev, b->join_ev})
+        if (e) cudaEventDestroy(e);
     for (auto& e : b->tev)
         if (e) cudaEventDestroy(e);
-    if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
+    for (cudaStream_t x : {b->cap_stream, b->side_stream})
+        if (x) cudaStreamDestroy(x);
     if (b->hst) cudaFreeHost(b->hst);
     delete b;
 }
@@ -636,7 +659,7 @@ lbm_status lbm_batch_fields(lbm_batch* b, int32_t i, double* h_rho, double* h_vx
     CK(cudaSetDevice(b->dev));
     double* sg = (double*)h.f[1 - b->cur];  // idle buffer: >= 4 N doubles
     const size_t N = h.N;
-    CK(launch_macro_mixed(h.f[b->cur], h.rh, h.rl, h.Fx, h.Fy, h.dxx /* holds mu-hat */,
+    CK(launch_macro_mixed(h.f[b->cur], h.rh, rl_of(h), h.Fx, h.Fy, h.dxx /* holds mu-hat */,
                           h_rho ? sg : nullptr, h_vx ? sg + N : nullptr,
                           h_vy ? sg + 2 * N : nullptr, h_mu ? sg + 3 * N : nullptr, h.nx, h.ny,
                           h.plane, b->stream));
@@ -657,7 +680,7 @@ lbm_status lbm_batch_diag(lbm_batch* b, double* mass, double* max_v, double* rho
     CK(cudaSetDevice(b->dev));
     for (int i = 0; i < b->n; ++i) {
         const InstHost& h = b->inst[i];
-        CK(launch_diag_mixed(h.f[b->cur], h.rh, h.rl, h.Fx, h.Fy, h.nx, h.ny, h.plane,
+        CK(launch_diag_mixed(h.f[b->cur], h.rh, rl_of(h), h.Fx, h.Fy, h.nx, h.ny, h.plane,
                              h.partials, kParts, b->dst + i, b->stream));
     }
     lbm_status st = read_states(b);
@@ -689,7 +712,7 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int32_t reps) {
         int best_rows = 0;
         for (int rows : kRowChoices) {
             const CsArgs a =
-                cs_mixed_args(h.f[b->cur], h.f[1 - b->cur], h.Fx, h.Fy, h.rh, h.rl, h.nx, h.ny,
+                cs_mixed_args(h.f[b->cur], h.f[1 - b->cur], h.Fx, h.Fy, h.rh, rl_of(h), h.nx, h.ny,
                               h.plane, h.phys.omega, b->mrt ? &b->rates : nullptr, dst, rows);
             CK(launch_cs_mixed_args(a, s));  // warm-up
             CK(cudaEventRecord(b->tev[0], s));

@@ -190,7 +190,7 @@ EosC<T> eos_const(const PhysParams& p) {
                                      : p.a * p.alpha / p.b);
     return c;
 }
-constexpr int kMuBatchT = 256;  // threads per block of the batched mu-hat pass (4 nodes each)
+constexpr int kMuBatchT = 128;  // threads per block of the batched mu-hat pass (4 nodes each)
 struct MuBatchInst {
     const float* rh;
     float* mu;  // holds d_xx rho on entry
@@ -239,6 +239,7 @@ struct Geo32 {
 struct Dir32 {
     Geo32 g;
     const float* u;           // the field solved (density, or mu-hat)
+    const float* ul;          // its low part (double-float solves)
     const float *rho, *dr;    // force: density and its derivative along the line
     float *o1, *o2;           // first and second derivative, or the force
 };
@@ -262,6 +263,17 @@ int lines32_batch_blocks(int nx, int ny, int order, bool second, int nl);
 Lines32Inst lines32_batch_inst(const MixedLinesView& v, int order, bool second, int blk0, int nl);
 cudaError_t lines32_batch_launch(const Lines32Inst* d, const int* map, int nblocks, int order,
                                  bool second, int bump, int nl, cudaStream_t s);
+
+// Double-float density lines (lines_df.cu): x and y in one launch, stand-alone, batches.
+cudaError_t lines_df_rho(const float* rh, const float* rl, float* dxr, float* dxx, float* dyr,
+                         float* dyy, int nx, int ny, int order, DevState* st, int bump,
+                         cudaStream_t s, bool walls_y = false);
+cudaError_t lines_df_plain(const float* uh, const float* ul, float* d1, float* d2, int nx, int ny,
+                           int axis, int order, cudaStream_t s);
+int lines_df_batch_blocks(int nx, int ny, int order);
+Lines32Inst lines_df_batch_inst(const MixedLinesView& v, int order, int blk0);
+cudaError_t lines_df_batch_launch(const Lines32Inst* d, const int* map, int nblocks, int order,
+                                  int bump, cudaStream_t s);
 
 // Whole steps of a small periodic grid in one launch (FP32 density lines).
 struct SmallStep {

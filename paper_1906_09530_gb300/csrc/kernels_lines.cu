@@ -952,11 +952,26 @@ __global__ void __launch_bounds__(NL * 32, (xy_min_blocks<NL, SECOND, P1>()))
     if (bump && blockIdx.x == 0 && threadIdx.x == 0) st->t += 1;
     // y_first: the y-line blocks take the low block indices, so they are
     // dispatched first (in a launch of about one wave the slower y-windows then
-    // do not form the tail); otherwise the x-line blocks do
+    // do not form the tail); otherwise by tiles
     const int nby = (int)gridDim.x - nbx;
-    const bool x = y_first ? (int)blockIdx.x >= nby : (int)blockIdx.x < nbx;
-    const int local = y_first ? (x ? (int)blockIdx.x - nby : (int)blockIdx.x)
-                              : (x ? (int)blockIdx.x : (int)blockIdx.x - nbx);
+    bool x;
+    int local;
+    if (y_first) {
+        x = (int)blockIdx.x >= nby;
+        local = x ? (int)blockIdx.x - nby : (int)blockIdx.x;
+    } else {
+        // line groups across a tile (windows of a longer line own a multiple of NL)
+        const int gr = gy.nwin == 1 ? gx.ngroups : gy.own / NL;
+        const int gc = gx.nwin == 1 ? gy.ngroups : gx.own / NL;
+        const int row = gx.nwin * gr + gy.ngroups;     // blocks of a full row of tiles
+        const int ty = min((int)blockIdx.x / row, gy.nwin - 1);
+        int r = (int)blockIdx.x - ty * row;
+        const int cx = min(gr, gx.ngroups - ty * gr);
+        const int tx = min(r / (cx + gc), gx.nwin - 1);
+        r -= tx * (cx + gc);
+        x = r < cx;
+        local = x ? tx * gx.ngroups + ty * gr + r : ty * gy.ngroups + tx * gc + r - cx;
+    }
     if (x) {
         ex.init(st);
         inx.init(st);

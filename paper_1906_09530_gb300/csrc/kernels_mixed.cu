@@ -151,7 +151,7 @@ __device__ __forceinline__ void cs_mixed_body(const CsArgs& a, int wid) {
             for (int i = 0; i < 9; ++i) fout[i * plane + n] = g[i];
             const df r = sum9_exact(g);
             a.rh[n] = r.hi;
-            a.rl[n] = r.lo;
+            if (a.rl) a.rl[n] = r.lo;
         }
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(kRingT) k_cs_mixed_ring(CsArgs a) {
             for (int i = 0; i < 9; ++i) a.fout[i * plane + n] = g[i];
             const df rr = sum9_exact(g);
             a.rh[n] = rr.hi;
-            a.rl[n] = rr.lo;
+            if (a.rl) a.rl[n] = rr.lo;
         }
     }
     ring_wait_groups<0>();
@@ -378,6 +378,14 @@ __device__ __forceinline__ void velocity_mixed(const float (&g)[9], df r, float 
     vy = tf_div(jy, r, inv);
 }
 
+// The density of a node as hi + lo: the stored planes, or (rl null: a context whose line
+// solves read the hi part alone does not write the other, 4 of 88 bytes a node and step)
+// the exact sum of the populations again, which is what the planes hold.
+__device__ __forceinline__ df density_mixed(const float (&g)[9], const float* rh, const float* rl,
+                                            size_t n) {
+    return rl ? df{rh[n], rl[n]} : sum9_exact(g);
+}
+
 // FP64 outputs of the mixed state: rho = hi + lo, v = u + F/(2 rho), mu-hat; each output
 // may be null (vx and vy together).
 __global__ void k_macro_mixed(const float* __restrict__ f, const float* __restrict__ rh,
@@ -387,12 +395,12 @@ __global__ void k_macro_mixed(const float* __restrict__ f, const float* __restri
                               size_t plane) {
     for (size_t n = blockIdx.x * (size_t)blockDim.x + threadIdx.x; n < N;
          n += (size_t)gridDim.x * blockDim.x) {
-        const df r{rh[n], rl[n]};
         const float m = mu_o ? mu[n] : 0.0f;
-        if (vx || vy) {
-            float g[9];
+        float g[9];
 #pragma unroll
-            for (int i = 1; i < 9; ++i) g[i] = f[i * plane + n];
+        for (int i = 0; i < 9; ++i) g[i] = f[i * plane + n];
+        const df r = density_mixed(g, rh, rl, n);
+        if (vx || vy) {
             double u, v;
             velocity_mixed(g, r, Fx[n], Fy[n], u, v);
             if (vx) vx[n] = u;
@@ -463,8 +471,8 @@ __global__ void __launch_bounds__(kDiagT)
          n += (size_t)gridDim.x * blockDim.x) {
         float g[9];
 #pragma unroll
-        for (int i = 1; i < 9; ++i) g[i] = f[i * plane + n];
-        const df rd{rh[n], rl[n]};
+        for (int i = 0; i < 9; ++i) g[i] = f[i * plane + n];
+        const df rd = density_mixed(g, rh, rl, n);
         double u, v;
         velocity_mixed(g, rd, Fx[n], Fy[n], u, v);
         const double r = __dadd_rn(widen(rd.hi), widen(rd.lo));

@@ -20,7 +20,9 @@ double lambda(int order) {
     return (1.0 - std::sqrt(1.0 - 4.0 * alpha * alpha)) / (2.0 * alpha);
 }
 
-Line32 constants(int order) {
+}  // namespace
+
+Line32 line32_constants(int order) {
     const double alpha = order == 6 ? 1.0 / 3.0 : 0.25, lam = lambda(order);
     const double a = 2.0 / 3.0 * (alpha + 2.0), b = (4.0 * alpha - 1.0) / 3.0;  // Eq. 38
     Line32 k;
@@ -37,24 +39,22 @@ Line32 constants(int order) {
     return k;
 }
 
-// Halo: lam^H (single recursion) or (H+1) lam^H (double) below kEps, rounded up to a
-// multiple of 4 so that windows start on 16-byte boundaries.
-int halo(int order, bool second) {
+// eps1, eps2: what the recursions of the first and second derivative are cut at (eps2 0: no
+// second).  Halo: lam^H (single recursion) or (H+1) lam^H (double) below them, rounded up to
+// a multiple of 4 so that windows start on 16-byte boundaries.
+Geo32 line32_geometry(int nx, int ny, int axis, int order, double eps1, double eps2,
+                      bool walls_y) {
     const double lam = lambda(order);
-    int h = 1;
-    while (std::pow(lam, h) >= kEps) ++h;
-    if (second)
-        while ((h + 1) * std::pow(lam, h) >= kEps) ++h;
-    return (h + 1 + 3) / 4 * 4;
-}
-
-Geo32 geometry(int nx, int ny, int axis, int order, bool second, bool walls_y) {
+    int h1 = 1, h2 = 0;
+    while (std::pow(lam, h1) >= eps1) ++h1;
+    if (eps2 > 0.0)
+        while ((h2 + 1) * std::pow(lam, h2) >= eps2) ++h2;
     Geo32 g;
     g.n = axis == 0 ? nx : ny;
     g.nlines = axis == 0 ? ny : nx;
     g.ps = axis == 0 ? 1 : nx;
     g.ls = axis == 0 ? nx : 1;
-    g.H = halo(order, second);
+    g.H = (std::max(h1, h2) + 1 + 3) / 4 * 4;
     g.own = kW - 2 * g.H;
     if (g.own > g.n) g.own = g.n;
     g.nwin = (g.n + g.own - 1) / g.own;
@@ -69,6 +69,12 @@ Geo32 geometry(int nx, int ny, int axis, int order, bool second, bool walls_y) {
     const int nch = (g.H + g.own - 1) / kC + 1 + 4;
     g.nch = nch >= 32 ? 32 : (nch + 3) / 4 * 4;
     return g;
+}
+
+namespace {
+
+Geo32 geometry(int nx, int ny, int axis, int order, bool second, bool walls_y) {
+    return line32_geometry(nx, ny, axis, order, kEps, second ? kEps : 0.0, walls_y);
 }
 
 // lines a block of T threads takes; y-lines: a power of two of adjacent columns
@@ -166,7 +172,7 @@ cudaError_t run(Dir32 x, Dir32 y, int nx, int ny, int order, bool walls_y, DevSt
     auto go = [&](auto kern) -> cudaError_t {
         const cudaError_t e = allow_smem(kern, smem);
         if (e != cudaSuccess) return e;
-        return launch_pdl(kern, dim3(nbx + nby), dim3(T), smem, s, x, y, constants(order), st,
+        return launch_pdl(kern, dim3(nbx + nby), dim3(T), smem, s, x, y, line32_constants(order), st,
                           bump, nbx);
     };
     return order == 6 ? go(k_lines32<MODE, true>) : go(k_lines32<MODE, false>);
@@ -226,7 +232,7 @@ cudaError_t lines32_batch_launch(const Lines32Inst* d, const int* map, int nbloc
     auto go = [&](auto kern) -> cudaError_t {
         const cudaError_t e = allow_smem(kern, smem);
         if (e != cudaSuccess) return e;
-        kern<<<nblocks, T, smem, s>>>(d, map, constants(order), bump);
+        kern<<<nblocks, T, smem, s>>>(d, map, line32_constants(order), bump);
         return cudaGetLastError();
     };
     if (second)
@@ -249,7 +255,7 @@ namespace {
 constexpr int kCl = 16, kSmallT = 256;
 struct SmallArgs {
     float* f[2];
-    float *Fx, *Fy, *rh, *rl, *dxx, *dyy;
+    float *Fx, *Fy, *rh, *dxx, *dyy;
     int nx, ny;
     size_t plane;
     float omega, se, seps, sq;
@@ -308,9 +314,7 @@ __global__ void __launch_bounds__(kSmallT, 1) k_small(const __grid_constant__ Sm
             const size_t o = (size_t)y0 * nx + n;
 #pragma unroll
             for (int q = 0; q < 9; ++q) fout[q * a.plane + o] = g[q];
-            const df r = sum9_exact(g);
-            a.rh[o] = r.hi;
-            a.rl[o] = r.lo;
+            a.rh[o] = sum9_exact(g).hi;
         }
         cluster_sync();
         for (int b = rank; b < a.nb_r; b += kCl) {
@@ -352,7 +356,6 @@ SmallArgs small_args(const SmallStep& p) {
     a.Fx = p.v.Fx;
     a.Fy = p.v.Fy;
     a.rh = const_cast<float*>(p.v.rh);
-    a.rl = const_cast<float*>(p.v.rl);
     a.dxx = p.v.dxx;
     a.dyy = p.v.dyy;
     a.nx = p.v.nx;
@@ -374,7 +377,7 @@ SmallArgs small_args(const SmallStep& p) {
     a.nb_r = a.nb_rx + blocks_of(a.ry.g);
     a.nb_fx = blocks_of(a.fx.g);
     a.nb_f = a.nb_fx + blocks_of(a.fy.g);
-    a.k = constants(p.order);
+    a.k = line32_constants(p.order);
     a.mu = mu_mixed_const(p.phys);
     a.st = p.v.st;
     return a;

@@ -41,6 +41,10 @@ struct Line32 {
     float Cm1, Cm2;      // C (-lam)^C, 2C (-lam)^(2C)  (double-recursion joins)
 };
 
+Line32 line32_constants(int order);
+Geo32 line32_geometry(int nx, int ny, int axis, int order, double eps1, double eps2,
+                      bool walls_y);
+
 namespace l32 {
 
 constexpr int kC = kC32;

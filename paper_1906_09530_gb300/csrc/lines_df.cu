@@ -1,0 +1,497 @@
+// lines_df.cu -- line solves of the density in double-float (df.cuh): first derivatives in
+// double-float wherever a window crosses an interface, second derivatives in FP32 (see
+// kernels_mixed.cu for why), for the mixed path above a density ratio of 1e4 and the
+// stand-alone lbm_cfd_df.
+//
+// Windows, chunks and joins are those of lines32.cuh, with a halo of 40 (6th order) so that
+// the double-float recursions are cut at 1e-15.  A block takes groups of eight lines; a
+// group whose staged densities all lie within a factor 32 is solved in FP32 on the hi part
+// (FP32 rounding then stays below ~2e-6 of the local values, as accurate as the FP32 result
+// that is stored).  Both axes are staged by 16-byte copies, x-lines line by line, y-lines
+// row by row ([slot][lines]).
+//
+// What bounded it was instruction fetch: with the chunk in registers everything is unrolled
+// over 19 positions, about 100 operations each in double-float, for either axis (4.6 of 8
+// stalled warps waited for instructions).  So the chunk stays in shared memory, in place of
+// the staged window, and the loops are loops; the right-hand side's hi part, which the second
+// derivative starts from, goes to a plane of its own.  Density lines of 1000^2 at ratio 8e4:
+// 33.4 us unrolled in registers, 25.2 so (a step 54.5 -> 47.6).  What is left is uneven: 500
+// blocks, half of them crossing the interface, on 456 places.  Half groups (128 threads, one
+// wave) were no faster: 51.7 against 49.9 us a step.
+#include <algorithm>
+#include <cfloat>
+#include <cmath>
+
+#include "df.cuh"
+#include "lines32.cuh"
+
+namespace cplbm {
+namespace {
+
+constexpr int kC = kC32, kT = 256, kGroup = 8;
+constexpr double kEpsDF = 1e-15, kEpsF = 1e-8;
+
+struct LineDF {
+    Line32 f;
+    df c1, c2, nlam, pw[kC], m1, m2;
+};
+
+__device__ __forceinline__ df fma_df(df x, df c, df y) { return df_fma(x, c.hi, c.lo, y); }
+
+// join1<0> in double-float: forward s > 0, backward s < 0, `have` chunks on that side
+__device__ __forceinline__ df join_df(const LineDF& k, const float* h, const float* l, int s,
+                                      int have) {
+    auto at = [&](int i) { return df{h[-i * s], l[-i * s]}; };
+    if (have < 1) return df{0.0f, 0.0f};
+    df c = at(1);
+    if (have >= 2) c = fma_df(at(2), k.m1, c);
+    if (have >= 3) {
+        df d = at(3);
+        if (have >= 4) d = fma_df(at(4), k.m1, d);
+        c = fma_df(d, k.m2, c);
+    }
+    return c;
+}
+
+// Shared memory: eight join arrays of kT floats, the two planes of the staged window (hi, lo),
+// whose places the first derivative takes, and the second derivative's plane.
+template <bool SIXTH>
+__device__ __forceinline__ void block_df(const Dir32& d, const LineDF& k, int axis, int bid,
+                                         float* sh) {
+    const Geo32& g = d.g;
+    const int t = threadIdx.x;
+    const int grp = bid % g.ngroups, win = bid / g.ngroups;
+    const int s0 = win * g.own, nown = min(g.own, g.n - s0);
+    const int nch = g.nch, nl = g.nl;
+    const int ln = axis == 0 ? t / nch : t % nl;
+    const int c = axis == 0 ? t - ln * nch : t / nl;
+    const int line = grp * nl + ln;
+    const bool live = ln < nl && c < nch && line < g.nlines;
+    const int js = axis == 0 ? 1 : nl;
+    // end states: first derivative (hi, lo) and second (v, w), forward and backward
+    float *eh = sh + t, *el = eh + kT, *ev = el + kT, *ew = ev + kT;
+    float *zh = ew + kT, *zl = zh + kT, *zv = zl + kT, *zw = zv + kT;
+    const int LW = l32::line_stride(nch), nq = kC * nch + 8;
+    float* hi = sh + 8 * kT;
+    float* lo = hi + nl * LW;
+    float* p2 = lo + nl * LW;
+    __shared__ int lowest[kT / 8 / kGroup], highest[kT / 8 / kGroup];
+    if (t < kT / 8 / kGroup) {
+        lowest[t] = __float_as_int(FLT_MAX);
+        highest[t] = 0;
+    }
+    auto wrap = [&](int p) {
+        if (g.magic) p -= g.period * (int)__umulhi((unsigned)p, g.magic);
+        else if (p >= g.period) p -= g.period;
+        return g.period == 1 ? 0 : p;
+    };
+    const int p0 = wrap(s0 - g.H - 4 + g.lift);
+    // ---- stage ----
+    if (axis == 0) {
+        if (live) {
+            const size_t base = (size_t)line * g.ls;
+            const int w = g.vec ? 4 : 1;
+            for (int q = w * c; q < nq; q += w * nch) {
+                const size_t o = base + (size_t)wrap(p0 + q);
+                if (g.vec) {
+                    l32::cp16(hi + ln * LW + q, d.u + o);
+                    l32::cp16(lo + ln * LW + q, d.ul + o);
+                } else {
+                    l32::cp4(hi + ln * LW + q, d.u + o);
+                    l32::cp4(lo + ln * LW + q, d.ul + o);
+                }
+            }
+        }
+    } else {
+        // pieces of four columns (one where rows are not whole 16-byte pieces)
+        const int w = g.vec ? 4 : 1, pr = nl / w;
+        for (int i = t; i < nq * pr; i += kT) {
+            const int q = i / pr, x = w * (i - q * pr), col = grp * nl + x;
+            if (col >= g.nlines) continue;  // (whole pieces: nlines is a multiple of w)
+            int p = wrap(p0 + q);
+            if (g.mirror && p >= g.n) p = 2 * g.n - 1 - p;
+            const size_t o = (size_t)p * g.ps + (size_t)col;
+            if (g.vec) {
+                l32::cp16(hi + q * nl + x, d.u + o);
+                l32::cp16(lo + q * nl + x, d.ul + o);
+            } else {
+                l32::cp4(hi + q * nl + x, d.u + o);
+                l32::cp4(lo + q * nl + x, d.ul + o);
+            }
+        }
+    }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    __syncthreads();
+    // chunk position j at base + j ps
+    const int ps = axis == 0 ? 1 : nl;
+    const int base = axis == 0 ? ln * LW + c * kC + 4 : (c * kC + 4) * nl + ln;
+    float *uh = hi + base, *ul = lo + base, *q2 = p2 + base;
+    // ---- which groups need double-float ----
+    if (live) {
+        float mn = FLT_MAX, mx = 0.0f;
+#pragma unroll 9
+        for (int j = -4; j < kC + 4; ++j) {
+            mn = fminf(mn, uh[j * ps]);
+            mx = fmaxf(mx, uh[j * ps]);
+        }
+        // non-negative floats order as integers
+        atomicMin(&lowest[ln / kGroup], __float_as_int(fmaxf(mn, 0.0f)));
+        atomicMax(&highest[ln / kGroup], __float_as_int(mx));
+    }
+    __syncthreads();
+    bool wide = true;
+    if (live) {
+        const float mn = __int_as_float(lowest[ln / kGroup]),
+                    mx = __int_as_float(highest[ln / kGroup]);
+        // (a group cut short by the grid's edge is always solved in double-float)
+        const bool whole = (line / kGroup + 1) * kGroup <= g.nlines;
+        wide = !(whole && mn > 0.0f && mx <= 32.0f * mn);
+    }
+    auto U = [&](int j) { return df{uh[j * ps], ul[j * ps]}; };
+    auto rhs = [&](df am2, df am1, df ap1, df ap2) {
+        df b = df_mul(df_sub(ap1, am1), k.c1.hi, k.c1.lo);
+        if (SIXTH) b = fma_df(df_sub(ap2, am2), k.c2, b);
+        return b;
+    };
+    auto rhs_f = [&](float am2, float am1, float ap1, float ap2) {
+        float b = (ap1 - am1) * k.f.c1;
+        if (SIXTH) b = rn_fma(ap2 - am2, k.f.c2, b);
+        return b;
+    };
+    auto at_f = [&](int j) {
+        return rhs_f(uh[(j - 2) * ps], uh[(j - 1) * ps], uh[(j + 1) * ps], uh[(j + 2) * ps]);
+    };
+    // what the chunk needs of its neighbours, before they overwrite it: the window two
+    // positions either side, and the first right-hand side there (FP32)
+    const bool second = d.o2 != nullptr;
+    df a{0.0f, 0.0f}, b = a, z1 = a, z2 = a;
+    float bm2 = 0.0f, bm1 = 0.0f, bp1 = 0.0f, bp2 = 0.0f;
+    if (live) {
+        a = U(-2);
+        b = U(-1);
+        z1 = U(kC);
+        z2 = U(kC + 1);
+        if (second) {
+            bm2 = at_f(-2);
+            bm1 = at_f(-1);
+            bp1 = at_f(kC);
+            bp2 = at_f(kC + 1);
+        }
+    }
+    const int after = nch - 1 - c;
+    __syncthreads();
+    // ---- forward ----
+    if (live) {
+        df e = U(0), f = U(1);
+        if (wide) {
+            df w{0.0f, 0.0f};
+            float *ph = uh, *pl = ul, *p = q2;  // at position j
+            auto step = [&](df h) {
+                const df r = rhs(a, b, f, h);
+                w = fma_df(w, k.nlam, r);
+                *p = r.hi;
+                *ph = w.hi;
+                *pl = w.lo;
+                p += ps;
+                ph += ps;
+                pl += ps;
+                a = b;
+                b = e;
+                e = f;
+                f = h;
+            };
+#pragma unroll 4
+            for (int j = 0; j < kC - 3; ++j) step(df{ph[2 * ps], pl[2 * ps]});
+            step(df{ph[2 * ps], pl[2 * ps]});
+            step(z1);
+            step(z2);
+            *eh = w.hi;
+            *el = w.lo;
+        } else {
+            float w = 0.0f;
+            float *ph = uh, *p = q2;
+            auto step = [&](float h) {
+                const float r = rhs_f(a.hi, b.hi, f.hi, h);
+                w = rn_fma(w, k.f.nlam, r);
+                *p = r;
+                *ph = w;
+                p += ps;
+                ph += ps;
+                a.hi = b.hi;
+                b.hi = e.hi;
+                e.hi = f.hi;
+                f.hi = h;
+            };
+#pragma unroll 4
+            for (int j = 0; j < kC - 3; ++j) step(ph[2 * ps]);
+            step(ph[2 * ps]);
+            step(z1.hi);
+            step(z2.hi);
+            *eh = w;
+        }
+        if (second) {
+            float p = bm2, q = bm1, r = q2[0], x = q2[ps], v = 0.0f, w = 0.0f;
+            float* o = q2;
+            auto step = [&](float h) {
+                float y = rn_mul(rn_sub(x, q), k.f.c1);
+                if (SIXTH) y = rn_fma(rn_sub(h, p), k.f.c2, y);
+                v = rn_fma(v, k.f.nlam, y);
+                *o = w = rn_fma(w, k.f.nlam, v);
+                o += ps;
+                p = q;
+                q = r;
+                r = x;
+                x = h;
+            };
+#pragma unroll 8
+            for (int j = 0; j < kC - 3; ++j) step(o[2 * ps]);
+            step(o[2 * ps]);
+            step(bp1);
+            step(bp2);
+            *ev = v;
+            *ew = w;
+        }
+    }
+    __syncthreads();
+    // ---- backward ----
+    if (live) {
+        if (wide) {
+            const df cf = join_df(k, eh, el, js, c);
+            df z{0.0f, 0.0f};
+            float *ph = uh + (kC - 1) * ps, *pl = ul + (kC - 1) * ps;
+#pragma unroll 4
+            for (int j = kC - 1; j >= 0; --j) {
+                z = fma_df(z, k.nlam, fma_df(cf, k.pw[j], df{*ph, *pl}));
+                *ph = z.hi;
+                *pl = z.lo;
+                ph -= ps;
+                pl -= ps;
+            }
+            *zh = z.hi;
+            *zl = z.lo;
+        } else {
+            const float cf = l32::join1<0>(k.f, eh, js, c);
+            float z = 0.0f;
+#pragma unroll 5
+            for (int j = kC - 1; j >= 0; --j)
+                uh[j * ps] = z = rn_fma(z, k.f.nlam, rn_fma(cf, k.f.pw[j], uh[j * ps]));
+            *zh = z;
+        }
+        if (second) {
+            float cv, cw, y = 0.0f, z = 0.0f;
+            l32::join2<0>(k.f, ev, ew, js, c, cv, cw);
+#pragma unroll 5
+            for (int j = kC - 1; j >= 0; --j) {
+                const float r = rn_fma(k.f.pw[j], rn_fma((float)(j + 1), cv, cw), q2[j * ps]);
+                y = rn_fma(y, k.f.nlam, r);
+                q2[j * ps] = z = rn_fma(z, k.f.nlam, y);
+            }
+            *zv = y;
+            *zw = z;
+        }
+    }
+    __syncthreads();
+    // ---- the state entering from after the chunk ----
+    if (live) {
+        if (wide) {
+            const df cb = join_df(k, zh, zl, -js, after);
+            float *ph = uh, *pl = ul;
+#pragma unroll 4
+            for (int j = 0; j < kC; ++j) {
+                *ph = df_round(fma_df(cb, k.pw[kC - 1 - j], df{*ph, *pl}));
+                ph += ps;
+                pl += ps;
+            }
+        } else {
+            const float cb = l32::join1<0>(k.f, zh, -js, after);
+#pragma unroll 5
+            for (int j = 0; j < kC; ++j) uh[j * ps] = rn_fma(cb, k.f.pw[kC - 1 - j], uh[j * ps]);
+        }
+        if (second) {
+            float cy, cz;
+            l32::join2<0>(k.f, zv, zw, -js, after, cy, cz);
+#pragma unroll 5
+            for (int j = 0; j < kC; ++j)
+                q2[j * ps] =
+                    rn_fma(k.f.pw[kC - 1 - j], rn_fma((float)(kC - j), cy, cz), q2[j * ps]);
+        }
+    }
+    __syncthreads();
+    // ---- out: window position q at slot q + 4 ----
+    const int H4 = g.H + 4;
+    if (axis == 0) {
+        if (live) {
+            const size_t o = (size_t)line * g.ls + (size_t)s0;
+            const float *r1 = hi + ln * LW + H4, *r2 = p2 + ln * LW + H4;
+            if (g.vec) {
+                for (int q = 4 * c; q < nown; q += 4 * nch) {
+                    *reinterpret_cast<float4*>(d.o1 + o + q) =
+                        *reinterpret_cast<const float4*>(r1 + q);
+                    if (d.o2)
+                        *reinterpret_cast<float4*>(d.o2 + o + q) =
+                            *reinterpret_cast<const float4*>(r2 + q);
+                }
+            } else {
+                for (int q = c; q < nown; q += nch) {
+                    d.o1[o + q] = r1[q];
+                    if (d.o2) d.o2[o + q] = r2[q];
+                }
+            }
+        }
+    } else {
+        const int w = g.vec ? 4 : 1, pr = nl / w;
+        for (int i = t; i < nown * pr; i += kT) {
+            const int q = i / pr, x = w * (i - q * pr), col = grp * nl + x;
+            if (col >= g.nlines) continue;
+            const size_t o = (size_t)(s0 + q) * g.ps + (size_t)col;
+            const int m = (q + H4) * nl + x;
+            if (g.vec) {
+                *reinterpret_cast<float4*>(d.o1 + o) = *reinterpret_cast<const float4*>(hi + m);
+                if (d.o2)
+                    *reinterpret_cast<float4*>(d.o2 + o) = *reinterpret_cast<const float4*>(p2 + m);
+            } else {
+                d.o1[o] = hi[m];
+                if (d.o2) d.o2[o] = p2[m];
+            }
+        }
+    }
+}
+
+template <bool SIXTH>
+__global__ void __launch_bounds__(kT, 3)
+    k_lines_df(Dir32 x, Dir32 y, const __grid_constant__ LineDF k, DevState* st, int bump,
+               int nbx) {
+    pdl_prologue();
+    extern __shared__ __align__(16) float shdf[];
+    if (bump && blockIdx.x == 0 && threadIdx.x == 0) st->t += 1;
+    const int nby = (int)gridDim.x - nbx, b = blockIdx.x;
+    const bool is_y = b < nby;
+    const Dir32& d = is_y ? y : x;
+    block_df<SIXTH>(d, k, is_y, is_y ? b : b - nby, shdf);
+}
+
+template <bool SIXTH>
+__global__ void __launch_bounds__(kT, 3)
+    k_lines_df_batch(const Lines32Inst* __restrict__ d, const int* __restrict__ map,
+                     const __grid_constant__ LineDF k, int bump) {
+    extern __shared__ __align__(16) float shdf[];
+    const Lines32Inst& D = d[map[blockIdx.x]];
+    const int local = (int)blockIdx.x - D.blk0;
+    if (bump && local == 0 && threadIdx.x == 0) D.st->t += 1;
+    const bool is_y = local >= D.nbx;
+    block_df<SIXTH>(is_y ? D.y : D.x, k, is_y, is_y ? local - D.nbx : local, shdf);
+}
+
+// ---- host side ----
+df split(double v) {
+    df r;
+    r.hi = (float)v;
+    r.lo = (float)(v - (double)r.hi);
+    return r;
+}
+LineDF constants_df(int order) {
+    const double alpha = order == 6 ? 1.0 / 3.0 : 0.25;
+    const double lam = (1.0 - std::sqrt(1.0 - 4.0 * alpha * alpha)) / (2.0 * alpha);
+    const double a = 2.0 / 3.0 * (alpha + 2.0), b = (4.0 * alpha - 1.0) / 3.0;  // Eq. 38
+    LineDF k;
+    k.f = line32_constants(order);
+    k.c1 = split(lam / alpha * a / 2.0);
+    k.c2 = split(lam / alpha * b / 4.0);
+    k.nlam = split(-lam);
+    double p = 1.0;
+    for (int j = 0; j < kC; ++j) k.pw[j] = split(p *= -lam);
+    const double m = std::pow(-lam, kC);
+    k.m1 = split(m);
+    k.m2 = split(m * m);
+    return k;
+}
+
+// Lines a block: groups of eight, as many as the block's threads hold.
+void divide_df(Geo32& g) {
+    g.nl = std::max(kGroup, kT / g.nch / kGroup * kGroup);
+    g.ngroups = (g.nlines + g.nl - 1) / g.nl;
+}
+Dir32 dir_df(const float* h, const float* l, float* d1, float* d2, int nx, int ny, int axis,
+             int order, bool second, bool walls_y) {
+    Dir32 d{};
+    d.u = h;
+    d.ul = l;
+    d.o1 = d1;
+    d.o2 = d2;
+    d.g = line32_geometry(nx, ny, axis, order, kEpsDF, second ? kEpsF : 0.0, walls_y);
+    divide_df(d.g);
+    return d;
+}
+int blocks_of(const Geo32& g) { return g.ngroups * g.nwin; }
+size_t smem_df(const Geo32& g) {
+    return ((size_t)8 * kT + 3 * (size_t)g.nl * l32::line_stride(g.nch)) * sizeof(float);
+}
+template <class K>
+cudaError_t allow_smem(K kern, size_t bytes) {
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+cudaError_t run_df(const Dir32& x, const Dir32& y, int nbx, int nby, int order, DevState* st,
+                   int bump, cudaStream_t s) {
+    const size_t smem = std::max(smem_df(x.g), smem_df(y.g));
+    auto go = [&](auto kern) -> cudaError_t {
+        const cudaError_t e = allow_smem(kern, smem);
+        if (e != cudaSuccess) return e;
+        return launch_pdl(kern, dim3(nbx + nby), dim3(kT), smem, s, x, y, constants_df(order), st,
+                          bump, nbx);
+    };
+    return order == 6 ? go(k_lines_df<true>) : go(k_lines_df<false>);
+}
+
+}  // namespace
+
+cudaError_t lines_df_rho(const float* rh, const float* rl, float* dxr, float* dxx, float* dyr,
+                         float* dyy, int nx, int ny, int order, DevState* st, int bump,
+                         cudaStream_t s, bool walls_y) {
+    const Dir32 x = dir_df(rh, rl, dxr, dxx, nx, ny, 0, order, true, false),
+                y = dir_df(rh, rl, dyr, dyy, nx, ny, 1, order, true, walls_y);
+    return run_df(x, y, blocks_of(x.g), blocks_of(y.g), order, st, bump, s);
+}
+
+cudaError_t lines_df_plain(const float* uh, const float* ul, float* d1, float* d2, int nx, int ny,
+                           int axis, int order, cudaStream_t s) {
+    const Dir32 d = dir_df(uh, ul, d1, d2, nx, ny, axis, order, d2 != nullptr, false);
+    const int nb = blocks_of(d.g);
+    return run_df(d, d, axis == 0 ? nb : 0, axis == 0 ? 0 : nb, order, nullptr, 0, s);
+}
+
+int lines_df_batch_blocks(int nx, int ny, int order) {
+    return blocks_of(dir_df(nullptr, nullptr, nullptr, nullptr, nx, ny, 0, order, true, false).g) +
+           blocks_of(dir_df(nullptr, nullptr, nullptr, nullptr, nx, ny, 1, order, true, false).g);
+}
+
+Lines32Inst lines_df_batch_inst(const MixedLinesView& v, int order, int blk0) {
+    Lines32Inst d{};
+    d.x = dir_df(v.rh, v.rl, v.dxr, v.dxx, v.nx, v.ny, 0, order, true, false);
+    d.y = dir_df(v.rh, v.rl, v.dyr, v.dyy, v.nx, v.ny, 1, order, true, false);
+    d.nbx = blocks_of(d.x.g);
+    d.blk0 = blk0;
+    d.st = v.st;
+    return d;
+}
+
+cudaError_t lines_df_batch_launch(const Lines32Inst* d, const int* map, int nblocks, int order,
+                                  int bump, cudaStream_t s) {
+    if (nblocks <= 0) return cudaSuccess;
+    size_t smem = 0;  // the most a block of any instance stages
+    for (int nch = 8; nch <= 32; nch += 4) {
+        Geo32 g{};
+        g.nch = nch;
+        divide_df(g);
+        smem = std::max(smem, smem_df(g));
+    }
+    auto go = [&](auto kern) -> cudaError_t {
+        const cudaError_t e = allow_smem(kern, smem);
+        if (e != cudaSuccess) return e;
+        kern<<<nblocks, kT, smem, s>>>(d, map, constants_df(order), bump);
+        return cudaGetLastError();
+    };
+    return order == 6 ? go(k_lines_df_batch<true>) : go(k_lines_df_batch<false>);
+}
+
+}  // namespace cplbm
