@@ -139,26 +139,18 @@ lbm_status enqueue_force(lbm_ctx* c, cudaStream_t s, int bump, int fcur,
     launch_pdl_on() = c->pdl_now;
     auto mark = [&](int i) { return ev ? cudaEventRecord(ev[i], s) : cudaSuccess; };
     if (!is_fp64(c)) {
-        const bool lines32 = (long long)nx * ny <= kLines32Nodes;
         // x|y lines of rho together, mu-hat pointwise, x|y lines of mu-hat + force
         if (c->rho_df)
             CK(lines_df_rho(c->m_rh, c->m_rl, c->m_dxr, c->m_dxx, c->m_dyr, c->m_dyy, nx, ny, o,
                             c->dst, bump, s, c->walls_y));
-        else if (lines32)
+        else
             CK(lines32_rho(c->m_rh, c->m_dxr, c->m_dxx, c->m_dyr, c->m_dyy, nx, ny, o, c->dst,
                            bump, s, c->walls_y));
-        else
-            CK(lines_mixed_rho_xy_f32(c->m_rh, c->m_dxr, c->m_dxx, c->m_dyr, c->m_dyy, nx, ny, o,
-                                      c->dst, bump, s, c->walls_y));
         CK(mark(0));
         CK(launch_mu_mixed(c->m_rh, c->m_dxx, c->m_dyy, nx, ny, c->phys, c->dst, s));
         CK(mark(1));
-        if (lines32)
-            CK(lines32_force(c->m_dxx, c->m_rh, c->m_dxr, c->m_dyr, c->m_Fx, c->m_Fy, nx, ny, o,
-                             c->dst, s, c->walls_y));
-        else
-            CK(lines_mixed_force_xy(c->m_dxx, c->m_rh, c->m_dxr, c->m_dyr, c->m_Fx, c->m_Fy, nx,
-                                    ny, o, s, c->walls_y, c->dst));
+        CK(lines32_force(c->m_dxx, c->m_rh, c->m_dxr, c->m_dyr, c->m_Fx, c->m_Fy, nx, ny, o,
+                         c->dst, s, c->walls_y));
         CK(mark(2));
         CK(mark(3));
         return LBM_OK;

@@ -72,23 +72,15 @@ int cs_blocks_for(int nx, int ny, int rows) {
 }
 int mu_blocks_for(size_t N) { return (int)(((N + 3) / 4 + kMuBatchT - 1) / kMuBatchT); }
 
-// Offsets of the table region, sized for the largest block counts (the
-// smallest strip height) so that autotuning never needs more room.
-// Line passes: where every grid is small enough (kLines32Nodes) the FP32 ones are
-// Lines32Inst and their launches, else the full windows' descriptors.
-size_t f32_desc_bytes(bool l32, LineBatchKind kind) {
-    return l32 ? sizeof(Lines32Inst) : lines_batch_desc_bytes(kind);
-}
-int f32_blocks(bool l32, int nx, int ny, int order, LineBatchKind kind, int nl) {
-    return l32 ? lines32_batch_blocks(nx, ny, order, kind == LineBatchKind::kRhoF32, nl)
-               : lines_batch_blocks(nx, ny, order, kind, nl);
-}
-bool small_lines(const lbm_instance* inst, int n) {
+// A batch with a grid above kLines32Nodes solves its FP32 lines in full windows.
+bool wide_lines(const lbm_instance* inst, int n) {
     for (int i = 0; i < n; ++i)
-        if ((long long)inst[i].grid.nx * inst[i].grid.ny > kLines32Nodes) return false;
-    return true;
+        if ((long long)inst[i].grid.nx * inst[i].grid.ny > kLines32Nodes) return true;
+    return false;
 }
 
+// Offsets of the table region, sized for the largest block counts (the
+// smallest strip height) so that autotuning never needs more room.
 struct Tables {
     size_t cs, mu, rho_df, rho_f32, force, state;
     size_t map_cs, map_mu, map_rho_df, map_rho_f32, map_force, end;
@@ -99,14 +91,14 @@ Tables table_layout(const lbm_instance* inst, int n, int order, size_t base) {
     // each density map is sized for every instance in it (the double-float
     // windows are the shorter ones, so their count bounds both kinds)
     long long cs_max = 0, mu = 0, rho = 0, force = 0;
-    const bool l32 = small_lines(inst, n);
+    const bool wide = wide_lines(inst, n);
     for (int i = 0; i < n; ++i) {
         const int nx = inst[i].grid.nx, ny = inst[i].grid.ny;
         cs_max += cs_blocks_for(nx, ny, kRowChoices[0]);
         mu += mu_blocks_for((size_t)nx * ny);
         rho += std::max(lines_df_batch_blocks(nx, ny, order),
-                        f32_blocks(l32, nx, ny, order, LineBatchKind::kRhoF32, 8));
-        force += f32_blocks(l32, nx, ny, order, LineBatchKind::kForce, 8);
+                        lines32_batch_blocks(nx, ny, order, true, 8, wide));
+        force += lines32_batch_blocks(nx, ny, order, false, 8, wide);
     }
     Tables t;
     size_t o = base;
@@ -118,8 +110,8 @@ Tables table_layout(const lbm_instance* inst, int n, int order, size_t base) {
     t.cs = take(n * sizeof(CsBatchInst));
     t.mu = take(n * sizeof(MuBatchInst));
     t.rho_df = take(n * sizeof(Lines32Inst));
-    t.rho_f32 = take(n * f32_desc_bytes(l32, LineBatchKind::kRhoF32));
-    t.force = take(n * f32_desc_bytes(l32, LineBatchKind::kForce));
+    t.rho_f32 = take(n * sizeof(Lines32Inst));
+    t.force = take(n * sizeof(Lines32Inst));
     t.state = take(n * sizeof(DevState));
     t.map_cs = take(cs_max * sizeof(int));
     t.map_mu = take(mu * sizeof(int));
@@ -148,7 +140,7 @@ bool instance_ok(const lbm_instance& in) {
 struct lbm_batch {
     int dev, n, order;
     bool mrt;  // MRT collision (Eq. 4) for every instance
-    bool l32;  // FP32 line passes by Lines32Inst (every grid small enough)
+    bool wide;  // FP32 lines in full windows (a grid above kLines32Nodes)
     MrtRates rates;
     cudaStream_t stream, cap_stream, side_stream;  // the last two for graph capture only
     cudaEvent_t ev, tev[5], fork_ev, join_ev;
@@ -202,25 +194,9 @@ MixedLinesView view_of(const lbm_batch* b, int i) {
 lbm_status upload_tables(lbm_batch* b) {
     Tables& t = b->tb;
     const int n = b->n;
-    const size_t bdf = sizeof(Lines32Inst);
-    const size_t bf = f32_desc_bytes(b->l32, LineBatchKind::kRhoF32);
-    const size_t bfo = f32_desc_bytes(b->l32, LineBatchKind::kForce);
-    // one instance's descriptor of an FP32 line pass, and its blocks in the map
-    auto fill = [&](LineBatchKind kind, int i, std::vector<int>& m, unsigned char* dst) {
-        const InstHost& h = b->inst[i];
-        const MixedLinesView v = view_of(b, i);
-        if (b->l32) {
-            const Lines32Inst d = lines32_batch_inst(v, b->order, kind == LineBatchKind::kRhoF32,
-                                                     (int)m.size(), b->line_nl);
-            std::memcpy(dst, &d, sizeof(d));
-        } else {
-            lines_batch_fill(kind, v, b->order, (int)m.size(), dst, b->line_nl);
-        }
-        m.insert(m.end(), f32_blocks(b->l32, h.nx, h.ny, b->order, kind, b->line_nl), i);
-    };
     std::vector<CsBatchInst> cs(n);
     std::vector<MuBatchInst> mu(n);
-    std::vector<unsigned char> rdf(n * bdf), rf(n * bf), force(n * bfo);
+    std::vector<Lines32Inst> rdf(n), rf(n), force(n);
     std::vector<int> mcs, mmu, mrdf, mrf, mforce;
     for (int i : b->order_by_size) {
         const InstHost& h = b->inst[i];
@@ -238,15 +214,18 @@ lbm_status upload_tables(lbm_batch* b) {
         mmu.insert(mmu.end(), mu_blocks_for(h.N), i);
         mu[i] = m;
 
+        const MixedLinesView v = view_of(b, i);
         if (h.rho_df) {
-            const Lines32Inst d =
-                lines_df_batch_inst(view_of(b, i), b->order, (int)mrdf.size());
-            std::memcpy(rdf.data() + i * bdf, &d, sizeof(d));
+            rdf[i] = lines_df_batch_inst(v, b->order, (int)mrdf.size());
             mrdf.insert(mrdf.end(), lines_df_batch_blocks(h.nx, h.ny, b->order), i);
         } else {
-            fill(LineBatchKind::kRhoF32, i, mrf, rf.data() + i * bf);
+            rf[i] = lines32_batch_inst(v, b->order, true, (int)mrf.size(), b->line_nl, b->wide);
+            mrf.insert(mrf.end(),
+                       lines32_batch_blocks(h.nx, h.ny, b->order, true, b->line_nl, b->wide), i);
         }
-        fill(LineBatchKind::kForce, i, mforce, force.data() + i * bfo);
+        force[i] = lines32_batch_inst(v, b->order, false, (int)mforce.size(), b->line_nl, b->wide);
+        mforce.insert(mforce.end(),
+                      lines32_batch_blocks(h.nx, h.ny, b->order, false, b->line_nl, b->wide), i);
     }
     // the table region was sized for the largest counts
     const size_t cap_cs = (t.map_mu - t.map_cs) / sizeof(int);
@@ -264,9 +243,9 @@ lbm_status upload_tables(lbm_batch* b) {
     };
     CK(put(t.cs, cs.data(), n * sizeof(CsBatchInst)));
     CK(put(t.mu, mu.data(), n * sizeof(MuBatchInst)));
-    CK(put(t.rho_df, rdf.data(), rdf.size()));
-    CK(put(t.rho_f32, rf.data(), rf.size()));
-    CK(put(t.force, force.data(), force.size()));
+    CK(put(t.rho_df, rdf.data(), n * sizeof(Lines32Inst)));
+    CK(put(t.rho_f32, rf.data(), n * sizeof(Lines32Inst)));
+    CK(put(t.force, force.data(), n * sizeof(Lines32Inst)));
     CK(put(t.map_cs, mcs.data(), mcs.size() * sizeof(int)));
     CK(put(t.map_mu, mmu.data(), mmu.size() * sizeof(int)));
     CK(put(t.map_rho_df, mrdf.data(), mrdf.size() * sizeof(int)));
@@ -281,17 +260,13 @@ const T* at(const lbm_batch* b, size_t off) {
     return reinterpret_cast<const T*>(b->ws + off);
 }
 
-// one FP32 line pass of the whole batch (kRhoF32 or kForce)
-cudaError_t f32_lines(const lbm_batch* b, LineBatchKind kind, int bump, cudaStream_t s) {
+// one FP32 line pass of the whole batch: the density's, or the force's
+cudaError_t f32_lines(const lbm_batch* b, bool rho, int bump, cudaStream_t s) {
     const Tables& t = b->tb;
-    const bool rho = kind == LineBatchKind::kRhoF32;
-    const char* d = b->ws + (rho ? t.rho_f32 : t.force);
-    const int* map = at<int>(b, rho ? t.map_rho_f32 : t.map_force);
-    const int nb = rho ? t.nb_rho_f32 : t.nb_force;
-    if (b->l32)
-        return lines32_batch_launch(reinterpret_cast<const Lines32Inst*>(d), map, nb, b->order,
-                                    rho, bump, b->line_nl, s);
-    return lines_batch_launch(kind, d, map, nb, b->order, bump, s, b->line_nl);
+    return lines32_batch_launch(at<Lines32Inst>(b, rho ? t.rho_f32 : t.force),
+                                at<int>(b, rho ? t.map_rho_f32 : t.map_force),
+                                rho ? t.nb_rho_f32 : t.nb_force, b->order, rho, bump, b->line_nl,
+                                b->wide, s);
 }
 
 // `side` (while capturing): another stream, on which the double-float density lines run
@@ -313,7 +288,7 @@ lbm_status enqueue_step(lbm_batch* b, cudaStream_t s, int from, cudaEvent_t* ev 
     }
     CK(lines_df_batch_launch(at<Lines32Inst>(b, t.rho_df), at<int>(b, t.map_rho_df), t.nb_rho_df,
                              b->order, 1, sd));
-    CK(f32_lines(b, LineBatchKind::kRhoF32, 1, s));
+    CK(f32_lines(b, true, 1, s));
     if (fork) {
         CK(cudaEventRecord(b->join_ev, side));
         CK(cudaStreamWaitEvent(s, b->join_ev, 0));
@@ -321,7 +296,7 @@ lbm_status enqueue_step(lbm_batch* b, cudaStream_t s, int from, cudaEvent_t* ev 
     CK(mark(2));
     CK(launch_mu_mixed_batch(at<MuBatchInst>(b, t.mu), at<int>(b, t.map_mu), t.nb_mu, s));
     CK(mark(3));
-    CK(f32_lines(b, LineBatchKind::kForce, 0, s));
+    CK(f32_lines(b, false, 0, s));
     CK(mark(4));
     return LBM_OK;
 }
@@ -396,16 +371,10 @@ lbm_status instance_force(lbm_batch* b, int i) {
     cudaStream_t s = b->stream;
     if (h.rho_df)
         CK(lines_df_rho(h.rh, h.rl, h.dxr, h.dxx, h.dyr, h.dyy, h.nx, h.ny, b->order, st, 0, s));
-    else if (b->l32)
+    else
         CK(lines32_rho(h.rh, h.dxr, h.dxx, h.dyr, h.dyy, h.nx, h.ny, b->order, st, 0, s));
-    else
-        CK(lines_mixed_rho_xy_f32(h.rh, h.dxr, h.dxx, h.dyr, h.dyy, h.nx, h.ny, b->order, st, 0,
-                                  s));
     CK(launch_mu_mixed(h.rh, h.dxx, h.dyy, h.nx, h.ny, h.phys, st, s));
-    if (b->l32)
-        CK(lines32_force(h.dxx, h.rh, h.dxr, h.dyr, h.Fx, h.Fy, h.nx, h.ny, b->order, st, s));
-    else
-        CK(lines_mixed_force_xy(h.dxx, h.rh, h.dxr, h.dyr, h.Fx, h.Fy, h.nx, h.ny, b->order, s));
+    CK(lines32_force(h.dxx, h.rh, h.dxr, h.dyr, h.Fx, h.Fy, h.nx, h.ny, b->order, st, s));
     return LBM_OK;
 }
 
@@ -457,7 +426,7 @@ lbm_status lbm_batch_init(lbm_batch** out, const lbm_instance* inst, int32_t n,
     if (!b) return LBM_ENOMEM;
     b->n = n;
     b->order = opts->fd_order;
-    b->l32 = small_lines(inst, n);
+    b->wide = wide_lines(inst, n);
     b->line_nl = 8;
     b->mrt = opts->collision == LBM_COLLIDE_MRT;
     b->rates = MrtRates{opts->s_e, opts->s_eps, opts->s_q};
@@ -744,8 +713,8 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int32_t reps) {
             st = upload_tables(b);
             if (st) return st;
             auto pass = [&]() -> cudaError_t {
-                const cudaError_t e = f32_lines(b, LineBatchKind::kRhoF32, 0, s);
-                return e != cudaSuccess ? e : f32_lines(b, LineBatchKind::kForce, 0, s);
+                const cudaError_t e = f32_lines(b, true, 0, s);
+                return e != cudaSuccess ? e : f32_lines(b, false, 0, s);
             };
             CK(pass());  // warm-up
             CK(cudaEventRecord(b->tev[0], s));

@@ -254,15 +254,20 @@ cudaError_t lines32_rho(const float* rh, float* dxr, float* dxx, float* dyr, flo
 cudaError_t lines32_force(const float* mu, const float* rh, const float* dxr, const float* dyr,
                           float* Fx, float* Fy, int nx, int ny, int order, DevState* st,
                           cudaStream_t s, bool walls_y = false);
-// Grids whose FP32 lines they solve.  Larger ones keep the full windows of
-// kernels_lines.cu: 1024^2 37.1 us a step against 35.4, 4096^2 499 against 471; 512^2 17.4
-// against 20.1.
+// Grids whose FP32 lines are solved by (line, chunk) pairs; larger ones take full windows
+// (lines32_wide.cu), which lines32_rho and lines32_force dispatch to.
 constexpr long long kLines32Nodes = 1LL << 19;
-// nl (8 or 16): blocks of 32 nl threads
-int lines32_batch_blocks(int nx, int ny, int order, bool second, int nl);
-Lines32Inst lines32_batch_inst(const MixedLinesView& v, int order, bool second, int blk0, int nl);
+cudaError_t lines32_wide(Dir32 x, Dir32 y, int nx, int ny, int order, bool second, DevState* st,
+                         int bump, cudaStream_t s);
+// Batches: nl (8 or 16): blocks of 32 nl threads; wide: full windows, nl lines a block
+int lines32_batch_blocks(int nx, int ny, int order, bool second, int nl, bool wide);
+Lines32Inst lines32_batch_inst(const MixedLinesView& v, int order, bool second, int blk0, int nl,
+                               bool wide);
 cudaError_t lines32_batch_launch(const Lines32Inst* d, const int* map, int nblocks, int order,
-                                 bool second, int bump, int nl, cudaStream_t s);
+                                 bool second, int bump, int nl, bool wide, cudaStream_t s);
+void lines32_wide_divide(Dir32& x, Dir32& y, int nl);
+cudaError_t lines32_wide_batch(const Lines32Inst* d, const int* map, int nblocks, int order,
+                               bool second, int bump, int nl, cudaStream_t s);
 
 // Double-float density lines (lines_df.cu): x and y in one launch, stand-alone, batches.
 cudaError_t lines_df_rho(const float* rh, const float* rl, float* dxr, float* dxx, float* dyr,
@@ -290,22 +295,6 @@ constexpr int64_t kSmallSteps = 512;        // steps a launch (a few millisecond
 bool small_steps_fit(const SmallStep& p);
 cudaError_t launch_small_steps(const SmallStep& p, int from, int64_t steps, cudaStream_t s);
 
-// Line passes: descriptor size per instance, blocks per instance, descriptor
-// written to host memory (copied to the device by the caller), the launches.
-enum class LineBatchKind {
-    kRhoDF,   // x|y lines of the density, double-float where a window needs it
-    kRhoF32,  // x|y lines of the density in FP32 (the hi part only)
-    kForce,   // x|y lines of mu-hat with the force epilogue
-};
-size_t lines_batch_desc_bytes(LineBatchKind kind);
-// nl: lines per block, 8 or 16 (the FP32 kinds; the double-float density lines
-// always take 8).  Results do not depend on it.
-int lines_batch_blocks(int nx, int ny, int order, LineBatchKind kind, int nl = 8);
-void lines_batch_fill(LineBatchKind kind, const MixedLinesView& v, int order, int blk0,
-                      void* host_dst, int nl = 8);
-cudaError_t lines_batch_launch(LineBatchKind kind, const void* d_desc, const int* map,
-                               int nblocks, int order, int bump, cudaStream_t s, int nl = 8);
-
 // Below this Maxwell density ratio the mixed path solves the density's lines in
 // FP32 (measured: coexistence densities within 2e-4 of the FP64 path); at and
 // above it, in double-float wherever a window spans more than a factor 32.
@@ -327,27 +316,10 @@ cudaError_t lines_fp64_force(const double* mu, const double* rho, const double* 
                              cudaStream_t s, bool walls_y = false);
 cudaError_t lines_fp64_plain(const double* u, double* d1, double* d2, int nx, int ny, int axis,
                              int order, cudaStream_t s);
-// Mixed path, merged launches: the x- and y-lines of rho together (first and
-// second derivatives); then, after launch_mu_mixed, the x- and y-lines of
-// mu-hat together with the force epilogue.
-cudaError_t lines_mixed_rho_xy(const float* rh, const float* rl, float* dxr, float* dxx,
-                               float* dyr, float* dyy, int nx, int ny, int order, DevState* st,
-                               int bump, cudaStream_t s, bool walls_y = false);
-// The same in FP32 on the hi part of the density (below kDfRatio).
-cudaError_t lines_mixed_rho_xy_f32(const float* rh, float* dxr, float* dxx, float* dyr,
-                                   float* dyy, int nx, int ny, int order, DevState* st, int bump,
-                                   cudaStream_t s, bool walls_y = false);
-cudaError_t lines_mixed_force_xy(const float* mu, const float* rh, const float* dxr,
-                                 const float* dyr, float* Fx, float* Fy, int nx, int ny,
-                                 int order, cudaStream_t s, bool walls_y = false,
-                                 DevState* st = nullptr);
 // mu-hat = k^2 mu0(rho) - kappa (d_xx + d_yy) rho (Eqs. 21, 33, Sec. 5.6), FP32,
 // written over d_xx rho (`dxx_mu`); flags bad values.
 cudaError_t launch_mu_mixed(const float* rh, float* dxx_mu, const float* dyy, int nx, int ny,
                             const PhysParams& p, DevState* st, cudaStream_t s);
-cudaError_t lines_mixed_plain(const float* uh, const float* ul, float* d1, float* d2, int nx,
-                              int ny, int axis, int order, cudaStream_t s);
-
 // Host thermodynamics of the product library (independent of the oracle), for
 // the EOS kinds LBM_EOS_* (Sec. 3.2).  Return 0 or -1 (invalid arguments, or
 // T outside (0, T_c) for the Maxwell pair).

@@ -167,13 +167,15 @@ cudaError_t run(Dir32 x, Dir32 y, int nx, int ny, int order, bool walls_y, DevSt
                 cudaStream_t s) {
     constexpr bool SECOND = MODE == l32::RHO;
     const int T = lay_out(x, y, nx, ny, order, SECOND, walls_y, 0);
+    if ((long long)nx * ny > kLines32Nodes)
+        return lines32_wide(x, y, nx, ny, order, SECOND, st, bump, s);
     const int nbx = blocks_of(x.g), nby = blocks_of(y.g);
     const size_t smem = smem_of(x.g, T, SECOND);
     auto go = [&](auto kern) -> cudaError_t {
         const cudaError_t e = allow_smem(kern, smem);
         if (e != cudaSuccess) return e;
-        return launch_pdl(kern, dim3(nbx + nby), dim3(T), smem, s, x, y, line32_constants(order), st,
-                          bump, nbx);
+        return launch_pdl(kern, dim3(nbx + nby), dim3(T), smem, s, x, y, line32_constants(order),
+                          st, bump, nbx);
     };
     return order == 6 ? go(k_lines32<MODE, true>) : go(k_lines32<MODE, false>);
 }
@@ -194,13 +196,15 @@ cudaError_t lines32_force(const float* mu, const float* rh, const float* dxr, co
 }
 
 // ---- batches ----
-int lines32_batch_blocks(int nx, int ny, int order, bool second, int nl) {
+int lines32_batch_blocks(int nx, int ny, int order, bool second, int nl, bool wide) {
     Dir32 x{}, y{};
     lay_out(x, y, nx, ny, order, second, false, 32 * nl);
+    if (wide) lines32_wide_divide(x, y, nl);
     return blocks_of(x.g) + blocks_of(y.g);
 }
 
-Lines32Inst lines32_batch_inst(const MixedLinesView& v, int order, bool second, int blk0, int nl) {
+Lines32Inst lines32_batch_inst(const MixedLinesView& v, int order, bool second, int blk0, int nl,
+                               bool wide) {
     Lines32Inst d{};
     if (second) {
         d.x = density_dir(v.rh, v.dxr, v.dxx);
@@ -210,6 +214,7 @@ Lines32Inst lines32_batch_inst(const MixedLinesView& v, int order, bool second, 
         d.y = force_dir(v.dxx, v.rh, v.dyr, v.Fy);
     }
     lay_out(d.x, d.y, v.nx, v.ny, order, second, false, 32 * nl);
+    if (wide) lines32_wide_divide(d.x, d.y, nl);
     d.nbx = blocks_of(d.x.g);
     d.blk0 = blk0;
     d.st = v.st;
@@ -219,8 +224,9 @@ Lines32Inst lines32_batch_inst(const MixedLinesView& v, int order, bool second, 
 // the largest shared memory a block of 32 nl threads can need: the shortest windows
 // (8 chunks) stage the most lines
 cudaError_t lines32_batch_launch(const Lines32Inst* d, const int* map, int nblocks, int order,
-                                 bool second, int bump, int nl, cudaStream_t s) {
+                                 bool second, int bump, int nl, bool wide, cudaStream_t s) {
     if (nblocks <= 0) return cudaSuccess;
+    if (wide) return lines32_wide_batch(d, map, nblocks, order, second, bump, nl, s);
     const int T = 32 * nl;
     size_t smem = 0;
     for (int nch = 8; nch <= 32; nch += 4) {
