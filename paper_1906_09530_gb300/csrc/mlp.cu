@@ -260,6 +260,7 @@ struct WgArgs {
     int chunks;       // K chunks (64 batch rows) in all
     int per_slice;    // K chunks per slice
     float* part;      // [slices][kWgTiles * 128][256]
+    double* next_sse; // squared-error sum of the next call, cleared here
     int* err;
 };
 
@@ -388,18 +389,28 @@ __device__ __forceinline__ void rows_store32(float* s, const float* x, float* ou
     __syncwarp();
 }
 
+// entries k .. k + 7 of row b of the input: x [B][4] FP32 -> BF16 [B][kK0], zero-padded
+__device__ __forceinline__ void input_piece(const float* x, __nv_bfloat16* x16, int b, int k) {
+    __align__(16) __nv_bfloat16 h[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        h[j] = __float2bfloat16_rn(k + j < kIn ? x[b * kIn + k + j] : 0.0f);
+    *reinterpret_cast<uint4*>(x16 + (long long)b * kK0 + k) = *reinterpret_cast<uint4*>(h);
+}
+
 // coalesced loads of this warp's 32 rows x kNC columns of a row-major FP32
 // matrix [M][256], issued ahead of use (rows >= M read as zero): piece j holds
 // row 4 j + lane / 8, columns 4 (lane % 8) .. + 3
+// (SELF: written earlier by this kernel, by the same lane: not through the read-only path)
+template <bool SELF = false>
 __device__ __forceinline__ void aux_fetch(float4* pf, const float* in, int r0, int c, int M,
                                           int lane) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const int rr = 4 * j + (lane >> 3), q = lane & 7;
-        pf[j] = r0 + rr < M
-                    ? __ldg(reinterpret_cast<const float4*>(in + (long long)(r0 + rr) * UN + c +
-                                                            4 * q))
-                    : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4* p =
+            reinterpret_cast<const float4*>(in + (long long)(r0 + rr) * UN + c + 4 * q);
+        pf[j] = r0 + rr >= M ? make_float4(0.f, 0.f, 0.f, 0.f) : (SELF ? *p : __ldg(p));
     }
 }
 // the fetched pieces into the staging block s, row r0 + i of the matrix in its row i
@@ -656,6 +667,208 @@ __global__ void __launch_bounds__(kRowsThreads, kRowsPerSm)
                      : "memory");
 }
 
+// ---------------------------------------------------------------------------
+// The whole chain of row products of one 128-row tile in a cluster of four CTAs, one per
+// 64-column block: the input conversion, the four layers and, in training, the three input
+// gradients.  A layer's rows need only their own tile's, so the cluster's barrier is all the
+// ordering they want: at batches of a few thousand, where each product is one round of
+// tiles, launching them one by one costs 5 us each.  Roles, tiles and epilogues are those of
+// k_umma_rows; all of a stage's A chunks are in flight at once, and the next stage's weights
+// arrive during this one.  Activations and signals pass through global memory: written by
+// ordinary stores, read by the next stage's tensor copies, hence the proxy fences on both
+// sides of the barrier.  A wait that runs out sets the abort flag; every thread still keeps
+// every barrier.  Bound by the latency of a stage, 4.7 us of fences, copies, MMAs and epilogue
+// one after another: 33 us a training pass of 256 rows, a fit step of them 46 us; with eight
+// launches 49 us.
+// ---------------------------------------------------------------------------
+constexpr int kChainCtas = UN / kNT, kChainStages = 2 * kLayers - 1;
+constexpr size_t kChainSmem = 1024 + 4 * kRowChunk + 2 * kRowB + (size_t)kRowEpi * 32 * kS32 * 4 +
+                              kLayers * kNT * 4 + (size_t)kRowEpi * (kNT / 2) * 4;
+static_assert(kChainSmem <= 227 * 1024 - 1024, "chain kernel shared memory");
+struct ChainMaps {
+    WgMaps wg;
+    CUtensorMap wt[kLayers], w[kLayers];
+};
+struct ChainArgs {
+    const float* x;
+    __nv_bfloat16* x16;
+    int n;                     // stages: 4 (inference) or 7
+    RowArgs st[kChainStages];  // layers 0..3, then the signals of layers 2, 1, 0
+};
+
+__device__ __forceinline__ void proxy_fence() {
+    asm volatile("fence.proxy.async;\n" ::: "memory");
+}
+__device__ __forceinline__ void chain_sync() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+
+__global__ void __launch_bounds__(kRowsThreads, 1)
+    k_umma_chain(const __grid_constant__ ChainMaps m, const __grid_constant__ ChainArgs g) {
+    extern __shared__ __align__(1024) unsigned char usm_raw[];
+    unsigned char* usm = usm_raw + ((1024u - (su32(usm_raw) & 1023u)) & 1023u);
+    unsigned char* bsm = usm + 4 * kRowChunk;  // two stages of Bt
+    float* st32 = reinterpret_cast<float*>(bsm + 2 * kRowB);
+    float* bias_s = st32 + kRowEpi * 32 * kS32;  // [layer][kNT]
+    float* bsum_s = bias_s + kLayers * kNT;
+    constexpr unsigned bbytes = kNT * kKC * 2;
+    // A chunk 0..3 there, Bt of even / odd stages there, accumulator 0/1 full
+    constexpr int FA = 0, FB = 4, AF = 6;
+    __shared__ __align__(8) uint64_t bar[8];
+    __shared__ uint32_t tbase;
+    __shared__ int abort_s;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = blockIdx.x, col0 = rank * kNT, t = blockIdx.y;
+    const int M = g.st[0].M;
+    int* err = g.st[0].err;
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                         su32(&tbase)),
+                     "r"(2 * kNT)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int q = 0; q < 8; ++q) mb_init(&bar[q], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        abort_s = 0;
+    }
+    pdl_prologue();  // what follows reads what the kernels before this one wrote
+    for (int i = tid; i < kLayers * kNT; i += kRowsThreads)
+        bias_s[i] = g.st[i / kNT].bias[col0 + i % kNT];
+    // this CTA's quarter of the tile's input rows, zero-padded to kK0 columns
+    if (tid < (UM / kChainCtas) * (kK0 / 8)) {
+        const int b = t * UM + rank * (UM / kChainCtas) + tid / (kK0 / 8);
+        const int k = 8 * (tid % (kK0 / 8));
+        if (b < M) input_piece(g.x, g.x16, b, k);
+    }
+    proxy_fence();
+    tc_fence_before();
+    __syncthreads();
+    chain_sync();
+    tc_fence_after();
+    const uint32_t tmem = tbase;
+    volatile int* abort_v = &abort_s;
+    auto give_up = [&] {
+        atomicExch(err, 1);
+        *abort_v = 1;
+    };
+    auto maps_of = [&](int s, const CUtensorMap*& a, const CUtensorMap*& b) {
+        a = s < kLayers ? &m.wg.a[s] : &m.wg.d[2 * kLayers - 1 - s];
+        b = s < kLayers ? &m.wt[s] : &m.w[2 * kLayers - 1 - s];
+    };
+    auto load_b = [&](int s) {
+        const CUtensorMap *a, *b;
+        maps_of(s, a, b);
+        const int nkc = s == 0 ? 1 : kW / kKC;
+        unsigned char* dst = bsm + (s & 1) * kRowB;
+        mb_expect(&bar[FB + (s & 1)], nkc * bbytes);
+        for (int j = 0; j < nkc; ++j) tma2(dst + j * bbytes, b, j * kKC, col0, &bar[FB + (s & 1)]);
+    };
+    static_assert(kNT == kBox, "a K chunk of Bt is one box");
+    double sse = 0.0;
+    int last_a = -1, last_b = -1;  // the loader's latest stages
+    for (int s = 0; s < g.n; ++s) {
+        const int nkc = s == 0 ? 1 : kW / kKC;  // K: kK0 in the first layer
+        if (warp == kRowEpi) {
+            if (lane == 0 && !*abort_v) {
+                proxy_fence();
+                if (s == 0) load_b(0);
+                const CUtensorMap *a, *b;
+                maps_of(s, a, b);
+                for (int j = 0; j < nkc; ++j) {
+                    mb_expect(&bar[FA + j], (unsigned)kRowChunk);
+                    for (int r = 0; r < UM; r += kBox)
+                        tma2(usm + j * kRowChunk + r * kKC * 2, a, j * kKC, t * UM + r,
+                             &bar[FA + j]);
+                }
+                if (s + 1 < g.n) load_b(s + 1);
+                last_a = s;
+                last_b = s + 1 < g.n ? s + 1 : s;
+            }
+            __syncwarp();
+        } else if (warp == kRowEpi + 1) {
+            if (lane == 0) {
+                const unsigned B = su32(bsm + (s & 1) * kRowB);
+                const uint32_t acc = tmem + (uint32_t)((s & 1) * kNT);
+                bool ok = mb_wait(&bar[FB + (s & 1)], (s >> 1) & 1, abort_v);
+                for (int j = 0; ok && j < nkc; ++j) {
+                    // chunk 0 is used by every stage, the others from the second on
+                    ok = mb_wait(&bar[FA + j], (j == 0 ? s : s - 1) & 1, abort_v);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const unsigned A = su32(usm + j * kRowChunk);
+                    for (int kk = 0; kk < kKC / 16; ++kk)
+                        umma<idesc(kNT, false)>(acc, umma_desc(A + kk * 32),
+                                                umma_desc(B + j * bbytes + kk * 32),
+                                                j > 0 || kk > 0);
+                }
+                if (!ok) give_up();
+                // (also after a failed wait: the MMAs issued complete before the CTA leaves)
+                umma_commit(&bar[AF + (s & 1)]);
+                if (!ok) mb_wait(&bar[AF + (s & 1)], (s >> 1) & 1, nullptr);
+            }
+            __syncwarp();
+        } else {
+            const RowArgs& r = g.st[s];
+            float* s32 = st32 + warp * 32 * kS32;
+            float* bsum = bsum_s + warp * (kNT / 2);
+            const int quarter = warp & 3, c0 = (warp >> 2) * (kNT / 2);
+            const int r0 = t * UM + quarter * 32;
+            float4 pf[8];
+            if (r.epi == EPI_TANH_BACK) aux_fetch<true>(pf, r.aprev, r0, col0 + c0, M, lane);
+            if (r.epi == EPI_LOSS) aux_fetch(pf, r.aprev, r0, col0 + c0, M, lane);
+            bool ok = mb_wait(&bar[AF + (s & 1)], (s >> 1) & 1, abort_v);
+            ok = __all_sync(0xffffffffu, ok);
+            if (ok) {
+                tc_fence_after();
+                const uint32_t acc =
+                    tmem + (uint32_t)((s & 1) * kNT) + ((uint32_t)(quarter * 32) << 16);
+                if (r.epi == EPI_TANH_BACK || r.epi == EPI_LOSS) aux_stage(pf, s32, lane);
+                float x[kNC];
+                tmem_ld(acc + (uint32_t)c0, x);
+                bsum[lane] = 0.0f;
+                __syncwarp();
+                rows_epilogue(r, x, bias_s + (s < kLayers ? s : 0) * kNT + c0, s32, r0, col0 + c0,
+                              lane, bsum, sse);
+                __syncwarp();
+                if (r.bpart) r.bpart[((long long)t * 4 + quarter) * UN + col0 + c0 + lane] = bsum[lane];
+            } else if (lane == 0) {
+                give_up();
+            }
+            tc_fence_before();
+        }
+        proxy_fence();
+        chain_sync();
+        tc_fence_after();
+    }
+    double* total = g.n > kLayers ? g.st[kLayers - 1].sse : nullptr;
+    if (total && warp < kRowEpi) {
+        for (int o = 16; o > 0; o >>= 1) sse += __shfl_down_sync(0xffffffffu, sse, o);
+        if (lane == 0) atomicAdd(total, sse);
+    }
+    if (lane == 0 && *abort_v) {
+        // what an abandoned stage has in flight completes before the CTA leaves (bounded)
+        if (warp == kRowEpi) {
+            const int s = last_a, nkc = s == 0 ? 1 : kW / kKC;
+            for (int j = 0; s >= 0 && j < nkc; ++j)
+                mb_wait(&bar[FA + j], (j == 0 ? s : s - 1) & 1, nullptr);
+            if (last_b >= 0) mb_wait(&bar[FB + (last_b & 1)], (last_b >> 1) & 1, nullptr);
+        } else if (warp == kRowEpi + 1) {
+            mb_wait(&bar[AF + ((g.n - 1) & 1)], ((g.n - 1) >> 1) & 1, nullptr);
+        }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
+                     "r"(2 * kNT)
+                     : "memory");
+}
+
 __global__ void __launch_bounds__(kWgThreads, 1)
     k_umma_wgrad(const __grid_constant__ WgMaps maps, WgArgs g) {
     extern __shared__ __align__(1024) unsigned char usm_raw[];
@@ -671,6 +884,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int mt = blockIdx.x, slice = blockIdx.y;
     const int layer = (mt + 1) / 2, m0 = mt == 0 ? 0 : ((mt - 1) & 1) * UM;
+    const bool clears = mt == 0 && slice == 0 && tid == 0;
     const int j0 = slice * g.per_slice;
     const int nk = min(g.per_slice, g.chunks - j0);  // >= 1 by the host's choice of slices
     if (warp == 0) {
@@ -686,6 +900,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         abort_s = 0;
     }
     pdl_prologue();
+    if (clears) *g.next_sse = 0.0;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -872,21 +1087,12 @@ __global__ void __launch_bounds__(256) k_gradient(GradArgs g) {
     }
 }
 
-// x [B][4] FP32 -> BF16 [B][kK0], zero-padded; the squared-error sum (not null) cleared
-__global__ void k_input(const float* __restrict__ x, __nv_bfloat16* __restrict__ x16, int B,
-                        double* sse) {
+// x [B][4] FP32 -> BF16 [B][kK0], zero-padded
+__global__ void k_input(const float* __restrict__ x, __nv_bfloat16* __restrict__ x16, int B) {
     pdl_prologue();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0 && sse) *sse = 0.0;
     // eight of a row's kK0 entries a thread
-    if (i < B * (kK0 / 8)) {
-        const int b = i / (kK0 / 8), k = 8 * (i - b * (kK0 / 8));
-        __align__(16) __nv_bfloat16 h[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-            h[j] = __float2bfloat16_rn(k + j < kIn ? x[b * kIn + k + j] : 0.0f);
-        *reinterpret_cast<uint4*>(x16 + (long long)b * kK0 + k) = *reinterpret_cast<uint4*>(h);
-    }
+    if (i < B * (kK0 / 8)) input_piece(x, x16, i / (kK0 / 8), 8 * (i % (kK0 / 8)));
 }
 
 // FP32 master weights -> BF16 copies ([fan_in padded][fan_out] for layer 0; the
@@ -976,8 +1182,9 @@ struct lbm_mlp {
     float *d32, *e32;            // the same in FP32 (mma.sync kernel only), alternating
     float* part;                 // weight-gradient partials [slices][kWgTiles * 128][256]
     float* bpart;                // bias-gradient partials [layers][kRowGridCap * 4][256]
-    double* sse;                 // device scalar
-    double* h_sse;               // pinned mirror of both
+    double* sse;                 // squared-error sums of this call and the next, in turn
+    int turn;                    // which of them is this call's
+    double* h_sse;               // pinned mirror of both and err
     long long step;
     bool tensor_cores;           // forward and input-gradient products by tcgen05
     TcMaps maps;
@@ -1034,7 +1241,7 @@ MlpLayout mlp_layout(int B0) {
     L.e32 = take(B * kW * 4);
     L.part = take(S * kWgTiles * UM * UN * 4);
     L.bpart = take((size_t)kLayers * kRowGridCap * 4 * UN * 4);
-    L.sse = take(16);  // the squared-error sum and the error word, read back together
+    L.sse = take(24);  // two squared-error sums and the error word, read back together
     L.total = o;
     return L;
 }
@@ -1061,7 +1268,7 @@ const __nv_bfloat16* w16t_of(const lbm_mlp* n, int l) {
 // Drain the stream; a tensor-core product whose bounded wait ran out since the
 // last check makes this LBM_ETIMEOUT (and the word is cleared).
 lbm_status sync(lbm_mlp* n) {
-    if (cudaMemcpyAsync(n->h_sse, n->sse, 16, cudaMemcpyDeviceToHost, n->stream) !=
+    if (cudaMemcpyAsync(n->h_sse, n->sse, 24, cudaMemcpyDeviceToHost, n->stream) !=
             cudaSuccess ||
         cudaStreamSynchronize(n->stream) != cudaSuccess)
         return LBM_ECUDA;
@@ -1135,26 +1342,33 @@ cudaError_t set_smem_attrs(int dev) {
     cudaError_t e = cudaFuncSetAttribute(k_umma_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kRowsSmem);
     if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_umma_chain, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kChainSmem);
+    if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_umma_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kWgSmem);
     if (e == cudaSuccess) done |= bit;
     return e;
 }
 
-// a launch with programmatic serialization (every kernel here starts with pdl_prologue)
+// a launch with programmatic serialization (every kernel here starts with pdl_prologue), in
+// clusters of `cluster` CTAs along x
 template <typename... KArgs, typename... Args>
 cudaError_t launch(void (*kern)(KArgs...), dim3 grid, int block, size_t smem, cudaStream_t s,
-                   Args&&... args) {
+                   int cluster, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
@@ -1170,57 +1384,48 @@ int row_walkers(const lbm_mlp* n, int M) {
 // D[M x 256] = A Bt^T with the epilogue of g
 cudaError_t rows_tc(lbm_mlp* n, const CUtensorMap& ta, const CUtensorMap& tb, const RowArgs& g) {
     return launch(k_umma_rows, dim3(row_walkers(n, g.M), UN / kNT), kRowsThreads, kRowsSmem,
-                  n->stream, ta, tb, g);
+                  n->stream, 1, ta, tb, g);
 }
 
 float* bpart_of(const lbm_mlp* n, int l) { return n->bpart + (size_t)l * kRowGridCap * 4 * UN; }
 
-// forward pass on tcgen05.  t null: inference, only the output (written to y).
-// t not null: training; the hidden layers keep what the backward pass needs
-// (FP32 activations), and the last layer's epilogue turns its output straight into
-// the loss signal dL/dy (BF16, column sums) and the squared-error sum, without
-// storing y.
-lbm_status forward_tc(lbm_mlp* n, const float* x, int B, const float* t, float* y) {
-    cudaStream_t s = n->stream;
-    const bool train = t != nullptr;
-    CK(launch(k_input, dim3((B * (kK0 / 8) + 255) / 256), 256, 0, s, x, n->x16, B,
-              train ? n->sse : nullptr));
+// The row products of a pass on tcgen05, in order: the four layers and, where there are
+// targets t (training), the signals of layers 2, 1, 0.  t null: inference, only the output
+// (written to y).  In training the hidden layers keep what the backward pass needs (FP32
+// activations), and the last layer's epilogue turns its output straight into the loss
+// signal dL/dy (BF16, column sums) and the squared-error sum, without storing y.
+int row_stages(lbm_mlp* n, int B, const float* t, float* y, RowArgs* st) {
     for (int l = 0; l < kLayers; ++l) {
-        const bool hidden = l < kLayers - 1;
-        RowArgs g{};
+        RowArgs& g = st[l];
+        g = RowArgs{};
         g.M = B;
         g.K = l == 0 ? kK0 : kW;
         g.bias = n->p + param_offset(l) + (long long)kFanIn[l] * kFanOut[l];
         g.ld32 = kW;
         g.ld16 = kW;
         g.err = n->err;
-        if (hidden) {
+        if (l < kLayers - 1) {
             g.epi = EPI_BIAS_TANH;
-            g.out32 = train ? n->a32[l] : nullptr;
+            g.out32 = t ? n->a32[l] : nullptr;
             g.out16 = n->a16[l];
-        } else if (train) {
+        } else if (t) {
             g.epi = EPI_LOSS;
             g.aprev = t;
             g.scale = 1.0f / ((float)B * kOut);
-            g.sse = n->sse;
+            g.sse = n->sse + n->turn;
             g.out16 = n->sig[l];
             g.bpart = bpart_of(n, l);
         } else {
             g.epi = EPI_BIAS;
             g.out32 = y;
         }
-        CK(rows_tc(n, n->maps.wg.a[l], n->maps.wt[l], g));
     }
-    return LBM_OK;
-}
-
-// the backward pass on tcgen05, after forward_tc with targets: the signals of the hidden
-// layers and the partial weight gradients
-lbm_status backward_tc(lbm_mlp* n, int B) {
+    if (!t) return kLayers;
     for (int l = kLayers - 1; l > 0; --l) {
         // D_{l-1} = (D_l W_l^T) (1 - A_{l-1}^2): K-major operands are D [B][fo] and
         // W_l itself ([fi][fo])
-        RowArgs g{};
+        RowArgs& g = st[2 * kLayers - 1 - l];
+        g = RowArgs{};
         g.M = B;
         g.K = kW;
         g.epi = EPI_TANH_BACK;
@@ -1229,30 +1434,59 @@ lbm_status backward_tc(lbm_mlp* n, int B) {
         g.ld16 = kW;
         g.bpart = bpart_of(n, l - 1);
         g.err = n->err;
-        CK(rows_tc(n, n->maps.wg.d[l], n->maps.w[l], g));
     }
+    return kChainStages;
+}
+
+// One chain launch where the row tiles are at most one round of clusters, else the input
+// conversion and the products one by one.
+lbm_status rows_pass(lbm_mlp* n, const float* x, int B, const float* t, float* y) {
+    ChainArgs c;
+    c.x = x;
+    c.x16 = n->x16;
+    c.n = row_stages(n, B, t, y, c.st);
+    const int tiles = (B + UM - 1) / UM;
+    if (tiles <= n->nsm / kChainCtas) {
+        ChainMaps m;
+        m.wg = n->maps.wg;
+        std::memcpy(m.wt, n->maps.wt, sizeof(m.wt));
+        std::memcpy(m.w, n->maps.w, sizeof(m.w));
+        CK(launch(k_umma_chain, dim3(kChainCtas, tiles), kRowsThreads, kChainSmem, n->stream,
+                  kChainCtas, m, c));
+        return LBM_OK;
+    }
+    CK(launch(k_input, dim3((B * (kK0 / 8) + 255) / 256), 256, 0, n->stream, 1, x, n->x16, B));
+    for (int s = 0; s < c.n; ++s) {
+        const int l = 2 * kLayers - 1 - s;  // of a signal stage
+        CK(rows_tc(n, s < kLayers ? n->maps.wg.a[s] : n->maps.wg.d[l],
+                   s < kLayers ? n->maps.wt[s] : n->maps.w[l], c.st[s]));
+    }
+    return LBM_OK;
+}
+
+// the partial weight gradients, after rows_pass with targets
+lbm_status wgrad_tc(lbm_mlp* n, int B) {
     const Slicing sl = slicing(B);
-    const WgArgs w{sl.chunks, sl.per_slice, n->part, n->err};
-    CK(launch(k_umma_wgrad, dim3(kWgTiles, sl.slices), kWgThreads, kWgSmem, n->stream,
+    const WgArgs w{sl.chunks, sl.per_slice, n->part, n->sse + (1 - n->turn), n->err};
+    CK(launch(k_umma_wgrad, dim3(kWgTiles, sl.slices), kWgThreads, kWgSmem, n->stream, 1,
               n->maps.wg, w));
     return LBM_OK;
 }
 
-// the gradient from the partial sums of backward_tc: into grad, or (grad null) into one
+// the gradient from the partial sums of wgrad_tc: into grad, or (grad null) into one
 // Adam step of the parameters
 lbm_status gradient_tc(lbm_mlp* n, int B, float* grad, float lr, float c1, float c2) {
     const GradArgs g{n->part, slicing(B).slices, n->bpart, 4 * row_walkers(n, B), grad,
                      n->p, n->m, n->v, lr, c1, c2, n->w16, n->w16t};
     CK(launch(grad ? k_gradient<false> : k_gradient<true>, dim3(kGradW + kGradB), 256, 0,
-              n->stream, g));
+              n->stream, 1, g));
     return LBM_OK;
 }
 
 // the mma.sync forward pass (every layer's FP32 output kept)
 lbm_status forward_ms(lbm_mlp* n, const float* x, int B) {
     cudaStream_t s = n->stream;
-    CK(launch(k_input, dim3((B * (kK0 / 8) + 255) / 256), 256, 0, s, x, n->x16, B,
-              (double*)nullptr));
+    CK(launch(k_input, dim3((B * (kK0 / 8) + 255) / 256), 256, 0, s, 1, x, n->x16, B));
     for (int l = 0; l < kLayers; ++l) {
         GemmArgs g{};
         g.A = l == 0 ? n->x16 : n->a16[l - 1];
@@ -1290,10 +1524,10 @@ bool use_tc(lbm_mlp* n, int B, lbm_status* st) {
 // loss and gradient into n->g (device) on the mma.sync kernel, after forward_ms()
 lbm_status backward_ms(lbm_mlp* n, const float* t, int B) {
     cudaStream_t s = n->stream;
-    CK(cudaMemsetAsync(n->sse, 0, sizeof(double), s));
+    CK(cudaMemsetAsync(n->sse, 0, 2 * sizeof(double), s));
     const int total = B * kOut;
     k_loss_grad<<<(total + 255) / 256 < 1024 ? (total + 255) / 256 : 1024, 256, 0, s>>>(
-        n->a32[kLayers - 1], t, total, 1.0f / (float)total, n->d32, n->sig[1], n->sse);
+        n->a32[kLayers - 1], t, total, 1.0f / (float)total, n->d32, n->sig[1], n->sse + n->turn);
     CK(cudaGetLastError());
     float* d32 = n->d32;
     __nv_bfloat16* d16 = n->sig[1];
@@ -1359,11 +1593,12 @@ lbm_status train(lbm_mlp* n, const float* x, const float* t, int B, float lr, fl
     lbm_status st = LBM_OK;
     const bool tc = use_tc(n, B, &st);
     if (st) return st;
+    n->turn = 1 - n->turn;  // (zero: cleared by the call before)
     auto loss = [&]() -> lbm_status {
         if (!h_loss) return LBM_OK;
         const lbm_status w = sync(n);
         if (w) return w;
-        *h_loss = *n->h_sse / ((double)B * kOut);
+        *h_loss = n->h_sse[n->turn] / ((double)B * kOut);
         return LBM_OK;
     };
     float c1 = 0.0f, c2 = 0.0f;
@@ -1373,8 +1608,8 @@ lbm_status train(lbm_mlp* n, const float* x, const float* t, int B, float lr, fl
         c2 = (float)(1.0 - std::pow(0.999, (double)n->step));
     };
     if (tc) {
-        st = forward_tc(n, x, B, t, nullptr);
-        if (!st) st = backward_tc(n, B);
+        st = rows_pass(n, x, B, t, nullptr);
+        if (!st) st = wgrad_tc(n, B);
         if (!st && !(lr > 0)) st = gradient_tc(n, B, d_grad ? d_grad : n->g, 0.0f, 0.0f, 0.0f);
         if (!st) st = loss();  // (a wait that ran out is reported before the step is taken)
         if (st || !(lr > 0)) return st;
@@ -1440,7 +1675,8 @@ lbm_status lbm_mlp_init(lbm_mlp** out, int32_t max_batch, void* d_ws, size_t byt
     n->part = (float*)(w + L.part);
     n->bpart = (float*)(w + L.bpart);
     n->sse = (double*)(w + L.sse);
-    n->err = (int*)(n->sse + 1);
+    n->err = (int*)(n->sse + 2);
+    n->turn = 0;
     n->step = 0;
     n->tensor_cores = true;
     if (cudaDeviceGetAttribute(&n->nsm, cudaDevAttrMultiProcessorCount, n->dev) != cudaSuccess ||
@@ -1448,11 +1684,11 @@ lbm_status lbm_mlp_init(lbm_mlp** out, int32_t max_batch, void* d_ws, size_t byt
         delete n;
         return LBM_ECUDA;
     }
-    if (cudaMallocHost((void**)&n->h_sse, 16) != cudaSuccess) {
+    if (cudaMallocHost((void**)&n->h_sse, 24) != cudaSuccess) {
         delete n;
         return LBM_ECUDA;
     }
-    n->h_err = (int*)(n->h_sse + 1);
+    n->h_err = (int*)(n->h_sse + 2);
     if (cudaMemsetAsync(w, 0, L.total, n->stream) != cudaSuccess) {
         lbm_mlp_free(n);
         return LBM_ECUDA;
@@ -1499,7 +1735,7 @@ lbm_status lbm_mlp_forward(lbm_mlp* n, const float* d_x, int32_t batch, float* d
     if (!n || !d_x || !d_y || batch < 1 || batch > n->max_batch) return LBM_EINVAL;
     CK(cudaSetDevice(n->dev));
     lbm_status st = LBM_OK;
-    if (use_tc(n, batch, &st)) return st ? st : forward_tc(n, d_x, batch, nullptr, d_y);
+    if (use_tc(n, batch, &st)) return st ? st : rows_pass(n, d_x, batch, nullptr, d_y);
     if (st) return st;
     st = forward_ms(n, d_x, batch);
     if (st) return st;
