@@ -327,19 +327,37 @@ constexpr uint32_t idesc(int n, bool mn) {
     return (1u << 4) | (1u << 7) | (1u << 10) | (mn ? 3u << 15 : 0u) |
            ((uint32_t)(n >> 3) << 17) | ((uint32_t)(UM >> 4) << 24);
 }
+// The MMA issuer is a whole warp that stays together, in which one elected lane issues: with
+// operands that the compiler sees to be the same in every lane, four MMAs and a commit take
+// half the time that they do from one lane of a divergent branch (650 -> 390 cycles a
+// chunk of the chain kernel).
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t r;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(r));
+    return r;
+}
 template <uint32_t IDESC>
-__device__ __forceinline__ void umma(uint32_t tmem, uint64_t da, uint64_t db, bool acc) {
+__device__ __forceinline__ void umma(uint32_t lead, uint32_t tmem, uint64_t da, uint64_t db,
+                                     bool acc) {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-        "l"(da), "l"(db), "r"(IDESC), "r"(acc ? 1u : 0u)
+        "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 e, %5, 0;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+        "l"(da), "l"(db), "r"(IDESC), "r"(acc ? 1u : 0u), "r"(lead)
         : "memory");
 }
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
+__device__ __forceinline__ void umma_commit(uint32_t lead, uint64_t* bar) {
     asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-            su32(bar))
+        "{\n .reg .pred e;\n setp.ne.b32 e, %1, 0;\n"
+        " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::
+            "r"(su32(bar)),
+        "r"(lead)
         : "memory");
+}
+// mb_wait by a whole warp, with one answer for all of it
+__device__ __forceinline__ bool mb_wait_warp(uint64_t* bar, unsigned parity,
+                                             const volatile int* abort_flag) {
+    return __all_sync(0xffffffffu, mb_wait(bar, parity, abort_flag));
 }
 __device__ __forceinline__ void tc_fence_before() {
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -390,27 +408,26 @@ __device__ __forceinline__ void rows_store32(float* s, const float* x, float* ou
 }
 
 // entries k .. k + 7 of row b of the input: x [B][4] FP32 -> BF16 [B][kK0], zero-padded
-__device__ __forceinline__ void input_piece(const float* x, __nv_bfloat16* x16, int b, int k) {
+__device__ __forceinline__ uint4 input_piece(const float* x, int b, int k) {
     __align__(16) __nv_bfloat16 h[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j)
         h[j] = __float2bfloat16_rn(k + j < kIn ? x[b * kIn + k + j] : 0.0f);
-    *reinterpret_cast<uint4*>(x16 + (long long)b * kK0 + k) = *reinterpret_cast<uint4*>(h);
+    return *reinterpret_cast<uint4*>(h);
 }
 
 // coalesced loads of this warp's 32 rows x kNC columns of a row-major FP32
 // matrix [M][256], issued ahead of use (rows >= M read as zero): piece j holds
 // row 4 j + lane / 8, columns 4 (lane % 8) .. + 3
-// (SELF: written earlier by this kernel, by the same lane: not through the read-only path)
-template <bool SELF = false>
 __device__ __forceinline__ void aux_fetch(float4* pf, const float* in, int r0, int c, int M,
                                           int lane) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const int rr = 4 * j + (lane >> 3), q = lane & 7;
-        const float4* p =
-            reinterpret_cast<const float4*>(in + (long long)(r0 + rr) * UN + c + 4 * q);
-        pf[j] = r0 + rr >= M ? make_float4(0.f, 0.f, 0.f, 0.f) : (SELF ? *p : __ldg(p));
+        pf[j] = r0 + rr < M
+                    ? __ldg(reinterpret_cast<const float4*>(in + (long long)(r0 + rr) * UN + c +
+                                                            4 * q))
+                    : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
 // the fetched pieces into the staging block s, row r0 + i of the matrix in its row i
@@ -586,37 +603,40 @@ __global__ void __launch_bounds__(kRowsThreads, kRowsPerSm)
                 mb_wait(&bar[F0 + r % kRowStages], (r / kRowStages) & 1, nullptr);
         }
     } else if (warp == kRowEpi + 1) {
-        if (lane == 0) {
-            // MMA issuer: one accumulator per tile, alternating
-            int q = 0, i = 0, committed = -1;
-            const unsigned B = su32(bsm);
-            bool ok = mb_wait(&bar[BF], 0, abort_v);
-            for (int t = blockIdx.x; ok && t < ntiles; t += gridDim.x, ++i) {
-                if (i >= 2) ok = mb_wait(&bar[AE + (i & 1)], ((i - 2) >> 1) & 1, abort_v);
+        // MMA issuer: one accumulator per tile, alternating
+        const uint32_t lead = elect_one();
+        int q = 0, i = 0, committed = -1;
+        const uint64_t B = umma_desc(su32(bsm));
+        bool ok = mb_wait_warp(&bar[BF], 0, abort_v);
+        for (int t = blockIdx.x; ok && t < ntiles; t += gridDim.x, ++i) {
+            if (i >= 2) ok = mb_wait_warp(&bar[AE + (i & 1)], ((i - 2) >> 1) & 1, abort_v);
+            if (!ok) break;
+            const uint32_t acc = tmem + (uint32_t)((i & 1) * kNT);
+            for (int j = 0; j < nkc; ++j, ++q) {
+                const int st = q % kRowStages;
+                ok = mb_wait_warp(&bar[F0 + st], (q / kRowStages) & 1, abort_v);
                 if (!ok) break;
-                const uint32_t acc = tmem + (uint32_t)((i & 1) * kNT);
-                for (int j = 0; j < nkc; ++j, ++q) {
-                    const int st = q % kRowStages;
-                    ok = mb_wait(&bar[F0 + st], (q / kRowStages) & 1, abort_v);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const unsigned A = su32(usm + st * kRowChunk);
-                    for (int kk = 0; kk < kKC / 16; ++kk)
-                        umma<idesc(kNT, false)>(acc, umma_desc(A + kk * 32),
-                                                umma_desc(B + j * bbytes + kk * 32), j > 0 || kk > 0);
-                    umma_commit(&bar[E0 + st]);
-                    committed = q;
-                }
-                if (!ok) break;
-                umma_commit(&bar[AF + (i & 1)]);
+                tc_fence_after();
+                const uint64_t A = umma_desc(su32(usm + st * kRowChunk));
+#pragma unroll
+                for (int kk = 0; kk < kKC / 16; ++kk)
+                    umma<idesc(kNT, false)>(lead, acc, A + kk * 2,
+                                            B + (uint64_t)(j * (bbytes >> 4) + kk * 2),
+                                            j > 0 || kk > 0);
+                umma_commit(lead, &bar[E0 + st]);
+                committed = q;
             }
-            if (!ok) {
+            if (!ok) break;
+            umma_commit(lead, &bar[AF + (i & 1)]);
+        }
+        if (!ok) {
+            if (lead) {
                 atomicExch(g.err, 1);
                 *abort_v = 1;
-                if (committed >= 0)
-                    mb_wait(&bar[E0 + committed % kRowStages], (committed / kRowStages) & 1,
-                            nullptr);
             }
+            if (committed >= 0)
+                mb_wait_warp(&bar[E0 + committed % kRowStages], (committed / kRowStages) & 1,
+                             nullptr);
         }
     } else {
         float* s32 = st32 + warp * 32 * kS32;
@@ -668,26 +688,31 @@ __global__ void __launch_bounds__(kRowsThreads, kRowsPerSm)
 }
 
 // ---------------------------------------------------------------------------
-// The whole chain of row products of one 128-row tile in a cluster of four CTAs, one per
-// 64-column block: the input conversion, the four layers and, in training, the three input
-// gradients.  A layer's rows need only their own tile's, so the cluster's barrier is all the
-// ordering they want: at batches of a few thousand, where each product is one round of
-// tiles, launching them one by one costs 5 us each.  Roles, tiles and epilogues are those of
-// k_umma_rows; all of a stage's A chunks are in flight at once, and the next stage's weights
-// arrive during this one.  Activations and signals pass through global memory: written by
-// ordinary stores, read by the next stage's tensor copies, hence the proxy fences on both
-// sides of the barrier.  A wait that runs out sets the abort flag; every thread still keeps
-// every barrier.  Bound by the latency of a stage, 4.7 us of fences, copies, MMAs and epilogue
-// one after another: 33 us a training pass of 256 rows, a fit step of them 46 us; with eight
-// launches 49 us.
+// The whole chain of row products of 32 batch rows in one CTA: the input conversion, the
+// four layers and, in training, the three input gradients.  The products are transposed,
+// D^T = W^T A^T: 256 features are two 128-row tiles of weights, streamed through a ring, the
+// 32 batch rows the narrow operand, which stays in shared memory from one stage to the next,
+// so that no CTA needs another's results.  A thread of the epilogue has one feature of 16
+// rows: targets, outputs and biases are read and written in rows without staging; the
+// hidden activations that the backward stages need stay in tensor memory.  Global memory
+// gets what the weight gradient reads, written while the next products run.
+// Roles: warps 0..15 epilogue, then the loader and the MMA issuer.  A wait that runs out sets
+// the abort flag, on which every later wait gives up: the CTA goes through its stages
+// without waiting, and its results are void.
+// Bound by a stage's latency: @@M@@
 // ---------------------------------------------------------------------------
-constexpr int kChainCtas = UN / kNT, kChainStages = 2 * kLayers - 1;
-constexpr size_t kChainSmem = 1024 + 4 * kRowChunk + 2 * kRowB + (size_t)kRowEpi * 32 * kS32 * 4 +
-                              kLayers * kNT * 4 + (size_t)kRowEpi * (kNT / 2) * 4;
+constexpr int kChainRows = 32, kChainStages = 2 * kLayers - 1;
+constexpr int kChainEpi = 16, kChainThreads = 32 * (kChainEpi + 2), kChainRing = 11;
+constexpr int kCR = kChainRows / 2;  // rows of an epilogue thread
+constexpr size_t kActChunk = (size_t)kChainRows * kKC * 2, kAct = (kW / kKC) * kActChunk;
+constexpr size_t kChainSmem = 1024 + kChainRing * kRowChunk + 2 * kAct;
 static_assert(kChainSmem <= 227 * 1024 - 1024, "chain kernel shared memory");
+// tensor memory: [feature tile][row] of the accumulators, then of each hidden layer
+constexpr int kChainCols = kLayers * 2 * kChainRows;
+static_assert(kChainCols == 256, "an allocation is a power of two");
+static_assert(kK0 == kKC && kKC * 2 == 128 && UM == 2 * kBox && kW == 2 * UM, "chain layout");
 struct ChainMaps {
-    WgMaps wg;
-    CUtensorMap wt[kLayers], w[kLayers];
+    CUtensorMap w[kChainStages];  // each stage's weights, [feature][K]
 };
 struct ChainArgs {
     const float* x;
@@ -696,176 +721,235 @@ struct ChainArgs {
     RowArgs st[kChainStages];  // layers 0..3, then the signals of layers 2, 1, 0
 };
 
-__device__ __forceinline__ void proxy_fence() {
-    asm volatile("fence.proxy.async;\n" ::: "memory");
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* x) {
+    uint32_t v[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
+        "%13,%14,%15}, [%16];\n"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+          "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
+          "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+    for (int j = 0; j < 16; ++j) x[j] = __uint_as_float(v[j]);
 }
-__device__ __forceinline__ void chain_sync() {
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* x) {
+    uint32_t v[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(x[j]);
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,"
+        "%12,%13,%14,%15};\n" ::"r"(v[0]),
+        "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]),
+        "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]),
+        "r"(taddr)
+        : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
 }
 
-__global__ void __launch_bounds__(kRowsThreads, 1)
+__global__ void __launch_bounds__(kChainThreads, 1)
     k_umma_chain(const __grid_constant__ ChainMaps m, const __grid_constant__ ChainArgs g) {
     extern __shared__ __align__(1024) unsigned char usm_raw[];
     unsigned char* usm = usm_raw + ((1024u - (su32(usm_raw) & 1023u)) & 1023u);
-    unsigned char* bsm = usm + 4 * kRowChunk;  // two stages of Bt
-    float* st32 = reinterpret_cast<float*>(bsm + 2 * kRowB);
-    float* bias_s = st32 + kRowEpi * 32 * kS32;  // [layer][kNT]
-    float* bsum_s = bias_s + kLayers * kNT;
-    constexpr unsigned bbytes = kNT * kKC * 2;
-    // A chunk 0..3 there, Bt of even / odd stages there, accumulator 0/1 full
-    constexpr int FA = 0, FB = 4, AF = 6;
-    __shared__ __align__(8) uint64_t bar[8];
+    // the weights' ring, then two stages of the rows: [K chunk][row][128 bytes], swizzled
+    unsigned char* act = usm + kChainRing * kRowChunk;
+    // chunks there, chunks free, feature tile 0/1 done, rows there, all products done
+    constexpr int F0 = 0, E0 = kChainRing, TF = 2 * kChainRing, RF = TF + 2, DN = RF + 1;
+    __shared__ __align__(8) uint64_t bar[DN + 1];
+    __shared__ float half_s[2][kChainEpi / 2][32];  // (of two stages: a reader may lag by one)
     __shared__ uint32_t tbase;
     __shared__ int abort_s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int rank = blockIdx.x, col0 = rank * kNT, t = blockIdx.y;
-    const int M = g.st[0].M;
-    int* err = g.st[0].err;
+    const int R0 = blockIdx.x * kChainRows, M = g.st[0].M;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
                          su32(&tbase)),
-                     "r"(2 * kNT)
+                     "r"(kChainCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
     if (tid == 0) {
-        for (int q = 0; q < 8; ++q) mb_init(&bar[q], 1);
+        for (int q = 0; q <= DN; ++q) mb_init(&bar[q], q == RF ? kChainEpi : 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         abort_s = 0;
     }
     pdl_prologue();  // what follows reads what the kernels before this one wrote
-    for (int i = tid; i < kLayers * kNT; i += kRowsThreads)
-        bias_s[i] = g.st[i / kNT].bias[col0 + i % kNT];
-    // this CTA's quarter of the tile's input rows, zero-padded to kK0 columns
-    if (tid < (UM / kChainCtas) * (kK0 / 8)) {
-        const int b = t * UM + rank * (UM / kChainCtas) + tid / (kK0 / 8);
-        const int k = 8 * (tid % (kK0 / 8));
-        if (b < M) input_piece(g.x, g.x16, b, k);
+    if (tid < kChainRows * (kK0 / 8)) {
+        const int r = tid / (kK0 / 8), q = tid % (kK0 / 8), b = R0 + r;
+        const uint4 v = b < M ? input_piece(g.x, b, 8 * q) : make_uint4(0u, 0u, 0u, 0u);
+        *reinterpret_cast<uint4*>(act + r * 128 + ((q ^ (r & 7)) << 4)) = v;
+        if (b < M) *reinterpret_cast<uint4*>(g.x16 + (long long)b * kK0 + 8 * q) = v;
     }
-    proxy_fence();
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     tc_fence_before();
     __syncthreads();
-    chain_sync();
     tc_fence_after();
     const uint32_t tmem = tbase;
     volatile int* abort_v = &abort_s;
     auto give_up = [&] {
-        atomicExch(err, 1);
+        atomicExch(g.st[0].err, 1);
         *abort_v = 1;
     };
-    auto maps_of = [&](int s, const CUtensorMap*& a, const CUtensorMap*& b) {
-        a = s < kLayers ? &m.wg.a[s] : &m.wg.d[2 * kLayers - 1 - s];
-        b = s < kLayers ? &m.wt[s] : &m.w[2 * kLayers - 1 - s];
-    };
-    auto load_b = [&](int s) {
-        const CUtensorMap *a, *b;
-        maps_of(s, a, b);
-        const int nkc = s == 0 ? 1 : kW / kKC;
-        unsigned char* dst = bsm + (s & 1) * kRowB;
-        mb_expect(&bar[FB + (s & 1)], nkc * bbytes);
-        for (int j = 0; j < nkc; ++j) tma2(dst + j * bbytes, b, j * kKC, col0, &bar[FB + (s & 1)]);
-    };
-    static_assert(kNT == kBox, "a K chunk of Bt is one box");
-    double sse = 0.0;
-    int last_a = -1, last_b = -1;  // the loader's latest stages
-    for (int s = 0; s < g.n; ++s) {
-        const int nkc = s == 0 ? 1 : kW / kKC;  // K: kK0 in the first layer
-        if (warp == kRowEpi) {
-            if (lane == 0 && !*abort_v) {
-                proxy_fence();
-                if (s == 0) load_b(0);
-                const CUtensorMap *a, *b;
-                maps_of(s, a, b);
-                for (int j = 0; j < nkc; ++j) {
-                    mb_expect(&bar[FA + j], (unsigned)kRowChunk);
-                    for (int r = 0; r < UM; r += kBox)
-                        tma2(usm + j * kRowChunk + r * kKC * 2, a, j * kKC, t * UM + r,
-                             &bar[FA + j]);
-                }
-                if (s + 1 < g.n) load_b(s + 1);
-                last_a = s;
-                last_b = s + 1 < g.n ? s + 1 : s;
+    if (warp == kChainEpi) {
+        if (lane == 0) {
+            // loader: each stage's weights, tile after tile, through the ring
+            int q = 0;  // chunks issued
+            bool ok = true;
+            for (int s = 0; ok && s < g.n; ++s) {
+                const int nkc = s == 0 ? 1 : kW / kKC;  // K: kK0 in the first layer
+                for (int tile = 0; ok && tile < 2; ++tile)
+                    for (int j = 0; j < nkc; ++j, ++q) {
+                        const int st = q % kChainRing;
+                        if (q >= kChainRing)
+                            ok = mb_wait(&bar[E0 + st], ((q / kChainRing) - 1) & 1, abort_v);
+                        if (!ok) break;
+                        mb_expect(&bar[F0 + st], (unsigned)kRowChunk);
+                        for (int r = 0; r < UM; r += kBox)
+                            tma2(usm + st * kRowChunk + r * kKC * 2, &m.w[s], j * kKC,
+                                 tile * UM + r, &bar[F0 + st]);
+                    }
             }
-            __syncwarp();
-        } else if (warp == kRowEpi + 1) {
-            if (lane == 0) {
-                const unsigned B = su32(bsm + (s & 1) * kRowB);
-                const uint32_t acc = tmem + (uint32_t)((s & 1) * kNT);
-                bool ok = mb_wait(&bar[FB + (s & 1)], (s >> 1) & 1, abort_v);
-                for (int j = 0; ok && j < nkc; ++j) {
-                    // chunk 0 is used by every stage, the others from the second on
-                    ok = mb_wait(&bar[FA + j], (j == 0 ? s : s - 1) & 1, abort_v);
+            if (!ok) give_up();
+            // the copies issued last complete before the CTA leaves (bounded)
+            for (int r = (q > kChainRing ? q - kChainRing : 0); r < q; ++r)
+                mb_wait(&bar[F0 + r % kChainRing], (r / kChainRing) & 1, nullptr);
+        }
+    } else if (warp == kChainEpi + 1) {
+        const uint32_t lead = elect_one();
+        int st = 0;
+        unsigned phase = 0;
+        bool ok = true;
+        for (int s = 0; ok && s < g.n; ++s) {
+            const int nkc = s == 0 ? 1 : kW / kKC;
+            const uint64_t rows = umma_desc(su32(act + (s & 1) * kAct));
+            if (s > 0) ok = mb_wait_warp(&bar[RF], (s - 1) & 1, abort_v);
+            for (int tile = 0; ok && tile < 2; ++tile) {
+                for (int j = 0; j < nkc; ++j) {
+                    ok = mb_wait_warp(&bar[F0 + st], phase, abort_v);
                     if (!ok) break;
                     tc_fence_after();
-                    const unsigned A = su32(usm + j * kRowChunk);
+                    const uint64_t A = umma_desc(su32(usm + st * kRowChunk));
+                    const uint64_t B = rows + (uint64_t)j * (kActChunk >> 4);
+#pragma unroll
                     for (int kk = 0; kk < kKC / 16; ++kk)
-                        umma<idesc(kNT, false)>(acc, umma_desc(A + kk * 32),
-                                                umma_desc(B + j * bbytes + kk * 32),
-                                                j > 0 || kk > 0);
+                        umma<idesc(kChainRows, false)>(lead, tmem + (uint32_t)(tile * kChainRows),
+                                                       A + kk * 2, B + kk * 2, j > 0 || kk > 0);
+                    umma_commit(lead, &bar[E0 + st]);
+                    if (++st == kChainRing) {
+                        st = 0;
+                        phase ^= 1u;
+                    }
                 }
-                if (!ok) give_up();
-                // (also after a failed wait: the MMAs issued complete before the CTA leaves)
-                umma_commit(&bar[AF + (s & 1)]);
-                if (!ok) mb_wait(&bar[AF + (s & 1)], (s >> 1) & 1, nullptr);
+                if (ok) umma_commit(lead, &bar[TF + tile]);
             }
-            __syncwarp();
-        } else {
+        }
+        if (!ok && lead) give_up();
+        umma_commit(lead, &bar[DN]);
+        mb_wait_warp(&bar[DN], 0, nullptr);
+    } else {
+        const int quarter = warp & 3, tile = (warp >> 2) & 1, half = warp >> 3;
+        const int f0 = tile * UM + quarter * 32, f = f0 + lane;
+        const int r0 = R0 + half * kCR;  // this thread's rows r0 ..  of feature f
+        const int nr = M - r0;           // those below it are live
+        const uint32_t col = tmem + ((uint32_t)(quarter * 32) << 16) +
+                             (uint32_t)(tile * kChainRows + half * kCR);
+        // element f of a row of the narrow operand; this warp's 32 features of it
+        unsigned char* af = act + (f >> 6) * kActChunk + (f & 7) * 2;
+        const int piece = (f & 63) >> 3, piece0 = (f0 & 63) >> 3;
+        double sse = 0.0;
+        for (int s = 0; s < g.n; ++s) {
             const RowArgs& r = g.st[s];
-            float* s32 = st32 + warp * 32 * kS32;
-            float* bsum = bsum_s + warp * (kNT / 2);
-            const int quarter = warp & 3, c0 = (warp >> 2) * (kNT / 2);
-            const int r0 = t * UM + quarter * 32;
-            float4 pf[8];
-            if (r.epi == EPI_TANH_BACK) aux_fetch<true>(pf, r.aprev, r0, col0 + c0, M, lane);
-            if (r.epi == EPI_LOSS) aux_fetch(pf, r.aprev, r0, col0 + c0, M, lane);
-            bool ok = mb_wait(&bar[AF + (s & 1)], (s >> 1) & 1, abort_v);
-            ok = __all_sync(0xffffffffu, ok);
-            if (ok) {
-                tc_fence_after();
-                const uint32_t acc =
-                    tmem + (uint32_t)((s & 1) * kNT) + ((uint32_t)(quarter * 32) << 16);
-                if (r.epi == EPI_TANH_BACK || r.epi == EPI_LOSS) aux_stage(pf, s32, lane);
-                float x[kNC];
-                tmem_ld(acc + (uint32_t)c0, x);
-                bsum[lane] = 0.0f;
-                __syncwarp();
-                rows_epilogue(r, x, bias_s + (s < kLayers ? s : 0) * kNT + c0, s32, r0, col0 + c0,
-                              lane, bsum, sse);
-                __syncwarp();
-                if (r.bpart) r.bpart[((long long)t * 4 + quarter) * UN + col0 + c0 + lane] = bsum[lane];
-            } else if (lane == 0) {
+            const unsigned next = (unsigned)(((s + 1) & 1) * kAct);
+            float a[kCR], x[kCR];
+            const float bias = r.bias ? r.bias[f] : 0.0f;
+            if (r.epi == EPI_LOSS) {
+#pragma unroll
+                for (int j = 0; j < kCR; ++j)
+                    a[j] = j < nr ? __ldg(r.aprev + (long long)(r0 + j) * UN + f) : 0.0f;
+            }
+            if (!__all_sync(0xffffffffu, mb_wait(&bar[TF + tile], s & 1, abort_v)) && lane == 0)
                 give_up();
+            __syncwarp();
+            tc_fence_after();
+            tmem_ld16(col, x);
+            if (r.epi == EPI_TANH_BACK) {
+                tmem_ld16(col + (uint32_t)((kChainStages - s) * 2 * kChainRows), a);
+#pragma unroll
+                for (int j = 0; j < kCR; ++j) x[j] *= 1.0f - a[j] * a[j];
+            } else if (r.epi == EPI_BIAS_TANH) {
+#pragma unroll
+                for (int j = 0; j < kCR; ++j) x[j] = tanh_act(x[j] + bias);
+            } else if (r.epi == EPI_BIAS) {
+#pragma unroll
+                for (int j = 0; j < kCR; ++j) x[j] += bias;
+            } else {
+                float e2 = 0.0f;
+#pragma unroll
+                for (int j = 0; j < kCR; ++j) {
+                    const float e = j < nr ? x[j] + bias - a[j] : 0.0f;
+                    e2 = fmaf(e, e, e2);
+                    x[j] = 2.0f * e * r.scale;
+                }
+                sse += (double)e2;
+            }
+#pragma unroll
+            for (int j = 0; j < kCR; ++j)
+                if (j >= nr) x[j] = 0.0f;  // rows past M add nothing to the sums
+            if (r.out16) {
+#pragma unroll
+                for (int j = 0; j < kCR; ++j) {
+                    const int rr = half * kCR + j;
+                    *reinterpret_cast<__nv_bfloat16*>(af + next + rr * 128 +
+                                                      ((piece ^ (rr & 7)) << 4)) =
+                        __float2bfloat16_rn(x[j]);
+                }
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
             }
             tc_fence_before();
+            __syncwarp();
+            if (lane == 0 && s + 1 < g.n) mb_arrive(&bar[RF]);
+            // what the backward stages and the other kernels read
+            if (r.epi == EPI_BIAS_TANH && g.n > kLayers)
+                tmem_st16(col + (uint32_t)((s + 1) * 2 * kChainRows), x);
+            if (r.out16) {
+#pragma unroll
+                for (int i = 0; i < kCR * 4 / 32; ++i) {
+                    const int j = (lane + 32 * i) >> 2, p = lane & 3, rr = half * kCR + j;
+                    if (j < nr)
+                        *reinterpret_cast<uint4*>(r.out16 + (long long)(r0 + j) * kW + f0 +
+                                                  8 * p) =
+                            *reinterpret_cast<const uint4*>(
+                                act + (f0 >> 6) * kActChunk + next + rr * 128 +
+                                (((piece0 + p) ^ (rr & 7)) << 4));
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < kCR; ++j)
+                    if (j < nr) r.out32[(long long)(r0 + j) * kW + f] = x[j];
+            }
+            if (r.bpart) {
+                // rows 0 .. 15 and 16 .. 31, then the halves
+                float cs = 0.0f;
+#pragma unroll
+                for (int j = 0; j < kCR; ++j) cs += x[j];
+                if (half) half_s[s & 1][warp & 7][lane] = cs;
+                asm volatile("bar.sync %0, 64;\n" ::"r"(1 + (warp & 7)) : "memory");
+                if (!half)
+                    r.bpart[(long long)blockIdx.x * UN + f] = cs + half_s[s & 1][warp & 7][lane];
+            }
+            __syncwarp();
         }
-        proxy_fence();
-        chain_sync();
-        tc_fence_after();
-    }
-    double* total = g.n > kLayers ? g.st[kLayers - 1].sse : nullptr;
-    if (total && warp < kRowEpi) {
-        for (int o = 16; o > 0; o >>= 1) sse += __shfl_down_sync(0xffffffffu, sse, o);
-        if (lane == 0) atomicAdd(total, sse);
-    }
-    if (lane == 0 && *abort_v) {
-        // what an abandoned stage has in flight completes before the CTA leaves (bounded)
-        if (warp == kRowEpi) {
-            const int s = last_a, nkc = s == 0 ? 1 : kW / kKC;
-            for (int j = 0; s >= 0 && j < nkc; ++j)
-                mb_wait(&bar[FA + j], (j == 0 ? s : s - 1) & 1, nullptr);
-            if (last_b >= 0) mb_wait(&bar[FB + (last_b & 1)], (last_b >> 1) & 1, nullptr);
-        } else if (warp == kRowEpi + 1) {
-            mb_wait(&bar[AF + ((g.n - 1) & 1)], ((g.n - 1) >> 1) & 1, nullptr);
+        if (g.n > kLayers) {
+            for (int i = 16; i > 0; i >>= 1) sse += __shfl_down_sync(0xffffffffu, sse, i);
+            if (lane == 0) atomicAdd(g.st[kLayers - 1].sse, sse);
         }
     }
-    __syncwarp();
     tc_fence_before();
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
-                     "r"(2 * kNT)
+                     "r"(kChainCols)
                      : "memory");
 }
 
@@ -932,31 +1016,34 @@ __global__ void __launch_bounds__(kWgThreads, 1)
                 mb_wait(&bar[j % kStages], (j / kStages) & 1, nullptr);
         }
     } else if (warp == kWgEpi + 1) {
-        if (lane == 0) {
-            // MMA issuer
-            bool ok = true;
-            int issued = 0;
-            for (int j = 0; j < nk; ++j) {
-                const int s = j % kStages;
-                ok = mb_wait(&bar[s], (j / kStages) & 1, abort_v);
-                if (!ok) break;
-                tc_fence_after();
-                const unsigned A = su32(usm + (size_t)s * (kAbytes + kBbytes));
-                for (int kk = 0; kk < kKC / 16; ++kk)
-                    umma<idesc(UN, true)>(tmem, umma_desc_mn(A + kk * 2048),
-                                          umma_desc_mn(A + kAbytes + kk * 2048), j > 0 || kk > 0);
-                umma_commit(&bar[kStages + s]);
-                issued = j + 1;
-            }
-            if (ok) {
-                umma_commit(&bar[2 * kStages]);
-            } else {
+        // MMA issuer
+        const uint32_t lead = elect_one();
+        bool ok = true;
+        int issued = 0;
+        for (int j = 0; j < nk; ++j) {
+            const int s = j % kStages;
+            ok = mb_wait_warp(&bar[s], (j / kStages) & 1, abort_v);
+            if (!ok) break;
+            tc_fence_after();
+            const unsigned A = su32(usm + (size_t)s * (kAbytes + kBbytes));
+            const uint64_t da = umma_desc_mn(A), db = umma_desc_mn(A + kAbytes);
+#pragma unroll
+            for (int kk = 0; kk < kKC / 16; ++kk)
+                umma<idesc(UN, true)>(lead, tmem, da + kk * (2048 >> 4), db + kk * (2048 >> 4),
+                                      j > 0 || kk > 0);
+            umma_commit(lead, &bar[kStages + s]);
+            issued = j + 1;
+        }
+        if (ok) {
+            umma_commit(lead, &bar[2 * kStages]);
+        } else {
+            if (lead) {
                 atomicExch(g.err, 1);
                 *abort_v = 1;
-                if (issued > 0)
-                    mb_wait(&bar[kStages + (issued - 1) % kStages], ((issued - 1) / kStages) & 1,
-                            nullptr);
             }
+            if (issued > 0)
+                mb_wait_warp(&bar[kStages + (issued - 1) % kStages],
+                             ((issued - 1) / kStages) & 1, nullptr);
         }
     } else {
         bool ok = mb_wait(&bar[2 * kStages], 0, abort_v);
@@ -1092,7 +1179,8 @@ __global__ void k_input(const float* __restrict__ x, __nv_bfloat16* __restrict__
     pdl_prologue();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     // eight of a row's kK0 entries a thread
-    if (i < B * (kK0 / 8)) input_piece(x, x16, i / (kK0 / 8), 8 * (i % (kK0 / 8)));
+    if (i < B * (kK0 / 8))
+        reinterpret_cast<uint4*>(x16)[i] = input_piece(x, i / (kK0 / 8), 8 * (i % (kK0 / 8)));
 }
 
 // FP32 master weights -> BF16 copies ([fan_in padded][fan_out] for layer 0; the
@@ -1351,24 +1439,20 @@ cudaError_t set_smem_attrs(int dev) {
     return e;
 }
 
-// a launch with programmatic serialization (every kernel here starts with pdl_prologue), in
-// clusters of `cluster` CTAs along x
+// a launch with programmatic serialization (every kernel here starts with pdl_prologue)
 template <typename... KArgs, typename... Args>
 cudaError_t launch(void (*kern)(KArgs...), dim3 grid, int block, size_t smem, cudaStream_t s,
-                   int cluster, Args&&... args) {
+                   Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)cluster;
-    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
@@ -1384,7 +1468,7 @@ int row_walkers(const lbm_mlp* n, int M) {
 // D[M x 256] = A Bt^T with the epilogue of g
 cudaError_t rows_tc(lbm_mlp* n, const CUtensorMap& ta, const CUtensorMap& tb, const RowArgs& g) {
     return launch(k_umma_rows, dim3(row_walkers(n, g.M), UN / kNT), kRowsThreads, kRowsSmem,
-                  n->stream, 1, ta, tb, g);
+                  n->stream, ta, tb, g);
 }
 
 float* bpart_of(const lbm_mlp* n, int l) { return n->bpart + (size_t)l * kRowGridCap * 4 * UN; }
@@ -1438,24 +1522,23 @@ int row_stages(lbm_mlp* n, int B, const float* t, float* y, RowArgs* st) {
     return kChainStages;
 }
 
-// One chain launch where the row tiles are at most one round of clusters, else the input
+// One chain launch where the row tiles are at most one round of CTAs, else the input
 // conversion and the products one by one.
 lbm_status rows_pass(lbm_mlp* n, const float* x, int B, const float* t, float* y) {
     ChainArgs c;
     c.x = x;
     c.x16 = n->x16;
     c.n = row_stages(n, B, t, y, c.st);
-    const int tiles = (B + UM - 1) / UM;
-    if (tiles <= n->nsm / kChainCtas) {
+    // (whole 128-row tiles: the row kernels leave four rows of column sums for each)
+    const int ctas = (B + UM - 1) / UM * (UM / kChainRows);
+    if (ctas <= n->nsm) {
         ChainMaps m;
-        m.wg = n->maps.wg;
-        std::memcpy(m.wt, n->maps.wt, sizeof(m.wt));
-        std::memcpy(m.w, n->maps.w, sizeof(m.w));
-        CK(launch(k_umma_chain, dim3(kChainCtas, tiles), kRowsThreads, kChainSmem, n->stream,
-                  kChainCtas, m, c));
+        for (int s = 0; s < kChainStages; ++s)
+            m.w[s] = s < kLayers ? n->maps.wt[s] : n->maps.w[2 * kLayers - 1 - s];
+        CK(launch(k_umma_chain, dim3(ctas), kChainThreads, kChainSmem, n->stream, m, c));
         return LBM_OK;
     }
-    CK(launch(k_input, dim3((B * (kK0 / 8) + 255) / 256), 256, 0, n->stream, 1, x, n->x16, B));
+    CK(launch(k_input, dim3((B * (kK0 / 8) + 255) / 256), 256, 0, n->stream, x, n->x16, B));
     for (int s = 0; s < c.n; ++s) {
         const int l = 2 * kLayers - 1 - s;  // of a signal stage
         CK(rows_tc(n, s < kLayers ? n->maps.wg.a[s] : n->maps.wg.d[l],
@@ -1468,7 +1551,7 @@ lbm_status rows_pass(lbm_mlp* n, const float* x, int B, const float* t, float* y
 lbm_status wgrad_tc(lbm_mlp* n, int B) {
     const Slicing sl = slicing(B);
     const WgArgs w{sl.chunks, sl.per_slice, n->part, n->sse + (1 - n->turn), n->err};
-    CK(launch(k_umma_wgrad, dim3(kWgTiles, sl.slices), kWgThreads, kWgSmem, n->stream, 1,
+    CK(launch(k_umma_wgrad, dim3(kWgTiles, sl.slices), kWgThreads, kWgSmem, n->stream,
               n->maps.wg, w));
     return LBM_OK;
 }
@@ -1479,14 +1562,14 @@ lbm_status gradient_tc(lbm_mlp* n, int B, float* grad, float lr, float c1, float
     const GradArgs g{n->part, slicing(B).slices, n->bpart, 4 * row_walkers(n, B), grad,
                      n->p, n->m, n->v, lr, c1, c2, n->w16, n->w16t};
     CK(launch(grad ? k_gradient<false> : k_gradient<true>, dim3(kGradW + kGradB), 256, 0,
-              n->stream, 1, g));
+              n->stream, g));
     return LBM_OK;
 }
 
 // the mma.sync forward pass (every layer's FP32 output kept)
 lbm_status forward_ms(lbm_mlp* n, const float* x, int B) {
     cudaStream_t s = n->stream;
-    CK(launch(k_input, dim3((B * (kK0 / 8) + 255) / 256), 256, 0, s, 1, x, n->x16, B));
+    CK(launch(k_input, dim3((B * (kK0 / 8) + 255) / 256), 256, 0, s, x, n->x16, B));
     for (int l = 0; l < kLayers; ++l) {
         GemmArgs g{};
         g.A = l == 0 ? n->x16 : n->a16[l - 1];

@@ -1,5 +1,5 @@
-"""The one-launch chain of the surrogate's row products (batches whose 128-row tiles are at
-most one round of four-CTA clusters) at its edges: a single row, a tile's last and first
+"""The one-launch chain of the surrogate's row products (batches of at most one round of
+32-row CTAs, four to a 128-row tile) at its edges: a single row, a tile's last and first
 rows, the largest batch that takes it on 152 SMs (38 tiles, 4864 rows) and the first that
 does not.  Bounds are those of test_gpu_mlp: C_BOUND BF16 scales an entry."""
 import numpy as np
