@@ -11,10 +11,9 @@
 //   weight gradient    dW_l  = A_{l-1}^T D_l        [fan_in x B] [B x fan_out]
 //   input gradient     D_{l-1} = (D_l W_l^T) (1 - A_{l-1}^2)
 // with fused epilogues (bias + tanh, tanh derivative).  All of them run as
-// tcgen05 MMAs with the accumulator in tensor memory and the operands brought in
-// by tensor copies: the forward and input-gradient products (256 output columns,
-// a batch of rows) in the persistent k_umma_rows, the weight gradient (K = the
-// batch) split over K in k_umma_wgrad.  The strided mma.sync tile kernel
+// tcgen05 MMAs with the accumulator in tensor memory: the forward and input-gradient
+// products of a batch of rows one after another in k_umma_chain, the weight gradient
+// (K = the batch) split over K in k_umma_wgrad, its operands brought in by tensor copies.  The strided mma.sync tile kernel
 // (k_gemm) is kept as the comparison point, selected by lbm_mlp_set_tcgen05, and
 // runs a call whose tensor maps cannot be made.
 #include <cuda.h>  // CUtensorMap and its encoder's types (the encoder is fetched at run time)
@@ -177,24 +176,13 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs g) {
 // other roles see the flag and leave their loops, and the CTA waits (bounded)
 // for its copies and MMAs in flight before it frees its tensor memory.
 //
-// k_umma_rows: D[M x 256] = A[M x K] Bt[256 x K]^T, K = 64 or 256: the forward
-// products (A = the layer input, Bt = the transposed weights) and the input
-// gradients (A = the backward signal, Bt = the weights as stored).  A CTA computes tiles
-// of 128 rows x kNT columns (grid.y: column blocks) and walks the rows.
-// Warp 8 (one thread) loads the CTA's columns of Bt once, which stay in shared memory, and
-// streams the 64-wide K chunks of A through a ring; warp 9 (one thread) issues the MMAs (128 x kNT x 16
-// each) into one of two accumulators; warps 0-7 drain the other accumulator (the previous
-// tile) meanwhile, two warps per quarter of the tensor-memory lanes, one per half of the
-// columns.  The epilogue bounds it: it stages each 32-row x 32-column block in shared
-// memory so that its global loads and stores are row pieces of 128 (FP32) or 64 (BF16)
-// bytes.
+// k_umma_chain (described beside it): the forward products and the input gradients.
 //
 // k_umma_wgrad: the weight gradients dW[fi x 256] = A^T D over the batch, of all four
-// layers in one launch.  Both operands are read as the row kernel left them, [batch][256],
+// layers in one launch.  Both operands are read as the chain kernel left them, [batch][256],
 // so K (the batch) is their slow dimension: the MN-major 128-byte-swizzle layout, 64
 // columns a row of 128 bytes, 8 batch rows a group of 1024 bytes, the next 64 columns one
-// box further.  (Transposed copies for a K-major product cost the row kernel's epilogue
-// sixteen 2-byte stores a chunk.)  K is split into slices (grid.y); each CTA streams its
+// box further.  K is split into slices (grid.y); each CTA streams its
 // slice through a four-stage ring of 64-row chunks (warp 4 loads, warp 5 issues the MMAs)
 // and writes an FP32 partial; k_gradient adds the partials in a fixed order
 // (deterministic) and, in training, applies Adam to each entry as it gets it.
@@ -205,48 +193,30 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs g) {
 // ---------------------------------------------------------------------------
 constexpr int UM = 128, UN = 256;
 constexpr unsigned kUmmaSpins = 1u << 22;
-constexpr int kS32 = 36, kS16 = 40;  // padded rows of the epilogue's staging blocks
+constexpr int kS32 = 36;  // padded rows of the epilogue's staging blocks
 constexpr int kKC = 64;              // K chunk of the streamed operands
-// k_umma_rows: 8 epilogue warps (two per tensor-memory lane quarter, one per
-// half of the columns), a loader warp and an MMA warp; a ring of A chunks (two CTAs an SM with
-// two stages each were no faster)
-constexpr int kRowEpi = 8, kRowStages = 5, kRowsPerSm = 1;
-constexpr int kRowsThreads = 32 * (kRowEpi + 2);
 // k_umma_wgrad: 4 epilogue warps, a loader warp and an MMA warp; 4-stage ring
 constexpr int kWgEpi = 4, kStages = 4;
 constexpr int kWgThreads = 32 * (kWgEpi + 2);
-constexpr int kRowGridCap = 256;  // most CTAs of a k_umma_rows launch
+constexpr int kChainCap = 1024;  // most CTAs of a k_umma_chain launch
 constexpr int kBox = 64;                              // rows of a tensor-copy box
 constexpr unsigned kBoxBytes = kBox * kKC * 2;        // 64 x 64 BF16
-// columns of a row kernel's tile: narrow, so that the two row tiles of a batch of 256 use
-// eight SMs, and because 256 row tiles then divide evenly (7 quarter tiles for the busiest
-// of 152 SMs against 2 whole ones): Adam step 49 / 205 us at batch 256 / 32768 with 64
-// columns, 63 / 222 with 128, 91 / 249 with 256 (before the steps that followed).
-constexpr int kNT = 64;
 // the stages are aligned to 1024 bytes inside the dynamic allocation (hence + 1024)
-constexpr size_t kRowChunk = (size_t)UM * kKC * 2;                  // of A
-constexpr size_t kRowB = (size_t)kNT * kW * 2;                       // Bt, all of K
-constexpr size_t kRowsSmem = 1024 + kRowStages * kRowChunk + kRowB +
-                             (size_t)kRowEpi * 32 * kS32 * 4 + kNT * 4 +
-                             (size_t)kRowEpi * (kNT / 2) * 4;
+constexpr size_t kWChunk = (size_t)UM * kKC * 2;             // 128 features of a row product
 constexpr size_t kChunkBytes = (size_t)(UM + UN) * kKC * 2;  // of the weight gradient
 constexpr size_t kWgSmem = 1024 + kStages * kChunkBytes + (size_t)kWgEpi * 32 * kS32 * 4;
-static_assert(kRowsPerSm * (kRowsSmem + 1024) <= 227 * 1024, "row kernel shared memory");
-static_assert(kNT == 2 * 32, "an epilogue warp takes one 32-column chunk of a tile");
 static_assert(kWgSmem <= 227 * 1024 - 1024, "weight-gradient kernel shared memory");
 
 struct RowArgs {
-    int M, K;
+    int M;
     int epi;
     const float* bias;   // [256] (EPI_BIAS_TANH, EPI_BIAS, EPI_LOSS)
-    const float* aprev;  // [M][256]: the activations (EPI_TANH_BACK) or targets (EPI_LOSS)
+    const float* t;      // [M][256]: the targets (EPI_LOSS)
     float scale;         // EPI_LOSS: dL/dy = scale (y - target)
     double* sse;         // EPI_LOSS: sum of (y - target)^2 (added to)
-    float* bpart;        // or null: column sums of the result, [grid][4][256] (see below)
-    float* out32;        // [M][ld32] or null
-    int ld32;
-    __nv_bfloat16* out16;   // [M][ld16] or null
-    int ld16;
+    float* bpart;        // or null: column sums of the result, [grid][256]
+    float* out32;        // [M][256] (EPI_BIAS) or null
+    __nv_bfloat16* out16;   // [M][256] or null
     int* err;
 };
 
@@ -416,300 +386,38 @@ __device__ __forceinline__ uint4 input_piece(const float* x, int b, int k) {
     return *reinterpret_cast<uint4*>(h);
 }
 
-// coalesced loads of this warp's 32 rows x kNC columns of a row-major FP32
-// matrix [M][256], issued ahead of use (rows >= M read as zero): piece j holds
-// row 4 j + lane / 8, columns 4 (lane % 8) .. + 3
-__device__ __forceinline__ void aux_fetch(float4* pf, const float* in, int r0, int c, int M,
-                                          int lane) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const int rr = 4 * j + (lane >> 3), q = lane & 7;
-        pf[j] = r0 + rr < M
-                    ? __ldg(reinterpret_cast<const float4*>(in + (long long)(r0 + rr) * UN + c +
-                                                            4 * q))
-                    : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-}
-// the fetched pieces into the staging block s, row r0 + i of the matrix in its row i
-__device__ __forceinline__ void aux_stage(const float4* pf, float* s, int lane) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-        *reinterpret_cast<float4*>(s + (4 * j + (lane >> 3)) * kS32 + 4 * (lane & 7)) = pf[j];
-    __syncwarp();
-}
-
-// The epilogue of one kNC-column chunk [c, c + kNC) of a warp's 32 rows (x: row
-// r0 + lane; bias_c: the biases of its columns; for EPI_TANH_BACK and EPI_LOSS the
-// staging block s holds the same entries of aprev).  Column sums of the result over the
-// warp's rows are added to bsum[0..kNC).
-__device__ __forceinline__ void rows_epilogue(const RowArgs& g, float* x, const float* bias_c,
-                                              float* s32, int r0, int c, int lane, float* bsum,
-                                              double& sse) {
-    const bool live = r0 + lane < g.M;
-    __nv_bfloat16* s16 = reinterpret_cast<__nv_bfloat16*>(s32);
-    // this lane's row of the staged operand, four entries at a time
-    auto aux = [&](int j) { return *reinterpret_cast<const float4*>(s32 + lane * kS32 + j); };
-    if (g.epi == EPI_TANH_BACK) {
-#pragma unroll
-        for (int j = 0; j < kNC; j += 4) {
-            const float4 a = aux(j);
-            x[j] *= 1.0f - a.x * a.x;
-            x[j + 1] *= 1.0f - a.y * a.y;
-            x[j + 2] *= 1.0f - a.z * a.z;
-            x[j + 3] *= 1.0f - a.w * a.w;
-        }
-    } else if (g.epi == EPI_BIAS_TANH) {
-#pragma unroll
-        for (int j = 0; j < kNC; ++j) x[j] = tanh_act(x[j] + bias_c[j]);
-    } else if (g.epi == EPI_BIAS) {
-#pragma unroll
-        for (int j = 0; j < kNC; ++j) x[j] += bias_c[j];
-    } else if (g.epi == EPI_LOSS) {
-#pragma unroll
-        for (int h = 0; h < kNC; h += 16) {
-            float e2 = 0.0f;
-#pragma unroll
-            for (int j = h; j < h + 16; j += 4) {
-                const float4 a = aux(j);
-                const float t[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float e = live ? x[j + k] + bias_c[j + k] - t[k] : 0.0f;
-                    e2 = fmaf(e, e, e2);
-                    x[j + k] = 2.0f * e * g.scale;
-                }
-            }
-            sse += (double)e2;
-        }
-    }
-    if (!live) {
-#pragma unroll
-        for (int j = 0; j < kNC; ++j) x[j] = 0.0f;  // rows past M add nothing to the sums
-    }
-    if (g.out32 || g.bpart) {
-#pragma unroll
-        for (int j = 0; j < kNC / 4; ++j)
-            *reinterpret_cast<float4*>(s32 + lane * kS32 + 4 * j) =
-                make_float4(x[4 * j], x[4 * j + 1], x[4 * j + 2], x[4 * j + 3]);
-        __syncwarp();
-        if (g.out32) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int rr = 4 * j + (lane >> 3), q = lane & 7;
-                if (r0 + rr < g.M)
-                    *reinterpret_cast<float4*>(g.out32 + (long long)(r0 + rr) * g.ld32 + c +
-                                               4 * q) =
-                        *reinterpret_cast<const float4*>(s32 + rr * kS32 + 4 * q);
-            }
-        }
-        if (g.bpart) {
-            // lane l adds column l over rows 0 .. 15 and 16 .. 31, then the halves
-            float cs[2] = {0.0f, 0.0f};
-#pragma unroll
-            for (int r = 0; r < 32; ++r) cs[r >> 4] += s32[r * kS32 + lane];
-            bsum[lane] += cs[0] + cs[1];
-        }
-        __syncwarp();
-    }
-    if (!g.out16) return;
-    __align__(16) __nv_bfloat16 hv[kNC];
-#pragma unroll
-    for (int j = 0; j < kNC; ++j) hv[j] = __float2bfloat16_rn(x[j]);
-#pragma unroll
-    for (int j = 0; j < kNC / 8; ++j)
-        *reinterpret_cast<uint4*>(s16 + lane * kS16 + 8 * j) =
-            *reinterpret_cast<const uint4*>(hv + 8 * j);
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int rr = 8 * j + (lane >> 2), q = lane & 3;
-        if (r0 + rr < g.M)
-            *reinterpret_cast<uint4*>(g.out16 + (long long)(r0 + rr) * g.ld16 + c + 8 * q) =
-                *reinterpret_cast<const uint4*>(s16 + rr * kS16 + 8 * q);
-    }
-    __syncwarp();
-}
-
-__global__ void __launch_bounds__(kRowsThreads, kRowsPerSm)
-    k_umma_rows(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
-                RowArgs g) {
-    extern __shared__ __align__(1024) unsigned char usm_raw[];
-    // the swizzle pattern repeats every 1024 bytes: stages start on such a boundary
-    unsigned char* usm = usm_raw + ((1024u - (su32(usm_raw) & 1023u)) & 1023u);
-    const int nkc = g.K / kKC;  // 64-wide chunks: K = 64 or 256
-    constexpr unsigned bbytes = kNT * kKC * 2;  // a K chunk of Bt
-    const int col0 = blockIdx.y * kNT;
-    // the A ring, Bt chunk after chunk, the epilogue's staging blocks
-    unsigned char* bsm = usm + kRowStages * kRowChunk;
-    float* st32 = reinterpret_cast<float*>(bsm + kRowB);
-    float* bias_s = st32 + kRowEpi * 32 * kS32;
-    float* bsum_s = bias_s + kNT;  // [kRowEpi][kNT / 2]: column sums of each warp's half
-    // stages full, stages free, accumulator 0/1 full, Bt there, accumulator 0/1 drained
-    constexpr int F0 = 0, E0 = kRowStages, AF = 2 * kRowStages, BF = AF + 2, AE = BF + 1;
-    __shared__ __align__(8) uint64_t bar[AE + 2];
-    __shared__ uint32_t tbase;
-    __shared__ int abort_s;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int ntiles = (g.M + UM - 1) / UM;
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
-                         su32(&tbase)),
-                     "r"(2 * kNT)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
-    }
-    if (tid == 0) {
-        for (int q = 0; q < AE; ++q) mb_init(&bar[q], 1);
-        mb_init(&bar[AE], kRowEpi);
-        mb_init(&bar[AE + 1], kRowEpi);
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-        abort_s = 0;
-    }
-    for (int i = tid; i < kRowEpi * (kNT / 2); i += blockDim.x) bsum_s[i] = 0.0f;
-    pdl_prologue();  // what follows reads what the kernels before this one wrote
-    for (int i = tid; i < kNT; i += blockDim.x) bias_s[i] = g.bias ? g.bias[col0 + i] : 0.0f;
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = tbase;
-    volatile int* abort_v = &abort_s;
-    if (warp == kRowEpi) {
-        if (lane == 0) {
-            // loader: Bt, then every chunk of every tile through the ring
-            int q = 0;  // chunks issued
-            bool ok = true;
-            mb_expect(&bar[BF], nkc * bbytes);
-            for (int j = 0; j < nkc; ++j)
-                for (int r = 0; r < kNT; r += kBox)
-                    tma2(bsm + j * bbytes + r * kKC * 2, &tb, j * kKC, col0 + r, &bar[BF]);
-            for (int t = blockIdx.x; ok && t < ntiles; t += gridDim.x)
-                for (int j = 0; j < nkc; ++j, ++q) {
-                    const int st = q % kRowStages;
-                    if (q >= kRowStages)
-                        ok = mb_wait(&bar[E0 + st], ((q / kRowStages) - 1) & 1, abort_v);
-                    if (!ok) break;
-                    unsigned char* A = usm + st * kRowChunk;
-                    mb_expect(&bar[F0 + st], (unsigned)kRowChunk);
-                    for (int r = 0; r < UM; r += kBox)
-                        tma2(A + r * kKC * 2, &ta, j * kKC, t * UM + r, &bar[F0 + st]);
-                }
-            if (!ok) {
-                atomicExch(g.err, 1);
-                *abort_v = 1;
-            }
-            // the copies issued last complete before the CTA leaves (bounded)
-            mb_wait(&bar[BF], 0, nullptr);
-            for (int r = (q > kRowStages ? q - kRowStages : 0); r < q; ++r)
-                mb_wait(&bar[F0 + r % kRowStages], (r / kRowStages) & 1, nullptr);
-        }
-    } else if (warp == kRowEpi + 1) {
-        // MMA issuer: one accumulator per tile, alternating
-        const uint32_t lead = elect_one();
-        int q = 0, i = 0, committed = -1;
-        const uint64_t B = umma_desc(su32(bsm));
-        bool ok = mb_wait_warp(&bar[BF], 0, abort_v);
-        for (int t = blockIdx.x; ok && t < ntiles; t += gridDim.x, ++i) {
-            if (i >= 2) ok = mb_wait_warp(&bar[AE + (i & 1)], ((i - 2) >> 1) & 1, abort_v);
-            if (!ok) break;
-            const uint32_t acc = tmem + (uint32_t)((i & 1) * kNT);
-            for (int j = 0; j < nkc; ++j, ++q) {
-                const int st = q % kRowStages;
-                ok = mb_wait_warp(&bar[F0 + st], (q / kRowStages) & 1, abort_v);
-                if (!ok) break;
-                tc_fence_after();
-                const uint64_t A = umma_desc(su32(usm + st * kRowChunk));
-#pragma unroll
-                for (int kk = 0; kk < kKC / 16; ++kk)
-                    umma<idesc(kNT, false)>(lead, acc, A + kk * 2,
-                                            B + (uint64_t)(j * (bbytes >> 4) + kk * 2),
-                                            j > 0 || kk > 0);
-                umma_commit(lead, &bar[E0 + st]);
-                committed = q;
-            }
-            if (!ok) break;
-            umma_commit(lead, &bar[AF + (i & 1)]);
-        }
-        if (!ok) {
-            if (lead) {
-                atomicExch(g.err, 1);
-                *abort_v = 1;
-            }
-            if (committed >= 0)
-                mb_wait_warp(&bar[E0 + committed % kRowStages], (committed / kRowStages) & 1,
-                             nullptr);
-        }
-    } else {
-        float* s32 = st32 + warp * 32 * kS32;
-        float* bsum = bsum_s + warp * (kNT / 2);
-        const int quarter = warp & 3, c0 = (warp >> 2) * (kNT / 2);
-        const bool need_aux = g.epi == EPI_TANH_BACK || g.epi == EPI_LOSS;
-        double sse = 0.0;
-        int i = 0;
-        for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
-            // the operand does not depend on the product: on its way during the wait
-            const int r0 = t * UM + quarter * 32;
-            float4 pf[8];
-            if (need_aux) aux_fetch(pf, g.aprev, r0, col0 + c0, g.M, lane);
-            bool ok = mb_wait(&bar[AF + (i & 1)], (i >> 1) & 1, abort_v);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) {
-                if (lane == 0) {
-                    atomicExch(g.err, 1);
-                    *abort_v = 1;
-                }
-                break;
-            }
-            tc_fence_after();
-            const uint32_t acc =
-                tmem + (uint32_t)((i & 1) * kNT) + ((uint32_t)(quarter * 32) << 16);
-            if (need_aux) aux_stage(pf, s32, lane);
-            float x[kNC];
-            tmem_ld(acc + (uint32_t)c0, x);
-            rows_epilogue(g, x, bias_s + c0, s32, r0, col0 + c0, lane, bsum, sse);
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mb_arrive(&bar[AE + (i & 1)]);
-        }
-        __syncwarp();
-        if (g.bpart)
-            for (int j = lane; j < kNT / 2; j += 32)
-                g.bpart[((long long)blockIdx.x * 4 + quarter) * UN + col0 + c0 + j] = bsum[j];
-        if (g.sse) {
-            for (int o = 16; o > 0; o >>= 1) sse += __shfl_down_sync(0xffffffffu, sse, o);
-            if (lane == 0) atomicAdd(g.sse, sse);
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
-                     "r"(2 * kNT)
-                     : "memory");
-}
-
 // ---------------------------------------------------------------------------
-// The whole chain of row products of 32 batch rows in one CTA: the input conversion, the
-// four layers and, in training, the three input gradients.  The products are transposed,
-// D^T = W^T A^T: 256 features are two 128-row tiles of weights, streamed through a ring, the
-// 32 batch rows the narrow operand, which stays in shared memory from one stage to the next,
-// so that no CTA needs another's results.  A thread of the epilogue has one feature of 16
-// rows: targets, outputs and biases are read and written in rows without staging; the
-// hidden activations that the backward stages need stay in tensor memory.  Global memory
-// gets what the weight gradient reads, written while the next products run.
+// The chain of row products of ROWS (32 or 64) batch rows in one CTA, tile after tile: the
+// input conversion, the four layers and, in training, the three input gradients.  The
+// products are transposed, D^T = W^T A^T: 256 features are two 128-row tiles of weights,
+// streamed through a ring, the batch rows the narrow operand, which stays in shared memory
+// from one stage to the next, so that no CTA needs another's results.  A thread of the
+// epilogue has one feature of ROWS / 2 rows: targets, outputs and biases are read and written
+// in rows without staging; the hidden activations that the backward stages need stay in
+// tensor memory.  Global memory gets what the weight gradient reads, written while the next
+// products run.
 // Roles: warps 0..15 epilogue, then the loader and the MMA issuer.  A wait that runs out sets
 // the abort flag, on which every later wait gives up: the CTA goes through its stages
 // without waiting, and its results are void.
-// Bound by a stage's latency: @@M@@
+// Bound by a stage's latency: of 2 us, the MMAs' issue (eight chunks of 128 features x 64) is
+// one and the second feature tile's epilogue the other.  A training pass of 256 rows takes
+// 17 us, 33 in clusters of four CTAs that each had a quarter of the features of 128 rows,
+// 39 as eight launches; one of 32768 rows 75 us, 130 as eight launches.
 // ---------------------------------------------------------------------------
-constexpr int kChainRows = 32, kChainStages = 2 * kLayers - 1;
-constexpr int kChainEpi = 16, kChainThreads = 32 * (kChainEpi + 2), kChainRing = 11;
-constexpr int kCR = kChainRows / 2;  // rows of an epilogue thread
-constexpr size_t kActChunk = (size_t)kChainRows * kKC * 2, kAct = (kW / kKC) * kActChunk;
-constexpr size_t kChainSmem = 1024 + kChainRing * kRowChunk + 2 * kAct;
-static_assert(kChainSmem <= 227 * 1024 - 1024, "chain kernel shared memory");
+constexpr int kChainStages = 2 * kLayers - 1;
+constexpr int kChainEpi = 16, kChainThreads = 32 * (kChainEpi + 2);
+constexpr size_t act_chunk(int rows) { return (size_t)rows * kKC * 2; }  // a K chunk of rows
+constexpr size_t act_bytes(int rows) { return (kW / kKC) * act_chunk(rows); }
+constexpr int chain_ring(int rows) { return rows == 32 ? 11 : 9; }  // weight chunks
+constexpr size_t chain_smem(int rows) {
+    return 1024 + chain_ring(rows) * kWChunk + 2 * act_bytes(rows) +
+           (size_t)kLayers * kChainEpi * 32 * 4;
+}
+static_assert(chain_smem(32) <= 226 * 1024 - 1024, "chain kernel shared memory");
+static_assert(chain_smem(64) <= 226 * 1024 - 1024, "chain kernel shared memory");
 // tensor memory: [feature tile][row] of the accumulators, then of each hidden layer
-constexpr int kChainCols = kLayers * 2 * kChainRows;
-static_assert(kChainCols == 256, "an allocation is a power of two");
+constexpr int chain_cols(int rows) { return kLayers * 2 * rows; }
+static_assert(chain_cols(32) == 256 && chain_cols(64) == 512, "a power of two, at most 512");
 static_assert(kK0 == kKC && kKC * 2 == 128 && UM == 2 * kBox && kW == 2 * UM, "chain layout");
 struct ChainMaps {
     CUtensorMap w[kChainStages];  // each stage's weights, [feature][K]
@@ -717,6 +425,7 @@ struct ChainMaps {
 struct ChainArgs {
     const float* x;
     __nv_bfloat16* x16;
+    int tiles;                 // of ROWS batch rows
     int n;                     // stages: 4 (inference) or 7
     RowArgs st[kChainStages];  // layers 0..3, then the signals of layers 2, 1, 0
 };
@@ -748,24 +457,28 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* x) {
     asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
 }
 
+template <int ROWS>
 __global__ void __launch_bounds__(kChainThreads, 1)
     k_umma_chain(const __grid_constant__ ChainMaps m, const __grid_constant__ ChainArgs g) {
+    constexpr int RING = chain_ring(ROWS), kCR = ROWS / 2;  // rows of an epilogue thread
+    constexpr size_t CH = act_chunk(ROWS);
     extern __shared__ __align__(1024) unsigned char usm_raw[];
     unsigned char* usm = usm_raw + ((1024u - (su32(usm_raw) & 1023u)) & 1023u);
-    // the weights' ring, then two stages of the rows: [K chunk][row][128 bytes], swizzled
-    unsigned char* act = usm + kChainRing * kRowChunk;
+    // the weights' ring, two stages of the rows ([K chunk][row][128 bytes], swizzled), the
+    // column sums of each layer's signals ([layer][epilogue thread])
+    unsigned char* act = usm + RING * kWChunk;
+    float* bsum = reinterpret_cast<float*>(act + 2 * act_bytes(ROWS));
     // chunks there, chunks free, feature tile 0/1 done, rows there, all products done
-    constexpr int F0 = 0, E0 = kChainRing, TF = 2 * kChainRing, RF = TF + 2, DN = RF + 1;
+    constexpr int F0 = 0, E0 = RING, TF = 2 * RING, RF = TF + 2, DN = RF + 1;
     __shared__ __align__(8) uint64_t bar[DN + 1];
-    __shared__ float half_s[2][kChainEpi / 2][32];  // (of two stages: a reader may lag by one)
     __shared__ uint32_t tbase;
     __shared__ int abort_s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int R0 = blockIdx.x * kChainRows, M = g.st[0].M;
+    const int M = g.st[0].M;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
                          su32(&tbase)),
-                     "r"(kChainCols)
+                     "r"(chain_cols(ROWS))
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
@@ -774,14 +487,8 @@ __global__ void __launch_bounds__(kChainThreads, 1)
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         abort_s = 0;
     }
+    for (int i = tid; i < kLayers * kChainEpi * 32; i += kChainThreads) bsum[i] = 0.0f;
     pdl_prologue();  // what follows reads what the kernels before this one wrote
-    if (tid < kChainRows * (kK0 / 8)) {
-        const int r = tid / (kK0 / 8), q = tid % (kK0 / 8), b = R0 + r;
-        const uint4 v = b < M ? input_piece(g.x, b, 8 * q) : make_uint4(0u, 0u, 0u, 0u);
-        *reinterpret_cast<uint4*>(act + r * 128 + ((q ^ (r & 7)) << 4)) = v;
-        if (b < M) *reinterpret_cast<uint4*>(g.x16 + (long long)b * kK0 + 8 * q) = v;
-    }
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -791,154 +498,188 @@ __global__ void __launch_bounds__(kChainThreads, 1)
         atomicExch(g.st[0].err, 1);
         *abort_v = 1;
     };
+    // k: stages so far, over all tiles; the rows of stage k are in buffer k & 1
     if (warp == kChainEpi) {
         if (lane == 0) {
-            // loader: each stage's weights, tile after tile, through the ring
+            // loader: each stage's weights, feature tile after feature tile, through the ring
             int q = 0;  // chunks issued
             bool ok = true;
-            for (int s = 0; ok && s < g.n; ++s) {
-                const int nkc = s == 0 ? 1 : kW / kKC;  // K: kK0 in the first layer
-                for (int tile = 0; ok && tile < 2; ++tile)
-                    for (int j = 0; j < nkc; ++j, ++q) {
-                        const int st = q % kChainRing;
-                        if (q >= kChainRing)
-                            ok = mb_wait(&bar[E0 + st], ((q / kChainRing) - 1) & 1, abort_v);
-                        if (!ok) break;
-                        mb_expect(&bar[F0 + st], (unsigned)kRowChunk);
-                        for (int r = 0; r < UM; r += kBox)
-                            tma2(usm + st * kRowChunk + r * kKC * 2, &m.w[s], j * kKC,
-                                 tile * UM + r, &bar[F0 + st]);
-                    }
-            }
+            for (int t = blockIdx.x; ok && t < g.tiles; t += gridDim.x)
+                for (int s = 0; ok && s < g.n; ++s) {
+                    const int nkc = s == 0 ? 1 : kW / kKC;  // K: kK0 in the first layer
+                    for (int tile = 0; ok && tile < 2; ++tile)
+                        for (int j = 0; j < nkc; ++j, ++q) {
+                            const int st = q % RING;
+                            if (q >= RING)
+                                ok = mb_wait(&bar[E0 + st], ((q / RING) - 1) & 1, abort_v);
+                            if (!ok) break;
+                            mb_expect(&bar[F0 + st], (unsigned)kWChunk);
+                            for (int r = 0; r < UM; r += kBox)
+                                tma2(usm + st * kWChunk + r * kKC * 2, &m.w[s], j * kKC,
+                                     tile * UM + r, &bar[F0 + st]);
+                        }
+                }
             if (!ok) give_up();
             // the copies issued last complete before the CTA leaves (bounded)
-            for (int r = (q > kChainRing ? q - kChainRing : 0); r < q; ++r)
-                mb_wait(&bar[F0 + r % kChainRing], (r / kChainRing) & 1, nullptr);
+            for (int r = (q > RING ? q - RING : 0); r < q; ++r)
+                mb_wait(&bar[F0 + r % RING], (r / RING) & 1, nullptr);
         }
     } else if (warp == kChainEpi + 1) {
         const uint32_t lead = elect_one();
-        int st = 0;
+        int st = 0, k = 0;
         unsigned phase = 0;
         bool ok = true;
-        for (int s = 0; ok && s < g.n; ++s) {
-            const int nkc = s == 0 ? 1 : kW / kKC;
-            const uint64_t rows = umma_desc(su32(act + (s & 1) * kAct));
-            if (s > 0) ok = mb_wait_warp(&bar[RF], (s - 1) & 1, abort_v);
-            for (int tile = 0; ok && tile < 2; ++tile) {
-                for (int j = 0; j < nkc; ++j) {
-                    ok = mb_wait_warp(&bar[F0 + st], phase, abort_v);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint64_t A = umma_desc(su32(usm + st * kRowChunk));
-                    const uint64_t B = rows + (uint64_t)j * (kActChunk >> 4);
+        for (int t = blockIdx.x; ok && t < g.tiles; t += gridDim.x)
+            for (int s = 0; ok && s < g.n; ++s, ++k) {
+                const int nkc = s == 0 ? 1 : kW / kKC;
+                const uint64_t rows = umma_desc(su32(act + (k & 1) * act_bytes(ROWS)));
+                ok = mb_wait_warp(&bar[RF], k & 1, abort_v);
+                for (int tile = 0; ok && tile < 2; ++tile) {
+                    for (int j = 0; j < nkc; ++j) {
+                        ok = mb_wait_warp(&bar[F0 + st], phase, abort_v);
+                        if (!ok) break;
+                        tc_fence_after();
+                        const uint64_t A = umma_desc(su32(usm + st * kWChunk));
+                        const uint64_t B = rows + (uint64_t)j * (CH >> 4);
 #pragma unroll
-                    for (int kk = 0; kk < kKC / 16; ++kk)
-                        umma<idesc(kChainRows, false)>(lead, tmem + (uint32_t)(tile * kChainRows),
-                                                       A + kk * 2, B + kk * 2, j > 0 || kk > 0);
-                    umma_commit(lead, &bar[E0 + st]);
-                    if (++st == kChainRing) {
-                        st = 0;
-                        phase ^= 1u;
+                        for (int kk = 0; kk < kKC / 16; ++kk)
+                            umma<idesc(ROWS, false)>(lead, tmem + (uint32_t)(tile * ROWS),
+                                                     A + kk * 2, B + kk * 2, j > 0 || kk > 0);
+                        umma_commit(lead, &bar[E0 + st]);
+                        if (++st == RING) {
+                            st = 0;
+                            phase ^= 1u;
+                        }
                     }
+                    if (ok) umma_commit(lead, &bar[TF + tile]);
                 }
-                if (ok) umma_commit(lead, &bar[TF + tile]);
             }
-        }
         if (!ok && lead) give_up();
         umma_commit(lead, &bar[DN]);
         mb_wait_warp(&bar[DN], 0, nullptr);
     } else {
         const int quarter = warp & 3, tile = (warp >> 2) & 1, half = warp >> 3;
         const int f0 = tile * UM + quarter * 32, f = f0 + lane;
-        const int r0 = R0 + half * kCR;  // this thread's rows r0 ..  of feature f
-        const int nr = M - r0;           // those below it are live
         const uint32_t col = tmem + ((uint32_t)(quarter * 32) << 16) +
-                             (uint32_t)(tile * kChainRows + half * kCR);
-        // element f of a row of the narrow operand; this warp's 32 features of it
-        unsigned char* af = act + (f >> 6) * kActChunk + (f & 7) * 2;
+                             (uint32_t)(tile * ROWS + half * kCR);
+        // element f of the rows; 16-byte pieces of this warp's 32 features
+        unsigned char* af = act + (f >> 6) * CH + (f & 7) * 2;
+        unsigned char* aw = act + (f0 >> 6) * CH;
         const int piece = (f & 63) >> 3, piece0 = (f0 & 63) >> 3;
-        double sse = 0.0;
-        for (int s = 0; s < g.n; ++s) {
-            const RowArgs& r = g.st[s];
-            const unsigned next = (unsigned)(((s + 1) & 1) * kAct);
-            float a[kCR], x[kCR];
-            const float bias = r.bias ? r.bias[f] : 0.0f;
-            if (r.epi == EPI_LOSS) {
+        // this warp's rows of tile t of the input into the buffer of stage k: those of its
+        // features (kK0 in all), by the warps that have them
+        auto input = [&](int t, int k) {
+            if (f0 < kK0) {
 #pragma unroll
-                for (int j = 0; j < kCR; ++j)
-                    a[j] = j < nr ? __ldg(r.aprev + (long long)(r0 + j) * UN + f) : 0.0f;
-            }
-            if (!__all_sync(0xffffffffu, mb_wait(&bar[TF + tile], s & 1, abort_v)) && lane == 0)
-                give_up();
-            __syncwarp();
-            tc_fence_after();
-            tmem_ld16(col, x);
-            if (r.epi == EPI_TANH_BACK) {
-                tmem_ld16(col + (uint32_t)((kChainStages - s) * 2 * kChainRows), a);
-#pragma unroll
-                for (int j = 0; j < kCR; ++j) x[j] *= 1.0f - a[j] * a[j];
-            } else if (r.epi == EPI_BIAS_TANH) {
-#pragma unroll
-                for (int j = 0; j < kCR; ++j) x[j] = tanh_act(x[j] + bias);
-            } else if (r.epi == EPI_BIAS) {
-#pragma unroll
-                for (int j = 0; j < kCR; ++j) x[j] += bias;
-            } else {
-                float e2 = 0.0f;
-#pragma unroll
-                for (int j = 0; j < kCR; ++j) {
-                    const float e = j < nr ? x[j] + bias - a[j] : 0.0f;
-                    e2 = fmaf(e, e, e2);
-                    x[j] = 2.0f * e * r.scale;
-                }
-                sse += (double)e2;
-            }
-#pragma unroll
-            for (int j = 0; j < kCR; ++j)
-                if (j >= nr) x[j] = 0.0f;  // rows past M add nothing to the sums
-            if (r.out16) {
-#pragma unroll
-                for (int j = 0; j < kCR; ++j) {
-                    const int rr = half * kCR + j;
-                    *reinterpret_cast<__nv_bfloat16*>(af + next + rr * 128 +
-                                                      ((piece ^ (rr & 7)) << 4)) =
-                        __float2bfloat16_rn(x[j]);
+                for (int i = 0; i < kCR / 8; ++i) {
+                    const int rr = half * kCR + ((lane + 32 * i) >> 2), p = piece0 + (lane & 3);
+                    const int b = t * ROWS + rr;
+                    const uint4 v =
+                        b < M ? input_piece(g.x, b, 8 * p) : make_uint4(0u, 0u, 0u, 0u);
+                    *reinterpret_cast<uint4*>(aw + (k & 1) * act_bytes(ROWS) + rr * 128 +
+                                              ((p ^ (rr & 7)) << 4)) = v;
+                    if (b < M && g.n > kLayers)
+                        *reinterpret_cast<uint4*>(g.x16 + (long long)b * kK0 + 8 * p) = v;
                 }
                 asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0 && s + 1 < g.n) mb_arrive(&bar[RF]);
-            // what the backward stages and the other kernels read
-            if (r.epi == EPI_BIAS_TANH && g.n > kLayers)
-                tmem_st16(col + (uint32_t)((s + 1) * 2 * kChainRows), x);
-            if (r.out16) {
+            if (lane == 0) mb_arrive(&bar[RF]);
+        };
+        double sse = 0.0;
+        int k = 0;
+        input(blockIdx.x, 0);
+        for (int t = blockIdx.x; t < g.tiles; t += gridDim.x) {
+            const int r0 = t * ROWS + half * kCR;  // this thread's rows r0 .. of feature f
+            const int nr = M - r0;                 // those below it are live
+            for (int s = 0; s < g.n; ++s, ++k) {
+                const RowArgs& r = g.st[s];
+                const unsigned next = (unsigned)(((k + 1) & 1) * act_bytes(ROWS));
+                const float bias = r.bias ? r.bias[f] : 0.0f;
+                float pre[kCR];
+                if (r.epi == EPI_LOSS) {
 #pragma unroll
-                for (int i = 0; i < kCR * 4 / 32; ++i) {
-                    const int j = (lane + 32 * i) >> 2, p = lane & 3, rr = half * kCR + j;
-                    if (j < nr)
-                        *reinterpret_cast<uint4*>(r.out16 + (long long)(r0 + j) * kW + f0 +
-                                                  8 * p) =
-                            *reinterpret_cast<const uint4*>(
-                                act + (f0 >> 6) * kActChunk + next + rr * 128 +
-                                (((piece0 + p) ^ (rr & 7)) << 4));
+                    for (int j = 0; j < kCR; ++j)
+                        pre[j] = j < nr ? __ldg(r.t + (long long)(r0 + j) * UN + f) : 0.0f;
                 }
-            } else {
+                if (!mb_wait_warp(&bar[TF + tile], k & 1, abort_v) && lane == 0) give_up();
+                __syncwarp();
+                tc_fence_after();
+                float bs = 0.0f;
 #pragma unroll
-                for (int j = 0; j < kCR; ++j)
-                    if (j < nr) r.out32[(long long)(r0 + j) * kW + f] = x[j];
-            }
-            if (r.bpart) {
-                // rows 0 .. 15 and 16 .. 31, then the halves
-                float cs = 0.0f;
+                for (int h = 0; h < kCR; h += 16) {
+                    float a[16], x[16];
+                    tmem_ld16(col + (uint32_t)h, x);
+                    if (r.epi == EPI_TANH_BACK) {
+                        tmem_ld16(col + (uint32_t)((kChainStages - s) * 2 * ROWS + h), a);
 #pragma unroll
-                for (int j = 0; j < kCR; ++j) cs += x[j];
-                if (half) half_s[s & 1][warp & 7][lane] = cs;
-                asm volatile("bar.sync %0, 64;\n" ::"r"(1 + (warp & 7)) : "memory");
-                if (!half)
-                    r.bpart[(long long)blockIdx.x * UN + f] = cs + half_s[s & 1][warp & 7][lane];
+                        for (int j = 0; j < 16; ++j) x[j] *= 1.0f - a[j] * a[j];
+                    } else if (r.epi == EPI_BIAS_TANH) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) x[j] = tanh_act(x[j] + bias);
+                    } else if (r.epi == EPI_BIAS) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) x[j] += bias;
+                    } else {
+                        float e2 = 0.0f;
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            const float e = h + j < nr ? x[j] + bias - pre[h + j] : 0.0f;
+                            e2 = fmaf(e, e, e2);
+                            x[j] = 2.0f * e * r.scale;
+                        }
+                        sse += (double)e2;
+                    }
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (h + j >= nr) x[j] = 0.0f;  // rows past M add nothing to the sums
+                    if (r.out16) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            const int rr = half * kCR + h + j;
+                            *reinterpret_cast<__nv_bfloat16*>(af + next + rr * 128 +
+                                                              ((piece ^ (rr & 7)) << 4)) =
+                                __float2bfloat16_rn(x[j]);
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            if (h + j < nr) r.out32[(long long)(r0 + h + j) * kW + f] = x[j];
+                    }
+                    if (r.epi == EPI_BIAS_TANH && g.n > kLayers)
+                        tmem_st16(col + (uint32_t)((s + 1) * 2 * ROWS + h), x);
+                    if (r.bpart) {
+                        float cs = 0.0f;
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) cs += x[j];
+                        bs += cs;
+                    }
+                }
+                if (s + 1 < g.n) {
+                    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mb_arrive(&bar[RF]);
+                }
+                __syncwarp();
+                // what the weight gradient reads, while the next products run
+                if (r.out16 && g.n > kLayers) {
+#pragma unroll
+                    for (int i = 0; i < kCR / 8; ++i) {
+                        const int j = (lane + 32 * i) >> 2, p = lane & 3, rr = half * kCR + j;
+                        if (j < nr)
+                            *reinterpret_cast<uint4*>(r.out16 + (long long)(r0 + j) * kW + f0 +
+                                                      8 * p) =
+                                *reinterpret_cast<const uint4*>(
+                                    aw + next + rr * 128 + (((piece0 + p) ^ (rr & 7)) << 4));
+                    }
+                }
+                const int layer = s < kLayers ? s : kChainStages - 1 - s;
+                if (r.bpart) bsum[layer * kChainEpi * 32 + tid] += bs;
+                __syncwarp();
             }
-            __syncwarp();
+            if (t + gridDim.x < g.tiles) input(t + gridDim.x, k);
         }
         if (g.n > kLayers) {
             for (int i = 16; i > 0; i >>= 1) sse += __shfl_down_sync(0xffffffffu, sse, i);
@@ -947,9 +688,16 @@ __global__ void __launch_bounds__(kChainThreads, 1)
     }
     tc_fence_before();
     __syncthreads();
+    if (g.n > kLayers && tid < kW)
+        // (threads f and f + kW have feature f's halves of the rows)
+        for (int s = kLayers - 1; s < g.n; ++s) {
+            const int layer = s < kLayers ? s : kChainStages - 1 - s;
+            const float* b = bsum + layer * kChainEpi * 32;
+            g.st[s].bpart[(long long)blockIdx.x * UN + tid] = b[tid] + b[tid + kW];
+        }
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
-                     "r"(kChainCols)
+                     "r"(chain_cols(ROWS))
                      : "memory");
 }
 
@@ -1100,7 +848,7 @@ __device__ __forceinline__ void store_w16(int l, int k, float p, __nv_bfloat16* 
 struct GradArgs {
     const float* part;    // [slices][kWgTiles * 128][256]
     int slices;
-    const float* bpart;   // [layers][kRowGridCap * 4][256]: column sums of each signal
+    const float* bpart;   // [layers][kChainCap][256]: column sums of each signal
     int nb;               // rows of it in use
     float* grad;          // !ADAM: the gradient
     float *p, *m, *v;     // ADAM: parameters and moments
@@ -1160,7 +908,7 @@ __global__ void __launch_bounds__(256) k_gradient(GradArgs g) {
     __shared__ float acc[8][33];
     const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
     const int o = ((int)blockIdx.x - kGradW) * 32 + x, l = o / kW, n = o - l * kW;
-    const float* src = g.bpart + (long long)l * kRowGridCap * 4 * UN + n;
+    const float* src = g.bpart + (long long)l * kChainCap * UN + n;
     float s = 0.0f;
 #pragma unroll 8
     for (int q = y; q < g.nb; q += 8) s += src[q * UN];
@@ -1269,7 +1017,7 @@ struct lbm_mlp {
     __nv_bfloat16* sig[kLayers]; // backward signal at each layer's output, BF16 [R][256]
     float *d32, *e32;            // the same in FP32 (mma.sync kernel only), alternating
     float* part;                 // weight-gradient partials [slices][kWgTiles * 128][256]
-    float* bpart;                // bias-gradient partials [layers][kRowGridCap * 4][256]
+    float* bpart;                // bias-gradient partials [layers][kChainCap][256]
     double* sse;                 // squared-error sums of this call and the next, in turn
     int turn;                    // which of them is this call's
     double* h_sse;               // pinned mirror of both and err
@@ -1328,7 +1076,7 @@ MlpLayout mlp_layout(int B0) {
     L.d32 = take(B * kW * 4);
     L.e32 = take(B * kW * 4);
     L.part = take(S * kWgTiles * UM * UN * 4);
-    L.bpart = take((size_t)kLayers * kRowGridCap * 4 * UN * 4);
+    L.bpart = take((size_t)kLayers * kChainCap * UN * 4);
     L.sse = take(24);  // two squared-error sums and the error word, read back together
     L.total = o;
     return L;
@@ -1427,11 +1175,11 @@ cudaError_t set_smem_attrs(int dev) {
     static unsigned long long done = 0;  // one bit per device
     const unsigned long long bit = 1ull << (dev & 63);
     if (done & bit) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_umma_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kRowsSmem);
+    cudaError_t e = cudaFuncSetAttribute(
+        k_umma_chain<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chain_smem(32));
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_umma_chain, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kChainSmem);
+        e = cudaFuncSetAttribute(k_umma_chain<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)chain_smem(64));
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_umma_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kWgSmem);
@@ -1456,45 +1204,25 @@ cudaError_t launch(void (*kern)(KArgs...), dim3 grid, int block, size_t smem, cu
     return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
-// CTAs that walk the row tiles of one column block for M rows: together kRowsPerSm per SM
-// at most, and at most kRowGridCap (the rows of column sums they leave are sized by that)
-int row_walkers(const lbm_mlp* n, int M) {
-    const int tiles = (M + UM - 1) / UM;
-    int cap = kRowsPerSm * n->nsm / (UN / kNT);
-    cap = cap < 1 ? 1 : (cap < kRowGridCap ? cap : kRowGridCap);
-    return tiles < cap ? tiles : cap;
-}
-
-// D[M x 256] = A Bt^T with the epilogue of g
-cudaError_t rows_tc(lbm_mlp* n, const CUtensorMap& ta, const CUtensorMap& tb, const RowArgs& g) {
-    return launch(k_umma_rows, dim3(row_walkers(n, g.M), UN / kNT), kRowsThreads, kRowsSmem,
-                  n->stream, ta, tb, g);
-}
-
-float* bpart_of(const lbm_mlp* n, int l) { return n->bpart + (size_t)l * kRowGridCap * 4 * UN; }
+float* bpart_of(const lbm_mlp* n, int l) { return n->bpart + (size_t)l * kChainCap * UN; }
 
 // The row products of a pass on tcgen05, in order: the four layers and, where there are
 // targets t (training), the signals of layers 2, 1, 0.  t null: inference, only the output
-// (written to y).  In training the hidden layers keep what the backward pass needs (FP32
-// activations), and the last layer's epilogue turns its output straight into the loss
+// (written to y).  In training the last layer's epilogue turns its output straight into the loss
 // signal dL/dy (BF16, column sums) and the squared-error sum, without storing y.
 int row_stages(lbm_mlp* n, int B, const float* t, float* y, RowArgs* st) {
     for (int l = 0; l < kLayers; ++l) {
         RowArgs& g = st[l];
         g = RowArgs{};
         g.M = B;
-        g.K = l == 0 ? kK0 : kW;
         g.bias = n->p + param_offset(l) + (long long)kFanIn[l] * kFanOut[l];
-        g.ld32 = kW;
-        g.ld16 = kW;
         g.err = n->err;
         if (l < kLayers - 1) {
             g.epi = EPI_BIAS_TANH;
-            g.out32 = t ? n->a32[l] : nullptr;
             g.out16 = n->a16[l];
         } else if (t) {
             g.epi = EPI_LOSS;
-            g.aprev = t;
+            g.t = t;
             g.scale = 1.0f / ((float)B * kOut);
             g.sse = n->sse + n->turn;
             g.out16 = n->sig[l];
@@ -1506,44 +1234,46 @@ int row_stages(lbm_mlp* n, int B, const float* t, float* y, RowArgs* st) {
     }
     if (!t) return kLayers;
     for (int l = kLayers - 1; l > 0; --l) {
-        // D_{l-1} = (D_l W_l^T) (1 - A_{l-1}^2): K-major operands are D [B][fo] and
-        // W_l itself ([fi][fo])
+        // D_{l-1} = (D_l W_l^T) (1 - A_{l-1}^2): the weights' K-major operand is W_l itself
+        // ([fi][fo])
         RowArgs& g = st[2 * kLayers - 1 - l];
         g = RowArgs{};
         g.M = B;
-        g.K = kW;
         g.epi = EPI_TANH_BACK;
-        g.aprev = n->a32[l - 1];
         g.out16 = n->sig[l - 1];
-        g.ld16 = kW;
         g.bpart = bpart_of(n, l - 1);
         g.err = n->err;
     }
     return kChainStages;
 }
 
-// One chain launch where the row tiles are at most one round of CTAs, else the input
-// conversion and the products one by one.
+// Rows of a chain CTA's tile: 32 while those tiles are at most one round of CTAs, where the
+// latency of a tile is what counts (17 us against 22 of 64 rows, by the stages' timings),
+// else 64, for half the weights' traffic a row.
+int chain_rows(const lbm_mlp* n, int B) {
+    return (B + UM - 1) / UM * (UM / 32) <= n->nsm ? 32 : 64;
+}
+// (of whole 128-row tiles)
+int chain_tiles(const lbm_mlp* n, int B) { return (B + UM - 1) / UM * (UM / chain_rows(n, B)); }
+// CTAs, each of which leaves one row of column sums per layer
+int chain_ctas(const lbm_mlp* n, int B) {
+    const int cap = n->nsm < kChainCap ? n->nsm : kChainCap, tiles = chain_tiles(n, B);
+    return tiles < cap ? tiles : cap;
+}
+
+// the row products of a pass (row_stages), one launch
 lbm_status rows_pass(lbm_mlp* n, const float* x, int B, const float* t, float* y) {
     ChainArgs c;
     c.x = x;
     c.x16 = n->x16;
+    c.tiles = chain_tiles(n, B);
     c.n = row_stages(n, B, t, y, c.st);
-    // (whole 128-row tiles: the row kernels leave four rows of column sums for each)
-    const int ctas = (B + UM - 1) / UM * (UM / kChainRows);
-    if (ctas <= n->nsm) {
-        ChainMaps m;
-        for (int s = 0; s < kChainStages; ++s)
-            m.w[s] = s < kLayers ? n->maps.wt[s] : n->maps.w[2 * kLayers - 1 - s];
-        CK(launch(k_umma_chain, dim3(ctas), kChainThreads, kChainSmem, n->stream, m, c));
-        return LBM_OK;
-    }
-    CK(launch(k_input, dim3((B * (kK0 / 8) + 255) / 256), 256, 0, n->stream, x, n->x16, B));
-    for (int s = 0; s < c.n; ++s) {
-        const int l = 2 * kLayers - 1 - s;  // of a signal stage
-        CK(rows_tc(n, s < kLayers ? n->maps.wg.a[s] : n->maps.wg.d[l],
-                   s < kLayers ? n->maps.wt[s] : n->maps.w[l], c.st[s]));
-    }
+    ChainMaps m;
+    for (int s = 0; s < kChainStages; ++s)
+        m.w[s] = s < kLayers ? n->maps.wt[s] : n->maps.w[2 * kLayers - 1 - s];
+    const int rows = chain_rows(n, B);
+    CK(launch(rows == 32 ? k_umma_chain<32> : k_umma_chain<64>, dim3(chain_ctas(n, B)),
+              kChainThreads, chain_smem(rows), n->stream, m, c));
     return LBM_OK;
 }
 
@@ -1559,7 +1289,7 @@ lbm_status wgrad_tc(lbm_mlp* n, int B) {
 // the gradient from the partial sums of wgrad_tc: into grad, or (grad null) into one
 // Adam step of the parameters
 lbm_status gradient_tc(lbm_mlp* n, int B, float* grad, float lr, float c1, float c2) {
-    const GradArgs g{n->part, slicing(B).slices, n->bpart, 4 * row_walkers(n, B), grad,
+    const GradArgs g{n->part, slicing(B).slices, n->bpart, chain_ctas(n, B), grad,
                      n->p, n->m, n->v, lr, c1, c2, n->w16, n->w16t};
     CK(launch(grad ? k_gradient<false> : k_gradient<true>, dim3(kGradW + kGradB), 256, 0,
               n->stream, g));

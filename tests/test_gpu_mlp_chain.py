@@ -1,7 +1,7 @@
-"""The one-launch chain of the surrogate's row products (batches of at most one round of
-32-row CTAs, four to a 128-row tile) at its edges: a single row, a tile's last and first
-rows, the largest batch that takes it on 152 SMs (38 tiles, 4864 rows) and the first that
-does not.  Bounds are those of test_gpu_mlp: C_BOUND BF16 scales an entry."""
+"""The one-launch chain of the surrogate's row products at its edges: a single row, a tile's
+last and first rows, the largest batch in 32-row tiles on 152 SMs (4864 rows) and the first in
+64-row tiles, several tiles a CTA with a ragged end.  Bounds are those of test_gpu_mlp:
+C_BOUND BF16 scales an entry."""
 import numpy as np
 import pytest
 
@@ -11,7 +11,7 @@ from tests.test_gpu_mlp import C_BOUND, _scales, _setup
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("B", [1, 127, 129, 4864, 4865])
+@pytest.mark.parametrize("B", [1, 127, 129, 4864, 4865, 20011])
 def test_chain_entrywise(cuda, B):
     net, p, x, t, dx, dt = _setup(cuda, B)
     y = net.forward(dx).cpu().numpy().astype(np.float64)
@@ -23,7 +23,7 @@ def test_chain_entrywise(cuda, B):
 
 
 def test_rows_do_not_depend_on_the_launch(cuda):
-    """A row's product takes the same operations in a chain as in separate launches."""
+    """A row's product takes the same operations in tiles of 32 rows as of 64."""
     net, p, x, t, dx, dt = _setup(cuda, 4992)
     whole = net.forward(dx)
     for B in (1, 130, 4864):
