@@ -1,7 +1,7 @@
 // kernels_mixed.cu -- lattice kernels of the mixed-precision path: FP32
 // populations and collision, the density kept as a double-float pair; its line
-// solves are in kernels_lines.cu (double-float first derivatives of the density,
-// FP32 second derivatives, chemical potential and force).
+// solves are in lines32.cu, lines32_wide.cu (FP32) and lines_df.cu (double-float first
+// derivatives of the density).
 //
 // Why this split (GB300 runs FP64 at 1/64 of the FP32 rate, so FP64 arithmetic
 // in the line solves would bound the whole step):
@@ -127,12 +127,12 @@ __device__ __forceinline__ void cs_mixed_body(const CsArgs& a, int wid) {
     fetch(y0 + 1);
     if (WALLS && y0 == 0) reflect_into<true>(A, B, a.uw6[0]);
     for (int y = y0; y < y1; ++y) {
-        if (WALLS && y == ny - 1) {
+        if (WALLS && y + 1 == a.ny) {
             // row ny is solid: the pull takes only C[4], C[7], C[8] from it
             reflect_into<false>(C, B, a.uw6[1]);
         } else {
             collide_raw(C);  // row y+1
-            if (y + 1 < y1 && !(WALLS && y + 2 == ny)) fetch(y + 2);
+            if (y + 1 < y1 && !(WALLS && y + 2 == a.ny)) fetch(y + 2);
         }
         // gather row y: e = (ex, ey) comes from row y - ey, column x - ex
         float g[9];

@@ -26,7 +26,7 @@
 // reads its 23 (27) rows straight into registers and writes its rows, coalesced as they are.
 // Against one warp a line with all 32 chunks and staged y-windows: steps of 128^2 17.6 ->
 // 15.6 us, 512^2 20.1 -> 17.4, 333 x 277 26.4 -> 19.5.  On large grids, where every chunk is
-// needed and rows come from DRAM, those windows (kernels_lines.cu) stay ahead.
+// needed and rows come from DRAM, those windows (lines32_wide.cu) stay ahead.
 #pragma once
 
 #include "cplbm_internal.cuh"
