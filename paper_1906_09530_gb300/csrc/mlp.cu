@@ -399,18 +399,23 @@ __device__ __forceinline__ uint4 input_piece(const float* x, int b, int k) {
 // Roles: warps 0..15 epilogue, then the loader and the MMA issuer.  A wait that runs out sets
 // the abort flag, on which every later wait gives up: the CTA goes through its stages
 // without waiting, and its results are void.
-// Bound by a stage's latency: of 2 us, the MMAs' issue (eight chunks of 128 features x 64) is
-// one and the second feature tile's epilogue the other.  A training pass of 256 rows takes
-// 17 us, 33 in clusters of four CTAs that each had a quarter of the features of 128 rows,
-// 39 as eight launches; one of 32768 rows 75 us, 130 as eight launches.
+// Bound by a stage's latency: of 2.5 us, the MMA issuer's waits and MMAs are 1.6 and the
+// second feature tile's epilogue the rest.  A training pass of 256 rows takes 17 us, 33 in
+// clusters of four CTAs that each had a quarter of the features of 128 rows, 39 as eight
+// launches; one of 32768 rows 90 us, 130 as eight launches.  (Issuing the products of the
+// first half of K before the second half's epilogue, and a converged loader warp, were
+// slower: 496 and 516 us a fit epoch of 16 x 256 against 481.)
 // ---------------------------------------------------------------------------
 constexpr int kChainStages = 2 * kLayers - 1;
 constexpr int kChainEpi = 16, kChainThreads = 32 * (kChainEpi + 2);
 constexpr size_t act_chunk(int rows) { return (size_t)rows * kKC * 2; }  // a K chunk of rows
 constexpr size_t act_bytes(int rows) { return (kW / kKC) * act_chunk(rows); }
-constexpr int chain_ring(int rows) { return rows == 32 ? 11 : 9; }  // weight chunks
+// The weights' ring is of units of two K chunks: a wait, even for what is there, and the
+// commit that frees the place cost the MMA issuer some 300 cycles.
+constexpr size_t kWUnit = 2 * kWChunk;
+constexpr int chain_ring(int rows) { return rows == 32 ? 5 : 4; }
 constexpr size_t chain_smem(int rows) {
-    return 1024 + chain_ring(rows) * kWChunk + 2 * act_bytes(rows) +
+    return 1024 + chain_ring(rows) * kWUnit + 2 * act_bytes(rows) +
            (size_t)kLayers * kChainEpi * 32 * 4;
 }
 static_assert(chain_smem(32) <= 226 * 1024 - 1024, "chain kernel shared memory");
@@ -466,9 +471,9 @@ __global__ void __launch_bounds__(kChainThreads, 1)
     unsigned char* usm = usm_raw + ((1024u - (su32(usm_raw) & 1023u)) & 1023u);
     // the weights' ring, two stages of the rows ([K chunk][row][128 bytes], swizzled), the
     // column sums of each layer's signals ([layer][epilogue thread])
-    unsigned char* act = usm + RING * kWChunk;
+    unsigned char* act = usm + RING * kWUnit;
     float* bsum = reinterpret_cast<float*>(act + 2 * act_bytes(ROWS));
-    // chunks there, chunks free, feature tile 0/1 done, rows there, all products done
+    // units there, units free, feature tile 0/1 done, rows there, all products done
     constexpr int F0 = 0, E0 = RING, TF = 2 * RING, RF = TF + 2, DN = RF + 1;
     __shared__ __align__(8) uint64_t bar[DN + 1];
     __shared__ uint32_t tbase;
@@ -502,21 +507,22 @@ __global__ void __launch_bounds__(kChainThreads, 1)
     if (warp == kChainEpi) {
         if (lane == 0) {
             // loader: each stage's weights, feature tile after feature tile, through the ring
-            int q = 0;  // chunks issued
+            int q = 0;  // units issued
             bool ok = true;
             for (int t = blockIdx.x; ok && t < g.tiles; t += gridDim.x)
                 for (int s = 0; ok && s < g.n; ++s) {
                     const int nkc = s == 0 ? 1 : kW / kKC;  // K: kK0 in the first layer
                     for (int tile = 0; ok && tile < 2; ++tile)
-                        for (int j = 0; j < nkc; ++j, ++q) {
+                        for (int j = 0; j < nkc; j += 2, ++q) {
                             const int st = q % RING;
                             if (q >= RING)
                                 ok = mb_wait(&bar[E0 + st], ((q / RING) - 1) & 1, abort_v);
                             if (!ok) break;
-                            mb_expect(&bar[F0 + st], (unsigned)kWChunk);
-                            for (int r = 0; r < UM; r += kBox)
-                                tma2(usm + st * kWChunk + r * kKC * 2, &m.w[s], j * kKC,
-                                     tile * UM + r, &bar[F0 + st]);
+                            const int sub = nkc - j < 2 ? nkc - j : 2;
+                            mb_expect(&bar[F0 + st], sub * (unsigned)kWChunk);
+                            for (int r = 0; r < sub * UM; r += kBox)
+                                tma2(usm + st * kWUnit + r * kKC * 2, &m.w[s],
+                                     (j + r / UM) * kKC, tile * UM + r % UM, &bar[F0 + st]);
                         }
                 }
             if (!ok) give_up();
@@ -535,16 +541,20 @@ __global__ void __launch_bounds__(kChainThreads, 1)
                 const uint64_t rows = umma_desc(su32(act + (k & 1) * act_bytes(ROWS)));
                 ok = mb_wait_warp(&bar[RF], k & 1, abort_v);
                 for (int tile = 0; ok && tile < 2; ++tile) {
-                    for (int j = 0; j < nkc; ++j) {
+                    for (int j = 0; j < nkc; j += 2) {
                         ok = mb_wait_warp(&bar[F0 + st], phase, abort_v);
                         if (!ok) break;
                         tc_fence_after();
-                        const uint64_t A = umma_desc(su32(usm + st * kWChunk));
-                        const uint64_t B = rows + (uint64_t)j * (CH >> 4);
+                        for (int h = j; h < j + 2 && h < nkc; ++h) {
+                            const uint64_t A =
+                                umma_desc(su32(usm + st * kWUnit + (h - j) * kWChunk));
+                            const uint64_t B = rows + (uint64_t)h * (CH >> 4);
 #pragma unroll
-                        for (int kk = 0; kk < kKC / 16; ++kk)
-                            umma<idesc(ROWS, false)>(lead, tmem + (uint32_t)(tile * ROWS),
-                                                     A + kk * 2, B + kk * 2, j > 0 || kk > 0);
+                            for (int kk = 0; kk < kKC / 16; ++kk)
+                                umma<idesc(ROWS, false)>(lead, tmem + (uint32_t)(tile * ROWS),
+                                                         A + kk * 2, B + kk * 2,
+                                                         h > 0 || kk > 0);
+                        }
                         umma_commit(lead, &bar[E0 + st]);
                         if (++st == RING) {
                             st = 0;
