@@ -18,7 +18,9 @@
 // y-lines with mu-hat; this takes 55, the moment sum included, and 106.)  A join
 // reaches kPw positions into a chunk: beyond, lam^k is below 4e-24.
 //
-// Lines longer than kLMax are cut into overlapping windows, and lines between walls (the
+// Lines longer than kLWhole are cut into overlapping windows (whole, a line of 4096 leaves four
+// warps an SM: a 4096^2 step took 8.5 ms, in windows 5.3; on 1536^2 it is the same either
+// way), and lines between walls (the
 // even extension of period 2 n, Sec. 5.5) of more than 2 kHalo positions are one window
 // with a mirrored halo.  A window is solved as if it were periodic: what that gets wrong at
 // its ends has decayed by the owned positions.
@@ -34,7 +36,8 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kT = 128;       // threads a block; warps 0 .. nl-1 solve a line each
 constexpr int kPw = 57;       // powers (-lam)^0 .. (-lam)^56
 constexpr int kHalo = 96;     // two solves of kPw - 9 positions: lam^48 < 1e-20
-constexpr int kLMax = 6144;   // longest window: 4 lines of it are 198 KB of shared memory
+constexpr int kLWhole = 1600; // longest line solved whole
+constexpr int kLOwn = 1100;   // most positions a window of a longer one owns
 constexpr int kSMs = 152;
 
 struct Geo {
@@ -311,12 +314,13 @@ Geo geo64(int nx, int ny, int axis, bool walls_y, int lines_all) {
         g.H = kHalo;
         g.L = g.n + 2 * kHalo;
     }
-    if (g.L > kLMax) {
+    g.nwin = 1;
+    if (g.L > kLWhole) {
+        g.nwin = (g.n + kLOwn - 1) / kLOwn;
+        g.own = ((g.n + g.nwin - 1) / g.nwin + 3) / 4 * 4;
         g.H = kHalo;
-        g.L = kLMax;
-        g.own = kLMax - 2 * kHalo;
+        g.L = g.own + 2 * kHalo;
     }
-    g.nwin = (g.n + g.own - 1) / g.own;
     // Lines a block: the pipe is shared by all warps of an SM, so a launch takes as long as
     // the SM with most lines; 4 (32-byte pieces of the rows for y-lines) unless fewer
     // spread the lines better by more than a tenth (1024 lines: 7 an SM with one a block,

@@ -14,8 +14,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("order", [4, 6])
 @pytest.mark.parametrize("axis", [0, 1])
-@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 31, 32, 33, 56, 63, 65, 255, 1000, 1793, 6144, 6145,
-                               12100])
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 31, 32, 33, 56, 63, 65, 255, 1000, 1600, 1601, 1793,
+                               6144, 6145, 12100])
 def test_lines_of_every_chunking(cuda, order, axis, n):
     from oracle import cfd_alpha, cfd_line
     from paper_1906_09530_gb300 import lbm_cfd
@@ -39,10 +39,11 @@ def test_lines_of_every_chunking(cuda, order, axis, n):
     assert np.abs(d2 - r2).max() <= 1e-13 * max(np.abs(r2).max(), 1.0)
 
 
-@pytest.mark.parametrize("nx,ny", [(8, 8), (40, 31), (24, 192), (24, 193), (310, 300), (700, 40)])
+@pytest.mark.parametrize("nx,ny", [(8, 8), (40, 31), (24, 192), (24, 193), (310, 300), (700, 40),
+                                   (16, 1408), (16, 1409)])
 def test_walled_force_stage(cuda, nx, ny):
-    """The mirrored lines: whole periods up to 192 rows, one window with a halo above; 310 and
-    700 columns take 2 and 4 lines a block."""
+    """The mirrored lines: whole periods up to 192 rows, one window with a halo above, windows
+    above 1408; 310 and 700 columns take 2 and 4 lines a block."""
     from oracle import thermo
     from paper_1906_09530_gb300 import workloads as W
     rg, rl = thermo.maxwell(0.6)
