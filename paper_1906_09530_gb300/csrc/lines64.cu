@@ -345,10 +345,10 @@ Geo geo64(int nx, int ny, int axis, bool walls_y, int lines_all) {
 size_t smem64(const Geo& g) { return (size_t)g.nl * line_slots(g.L) * sizeof(double); }
 unsigned blocks64(const Geo& g) { return (unsigned)((long long)g.ngroups * g.nwin); }
 
+// Every launch tells the kernel its size, also below the 48 KB that need no telling: those
+// are of the dynamic and the static arrays together (pw, logs).
 template <class K>
 cudaError_t allow_smem(K kern, size_t bytes) {
-    // above the default 48 KB a kernel has to be told (per device: cheap, so each time)
-    if (bytes <= 48 * 1024) return cudaSuccess;
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
