@@ -46,6 +46,16 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t sme
     return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
+// Lets launches of a kernel have up to `most` bytes of dynamic shared memory.  The limit is
+// state of the device, which the launches of all grids, contexts and host threads share: every
+// caller gives the most that any grid needs of that kernel, never its own grid's size, so that
+// no thread lowers the limit between another's call and its launch.  (Also below 48 KB, which
+// need no telling only if the kernel's static arrays fit in them too.)
+template <class K>
+cudaError_t allow_smem(K kern, size_t most) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // Device-resident state block (one per context, inside the workspace).
 struct DevState {
     int64_t t;              // time level of the populations in f[cur]

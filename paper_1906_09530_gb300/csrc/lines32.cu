@@ -92,11 +92,24 @@ void divide(Geo32& g, int axis, int T) {
 // with 64 / 128 / 256 / 512: 512^2 23.3 / 19.1 / 17.4 / 19.7 us, 128^2 16.8 / 15.6 / 15.6 /
 // 17.5.  Rows that are not whole 16-byte pieces are staged four bytes at a time, which
 // wants more blocks: 333 x 277 20.2 / 19.5 / 20.5 / 23.5.
-int pick_threads(int nx) { return nx % 4 == 0 ? 256 : 128; }
+constexpr int kLoneT = 256;
+int pick_threads(int nx) { return nx % 4 == 0 ? kLoneT : 128; }
 
 size_t smem_of(const Geo32& gx, int T, bool second) {
     return ((size_t)6 * T + (size_t)gx.nl * l32::line_stride(gx.nch) * (second ? 2 : 1)) *
            sizeof(float);
+}
+// the most that a block of up to T threads can need: the shortest windows (8 chunks) stage
+// the most lines
+size_t most_smem(int T, bool second) {
+    size_t most = 0;
+    for (int nch = 8; nch <= 32; nch += 4) {
+        Geo32 g{};
+        g.nl = T / nch;
+        g.nch = nch;
+        most = std::max(most, smem_of(g, T, second));
+    }
+    return most;
 }
 int blocks_of(const Geo32& g) { return g.ngroups * g.nwin; }
 
@@ -128,12 +141,6 @@ __global__ void __launch_bounds__(kMaxT, 2)
         l32::block<MODE, SIXTH, 0>(D.x, k, local, sh32);
     else
         l32::block<MODE, SIXTH, 1>(D.y, k, local - D.nbx, sh32);
-}
-
-template <class K>
-cudaError_t allow_smem(K kern, size_t bytes) {
-    if (bytes <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 Dir32 density_dir(const float* rh, float* d1, float* d2) {
@@ -172,7 +179,7 @@ cudaError_t run(Dir32 x, Dir32 y, int nx, int ny, int order, bool walls_y, DevSt
     const int nbx = blocks_of(x.g), nby = blocks_of(y.g);
     const size_t smem = smem_of(x.g, T, SECOND);
     auto go = [&](auto kern) -> cudaError_t {
-        const cudaError_t e = allow_smem(kern, smem);
+        const cudaError_t e = allow_smem(kern, most_smem(kLoneT, SECOND));
         if (e != cudaSuccess) return e;
         return launch_pdl(kern, dim3(nbx + nby), dim3(T), smem, s, x, y, line32_constants(order),
                           st, bump, nbx);
@@ -221,22 +228,14 @@ Lines32Inst lines32_batch_inst(const MixedLinesView& v, int order, bool second, 
     return d;
 }
 
-// the largest shared memory a block of 32 nl threads can need: the shortest windows
-// (8 chunks) stage the most lines
 cudaError_t lines32_batch_launch(const Lines32Inst* d, const int* map, int nblocks, int order,
                                  bool second, int bump, int nl, bool wide, cudaStream_t s) {
     if (nblocks <= 0) return cudaSuccess;
     if (wide) return lines32_wide_batch(d, map, nblocks, order, second, bump, nl, s);
     const int T = 32 * nl;
-    size_t smem = 0;
-    for (int nch = 8; nch <= 32; nch += 4) {
-        Geo32 g{};
-        g.nl = T / nch;
-        g.nch = nch;
-        smem = std::max(smem, smem_of(g, T, second));
-    }
+    const size_t smem = most_smem(T, second);  // (of any of the batch's grids)
     auto go = [&](auto kern) -> cudaError_t {
-        const cudaError_t e = allow_smem(kern, smem);
+        const cudaError_t e = allow_smem(kern, most_smem(kMaxT, second));
         if (e != cudaSuccess) return e;
         kern<<<nblocks, T, smem, s>>>(d, map, line32_constants(order), bump);
         return cudaGetLastError();

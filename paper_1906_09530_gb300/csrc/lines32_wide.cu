@@ -406,11 +406,6 @@ void divide_wide(Dir32& d, int nl) {
     d.g.ngroups = (d.g.nlines + nl - 1) / nl;
 }
 int blocks_of(const Geo32& g) { return g.ngroups * g.nwin; }
-template <class K>
-cudaError_t allow_smem(K kern, size_t bytes) {
-    if (bytes <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
 
 template <bool SECOND, int NL>
 cudaError_t run_wide(Dir32 x, Dir32 y, int nx, int ny, int order, DevState* st, int bump,

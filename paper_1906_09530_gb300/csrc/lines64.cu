@@ -59,7 +59,7 @@ struct Scheme64 {
 // slot of window position q in shared memory: one spare slot in 32, so that lanes whose
 // chunks start a power of two apart do not meet in one bank
 __device__ __forceinline__ int slot(int q) { return q + (q >> 5); }
-__host__ __device__ __forceinline__ int line_slots(int L) { return L + (L >> 5) + 1; }
+__host__ __device__ constexpr int line_slots(int L) { return L + (L >> 5) + 1; }
 
 // One line, one warp: s holds u on entry and z on return.
 template <bool SIXTH>
@@ -342,21 +342,17 @@ Geo geo64(int nx, int ny, int axis, bool walls_y, int lines_all) {
     return g;
 }
 
+// (windows of longer lines, and windows with a mirrored halo, are no longer than kLWhole)
+constexpr size_t kMostSmem = 4 * (size_t)line_slots(kLWhole) * sizeof(double);
+static_assert(kLOwn % 4 == 0 && kLOwn + 2 * kHalo <= kLWhole, "the longest window");
 size_t smem64(const Geo& g) { return (size_t)g.nl * line_slots(g.L) * sizeof(double); }
 unsigned blocks64(const Geo& g) { return (unsigned)((long long)g.ngroups * g.nwin); }
-
-// Every launch tells the kernel its size, also below the 48 KB that need no telling: those
-// are of the dynamic and the static arrays together (pw, logs).
-template <class K>
-cudaError_t allow_smem(K kern, size_t bytes) {
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
 
 template <int MODE>
 cudaError_t launch64(const Args& a, const Geo& g, int order, cudaStream_t s) {
     const size_t smem = smem64(g);
     auto go = [&](auto kern) -> cudaError_t {
-        const cudaError_t e = allow_smem(kern, smem);
+        const cudaError_t e = allow_smem(kern, kMostSmem);
         if (e != cudaSuccess) return e;
         kern<<<blocks64(g), kT, smem, s>>>(a, g, scheme64(order, g.L));
         return cudaGetLastError();
@@ -393,7 +389,7 @@ cudaError_t lines_fp64_rho_y_mu(const double* rho, const double* zxx, double* zy
     const MuArgs m{eos_const<double>(p), p.k2, p.kappa * sc.c1 * sc.c1, p.mu_cap, p.cap_steps};
     const size_t smem = smem64(g);
     auto go = [&](auto kern) -> cudaError_t {
-        const cudaError_t e = allow_smem(kern, smem);
+        const cudaError_t e = allow_smem(kern, kMostSmem);
         if (e != cudaSuccess) return e;
         kern<<<blocks64(g), kT, smem, s>>>(a, g, sc, m, log_table());
         return cudaGetLastError();
@@ -417,7 +413,7 @@ cudaError_t lines_fp64_force(const double* mu, const double* rho, const double* 
     const unsigned nbx = zx ? blocks64(gx) : 0, nby = zy ? blocks64(gy) : 0;
     const size_t sx = smem64(gx), sy = smem64(gy), smem = sx > sy ? sx : sy;
     auto go = [&](auto kern) -> cudaError_t {
-        const cudaError_t e = allow_smem(kern, smem);
+        const cudaError_t e = allow_smem(kern, kMostSmem);
         if (e != cudaSuccess) return e;
         kern<<<nbx + nby, kT, smem, s>>>(args(zx, Fx), gx, scheme64(order, gx.L),
                                                   args(zy, Fy), gy, scheme64(order, gy.L),

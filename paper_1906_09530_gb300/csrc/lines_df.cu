@@ -426,16 +426,22 @@ int blocks_of(const Geo32& g) { return g.ngroups * g.nwin; }
 size_t smem_df(const Geo32& g) {
     return ((size_t)8 * kT + 3 * (size_t)g.nl * l32::line_stride(g.nch)) * sizeof(float);
 }
-template <class K>
-cudaError_t allow_smem(K kern, size_t bytes) {
-    if (bytes <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+// the most that a block stages, of any grid
+size_t most_smem_df() {
+    size_t most = 0;
+    for (int nch = 8; nch <= 32; nch += 4) {
+        Geo32 g{};
+        g.nch = nch;
+        divide_df(g);
+        most = std::max(most, smem_df(g));
+    }
+    return most;
 }
 cudaError_t run_df(const Dir32& x, const Dir32& y, int nbx, int nby, int order, DevState* st,
                    int bump, cudaStream_t s) {
     const size_t smem = std::max(smem_df(x.g), smem_df(y.g));
     auto go = [&](auto kern) -> cudaError_t {
-        const cudaError_t e = allow_smem(kern, smem);
+        const cudaError_t e = allow_smem(kern, most_smem_df());
         if (e != cudaSuccess) return e;
         return launch_pdl(kern, dim3(nbx + nby), dim3(kT), smem, s, x, y, constants_df(order), st,
                           bump, nbx);
@@ -478,13 +484,7 @@ Lines32Inst lines_df_batch_inst(const MixedLinesView& v, int order, int blk0) {
 cudaError_t lines_df_batch_launch(const Lines32Inst* d, const int* map, int nblocks, int order,
                                   int bump, cudaStream_t s) {
     if (nblocks <= 0) return cudaSuccess;
-    size_t smem = 0;  // the most a block of any instance stages
-    for (int nch = 8; nch <= 32; nch += 4) {
-        Geo32 g{};
-        g.nch = nch;
-        divide_df(g);
-        smem = std::max(smem, smem_df(g));
-    }
+    const size_t smem = most_smem_df();
     auto go = [&](auto kern) -> cudaError_t {
         const cudaError_t e = allow_smem(kern, smem);
         if (e != cudaSuccess) return e;
