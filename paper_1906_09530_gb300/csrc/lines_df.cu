@@ -419,6 +419,10 @@ Dir32 dir_df(const float* h, const float* l, float* d1, float* d2, int nx, int n
     d.o1 = d1;
     d.o2 = d2;
     d.g = line32_geometry(nx, ny, axis, order, kEpsDF, second ? kEpsF : 0.0, walls_y);
+    // 16-byte pieces want 16-byte pointers as well as whole pieces a row: lbm_cfd_df takes any
+    // that hold floats.  (The fields of contexts and batches are 256-byte aligned.)
+    for (const float* p : {h, l, (const float*)d1, (const float*)d2})
+        if ((uintptr_t)p % 16 != 0) d.g.vec = 0;
     divide_df(d.g);
     return d;
 }
