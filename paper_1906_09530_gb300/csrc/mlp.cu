@@ -213,7 +213,7 @@ struct RowArgs {
     const float* bias;   // [256] (EPI_BIAS_TANH, EPI_BIAS, EPI_LOSS)
     const float* t;      // [M][256]: the targets (EPI_LOSS)
     float scale;         // EPI_LOSS: dL/dy = scale (y - target)
-    double* sse;         // EPI_LOSS: sum of (y - target)^2 (added to)
+    double* sse;         // EPI_LOSS: sums of (y - target)^2, [grid]
     float* bpart;        // or null: column sums of the result, [grid][256]
     float* out32;        // [M][256] (EPI_BIAS) or null
     __nv_bfloat16* out16;   // [M][256] or null
@@ -230,7 +230,9 @@ struct WgArgs {
     int chunks;       // K chunks (64 batch rows) in all
     int per_slice;    // K chunks per slice
     float* part;      // [slices][kWgTiles * 128][256]
-    double* next_sse; // squared-error sum of the next call, cleared here
+    const double* sse_part;  // squared-error sums of the chain's CTAs
+    int nsse;                // how many
+    double* sse;             // their sum
     int* err;
 };
 
@@ -478,6 +480,7 @@ __global__ void __launch_bounds__(kChainThreads, 1)
     __shared__ __align__(8) uint64_t bar[DN + 1];
     __shared__ uint32_t tbase;
     __shared__ int abort_s;
+    __shared__ double wsse[kChainEpi];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int M = g.st[0].M;
     if (warp == 0) {
@@ -693,7 +696,7 @@ __global__ void __launch_bounds__(kChainThreads, 1)
         }
         if (g.n > kLayers) {
             for (int i = 16; i > 0; i >>= 1) sse += __shfl_down_sync(0xffffffffu, sse, i);
-            if (lane == 0) atomicAdd(g.st[kLayers - 1].sse, sse);
+            if (lane == 0) wsse[warp] = sse;
         }
     }
     tc_fence_before();
@@ -705,6 +708,11 @@ __global__ void __launch_bounds__(kChainThreads, 1)
             const float* b = bsum + layer * kChainEpi * 32;
             g.st[s].bpart[(long long)blockIdx.x * UN + tid] = b[tid] + b[tid + kW];
         }
+    if (g.n > kLayers && warp == kW / 32) {
+        double sse = lane < kChainEpi ? wsse[lane] : 0.0;
+        for (int i = kChainEpi / 2; i > 0; i >>= 1) sse += __shfl_down_sync(0xffffffffu, sse, i);
+        if (lane == 0) g.st[kLayers - 1].sse[blockIdx.x] = sse;
+    }
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
                      "r"(chain_cols(ROWS))
@@ -726,7 +734,6 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int mt = blockIdx.x, slice = blockIdx.y;
     const int layer = (mt + 1) / 2, m0 = mt == 0 ? 0 : ((mt - 1) & 1) * UM;
-    const bool clears = mt == 0 && slice == 0 && tid == 0;
     const int j0 = slice * g.per_slice;
     const int nk = min(g.per_slice, g.chunks - j0);  // >= 1 by the host's choice of slices
     if (warp == 0) {
@@ -742,7 +749,6 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         abort_s = 0;
     }
     pdl_prologue();
-    if (clears) *g.next_sse = 0.0;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -804,6 +810,13 @@ __global__ void __launch_bounds__(kWgThreads, 1)
                              ((issued - 1) / kStages) & 1, nullptr);
         }
     } else {
+        if (mt == 0 && slice == 0 && warp == 0) {
+            // the call's squared-error sum, in a fixed order, while the products run
+            double sse = 0.0;
+            for (int q = lane; q < g.nsse; q += 32) sse += g.sse_part[q];
+            for (int o = 16; o > 0; o >>= 1) sse += __shfl_down_sync(0xffffffffu, sse, o);
+            if (lane == 0) *g.sse = sse;
+        }
         bool ok = mb_wait(&bar[2 * kStages], 0, abort_v);
         ok = __all_sync(0xffffffffu, ok);
         if (ok) {
@@ -1028,9 +1041,9 @@ struct lbm_mlp {
     float *d32, *e32;            // the same in FP32 (mma.sync kernel only), alternating
     float* part;                 // weight-gradient partials [slices][kWgTiles * 128][256]
     float* bpart;                // bias-gradient partials [layers][kChainCap][256]
-    double* sse;                 // squared-error sums of this call and the next, in turn
-    int turn;                    // which of them is this call's
-    double* h_sse;               // pinned mirror of both and err
+    double* sse;                 // squared-error sum of the call
+    double* sse_part;            // those of the chain's CTAs, [kChainCap]
+    double* h_sse;               // pinned mirror of the sum and err
     long long step;
     bool tensor_cores;           // forward and input-gradient products by tcgen05
     TcMaps maps;
@@ -1041,7 +1054,8 @@ namespace {
 size_t al(size_t v) { return (v + 255) / 256 * 256; }
 
 struct MlpLayout {
-    size_t p, g, m, v, w16, w16t, x16, a32, a16, sig, d32, e32, part, bpart, sse, total;
+    size_t p, g, m, v, w16, w16t, x16, a32, a16, sig, d32, e32, part, bpart, sse, sse_part,
+        total;
 };
 
 int rows_of(int B) { return (B + 7) / 8 * 8; }  // rows of the batch-sized buffers
@@ -1087,7 +1101,8 @@ MlpLayout mlp_layout(int B0) {
     L.e32 = take(B * kW * 4);
     L.part = take(S * kWgTiles * UM * UN * 4);
     L.bpart = take((size_t)kLayers * kChainCap * UN * 4);
-    L.sse = take(24);  // two squared-error sums and the error word, read back together
+    L.sse = take(16);  // the squared-error sum and the error word, read back together
+    L.sse_part = take(kChainCap * sizeof(double));
     L.total = o;
     return L;
 }
@@ -1114,7 +1129,7 @@ const __nv_bfloat16* w16t_of(const lbm_mlp* n, int l) {
 // Drain the stream; a tensor-core product whose bounded wait ran out since the
 // last check makes this LBM_ETIMEOUT (and the word is cleared).
 lbm_status sync(lbm_mlp* n) {
-    if (cudaMemcpyAsync(n->h_sse, n->sse, 24, cudaMemcpyDeviceToHost, n->stream) !=
+    if (cudaMemcpyAsync(n->h_sse, n->sse, 16, cudaMemcpyDeviceToHost, n->stream) !=
             cudaSuccess ||
         cudaStreamSynchronize(n->stream) != cudaSuccess)
         return LBM_ECUDA;
@@ -1234,7 +1249,7 @@ int row_stages(lbm_mlp* n, int B, const float* t, float* y, RowArgs* st) {
             g.epi = EPI_LOSS;
             g.t = t;
             g.scale = 1.0f / ((float)B * kOut);
-            g.sse = n->sse + n->turn;
+            g.sse = n->sse_part;
             g.out16 = n->sig[l];
             g.bpart = bpart_of(n, l);
         } else {
@@ -1287,10 +1302,13 @@ lbm_status rows_pass(lbm_mlp* n, const float* x, int B, const float* t, float* y
     return LBM_OK;
 }
 
-// the partial weight gradients, after rows_pass with targets
+// the partial weight gradients, after rows_pass with targets, and the squared-error sum from
+// those of the chain's CTAs: each is stored, so that nothing is left of an earlier call, a
+// captured one or a replay
 lbm_status wgrad_tc(lbm_mlp* n, int B) {
     const Slicing sl = slicing(B);
-    const WgArgs w{sl.chunks, sl.per_slice, n->part, n->sse + (1 - n->turn), n->err};
+    const WgArgs w{sl.chunks, sl.per_slice, n->part, n->sse_part, chain_ctas(n, B), n->sse,
+                   n->err};
     CK(launch(k_umma_wgrad, dim3(kWgTiles, sl.slices), kWgThreads, kWgSmem, n->stream,
               n->maps.wg, w));
     return LBM_OK;
@@ -1347,10 +1365,10 @@ bool use_tc(lbm_mlp* n, int B, lbm_status* st) {
 // loss and gradient into n->g (device) on the mma.sync kernel, after forward_ms()
 lbm_status backward_ms(lbm_mlp* n, const float* t, int B) {
     cudaStream_t s = n->stream;
-    CK(cudaMemsetAsync(n->sse, 0, 2 * sizeof(double), s));
+    CK(cudaMemsetAsync(n->sse, 0, sizeof(double), s));
     const int total = B * kOut;
     k_loss_grad<<<(total + 255) / 256 < 1024 ? (total + 255) / 256 : 1024, 256, 0, s>>>(
-        n->a32[kLayers - 1], t, total, 1.0f / (float)total, n->d32, n->sig[1], n->sse + n->turn);
+        n->a32[kLayers - 1], t, total, 1.0f / (float)total, n->d32, n->sig[1], n->sse);
     CK(cudaGetLastError());
     float* d32 = n->d32;
     __nv_bfloat16* d16 = n->sig[1];
@@ -1416,12 +1434,11 @@ lbm_status train(lbm_mlp* n, const float* x, const float* t, int B, float lr, fl
     lbm_status st = LBM_OK;
     const bool tc = use_tc(n, B, &st);
     if (st) return st;
-    n->turn = 1 - n->turn;  // (zero: cleared by the call before)
     auto loss = [&]() -> lbm_status {
         if (!h_loss) return LBM_OK;
         const lbm_status w = sync(n);
         if (w) return w;
-        *h_loss = n->h_sse[n->turn] / ((double)B * kOut);
+        *h_loss = *n->h_sse / ((double)B * kOut);
         return LBM_OK;
     };
     float c1 = 0.0f, c2 = 0.0f;
@@ -1498,8 +1515,8 @@ lbm_status lbm_mlp_init(lbm_mlp** out, int32_t max_batch, void* d_ws, size_t byt
     n->part = (float*)(w + L.part);
     n->bpart = (float*)(w + L.bpart);
     n->sse = (double*)(w + L.sse);
-    n->err = (int*)(n->sse + 2);
-    n->turn = 0;
+    n->err = (int*)(n->sse + 1);
+    n->sse_part = (double*)(w + L.sse_part);
     n->step = 0;
     n->tensor_cores = true;
     if (cudaDeviceGetAttribute(&n->nsm, cudaDevAttrMultiProcessorCount, n->dev) != cudaSuccess ||
@@ -1507,11 +1524,11 @@ lbm_status lbm_mlp_init(lbm_mlp** out, int32_t max_batch, void* d_ws, size_t byt
         delete n;
         return LBM_ECUDA;
     }
-    if (cudaMallocHost((void**)&n->h_sse, 24) != cudaSuccess) {
+    if (cudaMallocHost((void**)&n->h_sse, 16) != cudaSuccess) {
         delete n;
         return LBM_ECUDA;
     }
-    n->h_err = (int*)(n->h_sse + 2);
+    n->h_err = (int*)(n->h_sse + 1);
     if (cudaMemsetAsync(w, 0, L.total, n->stream) != cudaSuccess) {
         lbm_mlp_free(n);
         return LBM_ECUDA;
