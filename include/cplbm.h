@@ -146,10 +146,10 @@ lbm_status lbm_set_fields_device(lbm_ctx *ctx, const double *d_rho, const double
                                  const double *d_uy);
 
 /* Advance n >= 0 time steps.  Steps are enqueued (in CUDA graphs of two
- * steps; small periodic MIXED grids run many steps in one launch); the call then waits for the stream and checks the device error
- * flag.  LBM_EUNSTABLE: some step produced a bad value, lbm_failed_step()
- * names the first time level flagged, and the state is undefined until the
- * next lbm_set_fields. */
+ * steps; small periodic MIXED grids run many steps in one launch); the call then
+ * waits for the stream and checks the device error flag.  LBM_EUNSTABLE: some
+ * step produced a bad value, lbm_failed_step() names the first time level
+ * flagged, and the state is undefined until the next lbm_set_fields. */
 lbm_status lbm_step(lbm_ctx *ctx, int64_t n);
 
 /* Like lbm_step but returns right after enqueuing; lbm_check() later waits
@@ -159,7 +159,9 @@ lbm_status lbm_check(lbm_ctx *ctx);
 
 /* Profiling: run one time step as direct launches (no graph) with a CUDA event
  * recorded on the stream before and after each of its passes, wait for it, and
- * return the passes' durations in milliseconds (5 slots).
+ * return the passes' durations in milliseconds (5 slots).  The passes are always
+ * launches of their own here, also on grids whose lbm_step runs whole steps in
+ * one launch (lbm_set_launch_mode), and FP64's last two, which lbm_step merges.
  * FP64: [0] collide-stream, [1] x-lines of rho, [2] y-lines of rho + mu-hat,
  *       [3] x-lines of mu-hat + F_x, [4] y-lines of mu-hat + F_y.
  * MIXED: [0] collide-stream, [1] x- and y-lines of rho, [2] mu-hat (pointwise),
@@ -186,7 +188,9 @@ int32_t lbm_path_flags(const lbm_ctx *ctx);
  *   > 0 the row-ring kernel wherever it applies, with that many rows a block
  *       (at most 4096).
  * Both give bit-identical results; LBM_PATH_CS_RING in lbm_path_flags says
- * which one runs.  LBM_EINVAL for other values. */
+ * which one runs.  Grids that run whole steps in one launch (lbm_set_launch_mode)
+ * do so in the default form only; with another, a step's passes are launches of
+ * their own.  LBM_EINVAL for other values. */
 lbm_status lbm_set_collide_form(lbm_ctx *ctx, int32_t ring_rows);
 
 /* How the passes of a step are launched (results are the same either way):
@@ -194,8 +198,9 @@ lbm_status lbm_set_collide_form(lbm_ctx *ctx, int32_t ring_rows);
  *                 step of a longer call) replays a captured one-step CUDA graph;
  *                 0: its passes are launched directly.  Longer calls always
  *                 replay graphs of 2 and 16 steps.  Periodic MIXED grids of a few
- *                 thousand nodes (at most 8192) with FP32 density lines run
- *                 whole steps in one cluster launch instead, in every mode.
+ *                 thousand nodes (at most 8192) with FP32 density lines and the
+ *                 default collide form run whole steps in one cluster launch
+ *                 instead, in every mode.
  *   pdl_direct, pdl_graphs  programmatic dependent launch between the kernels
  *                 of a mixed step, for direct launches and for graph-captured
  *                 ones: each kernel lets the next be scheduled once all of its

@@ -67,7 +67,7 @@ struct lbm_ctx {
     int64_t t;
     int64_t failed;
     bool ready;      // fields set
-    bool small;      // steps run whole in one launch (launch_small_steps)
+    bool small;      // steps can run whole in one launch (launch_small_steps)
     cudaGraphExec_t graph[2];    // two steps, starting from f[0] / f[1]
     cudaGraphExec_t graph16[2];  // kLongGraph steps, likewise (fewer graph launches)
     cudaGraphExec_t graph1[2];   // one step, for single steps when single_graph is set
@@ -544,7 +544,7 @@ lbm_status lbm_step_async(lbm_ctx* c, int64_t n) {
     lbm_status st = use_dev(c);
     if (st) return st;
     int64_t left = n;
-    if (c->small) {
+    if (c->small && c->ring_rows == 0) {  // (a form that was asked for runs as its own kernel)
         CK(launch_small_steps(small_step(c), c->cur, n, c->stream));
         c->cur = (int)((c->cur + n) & 1);
         c->t += n;
