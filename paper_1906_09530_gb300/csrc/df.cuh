@@ -87,9 +87,31 @@ __device__ __forceinline__ void tf_add(tf& s, float x) {
 }
 // n / r to about 68 bits, rounded once to double: three quotient digits of one float
 // each, the remainder after the first kept as hi + lo.  inv: 1 / r.hi to a float's
-// accuracy.  Finite n and finite r with r.hi > 0.
+// accuracy.  The digits' products reach 72 bits below the operands and need room in a
+// float's range: operands outside it (the gas at reduced temperatures below 0.13) are first
+// brought to about one by powers of 2^64, and the quotient's exponent is put back.
 __device__ __forceinline__ double tf_div(tf n, df r, float inv) {
     df s = quick_two_sum(n.a, n.b);  // normalised: the head holds a float's accuracy
+    int k = 0;                       // the quotient's exponent, in units of 64
+    const float size = fabsf(s.hi);
+    if (!(r.hi >= 0x1p-60f && r.hi <= 0x1p8f && size <= 0x1p32f &&
+          (size >= 0x1p-84f || size == 0.0f))) {
+#pragma unroll 1
+        for (int i = 0; i < 3; ++i) {  // (zero, infinite and NaN ones stay what they are)
+            const float a = fabsf(r.hi), b = fabsf(s.hi);
+            const int kr = a < 0x1p-32f ? 1 : (a > 0x1p32f ? -1 : 0);
+            const int kn = b < 0x1p-32f ? 1 : (b > 0x1p32f ? -1 : 0);
+            const float fr = __int_as_float((127 + 64 * kr) << 23);
+            const float fn = __int_as_float((127 + 64 * kn) << 23);
+            r.hi = __fmul_rn(r.hi, fr);
+            r.lo = __fmul_rn(r.lo, fr);
+            s.hi = __fmul_rn(s.hi, fn);
+            s.lo = __fmul_rn(s.lo, fn);
+            n.c = __fmul_rn(n.c, fn);
+            k += kr - kn;
+        }
+        inv = __frcp_rn(r.hi);
+    }
     const float q0 = __fmul_rn(s.hi, inv);
     const float p = __fmul_rn(q0, r.hi), t = __fmul_rn(q0, r.lo);
     float lo = __fsub_rn(n.c, fmaf(q0, r.lo, -t));
@@ -105,7 +127,10 @@ __device__ __forceinline__ double tf_div(tf n, df r, float inv) {
     rem = __fsub_rn(rem, fmaf(q1, r.hi, -p1));
     rem = __fadd_rn(rem, fmaf(-q1, r.lo, lo));
     const float q2 = __fmul_rn(rem, inv);
-    return __dadd_rn(widen(q0), __dadd_rn(widen(q1), widen(q2)));
+    const double q = __dadd_rn(widen(q0), __dadd_rn(widen(q1), widen(q2)));
+    return k == 0 || q == 0.0 ? q
+                              : __hiloint2double(__double2hiint(q) + k * (64 << 20),
+                                                 __double2loint(q));
 }
 
 }  // namespace cplbm

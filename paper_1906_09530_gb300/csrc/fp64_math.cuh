@@ -32,9 +32,23 @@ __device__ __forceinline__ double rcp64(double x) {
     const double z = __fma_rn(y, __fma_rn(-x, y, 1.0), y);
     return __fma_rn(z, __fma_rn(-x, z, 1.0), z);
 }
+// a / x; rcp: rcp64(x).  Finite a; finite x != 0 (the EOS denominators: 1 - b rho, which is
+// zero at the pole alone, and its like).
 __device__ __forceinline__ double div64(double a, double x, double rcp) {
     const double q = __dmul_rn(a, rcp);
     return __fma_rn(__fma_rn(-x, q, a), rcp, q);
+}
+// n / x twice, for densities x down to the smallest subnormal: those whose reciprocal, or
+// whose product's remainder, has no place in the type are scaled with their numerators.
+__device__ __forceinline__ void quotients64(double& a, double& b, double x) {
+    if (((unsigned)__double2hiint(x) & 0x7ff00000u) < (523u << 20)) {
+        x = __dmul_rn(x, 0x1p500);
+        a = __dmul_rn(a, 0x1p500);
+        b = __dmul_rn(b, 0x1p500);
+    }
+    const double inv = rcp64(x);
+    a = div64(a, x, inv);
+    b = div64(b, x, inv);
 }
 
 struct LogTable {

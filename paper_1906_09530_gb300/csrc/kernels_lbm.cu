@@ -131,9 +131,9 @@ __device__ __forceinline__ void node_velocity(const double* __restrict__ f, size
     for (int i = 1; i < 9; ++i) g[i] = f[i * plane + n];
     const double jx = (g[1] + g[5] + g[8]) - (g[3] + g[6] + g[7]);
     const double jy = (g[2] + g[5] + g[6]) - (g[4] + g[7] + g[8]);
-    const double inv = rcp64(rho);
-    vx = div64(jx + 0.5 * Fx, rho, inv);
-    vy = div64(jy + 0.5 * Fy, rho, inv);
+    vx = jx + 0.5 * Fx;
+    vy = jy + 0.5 * Fy;
+    quotients64(vx, vy, rho);
 }
 
 __global__ void k_macro(const double* __restrict__ f, const double* __restrict__ rho,
