@@ -40,9 +40,18 @@ __device__ __forceinline__ void collide_bgk(double (&f)[9], double rho, double F
     const double inv = rcp64(rho);
     const double mx = rn_add(jx, Fx), my = rn_add(jy, Fy);
     const double kx = rn_mul(keep, jx), ky = rn_mul(keep, jy);
-    const double pxx = rn_mul(rn_fma(mx, mx, -rn_mul(kx, jx)), inv);
-    const double pyy = rn_mul(rn_fma(my, my, -rn_mul(ky, jy)), inv);
-    const double pxy = rn_mul(rn_fma(mx, my, -rn_mul(kx, jy)), inv);
+    double pxx, pyy, pxy;
+    if (__double2hiint(rho) >= (1023 - 400) << 20) {  // 2^-400, without an FP64 comparison
+        pxx = rn_mul(rn_fma(mx, mx, -rn_mul(kx, jx)), inv);
+        pyy = rn_mul(rn_fma(my, my, -rn_mul(ky, jy)), inv);
+        pxy = rn_mul(rn_fma(mx, my, -rn_mul(kx, jy)), inv);
+    } else {  // m m would underflow
+        const double vx = rn_mul(mx, inv), vy = rn_mul(my, inv);
+        const double ux = rn_mul(kx, inv), uy = rn_mul(ky, inv);
+        pxx = rn_fma(mx, vx, -rn_mul(ux, jx));
+        pyy = rn_fma(my, vy, -rn_mul(uy, jy));
+        pxy = rn_fma(mx, vy, -rn_mul(ux, jy));
+    }
     const double s = rn_add(pxx, pyy);
     const double e1 = rn_mul(rn_fma(-1.5, s, rn_mul(omega, rho)), 1.0 / 9.0);
     f[0] = rn_fma(keep, f[0], rn_mul(4.0, e1));

@@ -48,3 +48,23 @@ def test_velocity_is_the_quotient(cuda, precision, k):
         assert np.all(np.abs(v - w) <= np.spacing(np.abs(w)))
     assert abs(vmax - np.sqrt(wx**2 + wy**2).max()) <= 4 * np.spacing(vmax)
     assert rmin == rmax == r[0, 0] and abs(mass - r.sum()) <= 1e-12 * mass
+
+
+@pytest.mark.parametrize("collision", ["bgk", "mrt"])
+@pytest.mark.parametrize("k", [-300, -600, -900])
+def test_collision_at_any_scale(cuda, collision, k):
+    """A uniform flow relaxes alike at every density: one step of the FP64 path, to 16 units
+    of the largest population (the collision has some 60 roundings, most of smaller terms).
+    Its terms u u rho are of size 0.01 rho here, not of (u rho)^2, which has no place in the
+    type."""
+    def stepped(k):
+        f = np.repeat(np.repeat(populations(1, 1, 0), 16, 1), 16, 2)
+        sim = simulation(16, 16, 0, "fp64", collision=collision)
+        sim.set_populations(np.ldexp(f, k))
+        sim.step(1)
+        out = sim.get_populations()[0]
+        sim.close()
+        return np.ldexp(out, -k)
+
+    want, got = stepped(0), stepped(k)
+    assert np.abs(got - want).max() <= 16 * 2.0**-53 * want.max()
