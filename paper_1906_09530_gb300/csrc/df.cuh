@@ -128,9 +128,11 @@ __device__ __forceinline__ double tf_div(tf n, df r, float inv) {
     rem = __fadd_rn(rem, fmaf(-q1, r.lo, lo));
     const float q2 = __fmul_rn(rem, inv);
     const double q = __dadd_rn(widen(q0), __dadd_rn(widen(q1), widen(q2)));
-    return k == 0 || q == 0.0 ? q
-                              : __hiloint2double(__double2hiint(q) + k * (64 << 20),
-                                                 __double2loint(q));
+    // (a NaN keeps its exponent: its high word has bits 19 to 30 set)
+    const unsigned hi = (unsigned)__double2hiint(q);
+    return k == 0 || q == 0.0 || (~hi & 0x7ff80000u) == 0u
+               ? q
+               : __hiloint2double((int)hi + k * (64 << 20), __double2loint(q));
 }
 
 }  // namespace cplbm

@@ -68,3 +68,21 @@ def test_collision_at_any_scale(cuda, collision, k):
 
     want, got = stepped(0), stepped(k)
     assert np.abs(got - want).max() <= 16 * 2.0**-53 * want.max()
+
+
+@pytest.mark.parametrize("precision", ["mixed", "mixed_df", "fp64"])
+@pytest.mark.parametrize("k,node", [(0, 0.0), (-100, 0.0), (-100, np.nan), (0, np.nan)])
+def test_velocity_without_a_value_is_nan(cuda, precision, k, node):
+    """A node without a density makes the state unstable, which the next check says; what is
+    read on the device before it has no velocity at that node, and not a number that looks
+    like one."""
+    from paper_1906_09530_gb300 import LbmError
+    rho = np.full((29, 37), 2.0**k)
+    rho[11, 17] = node
+    sim = simulation(37, 29, k, precision)
+    sim.set_fields_device(cuda.from_numpy(rho).cuda())
+    _, vx, vy, _ = (a.cpu().numpy() for a in sim.fields_device())
+    assert np.isnan(vx[11, 17]) and np.isnan(vy[11, 17])
+    with pytest.raises(LbmError):
+        sim.check()
+    sim.close()
