@@ -77,17 +77,22 @@ __device__ __forceinline__ float force_term(float r, float dmu, float d) {
 
 // Right-hand sides of a chunk from u at chunk positions -4 .. kC + 3 (first derivative
 // alone: -2 .. kC + 1), and the recursions forward from a zero state.
+// Explicitly rounded, as everything here: with contraction left to the compiler, the same
+// line could have other bits in another kernel.  At 4th order the chunk's two outermost
+// right-hand sides have one use each, and go into it as a multiply-add.
 template <bool SIXTH, bool SECOND, class U>
 __device__ __forceinline__ void chunk_forward(U u, const Line32& k, float (&r)[kC],
                                               float (&r2)[kC], float& w1, float& v2, float& w2) {
     auto rhs = [&](float am2, float am1, float ap1, float ap2) {
-        float b = (ap1 - am1) * k.c1;
+        float b = rn_mul(rn_sub(ap1, am1), k.c1);
         if (SIXTH) b = rn_fma(rn_sub(ap2, am2), k.c2, b);
         return b;
     };
 #pragma unroll
     for (int j = 0; j < kC; ++j) r[j] = rhs(u(j - 2), u(j - 1), u(j + 1), u(j + 2));
     if (SECOND) {
+        // the first right-hand side at j - 2, without its factor (4th order)
+        auto dif = [&](int j) { return rn_sub(u(j - 1), u(j - 3)); };
         float b[kC + 4];  // the first right-hand side at -2 .. kC + 1
 #pragma unroll
         for (int j = 0; j < kC + 4; ++j)
@@ -95,7 +100,9 @@ __device__ __forceinline__ void chunk_forward(U u, const Line32& k, float (&r)[k
 #pragma unroll
         for (int j = 0; j < kC; ++j) {
             if (SIXTH) r2[j] = rhs(b[j], b[j + 1], b[j + 3], b[j + 4]);
-            else r2[j] = (b[j + 3] - b[j + 1]) * k.c1;
+            else if (j == 0) r2[j] = rn_mul(rn_fma(-dif(1), k.c1, b[3]), k.c1);
+            else if (j == kC - 1) r2[j] = rn_mul(rn_fma(dif(kC + 2), k.c1, -b[kC]), k.c1);
+            else r2[j] = rn_mul(rn_sub(b[j + 3], b[j + 1]), k.c1);
         }
     }
     w1 = 0.0f;
