@@ -38,6 +38,8 @@ constexpr int kPw = 57;       // powers (-lam)^0 .. (-lam)^56
 constexpr int kHalo = 96;     // two solves of kPw - 9 positions: lam^48 < 1e-20
 constexpr int kLWhole = 1600; // longest line solved whole
 constexpr int kLOwn = 1100;   // most positions a window of a longer one owns
+// ... and of a launch of few lines (see geo64)
+constexpr int kLFew = kLOwn + 2 * kHalo;
 constexpr int kSMs = 152;
 
 struct Geo {
@@ -315,7 +317,11 @@ Geo geo64(int nx, int ny, int axis, bool walls_y, int lines_all) {
         g.L = g.n + 2 * kHalo;
     }
     g.nwin = 1;
-    if (g.L > kLWhole) {
+    // Where an SM has one or two lines a line's length is the time, and windows are shorter:
+    // 7, 200 and 300 stand-alone lines of 1500, both derivatives, 37.1, 41.2 and 41.2 us whole
+    // and 24.9, 26.8 and 35.0 in two windows; of 1600 39.1, 43.2 and 43.1, and 32.9, 33.0 and
+    // 41.2.  (From 1293 on: then a window is shorter than the longest of a longer line.)
+    if (g.L > (lines_all <= 2 * kSMs ? kLFew : kLWhole)) {
         g.nwin = (g.n + kLOwn - 1) / kLOwn;
         g.own = ((g.n + g.nwin - 1) / g.nwin + 3) / 4 * 4;
         g.H = kHalo;

@@ -86,3 +86,22 @@ def test_chemical_potential_over_twelve_decades(cuda):
             tol = 8 * 2.0**-53 * np.abs(terms).max()
             assert np.all(np.abs(mu - sum(terms)) <= tol), (kind, r)
         sim.close()
+
+
+# 304 lines are the most that count as few, 1292 positions the longest they are solved whole
+@pytest.mark.parametrize("axis", [0, 1])
+@pytest.mark.parametrize("lines", [304, 305])
+@pytest.mark.parametrize("n", [1292, 1293, 1599])
+def test_few_lines_in_windows(cuda, n, lines, axis):
+    """Tolerance 1e-13 of the largest derivative, as for single lines."""
+    from oracle import cfd_alpha, cfd_line
+    from paper_1906_09530_gb300 import lbm_cfd
+    u = np.random.default_rng(n).standard_normal((lines, n)) + 3.0
+    v = u if axis == 0 else np.ascontiguousarray(u.T)
+    d1, d2 = (d.cpu().numpy() for d in lbm_cfd(cuda.from_numpy(v).cuda(), axis, 6, True))
+    if axis == 1:
+        d1, d2 = d1.T, d2.T
+    r1 = np.stack([cfd_line(x, cfd_alpha(6)) for x in u])
+    r2 = np.stack([cfd_line(x, cfd_alpha(6)) for x in r1])
+    assert np.abs(d1 - r1).max() <= 1e-13 * np.abs(r1).max()
+    assert np.abs(d2 - r2).max() <= 1e-13 * np.abs(r2).max()
