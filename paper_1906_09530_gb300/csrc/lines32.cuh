@@ -79,8 +79,9 @@ __device__ __forceinline__ float force_term(float r, float dmu, float d) {
 // alone: -2 .. kC + 1), and the recursions forward from a zero state.
 // Explicitly rounded, as everything here: with contraction left to the compiler, the same
 // line could have other bits in another kernel.  At 4th order the chunk's two outermost
-// right-hand sides have one use each, and go into it as a multiply-add.
-template <bool SIXTH, bool SECOND, class U>
+// right-hand sides have one use each, and go into it as a multiply-add (EDGE; not in
+// lines_df.cu).
+template <bool SIXTH, bool SECOND, bool EDGE = true, class U>
 __device__ __forceinline__ void chunk_forward(U u, const Line32& k, float (&r)[kC],
                                               float (&r2)[kC], float& w1, float& v2, float& w2) {
     auto rhs = [&](float am2, float am1, float ap1, float ap2) {
@@ -100,8 +101,8 @@ __device__ __forceinline__ void chunk_forward(U u, const Line32& k, float (&r)[k
 #pragma unroll
         for (int j = 0; j < kC; ++j) {
             if (SIXTH) r2[j] = rhs(b[j], b[j + 1], b[j + 3], b[j + 4]);
-            else if (j == 0) r2[j] = rn_mul(rn_fma(-dif(1), k.c1, b[3]), k.c1);
-            else if (j == kC - 1) r2[j] = rn_mul(rn_fma(dif(kC + 2), k.c1, -b[kC]), k.c1);
+            else if (EDGE && j == 0) r2[j] = rn_mul(rn_fma(-dif(1), k.c1, b[3]), k.c1);
+            else if (EDGE && j == kC - 1) r2[j] = rn_mul(rn_fma(dif(kC + 2), k.c1, -b[kC]), k.c1);
             else r2[j] = rn_mul(rn_sub(b[j + 3], b[j + 1]), k.c1);
         }
     }

@@ -18,6 +18,8 @@
 // 33.4 us unrolled in registers, 25.2 so (a step 54.5 -> 47.6).  What is left is uneven: 500
 // blocks, half of them crossing the interface, on 456 places.  Half groups (128 threads, one
 // wave) were no faster: 51.7 against 49.9 us a step.
+// Where a launch has more blocks than that, groups solved in FP32 run as in lines32.cuh, with
+// the chunk in registers (kPlaces): their unrolled code is a tenth of the double-float one's.
 #include <algorithm>
 #include <cfloat>
 #include <cmath>
@@ -55,7 +57,8 @@ __device__ __forceinline__ df join_df(const LineDF& k, const float* h, const flo
 
 // Shared memory: eight join arrays of kT floats, the two planes of the staged window (hi, lo),
 // whose places the first derivative takes, and the second derivative's plane.
-template <bool SIXTH>
+// REGS: groups solved in FP32 have their chunks in registers (see kPlaces).
+template <bool SIXTH, bool SECOND, bool REGS>
 __device__ __forceinline__ void block_df(const Dir32& d, const LineDF& k, int axis, int bid,
                                          float* sh) {
     const Geo32& g = d.g;
@@ -161,29 +164,46 @@ __device__ __forceinline__ void block_df(const Dir32& d, const LineDF& k, int ax
     auto at_f = [&](int j) {
         return rhs_f(uh[(j - 2) * ps], uh[(j - 1) * ps], uh[(j + 1) * ps], uh[(j + 2) * ps]);
     };
-    // what the chunk needs of its neighbours, before they overwrite it: the window two
-    // positions either side, and the first right-hand side there (FP32)
-    const bool second = d.o2 != nullptr;
-    df a{0.0f, 0.0f}, b = a, z1 = a, z2 = a;
-    float bm2 = 0.0f, bm1 = 0.0f, bp1 = 0.0f, bp2 = 0.0f;
-    if (live) {
-        a = U(-2);
-        b = U(-1);
-        z1 = U(kC);
-        z2 = U(kC + 1);
-        if (second) {
-            bm2 = at_f(-2);
-            bm1 = at_f(-1);
-            bp1 = at_f(kC);
-            bp2 = at_f(kC + 1);
+    // What the chunk needs of its neighbours, before they overwrite it: the window two
+    // positions either side, and the first right-hand side there (FP32), in r; or the chunk
+    // itself.
+    const bool regs = REGS && live && !wide, loops = live && !regs;
+    float r[kC], r2[REGS ? kC : 1];
+    if constexpr (REGS) {
+        if (regs) {
+            float w1, v2, w2;
+            l32::chunk_forward<SIXTH, SECOND, false>([&](int j) { return uh[j * ps]; }, k.f, r,
+                                                     r2, w1, v2, w2);
+            *eh = w1;
+            if (SECOND) {
+                *ev = v2;
+                *ew = w2;
+            }
+        }
+    }
+    if (loops) {
+        auto keep = [&](int i, df x) {
+            r[i] = x.hi;
+            r[i + 1] = x.lo;
+        };
+        keep(0, U(-2));
+        keep(2, U(-1));
+        keep(4, U(kC));
+        keep(6, U(kC + 1));
+        if (SECOND) {
+            r[8] = at_f(-2);
+            r[9] = at_f(-1);
+            r[10] = at_f(kC);
+            r[11] = at_f(kC + 1);
         }
     }
     const int after = nch - 1 - c;
     __syncthreads();
     // ---- forward ----
-    if (live) {
-        df e = U(0), f = U(1);
-        if (wide) {
+    if (loops) {
+        df a{r[0], r[1]}, b{r[2], r[3]}, e = U(0), f = U(1);
+        const df z1{r[4], r[5]}, z2{r[6], r[7]};
+        if (REGS || wide) {
             df w{0.0f, 0.0f};
             float *ph = uh, *pl = ul, *p = q2;  // at position j
             auto step = [&](df h) {
@@ -229,8 +249,8 @@ __device__ __forceinline__ void block_df(const Dir32& d, const LineDF& k, int ax
             step(z2.hi);
             *eh = w;
         }
-        if (second) {
-            float p = bm2, q = bm1, r = q2[0], x = q2[ps], v = 0.0f, w = 0.0f;
+        if (SECOND) {
+            float p = r[8], q = r[9], u = q2[0], x = q2[ps], v = 0.0f, w = 0.0f;
             float* o = q2;
             auto step = [&](float h) {
                 float y = rn_mul(rn_sub(x, q), k.f.c1);
@@ -239,23 +259,35 @@ __device__ __forceinline__ void block_df(const Dir32& d, const LineDF& k, int ax
                 *o = w = rn_fma(w, k.f.nlam, v);
                 o += ps;
                 p = q;
-                q = r;
-                r = x;
+                q = u;
+                u = x;
                 x = h;
             };
 #pragma unroll 8
             for (int j = 0; j < kC - 3; ++j) step(o[2 * ps]);
             step(o[2 * ps]);
-            step(bp1);
-            step(bp2);
+            step(r[10]);
+            step(r[11]);
             *ev = v;
             *ew = w;
         }
     }
     __syncthreads();
     // ---- backward ----
-    if (live) {
-        if (wide) {
+    if constexpr (REGS) {
+        if (regs) {
+            const float cf = l32::join1<0>(k.f, eh, js, c);
+            float cv = 0.0f, cw = 0.0f, y, z;
+            if (SECOND) l32::join2<0>(k.f, ev, ew, js, c, cv, cw);
+            l32::chunk_backward<SECOND>(k.f, cf, cv, cw, r, r2, *zh, y, z);
+            if (SECOND) {
+                *zv = y;
+                *zw = z;
+            }
+        }
+    }
+    if (loops) {
+        if (REGS || wide) {
             const df cf = join_df(k, eh, el, js, c);
             df z{0.0f, 0.0f};
             float *ph = uh + (kC - 1) * ps, *pl = ul + (kC - 1) * ps;
@@ -277,7 +309,7 @@ __device__ __forceinline__ void block_df(const Dir32& d, const LineDF& k, int ax
                 uh[j * ps] = z = rn_fma(z, k.f.nlam, rn_fma(cf, k.f.pw[j], uh[j * ps]));
             *zh = z;
         }
-        if (second) {
+        if (SECOND) {
             float cv, cw, y = 0.0f, z = 0.0f;
             l32::join2<0>(k.f, ev, ew, js, c, cv, cw);
 #pragma unroll 5
@@ -292,8 +324,21 @@ __device__ __forceinline__ void block_df(const Dir32& d, const LineDF& k, int ax
     }
     __syncthreads();
     // ---- the state entering from after the chunk ----
-    if (live) {
-        if (wide) {
+    if constexpr (REGS) {
+        if (regs) {
+            const float cb = l32::join1<0>(k.f, zh, -js, after);
+            float cy = 0.0f, cz = 0.0f;
+            if (SECOND) l32::join2<0>(k.f, zv, zw, -js, after, cy, cz);
+            l32::chunk_finish<SECOND>(k.f, cb, cy, cz, r, r2);
+#pragma unroll
+            for (int j = 0; j < kC; ++j) {
+                uh[j * ps] = r[j];
+                if (SECOND) q2[j * ps] = r2[j];
+            }
+        }
+    }
+    if (loops) {
+        if (REGS || wide) {
             const df cb = join_df(k, zh, zl, -js, after);
             float *ph = uh, *pl = ul;
 #pragma unroll 4
@@ -307,7 +352,7 @@ __device__ __forceinline__ void block_df(const Dir32& d, const LineDF& k, int ax
 #pragma unroll 5
             for (int j = 0; j < kC; ++j) uh[j * ps] = rn_fma(cb, k.f.pw[kC - 1 - j], uh[j * ps]);
         }
-        if (second) {
+        if (SECOND) {
             float cy, cz;
             l32::join2<0>(k.f, zv, zw, -js, after, cy, cz);
 #pragma unroll 5
@@ -327,14 +372,14 @@ __device__ __forceinline__ void block_df(const Dir32& d, const LineDF& k, int ax
                 for (int q = 4 * c; q < nown; q += 4 * nch) {
                     *reinterpret_cast<float4*>(d.o1 + o + q) =
                         *reinterpret_cast<const float4*>(r1 + q);
-                    if (d.o2)
+                    if (SECOND)
                         *reinterpret_cast<float4*>(d.o2 + o + q) =
                             *reinterpret_cast<const float4*>(r2 + q);
                 }
             } else {
                 for (int q = c; q < nown; q += nch) {
                     d.o1[o + q] = r1[q];
-                    if (d.o2) d.o2[o + q] = r2[q];
+                    if (SECOND) d.o2[o + q] = r2[q];
                 }
             }
         }
@@ -347,17 +392,17 @@ __device__ __forceinline__ void block_df(const Dir32& d, const LineDF& k, int ax
             const int m = (q + H4) * nl + x;
             if (g.vec) {
                 *reinterpret_cast<float4*>(d.o1 + o) = *reinterpret_cast<const float4*>(hi + m);
-                if (d.o2)
+                if (SECOND)
                     *reinterpret_cast<float4*>(d.o2 + o) = *reinterpret_cast<const float4*>(p2 + m);
             } else {
                 d.o1[o] = hi[m];
-                if (d.o2) d.o2[o] = p2[m];
+                if (SECOND) d.o2[o] = p2[m];
             }
         }
     }
 }
 
-template <bool SIXTH>
+template <bool SIXTH, bool SECOND, bool REGS>
 __global__ void __launch_bounds__(kT, 3)
     k_lines_df(Dir32 x, Dir32 y, const __grid_constant__ LineDF k, DevState* st, int bump,
                int nbx) {
@@ -367,10 +412,10 @@ __global__ void __launch_bounds__(kT, 3)
     const int nby = (int)gridDim.x - nbx, b = blockIdx.x;
     const bool is_y = b < nby;
     const Dir32& d = is_y ? y : x;
-    block_df<SIXTH>(d, k, is_y, is_y ? b : b - nby, shdf);
+    block_df<SIXTH, SECOND, REGS>(d, k, is_y, is_y ? b : b - nby, shdf);
 }
 
-template <bool SIXTH>
+template <bool SIXTH, bool REGS>
 __global__ void __launch_bounds__(kT, 3)
     k_lines_df_batch(const Lines32Inst* __restrict__ d, const int* __restrict__ map,
                      const __grid_constant__ LineDF k, int bump) {
@@ -379,7 +424,7 @@ __global__ void __launch_bounds__(kT, 3)
     const int local = (int)blockIdx.x - D.blk0;
     if (bump && local == 0 && threadIdx.x == 0) D.st->t += 1;
     const bool is_y = local >= D.nbx;
-    block_df<SIXTH>(is_y ? D.y : D.x, k, is_y, is_y ? local - D.nbx : local, shdf);
+    block_df<SIXTH, true, REGS>(is_y ? D.y : D.x, k, is_y, is_y ? local - D.nbx : local, shdf);
 }
 
 // ---- host side ----
@@ -441,6 +486,13 @@ size_t most_smem_df() {
     }
     return most;
 }
+// More blocks than the chip has places (three an SM): then what counts is a block's work, and
+// groups solved in FP32 keep their chunks in registers, unrolled; below it is the latency,
+// which the fetch of that code adds to.  Steps at ratio 8e4 in loops and in registers:
+// 512^2 22.4 and 22.8 us, 1001 x 603 (404 blocks) 47.1 and 47.9, 3000 x 200 (525) 37.0 and
+// 35.4, 1500^2 96.5 and 93.3, 4096^2 572 and 536; the density alone, 2048^2 along x 26.8 and
+// 20.5 us.
+constexpr int kPlaces = 3 * 152;
 cudaError_t run_df(const Dir32& x, const Dir32& y, int nbx, int nby, int order, DevState* st,
                    int bump, cudaStream_t s) {
     const size_t smem = std::max(smem_df(x.g), smem_df(y.g));
@@ -450,7 +502,17 @@ cudaError_t run_df(const Dir32& x, const Dir32& y, int nbx, int nby, int order, 
         return launch_pdl(kern, dim3(nbx + nby), dim3(kT), smem, s, x, y, constants_df(order), st,
                           bump, nbx);
     };
-    return order == 6 ? go(k_lines_df<true>) : go(k_lines_df<false>);
+    const bool regs = nbx + nby > kPlaces;
+    if (x.o2) {
+        if (regs) return order == 6 ? go(k_lines_df<true, true, true>)
+                                    : go(k_lines_df<false, true, true>);
+        return order == 6 ? go(k_lines_df<true, true, false>)
+                          : go(k_lines_df<false, true, false>);
+    }
+    if (regs) return order == 6 ? go(k_lines_df<true, false, true>)
+                                : go(k_lines_df<false, false, true>);
+    return order == 6 ? go(k_lines_df<true, false, false>)
+                      : go(k_lines_df<false, false, false>);
 }
 
 }  // namespace
@@ -495,7 +557,9 @@ cudaError_t lines_df_batch_launch(const Lines32Inst* d, const int* map, int nblo
         kern<<<nblocks, kT, smem, s>>>(d, map, constants_df(order), bump);
         return cudaGetLastError();
     };
-    return order == 6 ? go(k_lines_df_batch<true>) : go(k_lines_df_batch<false>);
+    if (nblocks > kPlaces)
+        return order == 6 ? go(k_lines_df_batch<true, true>) : go(k_lines_df_batch<false, true>);
+    return order == 6 ? go(k_lines_df_batch<true, false>) : go(k_lines_df_batch<false, false>);
 }
 
 }  // namespace cplbm

@@ -1,0 +1,36 @@
+"""Double-float line solves (lbm_cfd_df): groups of lines that are solved in FP32 have their
+chunks in registers where a launch has more blocks than the chip has places, and in shared
+memory else.  Both give the same bits: many lines at once against the same lines a few at a
+time, with smooth groups and groups across an interface side by side."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("order", [4, 6])
+@pytest.mark.parametrize("axis", [0, 1])
+@pytest.mark.parametrize("n,lines", [(1000, 2400), (1001, 2397), (40, 16000), (2500, 760)])
+def test_many_lines_equal_few(cuda, n, lines, axis, order):
+    from paper_1906_09530_gb300 import lbm_cfd_df
+    torch = cuda
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    u = torch.rand((lines, n), generator=gen, device="cuda", dtype=torch.float64) + 1.0
+    steep = torch.arange(lines, device="cuda") // 24 % 3 == 1
+    u[steep, : n // 2] *= 1e-5
+    hi = u.float()
+    lo = (u - hi.double()).float()
+
+    def solve(a, b, second):
+        h, lw = hi[a:b], lo[a:b]
+        if axis == 1:
+            h, lw = h.t(), lw.t()
+        out = lbm_cfd_df(h.contiguous(), lw.contiguous(), axis, order, second)
+        out = out if second else (out,)
+        return [o.t() if axis == 1 else o for o in out]
+
+    for second in (True, False):
+        whole = solve(0, lines, second)
+        few = [solve(a, min(a + 192, lines), second) for a in range(0, lines, 192)]
+        for i, w in enumerate(whole):
+            assert torch.isfinite(w).all()
+            assert torch.equal(w, torch.cat([f[i] for f in few]))
