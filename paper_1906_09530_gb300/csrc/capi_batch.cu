@@ -85,6 +85,7 @@ struct Tables {
     size_t cs, mu, rho_df, rho_f32, force, state;
     size_t map_cs, map_mu, map_rho_df, map_rho_f32, map_force, end;
     int nb_cs, nb_mu, nb_rho_df, nb_rho_f32, nb_force;  // current counts
+    size_t smem_df;  // shared memory of a block of the double-float density lines
 };
 
 Tables table_layout(const lbm_instance* inst, int n, int order, size_t base) {
@@ -120,6 +121,7 @@ Tables table_layout(const lbm_instance* inst, int n, int order, size_t base) {
     t.map_force = take(force * sizeof(int));
     t.end = o;
     t.nb_cs = t.nb_mu = t.nb_rho_df = t.nb_rho_f32 = t.nb_force = 0;
+    t.smem_df = 0;
     return t;
 }
 
@@ -217,6 +219,7 @@ lbm_status upload_tables(lbm_batch* b) {
         const MixedLinesView v = view_of(b, i);
         if (h.rho_df) {
             rdf[i] = lines_df_batch_inst(v, b->order, (int)mrdf.size());
+            t.smem_df = std::max(t.smem_df, lines_df_batch_smem(rdf[i]));
             mrdf.insert(mrdf.end(), lines_df_batch_blocks(h.nx, h.ny, b->order), i);
         } else {
             rf[i] = lines32_batch_inst(v, b->order, true, (int)mrf.size(), b->line_nl, b->wide);
@@ -287,7 +290,7 @@ lbm_status enqueue_step(lbm_batch* b, cudaStream_t s, int from, cudaEvent_t* ev 
         CK(cudaStreamWaitEvent(side, b->fork_ev, 0));
     }
     CK(lines_df_batch_launch(at<Lines32Inst>(b, t.rho_df), at<int>(b, t.map_rho_df), t.nb_rho_df,
-                             b->order, 1, sd));
+                             b->order, t.smem_df, 1, sd));
     CK(f32_lines(b, true, 1, s));
     if (fork) {
         CK(cudaEventRecord(b->join_ev, side));

@@ -547,12 +547,18 @@ Lines32Inst lines_df_batch_inst(const MixedLinesView& v, int order, int blk0) {
     return d;
 }
 
+size_t lines_df_batch_smem(const Lines32Inst& d) {
+    return std::max(smem_df(d.x.g), smem_df(d.y.g));
+}
+
 cudaError_t lines_df_batch_launch(const Lines32Inst* d, const int* map, int nblocks, int order,
-                                  int bump, cudaStream_t s) {
+                                  size_t smem, int bump, cudaStream_t s) {
     if (nblocks <= 0) return cudaSuccess;
-    const size_t smem = most_smem_df();
+    // (two blocks an SM fit with the most any grid stages, and 256 of them are faster so: two
+    // 512^2 at ratio 8e4 35.6 us a step against 36.6)
+    if (nblocks <= 2 * 152) smem = most_smem_df();
     auto go = [&](auto kern) -> cudaError_t {
-        const cudaError_t e = allow_smem(kern, smem);
+        const cudaError_t e = allow_smem(kern, most_smem_df());
         if (e != cudaSuccess) return e;
         kern<<<nblocks, kT, smem, s>>>(d, map, constants_df(order), bump);
         return cudaGetLastError();
