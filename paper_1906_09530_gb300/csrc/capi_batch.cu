@@ -72,11 +72,25 @@ int cs_blocks_for(int nx, int ny, int rows) {
 }
 int mu_blocks_for(size_t N) { return (int)(((N + 3) / 4 + kMuBatchT - 1) / kMuBatchT); }
 
-// A batch with a grid above kLines32Nodes solves its FP32 lines in full windows.
-bool wide_lines(const lbm_instance* inst, int n) {
-    for (int i = 0; i < n; ++i)
-        if ((long long)inst[i].grid.nx * inst[i].grid.ny > kLines32Nodes) return true;
-    return false;
+// Whether a batch solves its FP32 lines in full windows (lines32_wide.cu) instead of by (line,
+// chunk) pairs, which saves chunks and spreads over more threads: with a grid above
+// kLines32Nodes; and where all rows are whole 16-byte pieces (else it always lost: 24 odd
+// members up to 400^2 63 us a step against 73), if most chunks are needed (16 of 512^2 147 us
+// by pairs and 140 in windows, 24 members up to 512^2 that use 84 of 100 chunks 111 and 109;
+// 24 that use 67 of 100 64 and 66, 256 of 128^2 174 and 233), or if the launch is about one
+// round of blocks, where a full window is done no later than a part of one (one 700^2 28.2
+// and 26.1, 8 members up to 400^2 28.4 and 25.3, 4 up to 256^2 20.2 and 18.0).
+bool wide_lines(const lbm_instance* inst, int n, int order) {
+    constexpr long long kRound = 4 * 152 * 8;  // windows of one line
+    long long chunks = 0, windows = 0;
+    bool vec = true;
+    for (int i = 0; i < n; ++i) {
+        const int nx = inst[i].grid.nx, ny = inst[i].grid.ny;
+        if ((long long)nx * ny > kLines32Nodes) return true;
+        vec = vec && nx % 4 == 0;
+        lines32_window_use(nx, ny, order, chunks, windows);
+    }
+    return vec && (windows <= kRound || 10 * chunks >= 8 * 32 * windows);
 }
 
 // Offsets of the table region, sized for the largest block counts (the
@@ -92,7 +106,7 @@ Tables table_layout(const lbm_instance* inst, int n, int order, size_t base) {
     // each density map is sized for every instance in it (the double-float
     // windows are the shorter ones, so their count bounds both kinds)
     long long cs_max = 0, mu = 0, rho = 0, force = 0;
-    const bool wide = wide_lines(inst, n);
+    const bool wide = wide_lines(inst, n, order);
     for (int i = 0; i < n; ++i) {
         const int nx = inst[i].grid.nx, ny = inst[i].grid.ny;
         cs_max += cs_blocks_for(nx, ny, kRowChoices[0]);
@@ -142,7 +156,7 @@ bool instance_ok(const lbm_instance& in) {
 struct lbm_batch {
     int dev, n, order;
     bool mrt;  // MRT collision (Eq. 4) for every instance
-    bool wide;  // FP32 lines in full windows (a grid above kLines32Nodes)
+    bool wide;  // FP32 lines in full windows
     MrtRates rates;
     cudaStream_t stream, cap_stream, side_stream;  // the last two for graph capture only
     cudaEvent_t ev, tev[5], fork_ev, join_ev;
@@ -429,7 +443,7 @@ lbm_status lbm_batch_init(lbm_batch** out, const lbm_instance* inst, int32_t n,
     if (!b) return LBM_ENOMEM;
     b->n = n;
     b->order = opts->fd_order;
-    b->wide = wide_lines(inst, n);
+    b->wide = wide_lines(inst, n, b->order);
     b->line_nl = 8;
     b->mrt = opts->collision == LBM_COLLIDE_MRT;
     b->rates = MrtRates{opts->s_e, opts->s_eps, opts->s_q};

@@ -269,6 +269,9 @@ cudaError_t lines32_force(const float* mu, const float* rh, const float* dxr, co
 constexpr long long kLines32Nodes = 1LL << 19;
 cudaError_t lines32_wide(Dir32 x, Dir32 y, int nx, int ny, int order, bool second, DevState* st,
                          int bump, cudaStream_t s);
+// adds the windows (one line each) of a grid's density lines, and the chunks of them, of 32 a
+// window, that (line, chunk) pairs solve
+void lines32_window_use(int nx, int ny, int order, long long& chunks, long long& windows);
 // Batches: nl (8 or 16): blocks of 32 nl threads; wide: full windows, nl lines a block
 int lines32_batch_blocks(int nx, int ny, int order, bool second, int nl, bool wide);
 Lines32Inst lines32_batch_inst(const MixedLinesView& v, int order, bool second, int blk0, int nl,

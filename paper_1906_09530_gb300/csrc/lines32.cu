@@ -203,6 +203,14 @@ cudaError_t lines32_force(const float* mu, const float* rh, const float* dxr, co
 }
 
 // ---- batches ----
+void lines32_window_use(int nx, int ny, int order, long long& chunks, long long& windows) {
+    for (int axis = 0; axis < 2; ++axis) {
+        const Geo32 g = geometry(nx, ny, axis, order, true, false);
+        windows += (long long)g.nlines * g.nwin;
+        chunks += (long long)g.nlines * g.nwin * g.nch;
+    }
+}
+
 int lines32_batch_blocks(int nx, int ny, int order, bool second, int nl, bool wide) {
     Dir32 x{}, y{};
     lay_out(x, y, nx, ny, order, second, false, 32 * nl);

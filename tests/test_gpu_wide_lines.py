@@ -1,5 +1,4 @@
-"""FP32 lines in full windows (grids above 2^19 nodes, and every member of a batch that holds
-one): the bits of the chunked kernels on the same lines, and the oracle's derivatives where
+"""FP32 lines in full windows (grids above 2^19 nodes, and batches that want them): the bits of the chunked kernels on the same lines, and the oracle's derivatives where
 their geometry changes (rows that are not whole 16-byte pieces, a ragged last line group, one
 window on one axis and many on the other, mirrored lines)."""
 import numpy as np
@@ -23,11 +22,15 @@ def start(nx, ny, seed):
 
 @pytest.mark.parametrize("order", [4, 6])
 @pytest.mark.parametrize("nl", [8, 16])
-def test_batch_with_a_large_member(cuda, nl, order):
-    """Small members are solved in the large one's full windows here and by (line, chunk) pairs,
-    or in one cluster launch, alone: bit for bit the same."""
+@pytest.mark.parametrize("sizes", [
+    [(1001, 600), (8, 400), (37, 29), (128, 96), (300, 700)],  # a large member
+    [(64, 64), (8, 400), (300, 132)],                          # about one round of blocks
+    [(512, 504)] * 10,                                         # most chunks needed
+    [(256, 244)] * 20 + [(37, 29)]])                           # none of these: by pairs
+def test_batch_in_full_windows(cuda, sizes, nl, order):
+    """Batch members are solved in full windows or by (line, chunk) pairs as the whole batch
+    wants it, a lone grid as it wants, or in one cluster launch: bit for bit the same."""
     from paper_1906_09530_gb300 import Batch, Simulation
-    sizes = [(1001, 600), (8, 400), (37, 29), (128, 96), (300, 700)]
     kw = dict(T_r=0.6, kappa=0.1, tau=1.0, k=0.4)
     rhos = [start(nx, ny, 3 + i) for i, (nx, ny) in enumerate(sizes)]
     b = Batch([dict(nx=nx, ny=ny, **kw) for nx, ny in sizes], fd_order=order)
@@ -35,7 +38,7 @@ def test_batch_with_a_large_member(cuda, nl, order):
     for i, r in enumerate(rhos):
         b.set_fields(i, r)
     b.step(5)
-    for i, (nx, ny) in enumerate(sizes):
+    for i, (nx, ny) in list(enumerate(sizes))[:5]:
         s = Simulation(nx, ny, 0.6, 0.1, 1.0, 0.4, fd_order=order, precision="mixed")
         s.set_fields(rhos[i])
         s.step(5)
