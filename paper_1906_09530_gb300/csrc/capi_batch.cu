@@ -304,7 +304,7 @@ lbm_status enqueue_step(lbm_batch* b, cudaStream_t s, int from, cudaEvent_t* ev 
         CK(cudaStreamWaitEvent(side, b->fork_ev, 0));
     }
     CK(lines_df_batch_launch(at<Lines32Inst>(b, t.rho_df), at<int>(b, t.map_rho_df), t.nb_rho_df,
-                             b->order, t.smem_df, 1, sd));
+                             b->order, t.smem_df, t.nb_rho_f32 > 0, 1, sd));
     CK(f32_lines(b, true, 1, s));
     if (fork) {
         CK(cudaEventRecord(b->join_ev, side));

@@ -291,11 +291,11 @@ cudaError_t lines_df_plain(const float* uh, const float* ul, float* d1, float* d
 int lines_df_batch_blocks(int nx, int ny, int order);
 Lines32Inst lines_df_batch_inst(const MixedLinesView& v, int order, int blk0);
 // smem: the largest lines_df_batch_smem of the batch's instances.  (Short lines stage the most,
-// 79 KB a block, of which an SM holds two: 2 x 2048^2 batches at ratio 8e4 took 134 us for
-// their density lines with it, and take 106 with the 70 of their own.)
+// 79 KB a block, of which an SM holds two: 16 x 256^2 at ratio 8e4 took 77 us a step with it and
+// 69 with the 70 of their own.)  beside: FP32 density lines run at the same time.
 size_t lines_df_batch_smem(const Lines32Inst& d);
 cudaError_t lines_df_batch_launch(const Lines32Inst* d, const int* map, int nblocks, int order,
-                                  size_t smem, int bump, cudaStream_t s);
+                                  size_t smem, bool beside, int bump, cudaStream_t s);
 
 // Whole steps of a small periodic grid in one launch (FP32 density lines).
 struct SmallStep {

@@ -10,19 +10,17 @@
 // that is stored).  Both axes are staged by 16-byte copies, x-lines line by line, y-lines
 // row by row ([slot][lines]).
 //
-// What bounded it was instruction fetch: with the chunk in registers everything is unrolled
-// over 19 positions, about 100 operations each in double-float, for either axis (4.6 of 8
-// stalled warps waited for instructions).  So the chunk stays in shared memory, in place of
-// the staged window, and the loops are loops; the right-hand side's hi part, which the second
-// derivative starts from, goes to a plane of its own.  Density lines of 1000^2 at ratio 8e4:
-// 33.4 us unrolled in registers, 25.2 so (a step 54.5 -> 47.6).  What is left is uneven: 500
-// blocks, half of them crossing the interface, on 456 places.  Half groups (128 threads, one
-// wave) were no faster: 51.7 against 49.9 us a step.
-// Where a launch has more blocks than that, groups solved in FP32 run as in lines32.cuh, with
-// the chunk in registers (kPlaces): their unrolled code is a tenth of the double-float one's.
+// A chunk is in registers from its right-hand side to its result, unrolled over its 19
+// positions, 128 registers and two blocks an SM.  In launches of many blocks (kManyBlocks) the
+// double-float chunks stay in shared memory, in place of the staged window, as loops: 80
+// registers and three blocks, for the groups solved in FP32, which are most of a large grid.
+// With those as loops too, density lines of 1000^2 at ratio 8e4 took 25.2 us and a step 47.2;
+// so it is 44.6.  (The chunk in registers within one kernel templated over all number types:
+// 33.4 and 54.4.)
 #include <algorithm>
 #include <cfloat>
 #include <cmath>
+#include <type_traits>
 
 #include "df.cuh"
 #include "lines32.cuh"
@@ -57,8 +55,8 @@ __device__ __forceinline__ df join_df(const LineDF& k, const float* h, const flo
 
 // Shared memory: eight join arrays of kT floats, the two planes of the staged window (hi, lo),
 // whose places the first derivative takes, and the second derivative's plane.
-// REGS: groups solved in FP32 have their chunks in registers (see kPlaces).
-template <bool SIXTH, bool SECOND, bool REGS>
+// LOOPS: double-float chunks are loops in shared memory (see kManyBlocks).
+template <bool SIXTH, bool SECOND, bool LOOPS>
 __device__ __forceinline__ void block_df(const Dir32& d, const LineDF& k, int axis, int bid,
                                          float* sh) {
     const Geo32& g = d.g;
@@ -167,49 +165,74 @@ __device__ __forceinline__ void block_df(const Dir32& d, const LineDF& k, int ax
     // What the chunk needs of its neighbours, before they overwrite it: the window two
     // positions either side, and the first right-hand side there (FP32), in r; or the chunk
     // itself.
-    const bool regs = REGS && live && !wide, loops = live && !regs;
-    float r[kC], r2[REGS ? kC : 1];
-    if constexpr (REGS) {
-        if (regs) {
-            float w1, v2, w2;
-            l32::chunk_forward<SIXTH, SECOND, false>([&](int j) { return uh[j * ps]; }, k.f, r,
-                                                     r2, w1, v2, w2);
-            *eh = w1;
+    float r[kC], r2[kC], rl[LOOPS ? 1 : kC];
+    if (live && !wide) {
+        float w1, v2, w2;
+        l32::chunk_forward<SIXTH, SECOND, false>([&](int j) { return uh[j * ps]; }, k.f, r, r2, w1,
+                                                 v2, w2);
+        *eh = w1;
+        if (SECOND) {
+            *ev = v2;
+            *ew = w2;
+        }
+    } else if (live) {
+        if constexpr (!LOOPS) {
+            df w{0.0f, 0.0f};
+            float b[kC + 4];  // the right-hand side's hi part at -2 .. kC + 1
+#pragma unroll
+            for (int j = 0; j < kC; ++j) {
+                const df h = rhs(U(j - 2), U(j - 1), U(j + 1), U(j + 2));
+                b[j + 2] = h.hi;
+                w = fma_df(w, k.nlam, h);
+                r[j] = w.hi;
+                rl[j] = w.lo;
+            }
+            *eh = w.hi;
+            *el = w.lo;
             if (SECOND) {
-                *ev = v2;
+                b[0] = at_f(-2);
+                b[1] = at_f(-1);
+                b[kC + 2] = at_f(kC);
+                b[kC + 3] = at_f(kC + 1);
+                float v = 0.0f, w2 = 0.0f;
+#pragma unroll
+                for (int j = 0; j < kC; ++j) {
+                    float y = rn_mul(rn_sub(b[j + 3], b[j + 1]), k.f.c1);
+                    if (SIXTH) y = rn_fma(rn_sub(b[j + 4], b[j]), k.f.c2, y);
+                    v = rn_fma(v, k.f.nlam, y);
+                    r2[j] = w2 = rn_fma(w2, k.f.nlam, v);
+                }
+                *ev = v;
                 *ew = w2;
+            }
+        } else {
+            auto keep = [&](int i, df x) {
+                r[i] = x.hi;
+                r[i + 1] = x.lo;
+            };
+            keep(0, U(-2));
+            keep(2, U(-1));
+            keep(4, U(kC));
+            keep(6, U(kC + 1));
+            if (SECOND) {
+                r[8] = at_f(-2);
+                r[9] = at_f(-1);
+                r[10] = at_f(kC);
+                r[11] = at_f(kC + 1);
             }
         }
     }
-    if (loops) {
-        auto keep = [&](int i, df x) {
-            r[i] = x.hi;
-            r[i + 1] = x.lo;
-        };
-        keep(0, U(-2));
-        keep(2, U(-1));
-        keep(4, U(kC));
-        keep(6, U(kC + 1));
-        if (SECOND) {
-            r[8] = at_f(-2);
-            r[9] = at_f(-1);
-            r[10] = at_f(kC);
-            r[11] = at_f(kC + 1);
-        }
-    }
     const int after = nch - 1 - c;
-    __syncthreads();
-    // ---- forward ----
-    if (loops) {
-        df a{r[0], r[1]}, b{r[2], r[3]}, e = U(0), f = U(1);
-        const df z1{r[4], r[5]}, z2{r[6], r[7]};
-        if (REGS || wide) {
-            df w{0.0f, 0.0f};
+    // ---- forward, in place of the staged window ----
+    if constexpr (LOOPS) {
+        __syncthreads();
+        if (live && wide) {
+            df a{r[0], r[1]}, b{r[2], r[3]}, e = U(0), f = U(1), w{0.0f, 0.0f};
             float *ph = uh, *pl = ul, *p = q2;  // at position j
             auto step = [&](df h) {
-                const df r = rhs(a, b, f, h);
-                w = fma_df(w, k.nlam, r);
-                *p = r.hi;
+                const df x = rhs(a, b, f, h);
+                w = fma_df(w, k.nlam, x);
+                *p = x.hi;
                 *ph = w.hi;
                 *pl = w.lo;
                 p += ps;
@@ -223,73 +246,56 @@ __device__ __forceinline__ void block_df(const Dir32& d, const LineDF& k, int ax
 #pragma unroll 4
             for (int j = 0; j < kC - 3; ++j) step(df{ph[2 * ps], pl[2 * ps]});
             step(df{ph[2 * ps], pl[2 * ps]});
-            step(z1);
-            step(z2);
+            step(df{r[4], r[5]});
+            step(df{r[6], r[7]});
             *eh = w.hi;
             *el = w.lo;
-        } else {
-            float w = 0.0f;
-            float *ph = uh, *p = q2;
-            auto step = [&](float h) {
-                const float r = rhs_f(a.hi, b.hi, f.hi, h);
-                w = rn_fma(w, k.f.nlam, r);
-                *p = r;
-                *ph = w;
-                p += ps;
-                ph += ps;
-                a.hi = b.hi;
-                b.hi = e.hi;
-                e.hi = f.hi;
-                f.hi = h;
-            };
-#pragma unroll 4
-            for (int j = 0; j < kC - 3; ++j) step(ph[2 * ps]);
-            step(ph[2 * ps]);
-            step(z1.hi);
-            step(z2.hi);
-            *eh = w;
-        }
-        if (SECOND) {
-            float p = r[8], q = r[9], u = q2[0], x = q2[ps], v = 0.0f, w = 0.0f;
-            float* o = q2;
-            auto step = [&](float h) {
-                float y = rn_mul(rn_sub(x, q), k.f.c1);
-                if (SIXTH) y = rn_fma(rn_sub(h, p), k.f.c2, y);
-                v = rn_fma(v, k.f.nlam, y);
-                *o = w = rn_fma(w, k.f.nlam, v);
-                o += ps;
-                p = q;
-                q = u;
-                u = x;
-                x = h;
-            };
+            if (SECOND) {
+                float p = r[8], q = r[9], u = q2[0], x = q2[ps], v = 0.0f, w = 0.0f;
+                float* o = q2;
+                auto step = [&](float h) {
+                    float y = rn_mul(rn_sub(x, q), k.f.c1);
+                    if (SIXTH) y = rn_fma(rn_sub(h, p), k.f.c2, y);
+                    v = rn_fma(v, k.f.nlam, y);
+                    *o = w = rn_fma(w, k.f.nlam, v);
+                    o += ps;
+                    p = q;
+                    q = u;
+                    u = x;
+                    x = h;
+                };
 #pragma unroll 8
-            for (int j = 0; j < kC - 3; ++j) step(o[2 * ps]);
-            step(o[2 * ps]);
-            step(r[10]);
-            step(r[11]);
-            *ev = v;
-            *ew = w;
+                for (int j = 0; j < kC - 3; ++j) step(o[2 * ps]);
+                step(o[2 * ps]);
+                step(r[10]);
+                step(r[11]);
+                *ev = v;
+                *ew = w;
+            }
         }
     }
     __syncthreads();
     // ---- backward ----
-    if constexpr (REGS) {
-        if (regs) {
-            const float cf = l32::join1<0>(k.f, eh, js, c);
-            float cv = 0.0f, cw = 0.0f, y, z;
-            if (SECOND) l32::join2<0>(k.f, ev, ew, js, c, cv, cw);
-            l32::chunk_backward<SECOND>(k.f, cf, cv, cw, r, r2, *zh, y, z);
-            if (SECOND) {
-                *zv = y;
-                *zw = z;
-            }
+    if (live && !wide) {
+        const float cf = l32::join1<0>(k.f, eh, js, c);
+        float cv = 0.0f, cw = 0.0f, y, z;
+        if (SECOND) l32::join2<0>(k.f, ev, ew, js, c, cv, cw);
+        l32::chunk_backward<SECOND>(k.f, cf, cv, cw, r, r2, *zh, y, z);
+        if (SECOND) {
+            *zv = y;
+            *zw = z;
         }
-    }
-    if (loops) {
-        if (REGS || wide) {
-            const df cf = join_df(k, eh, el, js, c);
-            df z{0.0f, 0.0f};
+    } else if (live) {
+        const df cf = join_df(k, eh, el, js, c);
+        df z{0.0f, 0.0f};
+        if constexpr (!LOOPS) {
+#pragma unroll
+            for (int j = kC - 1; j >= 0; --j) {
+                z = fma_df(z, k.nlam, fma_df(cf, k.pw[j], df{r[j], rl[j]}));
+                r[j] = z.hi;
+                rl[j] = z.lo;
+            }
+        } else {
             float *ph = uh + (kC - 1) * ps, *pl = ul + (kC - 1) * ps;
 #pragma unroll 4
             for (int j = kC - 1; j >= 0; --j) {
@@ -299,47 +305,53 @@ __device__ __forceinline__ void block_df(const Dir32& d, const LineDF& k, int ax
                 ph -= ps;
                 pl -= ps;
             }
-            *zh = z.hi;
-            *zl = z.lo;
-        } else {
-            const float cf = l32::join1<0>(k.f, eh, js, c);
-            float z = 0.0f;
-#pragma unroll 5
-            for (int j = kC - 1; j >= 0; --j)
-                uh[j * ps] = z = rn_fma(z, k.f.nlam, rn_fma(cf, k.f.pw[j], uh[j * ps]));
-            *zh = z;
         }
+        *zh = z.hi;
+        *zl = z.lo;
         if (SECOND) {
-            float cv, cw, y = 0.0f, z = 0.0f;
+            float cv, cw, y = 0.0f, x = 0.0f;
             l32::join2<0>(k.f, ev, ew, js, c, cv, cw);
+            auto step = [&](int j, float& v) {
+                y = rn_fma(y, k.f.nlam, rn_fma(k.f.pw[j], rn_fma((float)(j + 1), cv, cw), v));
+                v = x = rn_fma(x, k.f.nlam, y);
+            };
+            if constexpr (!LOOPS) {
+#pragma unroll
+                for (int j = kC - 1; j >= 0; --j) step(j, r2[j]);
+            } else {
 #pragma unroll 5
-            for (int j = kC - 1; j >= 0; --j) {
-                const float r = rn_fma(k.f.pw[j], rn_fma((float)(j + 1), cv, cw), q2[j * ps]);
-                y = rn_fma(y, k.f.nlam, r);
-                q2[j * ps] = z = rn_fma(z, k.f.nlam, y);
+                for (int j = kC - 1; j >= 0; --j) step(j, q2[j * ps]);
             }
             *zv = y;
-            *zw = z;
+            *zw = x;
         }
     }
     __syncthreads();
     // ---- the state entering from after the chunk ----
-    if constexpr (REGS) {
-        if (regs) {
-            const float cb = l32::join1<0>(k.f, zh, -js, after);
-            float cy = 0.0f, cz = 0.0f;
-            if (SECOND) l32::join2<0>(k.f, zv, zw, -js, after, cy, cz);
-            l32::chunk_finish<SECOND>(k.f, cb, cy, cz, r, r2);
+    if (live && !wide) {
+        const float cb = l32::join1<0>(k.f, zh, -js, after);
+        float cy = 0.0f, cz = 0.0f;
+        if (SECOND) l32::join2<0>(k.f, zv, zw, -js, after, cy, cz);
+        l32::chunk_finish<SECOND>(k.f, cb, cy, cz, r, r2);
+#pragma unroll
+        for (int j = 0; j < kC; ++j) {
+            uh[j * ps] = r[j];
+            if (SECOND) q2[j * ps] = r2[j];
+        }
+    } else if (live) {
+        const df cb = join_df(k, zh, zl, -js, after);
+        float cy = 0.0f, cz = 0.0f;
+        if (SECOND) l32::join2<0>(k.f, zv, zw, -js, after, cy, cz);
+        auto second = [&](int j, float v) {
+            return rn_fma(k.f.pw[kC - 1 - j], rn_fma((float)(kC - j), cy, cz), v);
+        };
+        if constexpr (!LOOPS) {
 #pragma unroll
             for (int j = 0; j < kC; ++j) {
-                uh[j * ps] = r[j];
-                if (SECOND) q2[j * ps] = r2[j];
+                uh[j * ps] = df_round(fma_df(cb, k.pw[kC - 1 - j], df{r[j], rl[j]}));
+                if (SECOND) q2[j * ps] = second(j, r2[j]);
             }
-        }
-    }
-    if (loops) {
-        if (REGS || wide) {
-            const df cb = join_df(k, zh, zl, -js, after);
+        } else {
             float *ph = uh, *pl = ul;
 #pragma unroll 4
             for (int j = 0; j < kC; ++j) {
@@ -347,18 +359,10 @@ __device__ __forceinline__ void block_df(const Dir32& d, const LineDF& k, int ax
                 ph += ps;
                 pl += ps;
             }
-        } else {
-            const float cb = l32::join1<0>(k.f, zh, -js, after);
+            if (SECOND) {
 #pragma unroll 5
-            for (int j = 0; j < kC; ++j) uh[j * ps] = rn_fma(cb, k.f.pw[kC - 1 - j], uh[j * ps]);
-        }
-        if (SECOND) {
-            float cy, cz;
-            l32::join2<0>(k.f, zv, zw, -js, after, cy, cz);
-#pragma unroll 5
-            for (int j = 0; j < kC; ++j)
-                q2[j * ps] =
-                    rn_fma(k.f.pw[kC - 1 - j], rn_fma((float)(kC - j), cy, cz), q2[j * ps]);
+                for (int j = 0; j < kC; ++j) q2[j * ps] = second(j, q2[j * ps]);
+            }
         }
     }
     __syncthreads();
@@ -402,8 +406,8 @@ __device__ __forceinline__ void block_df(const Dir32& d, const LineDF& k, int ax
     }
 }
 
-template <bool SIXTH, bool SECOND, bool REGS>
-__global__ void __launch_bounds__(kT, 3)
+template <bool SIXTH, bool SECOND, bool LOOPS>
+__global__ void __launch_bounds__(kT, LOOPS ? 3 : 2)
     k_lines_df(Dir32 x, Dir32 y, const __grid_constant__ LineDF k, DevState* st, int bump,
                int nbx) {
     pdl_prologue();
@@ -412,11 +416,11 @@ __global__ void __launch_bounds__(kT, 3)
     const int nby = (int)gridDim.x - nbx, b = blockIdx.x;
     const bool is_y = b < nby;
     const Dir32& d = is_y ? y : x;
-    block_df<SIXTH, SECOND, REGS>(d, k, is_y, is_y ? b : b - nby, shdf);
+    block_df<SIXTH, SECOND, LOOPS>(d, k, is_y, is_y ? b : b - nby, shdf);
 }
 
-template <bool SIXTH, bool REGS>
-__global__ void __launch_bounds__(kT, 3)
+template <bool SIXTH, bool LOOPS>
+__global__ void __launch_bounds__(kT, LOOPS ? 3 : 2)
     k_lines_df_batch(const Lines32Inst* __restrict__ d, const int* __restrict__ map,
                      const __grid_constant__ LineDF k, int bump) {
     extern __shared__ __align__(16) float shdf[];
@@ -424,7 +428,7 @@ __global__ void __launch_bounds__(kT, 3)
     const int local = (int)blockIdx.x - D.blk0;
     if (bump && local == 0 && threadIdx.x == 0) D.st->t += 1;
     const bool is_y = local >= D.nbx;
-    block_df<SIXTH, true, REGS>(is_y ? D.y : D.x, k, is_y, is_y ? local - D.nbx : local, shdf);
+    block_df<SIXTH, true, LOOPS>(is_y ? D.y : D.x, k, is_y, is_y ? local - D.nbx : local, shdf);
 }
 
 // ---- host side ----
@@ -486,13 +490,10 @@ size_t most_smem_df() {
     }
     return most;
 }
-// More blocks than the chip has places (three an SM): then what counts is a block's work, and
-// groups solved in FP32 keep their chunks in registers, unrolled; below it is the latency,
-// which the fetch of that code adds to.  Steps at ratio 8e4 in loops and in registers:
-// 512^2 22.4 and 22.8 us, 1001 x 603 (404 blocks) 47.1 and 47.9, 3000 x 200 (525) 37.0 and
-// 35.4, 1500^2 96.5 and 93.3, 4096^2 572 and 536; the density alone, 2048^2 along x 26.8 and
-// 20.5 us.
-constexpr int kPlaces = 3 * 152;
+// Steps at ratio 8e4 with double-float chunks in registers and as loops: 512^2 20.4 and 22.5
+// us, 1000^2 44.6 and 47.0, 1500^2 91.7 and 94.2, a batch of 4 x 1024^2 (2048 blocks) 177.6 and
+// 185.1, 2 x 2048^2 (4096) 335.5 and 335.0, 4096^2 (8192) 553.9 and 537.6.
+constexpr int kManyBlocks = 15 * 2 * 152;
 cudaError_t run_df(const Dir32& x, const Dir32& y, int nbx, int nby, int order, DevState* st,
                    int bump, cudaStream_t s) {
     const size_t smem = std::max(smem_df(x.g), smem_df(y.g));
@@ -502,17 +503,15 @@ cudaError_t run_df(const Dir32& x, const Dir32& y, int nbx, int nby, int order, 
         return launch_pdl(kern, dim3(nbx + nby), dim3(kT), smem, s, x, y, constants_df(order), st,
                           bump, nbx);
     };
-    const bool regs = nbx + nby > kPlaces;
-    if (x.o2) {
-        if (regs) return order == 6 ? go(k_lines_df<true, true, true>)
-                                    : go(k_lines_df<false, true, true>);
-        return order == 6 ? go(k_lines_df<true, true, false>)
-                          : go(k_lines_df<false, true, false>);
-    }
-    if (regs) return order == 6 ? go(k_lines_df<true, false, true>)
-                                : go(k_lines_df<false, false, true>);
-    return order == 6 ? go(k_lines_df<true, false, false>)
-                      : go(k_lines_df<false, false, false>);
+    const bool loops = nbx + nby > kManyBlocks;
+    auto pick = [&](auto sixth, auto second) {
+        constexpr bool S = decltype(sixth)::value, D = decltype(second)::value;
+        return loops ? go(k_lines_df<S, D, true>) : go(k_lines_df<S, D, false>);
+    };
+    using T = std::true_type;
+    using F = std::false_type;
+    if (x.o2) return order == 6 ? pick(T(), T()) : pick(F(), T());
+    return order == 6 ? pick(T(), F()) : pick(F(), F());
 }
 
 }  // namespace
@@ -552,18 +551,17 @@ size_t lines_df_batch_smem(const Lines32Inst& d) {
 }
 
 cudaError_t lines_df_batch_launch(const Lines32Inst* d, const int* map, int nblocks, int order,
-                                  size_t smem, int bump, cudaStream_t s) {
+                                  size_t smem, bool beside, int bump, cudaStream_t s) {
     if (nblocks <= 0) return cudaSuccess;
-    // (two blocks an SM fit with the most any grid stages, and 256 of them are faster so: two
-    // 512^2 at ratio 8e4 35.6 us a step against 36.6)
-    if (nblocks <= 2 * 152) smem = most_smem_df();
     auto go = [&](auto kern) -> cudaError_t {
         const cudaError_t e = allow_smem(kern, most_smem_df());
         if (e != cudaSuccess) return e;
         kern<<<nblocks, kT, smem, s>>>(d, map, constants_df(order), bump);
         return cudaGetLastError();
     };
-    if (nblocks > kPlaces)
+    // (beside the FP32 lines of other members the registers are shared: 12 members of 64^2 to
+    // 512^2, 8 of them at ratios above 1e4, 59.8 us a step in registers and 56.8 as loops)
+    if (nblocks > kManyBlocks || beside)
         return order == 6 ? go(k_lines_df_batch<true, true>) : go(k_lines_df_batch<false, true>);
     return order == 6 ? go(k_lines_df_batch<true, false>) : go(k_lines_df_batch<false, false>);
 }
