@@ -46,9 +46,9 @@ Geo32 line32_geometry(int nx, int ny, int axis, int order, double eps1, double e
                       bool walls_y) {
     const double lam = lambda(order);
     int h1 = 1, h2 = 0;
-    while (std::pow(lam, h1) >= eps1) ++h1;
+    for (double p = lam; p >= eps1; p *= lam) ++h1;
     if (eps2 > 0.0)
-        while ((h2 + 1) * std::pow(lam, h2) >= eps2) ++h2;
+        for (double p = 1.0; (h2 + 1) * p >= eps2; p *= lam) ++h2;
     Geo32 g;
     g.n = axis == 0 ? nx : ny;
     g.nlines = axis == 0 ? ny : nx;
