@@ -38,8 +38,9 @@ constexpr int kPw = 57;       // powers (-lam)^0 .. (-lam)^56
 constexpr int kHalo = 96;     // two solves of kPw - 9 positions: lam^48 < 1e-20
 constexpr int kLWhole = 1600; // longest line solved whole
 constexpr int kLOwn = 1100;   // most positions a window of a longer one owns
-// ... and of a launch of few lines (see geo64)
-constexpr int kLFew = kLOwn + 2 * kHalo;
+// in launches of few lines (see geo64): most positions a window owns where there is room for
+// more of them, and the longest lines solved whole, with such room and without
+constexpr int kLOwnRoom = 512, kLRoom = 1024, kLFew = kLOwn + 2 * kHalo;
 constexpr int kSMs = 152;
 
 struct Geo {
@@ -318,11 +319,13 @@ Geo geo64(int nx, int ny, int axis, bool walls_y, int lines_all) {
     }
     g.nwin = 1;
     // Where an SM has one or two lines a line's length is the time, and windows are shorter:
-    // 7, 200 and 300 stand-alone lines of 1500, both derivatives, 37.1, 41.2 and 41.2 us whole
-    // and 24.9, 26.8 and 35.0 in two windows; of 1600 39.1, 43.2 and 43.1, and 32.9, 33.0 and
-    // 41.2.  (From 1293 on: then a window is shorter than the longest of a longer line.)
-    if (g.L > (lines_all <= 2 * kSMs ? kLFew : kLWhole)) {
-        g.nwin = (g.n + kLOwn - 1) / kLOwn;
+    // 100 and 200 stand-alone lines of 1500, both derivatives, 37.1 and 41.2 us whole and 28.9
+    // and 26.8 in two windows (300: 41.2 and 35.0, but steps of 1600 x 304 205 and 207); where
+    // no SM gets two, short ones: 7 of 1500 37.2 and 20.7.
+    const int room = (g.n + kLOwnRoom - 1) / kLOwnRoom;
+    const bool has_room = (long long)lines_all * room <= kSMs;
+    if (g.L > (has_room ? kLRoom : 2 * lines_all <= 3 * kSMs ? kLFew : kLWhole)) {
+        g.nwin = has_room ? room : (g.n + kLOwn - 1) / kLOwn;
         g.own = ((g.n + g.nwin - 1) / g.nwin + 3) / 4 * 4;
         g.H = kHalo;
         g.L = g.own + 2 * kHalo;

@@ -88,10 +88,11 @@ def test_chemical_potential_over_twelve_decades(cuda):
         sim.close()
 
 
-# 304 lines are the most that count as few, 1292 positions the longest they are solved whole
+# 228 lines are the most that count as few, solved whole up to 1292 positions; 76 and 50 have
+# room for two and three windows of 512, from 1025 positions on
 @pytest.mark.parametrize("axis", [0, 1])
-@pytest.mark.parametrize("lines", [304, 305])
-@pytest.mark.parametrize("n", [1292, 1293, 1599])
+@pytest.mark.parametrize("n,lines", [(n, m) for n in (1292, 1293, 1599) for m in (228, 229)] +
+                         [(1024, 76), (1025, 50), (1025, 51), (1536, 50), (1537, 50), (3001, 8)])
 def test_few_lines_in_windows(cuda, n, lines, axis):
     """Tolerance 1e-13 of the largest derivative, as for single lines."""
     from oracle import cfd_alpha, cfd_line
