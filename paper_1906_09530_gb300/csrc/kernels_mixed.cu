@@ -117,7 +117,7 @@ __device__ __forceinline__ void cs_mixed_body(const CsArgs& a, int wid) {
         if constexpr (MRT)
             ok &= collide_mrt<float>(out, raw[9], raw[10], omega, FLT_MAX, a.se, a.seps, a.sq);
         else
-            ok &= collide_pairs<float>(out, raw[9], raw[10], omega, FLT_MAX);
+            ok &= collide_pairs(out, raw[9], raw[10], omega, FLT_MAX);
     };
     float A[9], B[9], C[9];
     fetch(y0 - 1);
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(kRingT) k_cs_mixed_ring(CsArgs a) {
             if constexpr (MRT)
                 ok &= collide_mrt<float>(f, fx, fy, a.omega, FLT_MAX, a.se, a.seps, a.sq);
             else
-                ok &= collide_pairs<float>(f, fx, fy, a.omega, FLT_MAX);
+                ok &= collide_pairs(f, fx, fy, a.omega, FLT_MAX);
 #pragma unroll
             for (int i = 0; i < 9; ++i) post[r % 3][i][t] = f[i];
         }

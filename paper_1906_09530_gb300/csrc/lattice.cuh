@@ -1,6 +1,6 @@
-// lattice.cuh -- D2Q9 velocity set (Sec. 2) and the BGK collision with
-// exact-difference forcing (Eqs. 1, 2, 5), shared by the FP64 and FP32
-// collide-stream kernels.
+// lattice.cuh -- D2Q9 velocity set (Sec. 2); the BGK collision of the FP32 collide-stream
+// kernels (Eqs. 1, 2, 5; the FP64 kernel's is in kernels_lbm.cu) and the MRT collision (Eq. 4)
+// of both, with exact-difference forcing.
 #pragma once
 
 namespace cplbm {
@@ -52,43 +52,35 @@ __device__ __forceinline__ double rn_div(double a, double b) { return __ddiv_rn(
 // v = u + F/rho.  Opposite directions share the even terms and flip the odd
 // one, so each of the four pairs is evaluated once.  Returns false when rho is
 // not a finite positive number.
-template <typename T>
-__device__ __forceinline__ bool collide_pairs(T f[9], T Fx, T Fy, T omega, T big) {
-    const T rho = rn_add(rn_add(rn_add(rn_add(f[0], f[1]), rn_add(f[2], f[3])),
+__device__ __forceinline__ bool collide_pairs(float f[9], float Fx, float Fy, float omega,
+                                              float big) {
+    const float rho = rn_add(rn_add(rn_add(rn_add(f[0], f[1]), rn_add(f[2], f[3])),
                                 rn_add(rn_add(f[4], f[5]), rn_add(f[6], f[7]))),
                          f[8]);
-    const T d57 = rn_sub(f[5], f[7]);
-    const T jx = rn_add(rn_sub(f[1], f[3]), rn_add(d57, rn_sub(f[8], f[6])));
-    const T jy = rn_add(rn_sub(f[2], f[4]), rn_add(d57, rn_sub(f[6], f[8])));
-    const T inv = rn_div(T(1), rho);
-    const T ux = rn_mul(jx, inv), uy = rn_mul(jy, inv);
-    const T vx = rn_fma(Fx, inv, ux), vy = rn_fma(Fy, inv, uy);
-    const T keep = rn_sub(T(1), omega);
-    const T uu = rn_fma(ux, ux, rn_mul(uy, uy));
-    const T vv = rn_fma(vx, vx, rn_mul(vy, vy));
-    const T base = rn_fma(T(-1.5), rn_fma(-keep, uu, vv), omega);
-    T r0, r1, r2;
-    if constexpr (sizeof(T) == 4) {
-        // In FP32, 4/9, 1/9 and 1/36 share one mantissa and all round up by 7.5e-9.  Used as
-        // constants, that bias adds mass every step and sets the populations' pressure apart
-        // from the force's c_s^2 rho, which shifts the dilute gas at high density ratios.
-        // Instead rho w_i = 16, 4, 1 x rho/36, with rho/36 = rho (hi + lo) rounded once.
-        constexpr float hi = 1.0f / 36.0f;
-        constexpr float lo = (float)(1.0 / 36.0 - (double)hi);
-        r2 = rn_fma(rho, T(hi), rn_mul(rho, T(lo)));
-        r1 = rn_mul(r2, T(4));
-        r0 = rn_mul(r2, T(16));
-    } else {
-        r0 = rn_mul(rho, T(4.0 / 9.0));
-        r1 = rn_mul(rho, T(1.0 / 9.0));
-        r2 = rn_mul(rho, T(1.0 / 36.0));
-    }
+    const float d57 = rn_sub(f[5], f[7]);
+    const float jx = rn_add(rn_sub(f[1], f[3]), rn_add(d57, rn_sub(f[8], f[6])));
+    const float jy = rn_add(rn_sub(f[2], f[4]), rn_add(d57, rn_sub(f[6], f[8])));
+    const float inv = rn_div(1.0f, rho);
+    const float ux = rn_mul(jx, inv), uy = rn_mul(jy, inv);
+    const float vx = rn_fma(Fx, inv, ux), vy = rn_fma(Fy, inv, uy);
+    const float keep = rn_sub(1.0f, omega);
+    const float uu = rn_fma(ux, ux, rn_mul(uy, uy));
+    const float vv = rn_fma(vx, vx, rn_mul(vy, vy));
+    const float base = rn_fma(-1.5f, rn_fma(-keep, uu, vv), omega);
+    // In FP32, 4/9, 1/9 and 1/36 share one mantissa and all round up by 7.5e-9.  Used as
+    // constants, that bias adds mass every step and sets the populations' pressure apart
+    // from the force's c_s^2 rho, which shifts the dilute gas at high density ratios.
+    // Instead rho w_i = 16, 4, 1 x rho/36, with rho/36 = rho (hi + lo) rounded once.
+    constexpr float hi = 1.0f / 36.0f;
+    constexpr float lo = (float)(1.0 / 36.0 - (double)hi);
+    const float r2 = rn_fma(rho, hi, rn_mul(rho, lo));
+    const float r1 = rn_mul(r2, 4.0f), r0 = rn_mul(r2, 16.0f);
     f[0] = rn_fma(keep, f[0], rn_mul(r0, base));
-    auto pair = [&](int i, int j, T w, T eu, T ev) {
-        const T s = rn_fma(-keep, eu, ev);
-        const T q = rn_fma(ev, ev, -rn_mul(keep, rn_mul(eu, eu)));
-        const T A = rn_mul(w, rn_fma(T(4.5), q, base));
-        const T B = rn_mul(w, rn_mul(T(3), s));
+    auto pair = [&](int i, int j, float w, float eu, float ev) {
+        const float s = rn_fma(-keep, eu, ev);
+        const float q = rn_fma(ev, ev, -rn_mul(keep, rn_mul(eu, eu)));
+        const float A = rn_mul(w, rn_fma(4.5f, q, base));
+        const float B = rn_mul(w, rn_mul(3.0f, s));
         f[i] = rn_fma(keep, f[i], rn_add(A, B));
         f[j] = rn_fma(keep, f[j], rn_sub(A, B));
     };
@@ -96,7 +88,7 @@ __device__ __forceinline__ bool collide_pairs(T f[9], T Fx, T Fy, T omega, T big
     pair(2, 4, r1, uy, vy);
     pair(5, 7, r2, rn_add(ux, uy), rn_add(vx, vy));
     pair(6, 8, r2, rn_sub(uy, ux), rn_sub(vy, vx));
-    return rho > T(0) && rho < big;
+    return rho > 0.0f && rho < big;
 }
 
 // MRT collision of Eq. 4 with exact-difference forcing (Eq. 5), in moment space:

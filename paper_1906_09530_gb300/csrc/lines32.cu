@@ -89,9 +89,9 @@ void divide(Geo32& g, int axis, int T) {
 }
 
 // Threads a block: 256 (8 full windows or 8 columns, 32-byte row pieces).  Measured steps
-// with 64 / 128 / 256 / 512: 512^2 23.3 / 19.1 / 17.4 / 19.7 us, 128^2 16.8 / 15.6 / 15.6 /
-// 17.5.  Rows that are not whole 16-byte pieces are staged four bytes at a time, which
-// wants more blocks: 333 x 277 20.2 / 19.5 / 20.5 / 23.5.
+// with 64 / 128 / 256 / 512: 512^2 22.5 / 17.7 / 16.0 / 18.2 us, 128^2 12.9 / 11.4 / 11.6 /
+// 13.5.  Rows that are not whole 16-byte pieces are staged four bytes at a time, which
+// wants more blocks: 333 x 277 18.0 / 17.2 / 18.1 / 21.2.
 constexpr int kLoneT = 256;
 int pick_threads(int nx) { return nx % 4 == 0 ? kLoneT : 128; }
 
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(kSmallT, 1) k_small(const __grid_constant__ Sm
             if constexpr (MRT)
                 bad_rho |= !collide_mrt<float>(f, fx, fy, a.omega, FLT_MAX, a.se, a.seps, a.sq);
             else
-                bad_rho |= !collide_pairs<float>(f, fx, fy, a.omega, FLT_MAX);
+                bad_rho |= !collide_pairs(f, fx, fy, a.omega, FLT_MAX);
 #pragma unroll
             for (int q = 0; q < 9; ++q) sh32[q * nh + n] = f[q];
         }

@@ -24,9 +24,9 @@
 // x-lines are staged in shared memory in 16-byte pieces and written back through it;
 // y-lines need no staging: the threads of a warp are adjacent columns of one chunk, so each
 // reads its 23 (27) rows straight into registers and writes its rows, coalesced as they are.
-// Against one warp a line with all 32 chunks and staged y-windows: steps of 128^2 17.6 ->
-// 15.6 us, 512^2 20.1 -> 17.4, 333 x 277 26.4 -> 19.5.  On large grids, where every chunk is
-// needed and rows come from DRAM, those windows (lines32_wide.cu) stay ahead.
+// Against full windows for every line (lines32_wide.cu): steps of 128^2 12.2 -> 11.6 us, 512^2
+// 17.2 -> 16.0, 333 x 277 20.8 -> 17.2.  On large grids, where every chunk is needed and rows
+// come from DRAM, those windows stay ahead.
 #pragma once
 
 #include "cplbm_internal.cuh"

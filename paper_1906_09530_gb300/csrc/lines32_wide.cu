@@ -1,8 +1,8 @@
 // lines32_wide.cu -- FP32 line solves (Eqs. 37-39) of large grids, with the fused force
 // (Eq. 12) epilogue: full windows of 32 chunks, NL lines (NL warps) a block.  Windows,
 // chunks, joins and rounding are those of lines32.cuh, so both give the same bits; on grids
-// above kLines32Nodes these are faster (1024^2 35.4 us a step against 37.1, 4096^2 471
-// against 499).
+// above kLines32Nodes these are faster (1024^2 33.9 us a step against 36.6, 4096^2 454
+// against 487), and in batches by the rule in capi_batch.cu.
 //
 //   x-lines  warp w owns line w and lane l chunk l, staged in 16-byte pieces line by line;
 //            chunk states are joined by warp shuffles.

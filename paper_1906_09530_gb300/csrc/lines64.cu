@@ -20,8 +20,8 @@
 //
 // Lines longer than kLWhole are cut into overlapping windows (whole, a line of 4096 leaves four
 // warps an SM: a 4096^2 step took 8.5 ms, in windows 5.3; on 1536^2 it is the same either
-// way), and lines between walls (the
-// even extension of period 2 n, Sec. 5.5) of more than 2 kHalo positions are one window
+// way), shorter ones too where a launch has few of them (geo64), and lines between walls
+// (the even extension of period 2 n, Sec. 5.5) of more than 2 kHalo positions are one window
 // with a mirrored halo.  A window is solved as if it were periodic: what that gets wrong at
 // its ends has decayed by the owned positions.
 #include "cplbm_internal.cuh"
