@@ -559,9 +559,11 @@ cudaError_t lines_df_batch_launch(const Lines32Inst* d, const int* map, int nblo
         kern<<<nblocks, kT, smem, s>>>(d, map, constants_df(order), bump);
         return cudaGetLastError();
     };
-    // (beside the FP32 lines of other members the registers are shared: 12 members of 64^2 to
-    // 512^2, 8 of them at ratios above 1e4, 59.8 us a step in registers and 56.8 as loops)
-    if (nblocks > kManyBlocks || beside)
+    // (beside the FP32 lines of other members the registers are shared: 24 members, 232 of the
+    // blocks these, 83.0 us a step in registers and 81.3 as loops; 17 members, 34 of the blocks,
+    // 35.7 and 37.5; 8, 164, 36.6 and 39.1)
+    constexpr int kManyBeside = 200;
+    if (nblocks > (beside ? kManyBeside : kManyBlocks))
         return order == 6 ? go(k_lines_df_batch<true, true>) : go(k_lines_df_batch<false, true>);
     return order == 6 ? go(k_lines_df_batch<true, false>) : go(k_lines_df_batch<false, false>);
 }
